@@ -439,8 +439,9 @@ def roofline(prof, info, steps, clk, pk, pk_kind, workload, nrhs=1):
         peak = SM_COUNT * 128 * 2 * clk_hz
         out.update({"bound": "alu", "pipe": "FP32 (FMA)", "unit": "TFLOP/s", "units_per_step": units,
                     "peak_basis": basis % "128 FMA lanes/clk x 2 FLOP"})
-    elif "k_lag_gemm" in name:
-        variant = 2 if "_ts" in name else 1 if "_tc" in name else 0
+    elif "k_lag_gemm" in name or "k_lag_pairs" in name:
+        f16 = "k_lag_pairs" in name
+        variant = 1 if f16 else 2 if "_ts" in name else 1 if "_tc" in name else 0
 
         def lag_units(l):
             # (flops, transfer variant) of a Lagrange level: a dense r x r (x kfac) GEMM per
@@ -448,13 +449,13 @@ def roofline(prof, info, steps, clk, pk, pk_kind, workload, nrhs=1):
             r, rk = info["r1"][l] ** 3, info["aca_rank"][l]
             if rk > 0:
                 return 4.0 * r * info["aca_pair_terms"][l], info["tune_tc"][l]
-            return 2.0 * kfac * r * r * info["n_adm"][l], info["tune_tc"][l]
+            return (8.0 if helm else 2.0) * kfac * r * r * nrhs * info["n_adm"][l], info["tune_tc"][l]
 
         units = sum(u for l in range(22) if info["mode"][l] == 1 for u, v in [lag_units(l)] if v == variant)
-        peak = pk.get("bf16_tflops", 1900.0) * 1e12 * (1.1 / 2.25)
-        out.update({"bound": "tensor", "pipe": "TF32", "unit": "TFLOP/s", "units_per_step": units,
-                    "peak_basis": "measured BF16 %.1f TFLOP/s x 1.1/2.25 (%s peaks file)"
-                                  % (pk.get("bf16_tflops", 1900.0), pk_kind)})
+        peak = pk.get("bf16_tflops", 1900.0) * 1e12 * (1.0 if f16 else 1.1 / 2.25)
+        out.update({"bound": "tensor", "pipe": "F16" if f16 else "TF32", "unit": "TFLOP/s", "units_per_step": units,
+                    "peak_basis": "measured BF16 %.1f TFLOP/s%s (%s peaks file)"
+                                  % (pk.get("bf16_tflops", 1900.0), "" if f16 else " x 1.1/2.25", pk_kind)})
     elif name == "k_lag_aca":
         # ACA of the transfer matrices: per term, the rank-one update of the r x r residual
         # with its squared norm (3 FP64 operations per entry), plus filling the matrix

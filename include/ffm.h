@@ -102,10 +102,11 @@ typedef struct {
     const char *autotune_cache; /* NULL, or a file written by ffm_autotune: the plan takes the
                                    picks stored for its sizes (single right-hand side picks;
                                    several-RHS picks from 64, else 8 RHS), timing nothing */
-    int lagrange_transfer;      /* Laplace Lagrange levels' transfer: 0 default (tcgen05 per
+    int lagrange_transfer;      /* Lagrange levels' transfer: 0 default (tcgen05 per
                                    translation, or ffm_autotune's pick), 1 CUDA-core GEMM per
                                    translation, 2 tcgen05 per translation, 3 tcgen05
-                                   target-stationary (r <= 64) */
+                                   target-stationary (FFM_LAPLACE, r <= 64; per translation
+                                   elsewhere) */
     const void *normals;        /* FFM_LAPLACE_DL: N_Y x 3 row-major source normals (any
                                    length; the kernel is linear in n), host or device; copied */
     ffm_dtype normals_dtype;    /* FFM_F32 or FFM_F64 */

@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libffm_gb300.so")
 SOURCES = ["tree.cu", "tables.cu", "farfield.cu", "nearfield.cu", "ffm_api.cu", "noalloc.cu", "autotune.cu",
-           "nufft.cu", "bem.cu"]
+           "nufft.cu", "bem.cu", "transfer.cu"]
 ARCH = os.environ.get("FFM_CUDA_ARCH", "103a")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_%s,code=sm_%s" % (ARCH, ARCH), "-O3", "-lineinfo", "-std=c++17",
@@ -34,7 +34,7 @@ def _stale(obj, src):
     if not os.path.exists(obj):
         return True
     t = os.path.getmtime(obj)
-    deps = [src, os.path.join(CSRC, "ffm_internal.cuh"), os.path.join(HERE, "..", "include", "ffm.h"), __file__]
+    deps = [src, *(os.path.join(CSRC, h) for h in ("ffm_internal.cuh", "dfloat.cuh", "tc_common.cuh")), os.path.join(HERE, "..", "include", "ffm.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

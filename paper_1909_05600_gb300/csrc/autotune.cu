@@ -170,8 +170,10 @@ void apply_cached_picks(ffm_plan_s *p, const char *cache_path, cudaStream_t s) {
         if (F.n_adm == 0) continue;
         int a, b, c;
         if (F.mode == 1) {
-            if (cache.get(lag_key(p, l, dev, 1), v) && parse_lag(v, a)) {
+            if (p->kind != FFM_HELMHOLTZ && !F.aca && cache.get(lag_key(p, l, dev, 1), v) && parse_lag(v, a)) {
                 if (a == 2) prepare_target_stationary(p, l, s);
+                if (a != 2 || !F.ts_ok) build_translation_groups(p, l, s);
+                if (a == 0) build_group_tiles(p, l, s);
                 if (a != 2 || F.ts_ok) F.tune_tc = a;
             }
         } else if (F.prec != FFM_PREC_F64) {
@@ -244,10 +246,8 @@ void autotune(ffm_plan_s *p, int nrhs, const char *cache_path, cudaStream_t s) {
         };
         std::string v;
         if (F.mode == 1) {
-            int r = F.r1 * F.r1 * F.r1;
-            if (!helm && !F.aca) build_translation_groups(p, l, s);  // the per-translation candidates
-            bool tc_ok = !helm && F.tc_tiles > 0 && !F.aca;
-            if (!tc_ok) continue;
+            if (helm || F.aca) continue;
+            build_group_tiles(p, l, s);  // the per-translation candidates
             std::string key = lag_key(p, l, dev, rhs_bucket(nrhs));
             int pick = -1;
             bool cached = cache.get(key, v) && parse_lag(v, pick);

@@ -17,6 +17,7 @@
 
 #include "ffm_internal.cuh"
 #include "dfloat.cuh"
+#include "tc_common.cuh"
 
 namespace ffm {
 
@@ -375,54 +376,14 @@ __global__ void __launch_bounds__(LG_T) k_lag_gemm(const uint32_t *__restrict__ 
 // bounded wait that raises a device error flag instead of hanging.
 constexpr int TC_M = 128;
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 __device__ __forceinline__ uint32_t kmajor_off(int row, int k, int KT) {
     return (uint32_t)((((row >> 3) * (KT >> 2) + (k >> 2)) << 7) + ((row & 7) << 4) + ((k & 3) << 2));
-}
-
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
 
 __device__ __forceinline__ void tf32_split(float x, float &hi, float &lo) {
     hi = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
     lo = x - hi;
 }
-
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-
-// bulk copy global -> shared, completion counted in bytes on an mbarrier
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-
-// Bounded wait for the completion of phase `parity` of an mbarrier: at most `tries`
-// try_wait attempts (none for tries <= 0); false if it gave up.
-// With `abort` (the launch's device error flag), the wait also gives up once another CTA has
-// raised the flag (checked every 1024 attempts), so one failure does not make every later
-// CTA spend its whole limit.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int tries, const int *abort = nullptr) {
-    uint32_t done = 0;
-    for (int it = 0; it < tries && !done; ++it) {
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(smem_addr(bar)), "r"(parity));
-        if (!done && abort && (it & 1023) == 1023 && *reinterpret_cast<const volatile int *>(abort)) break;
-    }
-    return done != 0;
-}
-
-// After a wait has given up, a kernel still waits for the tensor-core operations it has
-// already committed before it releases TMEM and exits (they read its shared memory and
-// write its TMEM columns); that wait is bounded too, by this larger count.
-constexpr int DRAIN_TRIES = 1 << 28;
 
 __device__ __forceinline__ void store_split(float *hi, float *lo, uint32_t o, float4 x) {
     float4 h, l;
@@ -1334,12 +1295,18 @@ void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *a
     void *ut = tmp.raw(ub);
     void *vt = tmp.raw(vb);
     dim3 gg((unsigned)F.n_tiles, cdiv(r, LG_BM), nrhs);
+    // the transfer by translation runs on the tensor cores (transfer.cu) unless the CUDA-core GEMM is
+    // forced or picked by the autotuner
+    const bool use_tc = F.tune_tc != 0 && F.Th;
     FFM_CUDA(cudaMemsetAsync(ut, 0, ub, s));
     FFM_CUDA(cudaMemsetAsync(vt, 0, vb, s));
     if (cplx) {
         lagrange_points_r1<true>(p, F, AY, cb, true, q, nrhs, ut, s);
-        FFM_LAUNCH(k_lag_gemm<true>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, F.T, r, rk,
-                   nrhs, (const float2 *)ut, (float2 *)vt);
+        if (use_tc)
+            lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
+        else
+            FFM_LAUNCH(k_lag_gemm<true>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, F.T, r, rk,
+                       nrhs, (const float2 *)ut, (float2 *)vt);
         lagrange_points_r1<true>(p, F, AX, cb, false, vt, nrhs, accf, s);
     } else {
         if (p->kind == FFM_LAPLACE_DL)
@@ -1378,18 +1345,14 @@ void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *a
         const int ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
         const size_t tblk = (size_t)F.n_trans * r * rk;
         const size_t vblk = (size_t)r * nrhs * p->bx[l].nb;
-        float *upad = nullptr, *uts = nullptr;
-        const bool use_tc = !(F.ts_ok && F.Tsp && F.tune_tc == 2) && F.tc_tiles > 0 && F.tune_tc != 0 && F.Tsh;
-        if (use_tc) {
-            // u~ with rows padded to rkp floats (whole, aligned 16-byte segments for cp.async)
-            int64_t nrow = (int64_t)p->by[l].nb * nrhs;
-            upad = tmp.get<float>((size_t)nrow * F.rkp);
-            split_pad((const float *)ut, 1, (int)nrow, rk, (int)nrow, F.rkp, upad, nullptr, s);
-        }
+        float *uts = nullptr;
+        const bool use_ts = F.ts_ok && F.Tsp && F.tune_tc == 2;
+        // all components in one launch
+        if (!use_ts && use_tc) lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
         for (int d = 0; d < ncomp; ++d) {
             const float *Td = F.T + d * tblk;
             float *vtd = (float *)vt + d * vblk;
-        if (F.ts_ok && F.Tsp && F.tune_tc == 2) {
+        if (use_ts) {
             FFM_CUDA(cudaFuncSetAttribute(k_lag_gemm_ts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS_SMEM));
             const float *u64 = (const float *)ut;
             if (r < 64) {  // rows of 64 floats, once for all components
@@ -1404,19 +1367,12 @@ void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *a
             dim3 gts(cdiv(F.n_tgt, TS_M), nrhs);
             FFM_LAUNCH(k_lag_gemm_ts, gts, TS_NP + 32, TS_SMEM, s, F.tgt, F.n_tgt, F.adm_off, F.adm_src, F.adm_t,
                        F.n_trans, F.Tsp, r, nrhs, u64, vtd, p->dev_err, p->wait_tries);
-        } else if (use_tc) {
-            // tensor cores: 256-pair tiles, K chunks of 16 source nodes, row blocks of <= 224
-            const int rkp = F.rkp;
-            const size_t dsz = (size_t)F.n_trans * npad * rkp;
-            tc_transfer(F, F.bt_src, F.bt_tgt, F.Tsh + d * dsz, (int64_t)npad * rkp, r, rkp, r, nrhs, upad, vtd,
-                        p->dev_err, p->wait_tries, s);
-        } else {
+        } else if (!use_tc) {
             FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, Td, r,
                        rk, nrhs, (const float *)ut, vtd);
         }
             lagrange_points_r1<false>(p, F, AX, cb, false, vtd, nrhs, accf + (size_t)d * nrhs * p->nx, s);
         }
-        if (upad) tmp.drop(upad);
         if (uts) tmp.drop(uts);
     }
 }

@@ -160,7 +160,7 @@ struct FarLevel {
     uint32_t *bt_off = nullptr;     // n_trans+1: pairs grouped by translation (CSR)
     uint32_t *bt_src = nullptr;     // n_adm source box per pair, grouped by translation
     uint32_t *bt_tgt = nullptr;     // n_adm target box per pair, grouped by translation
-    int64_t n_tiles = 0;            // GEMM column tiles over all translations
+    int64_t n_tiles = 0;            // CUDA-core GEMM column tiles over all translations
     uint32_t *tile_t = nullptr;     // per tile: translation
     uint32_t *tile_p0 = nullptr;    // per tile: first pair (index into bt_*)
     int64_t n_src_chunks = 0, n_tgt_chunks = 0;
@@ -170,8 +170,12 @@ struct FarLevel {
                                     // partners sorted by translation within each target)
     float *Tsp = nullptr;           // target-stationary transfer (r <= 64): T_t split into TF32
                                     // hi and lo, 64 x 64 each, in the K-major core-matrix layout
-    float *Tsh = nullptr;           // tensor-core transfer: T_t padded to npad rows of rkp floats
-    int rkp = 0;                    // (per component block for the gradient)
+    // tensor-core transfer by translation: f16 hi / lo images of T_t (transfer.cu), h_bpc blocks of
+    // h_nb rows per component, h_nk chunks of 32 columns, 1 / scale
+    uint16_t *Th = nullptr;
+    int h_bpc = 0, h_nb = 0, h_nk = 0;
+    float h_inv = 0;
+    int rkp = 0;                    // ACA stage 1's K extent on the tensor cores
     // ACA of T (eq. 11, Laplace single layer with ffm_opts.aca_eps): T_t ~ A_t B_t^T with
     // rank_t <= aca_rank (the level's largest); the transfer runs as w_p = B_t^T u~_src(p)
     // per pair, then v~_tgt(p) += A_t w_p.  B^T as [t][aca_rp][K] and A as [t][rows][aca_rp]
@@ -181,7 +185,7 @@ struct FarLevel {
     int aca_rank = 0, aca_rp = 0;
     float *Aca = nullptr, *Bca = nullptr;
     uint32_t *pair_id = nullptr;    // n_adm: p -> p (pair-indexed rows of w)
-    int64_t tc_tiles = 0;           // 256-pair tiles for the tensor-core transfer
+    int64_t tc_tiles = 0;           // 256-pair tiles for the ACA factors on the tensor cores
     uint32_t *tc_tile_t = nullptr;
     uint32_t *tc_tile_p0 = nullptr;
     // plane waves: arithmetic (FFM_PREC_F32 / _F32C with FP32 tables, FFM_PREC_F64 with
@@ -271,9 +275,13 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
 // tree.cu: partners sorted by translation and T pre-split for the target-stationary
 // transfer of Lagrange level l (on demand); tables.cu: the T split
 void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s);
-// tree.cu: pairs of Lagrange level l grouped by translation and the per-translation tiles
-// (on demand; no-op if present)
+// tree.cu: pairs of Lagrange level l grouped by translation; column tiles of the CUDA-core
+// transfer and of the ACA factors (both on demand; no-ops if present)
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s);
+void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s);
+// transfer.cu: operator images of a Lagrange level; v~ += T u~ over its pairs by translation
+void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, cudaStream_t s);
+void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
 // autotune.cu: the transfer variant stored for Lagrange level l in the plan's autotune
 // cache (0 CUDA cores, 1 tcgen05 per translation, 2 target-stationary), or -1
 int cached_lag_pick(const ffm_plan_s *p, int l);

@@ -627,18 +627,12 @@ void build_tables(ffm_plan_s *p, int l, TableJob &tj) {
         g.kind = p->kind;
         for (int a = 0; a < F.r1; ++a) g.hnode[a] = (float)(0.5 * dl * std::cos((2.0 * a + 1.0) * PI / (2.0 * F.r1)));
         FFM_LAUNCH(k_lag_table, F.n_trans, 256, 0, s, F.trans_m, F.n_trans, g, F.T);
-        int rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r, npad = (r + 15) / 16 * 16;
-        if (!cplx) {
-            // the tensor-core transfer's operand: T_t with npad rows of rkp (a multiple of its
-            // 16-node K chunks) floats, padding zero; the gradient's three component blocks one
-            // after another
-            int nblk = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
-            F.rkp = (rk + 15) / 16 * 16;
-            size_t tsz = (size_t)nblk * F.n_trans * npad * F.rkp;
-            F.Tsh = p->mem.get<float>(tsz);
-            split_pad(F.T, (int64_t)nblk * F.n_trans, r, rk, npad, F.rkp, F.Tsh, nullptr, s);
+        if (p->aca_eps > 0.0 && p->kind == FFM_LAPLACE) {
+            F.rkp = (r + 15) / 16 * 16;
+            build_aca(p, l, oxy, dl, tj);
+        } else {
+            build_operator_image(p, l, oxy, dl, s);
         }
-        if (p->aca_eps > 0.0 && p->kind == FFM_LAPLACE) build_aca(p, l, oxy, dl, tj);
         return;
     }
     // plane waves: quadrature of eq. 17, (L+1) Gauss-Legendre nodes in cos(theta) times 2L

@@ -1147,10 +1147,9 @@ static int64_t build_tiles(ffm_plan_s *p, const FarLevel &F, uint32_t bn, uint32
 }
 
 // Pairs of Lagrange level l grouped by translation (CSR bt_off over translations, with each
-// pair's source and target box) and the column tiles of the per-translation transfer
-// kernels (32 pairs for the CUDA-core GEMM, 256 for tcgen05).  Made while the plan is built,
-// or later by the autotuner or when the target-stationary transfer cannot take the level;
-// a level that runs the target-stationary transfer does without them.
+// pair's source and target box).  Made while the plan is built, or later by the autotuner or
+// when the target-stationary transfer cannot take the level; a level that runs the
+// target-stationary transfer does without them.
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
     if (F.mode != 1 || F.n_adm == 0 || F.bt_off) return;
@@ -1170,8 +1169,19 @@ void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     FFM_LAUNCH(k_gather_u32, cdiv(na, 256), 256, 0, s, ptgt, pidx, na, F.bt_tgt);
     F.bt_off = p->mem.get<uint32_t>(F.n_trans + 1);
     FFM_LAUNCH(k_csr_offsets, cdiv(F.n_trans + 1, 256), 256, 0, s, tk, na, F.n_trans, F.bt_off);
+    tmp.release();
+}
+
+// Column tiles over those groups: 32 pairs for the CUDA-core GEMM, 256 for the ACA factors on
+// the tensor cores (the dense tensor-core transfer cuts its own).
+void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s) {
+    FarLevel &F = p->far[l];
+    if (F.mode != 1 || F.n_adm == 0 || F.tile_t) return;
+    build_translation_groups(p, l, s);
+    Alloc tmp;
+    tmp.stream = s;
     F.n_tiles = build_tiles(p, F, LAG_GEMM_BN, &F.tile_t, &F.tile_p0, tmp, s);
-    F.tc_tiles = build_tiles(p, F, 256, &F.tc_tile_t, &F.tc_tile_p0, tmp, s);
+    if (p->aca_eps > 0.0) F.tc_tiles = build_tiles(p, F, 256, &F.tc_tile_t, &F.tc_tile_p0, tmp, s);
     tmp.release();
 }
 
@@ -1238,6 +1248,7 @@ static void finish_far_level(ffm_plan_s *p, int l, uint32_t *aa, uint32_t *ab, i
         const bool ts_first = (p->lag_transfer == 3 || pick == 2) && p->kind == FFM_LAPLACE && F.r1 <= 4 &&
                               !(p->aca_eps > 0.0);
         if (!ts_first) build_translation_groups(p, l, s);
+        if (p->lag_transfer == 1 || pick == 0 || p->aca_eps > 0.0) build_group_tiles(p, l, s);
         F.src_chunks = build_chunks(p, F.src, F.n_src, p->by[l].start, &F.n_src_chunks, tmp, s);
         F.tgt_chunks = build_chunks(p, F.tgt, F.n_tgt, p->bx[l].start, &F.n_tgt_chunks, tmp, s);
     }
