@@ -439,9 +439,9 @@ def roofline(prof, info, steps, clk, pk, pk_kind, workload, nrhs=1):
         peak = SM_COUNT * 128 * 2 * clk_hz
         out.update({"bound": "alu", "pipe": "FP32 (FMA)", "unit": "TFLOP/s", "units_per_step": units,
                     "peak_basis": basis % "128 FMA lanes/clk x 2 FLOP"})
-    elif "k_lag_gemm" in name or "k_lag_pairs" in name:
-        f16 = "k_lag_pairs" in name
-        variant = 1 if f16 else 2 if "_ts" in name else 1 if "_tc" in name else 0
+    elif "k_lag_gemm" in name or "k_lag_pairs" in name or "k_lag_targets" in name:
+        f16 = "k_lag_gemm" not in name
+        variant = 2 if "_targets" in name else 1 if f16 or "_tc" in name else 0
 
         def lag_units(l):
             # (flops, transfer variant) of a Lagrange level: a dense r x r (x kfac) GEMM per

@@ -102,7 +102,8 @@ typedef struct {
     const char *autotune_cache; /* NULL, or a file written by ffm_autotune: the plan takes the
                                    picks stored for its sizes (single right-hand side picks;
                                    several-RHS picks from 64, else 8 RHS), timing nothing */
-    int lagrange_transfer;      /* Lagrange levels' transfer: 0 default (tcgen05 per
+    int lagrange_transfer;      /* Lagrange levels' transfer: 0 default (tcgen05, target-stationary
+                                   on levels with many pairs per translation and else per
                                    translation, or ffm_autotune's pick), 1 CUDA-core GEMM per
                                    translation, 2 tcgen05 per translation, 3 tcgen05
                                    target-stationary (FFM_LAPLACE, r <= 64; per translation

@@ -374,8 +374,6 @@ __global__ void __launch_bounds__(LG_T) k_lag_gemm(const uint32_t *__restrict__ 
 // (g, c) at byte (g * KT/4 + c) * 128, leading-dimension (K) stride 128 B, 8-row-group stride
 // KT/4 * 128 B.  One thread issues the MMAs; completion is tracked by an mbarrier with a
 // bounded wait that raises a device error flag instead of hanging.
-constexpr int TC_M = 128;
-
 __device__ __forceinline__ uint32_t kmajor_off(int row, int k, int KT) {
     return (uint32_t)((((row >> 3) * (KT >> 2) + (k >> 2)) << 7) + ((row & 7) << 4) + ((k & 3) << 2));
 }
@@ -613,360 +611,11 @@ __global__ void k_split_pad(const float *__restrict__ src, int64_t nmat, int row
     }
 }
 
-// ---- target-stationary tensor-core transfer (r <= 64)
-//
-// A CTA owns TS_M = 128 consecutive target boxes of the level (TMEM lane = box) and runs
-// over every translation t present among their admissible pairs, in increasing order
-// (partners are sorted by translation within each target, so a per-row cursor finds the
-// row's source box for t, or none).  For each t it multiplies the source rows u~_b (zero
-// rows for boxes without a partner at t) by T_t (N = 64 target nodes, K = 64 source nodes,
-// zero padded beyond r) and accumulates D(a, i) = sum_t sum_j u~_{b(a,t)}(j) T_t(i, j) in
-// TMEM; each target's v~ is written once, with no atomics.  TF32 hi/lo split with three
-// MMAs per K step (hi hi + hi lo + lo hi), FP32 accumulation.
-//
-// Operands.  The A operand (the gathered source rows) lives in tensor memory: the MMAs read
-// it from TMEM, so shared memory only carries T_t (the B operand), and the operand reads of
-// the tensor cores from shared memory drop to a third.  A step is one translation (K = 64
-// source nodes, 24 MMAs).  Warps 1-8 produce; the two producers of a target row each own 32
-// of the row's 64 values.  A producer loads its values of the row's source (zero where the
-// row has no partner) from global memory into registers TS_P steps ahead, splits them into
-// TF32 hi and lo parts and writes them into one of TS_NA TMEM operand stages (tcgen05.st),
-// then arrives on that stage's "A full" mbarrier.  The first producer also starts a bulk copy
-// of T_t's pre-split image (32 KB) into one of TS_NB shared stages, TS_DB steps ahead,
-// counted in bytes on that stage's "B full" mbarrier.  One thread of
-// warp 0 waits on both, issues the step's 24 MMAs and commits them to the B stage's "empty"
-// mbarrier; the producers wait on it (TS_NA steps later) before they reuse the A and B
-// stages.  Each barrier round trip thus serves 24 MMAs.
-//
-// Accumulation.  One long tcgen05 accumulation loses accuracy, so the tile alternates
-// between two TMEM accumulators (64 columns each) every TS_DRAIN translations; the producers
-// add each finished accumulator into FP32 registers (tcgen05.ld) while the tensor cores fill
-// the other one, and the MMA thread waits for that drain before it reuses the accumulator.
-// Every wait is bounded; a give-up raises the device error flag, the CTA then waits for its
-// copies and committed MMAs, skips its results and frees TMEM.
-constexpr int TS_M = 128;
-constexpr int TS_K = 64;              // source nodes (K) per step: one translation
-constexpr int TS_BH = 64 * 32;        // floats per B hi or lo block of one half of K
-constexpr int TS_BST = 4 * TS_BH;     // floats per B stage: T_t's whole image (32 KB)
-constexpr int TS_NA = 3;              // A stages (tensor memory); producers run TS_NA steps ahead
-constexpr int TS_DB = 2;              // steps the copies of T_t's image run ahead
-constexpr int TS_NB = TS_NA + TS_DB;  // B stages (shared memory)
-constexpr int TS_P = 2;               // steps the source loads run ahead (registers)
-constexpr int TS_MAXT = 4096;         // translation codes lie in a 16^3 range
-constexpr int TS_DRAIN = 8;           // translations per TMEM accumulator fill
-constexpr int TS_NP = 2 * TS_M;       // producer threads (warps 1-8)
-constexpr int TS_TCOLS = 512;         // TMEM: 2 accumulators x 64 columns, TS_NA A stages x 128 (hi, lo)
-constexpr size_t TS_SMEM = sizeof(float) * (size_t)TS_NB * TS_BST;
-
-// 16 values of one lane into consecutive TMEM columns of the warp's lanes
-__device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(ta),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-        : "memory");
-}
-
-// eight floats from a 32-byte aligned global address, one 256-bit load through the read-only path
-__device__ __forceinline__ void ldg8(const float *p, float4 &a, float4 &b) {
-    asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-                 : "l"(p));
-}
-
 // 8 values of one lane into consecutive TMEM columns of the warp's lanes
 __device__ __forceinline__ void tmem_st8(uint32_t ta, const uint32_t (&v)[8]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(ta), "r"(v[0]),
                  "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
-}
-
-// u holds rows of 64 floats (r <= 64, zero padded): row (b, m) at ((b nrhs + m) 64).
-__global__ void __launch_bounds__(TS_NP + 32, 1) k_lag_gemm_ts(const uint32_t *__restrict__ tgt, int64_t n_tgt,
-                                                              const uint32_t *__restrict__ adm_off,
-                                                              const uint32_t *__restrict__ adm_src,
-                                                              const uint32_t *__restrict__ adm_t, int n_trans,
-                                                              const float *__restrict__ Tsp, int r, int nrhs,
-                                                              const float *__restrict__ u, float *__restrict__ vt,
-                                                              int *__restrict__ err, int tries) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    float *bring = reinterpret_cast<float *>(smem);
-    __shared__ uint32_t s_bits[TS_MAXT / 32];
-    __shared__ uint16_t s_tl[TS_MAXT];  // the translations present, in increasing order
-    __shared__ uint32_t s_wpre[TS_MAXT / 32 + 1];
-    __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_bfull[TS_NB], s_empty[TS_NB], s_afull[TS_NA], s_drained;
-    __shared__ int s_bad;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m = blockIdx.y;
-    const int64_t x0 = (int64_t)blockIdx.x * TS_M;
-    const int nw = (n_trans + 31) / 32;
-    for (int w = tid; w < TS_MAXT / 32; w += blockDim.x) s_bits[w] = 0u;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
-                     "r"(TS_TCOLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    if (tid == 0) {
-        s_bad = 0;
-        for (int i = 0; i < TS_NB; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_bfull[i])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_empty[i])));
-        }
-        for (int i = 0; i < TS_NA; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_afull[i])), "r"(TS_NP));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_drained)), "r"(TS_NP));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = s_tmem;
-    // producers: warp w (1-8) holds TMEM lanes 32 (w % 4) .. + 31, one target row per lane,
-    // and values 32 qh .. 32 qh + 31 of each step
-    const bool prod = warp >= 1;
-    const int dq = warp & 3, qh = (warp - 1) >> 2, row = dq * 32 + lane;
-    const int64_t x = x0 + row;
-    const bool has = prod && x < n_tgt;
-    uint32_t cur = has ? adm_off[x] : 0u, end = has ? adm_off[x + 1] : 0u;
-    if (has && qh == 0)
-        for (uint32_t e = cur; e < end; ++e) {
-            uint32_t t = adm_t[e];
-            atomicOr(&s_bits[t >> 5], 1u << (t & 31));
-        }
-    __syncthreads();
-    // list of the translations present: word counts, their prefix, then the set bits in order
-    if (tid < TS_MAXT / 32) s_wpre[tid + 1] = __popc(s_bits[tid]);
-    if (tid == 0) s_wpre[0] = 0u;
-    __syncthreads();
-    if (tid == 0)
-        for (int w = 1; w <= TS_MAXT / 32; ++w) s_wpre[w] += s_wpre[w - 1];
-    __syncthreads();
-    if (tid < nw) {
-        uint32_t bits = s_bits[tid], o = s_wpre[tid];
-        while (bits) {
-            s_tl[o++] = (uint16_t)(tid * 32 + __ffs(bits) - 1);
-            bits &= bits - 1;
-        }
-    }
-    __syncthreads();
-    const int nsteps = (int)s_wpre[TS_MAXT / 32];
-    bool ok = true;
-    if (prod) {
-        const int p = tid - 32;
-        float sum[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) sum[c] = 0.f;
-        int drained = 0;  // accumulator fills added into sum (columns 32 qh .. + 31)
-        auto drain = [&](int k) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t base = tmem + (uint32_t)((k & 1) * 64 + qh * 32) + ((uint32_t)(dq * 32) << 16);
-#pragma unroll
-            for (int c0 = 0; c0 < 32; c0 += 8) {
-                uint32_t v[8];
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                               "=r"(v[7])
-                             : "r"(base + (uint32_t)c0));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int q = 0; q < 8; ++q) sum[c0 + q] += __uint_as_float(v[q]);
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&s_drained)) : "memory");
-        };
-        // T_t's image of step sp into B stage sp % TS_NB: one bulk copy (32 KB) by the first
-        // producer, counted in bytes on the stage's "B full" barrier
-        int last_b = -1;
-        auto copy_b = [&](int sp) {
-            if (p != 0 || sp >= nsteps) return;
-            uint64_t *bar = &s_bfull[sp % TS_NB];
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
-                         "r"((uint32_t)(TS_BST * sizeof(float)))
-                         : "memory");
-            bulk_g2s(bring + (size_t)(sp % TS_NB) * TS_BST, Tsp + (size_t)s_tl[sp] * TS_BST,
-                     (uint32_t)(TS_BST * sizeof(float)), bar);
-            last_b = sp;
-        };
-        // this row's source values of step sp (zero without a partner), into registers.  The
-        // row's next two partners (translation, source) are held in registers and the one after
-        // is loaded as one is used, so the source row's address never waits on a list load.
-        uint32_t t0 = 0xffffffffu, b0 = 0u, t1 = 0xffffffffu, b1 = 0u;
-        if (cur < end) {
-            t0 = adm_t[cur];
-            b0 = adm_src[cur];
-        }
-        if (cur + 1 < end) {
-            t1 = adm_t[cur + 1];
-            b1 = adm_src[cur + 1];
-        }
-        float4 ring[TS_P][8];
-        auto load_a = [&](int sp, float4 *dst) {
-            bool use = false;
-            uint32_t src = 0u;
-            if (sp < nsteps && t0 == (uint32_t)s_tl[sp]) {
-                use = true;
-                src = b0;
-                t0 = t1;
-                b0 = b1;
-                ++cur;
-                t1 = 0xffffffffu;
-                if (cur + 1 < end) {
-                    t1 = adm_t[cur + 1];
-                    b1 = adm_src[cur + 1];
-                }
-            }
-            // 256-bit loads: half the load instructions (and L1 wavefronts) of 128-bit ones
-            const float *g = u + ((size_t)src * nrhs + m) * 64 + qh * 32;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                if (use) {
-                    ldg8(g + 8 * c, dst[2 * c], dst[2 * c + 1]);
-                } else {
-                    dst[2 * c] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    dst[2 * c + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-        };
-#pragma unroll
-        for (int k = 0; k < TS_P; ++k) load_a(k, ring[k]);
-        for (int sp = 0; sp < TS_DB; ++sp) copy_b(sp);
-        for (int s0 = 0; s0 < nsteps && ok; s0 += TS_P) {
-#pragma unroll
-            for (int k = 0; k < TS_P; ++k) {
-                const int s = s0 + k;
-                // (no break in this loop: it is unrolled so that the ring slot k is static)
-                if (s >= nsteps || !ok) continue;
-                if (s >= TS_NA) {
-                    // the MMAs of step s - TS_NA are done: its A and B stages are free.  A fill k
-                    // is drained once the first step of fill k + 1 is done: then the fill is
-                    // final, and the MMA thread has passed its wait for the drain of fill k - 1,
-                    // so the drain barrier is never two phases ahead of that wait (a give-up
-                    // is made warp-uniform: the drains are warp-wide TMEM loads)
-                    const int sb = s - TS_NA;
-                    bool w_ok = mbar_wait(&s_empty[sb % TS_NB], (uint32_t)((sb / TS_NB) & 1), tries, err);
-                    if (!__all_sync(0xffffffffu, w_ok)) {
-                        ok = false;
-                        continue;
-                    }
-                    const int done = sb / TS_DRAIN;
-                    while (drained < done) drain(drained++);
-                }
-                // split into TF32 hi and lo and write A stage s % TS_NA: columns 128 + 128 (s % TS_NA)
-                // + 32 qh (hi) and + 64 (lo), lane = row
-                const uint32_t ta =
-                    tmem + (uint32_t)(128 + (s % TS_NA) * 128 + qh * 32) + ((uint32_t)(dq * 32) << 16);
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {  // 16 values at a time: fewer live registers
-                    uint32_t hv[16], lv[16];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float4 f4 = ring[k][4 * hh + c];
-                        const float v4[4] = {f4.x, f4.y, f4.z, f4.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            float h, l;
-                            tf32_split(v4[q], h, l);
-                            hv[4 * c + q] = __float_as_uint(h);
-                            lv[4 * c + q] = __float_as_uint(l);
-                        }
-                    }
-                    tmem_st16(ta + 16u * hh, hv);
-                    tmem_st16(ta + 64u + 16u * hh, lv);
-                }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&s_afull[s % TS_NA])) : "memory");
-                copy_b(s + TS_DB);          // its stage held step s - TS_NA's image
-                load_a(s + TS_P, ring[k]);  // this ring slot's next step
-            }
-        }
-        if (ok && nsteps > 0) {
-            // the last step's MMAs complete after all others: then the last fills
-            const int l = nsteps - 1;
-            bool w_ok = mbar_wait(&s_empty[l % TS_NB], (uint32_t)((l / TS_NB) & 1), tries, err);
-            if (!__all_sync(0xffffffffu, w_ok)) ok = false;
-            const int fills = (nsteps + TS_DRAIN - 1) / TS_DRAIN;
-            while (ok && drained < fills) drain(drained++);
-        }
-        if (!ok) {
-            s_bad = 1;
-            for (int sp = max(0, last_b - TS_NB + 1); sp <= last_b; ++sp)  // copies still in flight
-                mbar_wait(&s_bfull[sp % TS_NB], (uint32_t)((sp / TS_NB) & 1), DRAIN_TRIES);
-        }
-        if (ok && x < n_tgt) {
-            float *dst = vt + ((size_t)tgt[x] * nrhs + m) * r + qh * 32;
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-                if (qh * 32 + c < r) dst[c] = sum[c];
-        }
-    } else if (lane == 0) {
-        // ---- MMA thread
-        const uint32_t lbo = 128, sbo = 8 * 128;  // B image: per half of K, 64 rows x 32 in core matrices
-        const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(64 >> 3) << 17) |
-                               ((uint32_t)(TS_M >> 4) << 24);
-        int issued = 0;
-        for (int s = 0; s < nsteps; ++s) {
-            const int fill = s / TS_DRAIN;
-            // the accumulator of fill - 2 must have been added into the producers' sums
-            if (s % TS_DRAIN == 0 && fill >= 2 && !mbar_wait(&s_drained, (uint32_t)((fill - 2) & 1), tries, err)) {
-                ok = false;
-                break;
-            }
-            const int b = s % TS_NB;
-            if (!mbar_wait(&s_bfull[b], (uint32_t)((s / TS_NB) & 1), tries, err) ||
-                !mbar_wait(&s_afull[s % TS_NA], (uint32_t)((s / TS_NA) & 1), tries, err)) {
-                ok = false;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t d = tmem + (uint32_t)((fill & 1) * 64);
-            const uint32_t a0 = tmem + (uint32_t)(128 + (s % TS_NA) * 128);
-            const uint32_t bst = smem_addr(bring + (size_t)b * TS_BST);
-#pragma unroll
-            for (int ks = 0; ks < TS_K / 8; ++ks) {
-                // K step ks: A columns 8 ks (hi) and 64 + 8 ks (lo); B in half ks / 4 of the image
-                // (hi block, then lo block), core matrices 2 (ks % 4) and 2 (ks % 4) + 1
-                const uint32_t ah = a0 + (uint32_t)(ks * 8), al = a0 + 64u + (uint32_t)(ks * 8);
-                const uint32_t bh0 = bst + (uint32_t)((ks >> 2) * 2 * TS_BH * 4 + (ks & 3) * 256);
-                const uint64_t bh = umma_desc(bh0, lbo, sbo), bl = umma_desc(bh0 + TS_BH * 4, lbo, sbo);
-                const uint32_t acc0 = (s % TS_DRAIN != 0 || ks > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                    "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-                    "r"(ah), "l"(bh), "r"(idesc), "r"(acc0));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;\n" ::"r"(d), "r"(ah), "l"(bl),
-                             "r"(idesc));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;\n" ::"r"(d), "r"(al), "l"(bh),
-                             "r"(idesc));
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_addr(&s_empty[b]))
-                         : "memory");
-            issued = s + 1;
-        }
-        // after a give-up: keep TMEM and the stages owned until the committed MMAs are done
-        if (!ok) {
-            s_bad = 1;
-            if (issued > 0)
-                mbar_wait(&s_empty[(issued - 1) % TS_NB], (uint32_t)(((issued - 1) / TS_NB) & 1), DRAIN_TRIES);
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid == 0 && s_bad) atomicOr(err, 1);
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TS_TCOLS));
-}
-
-// u~ rows of r < 64 floats copied into rows of 64 (zero padded), the row layout the
-// target-stationary transfer reads.
-__global__ void k_pad_rows64(const float *__restrict__ u, int64_t nrow, int r, float *__restrict__ out) {
-    int64_t n = nrow * 64;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t row = i >> 6;
-        int k = (int)(i & 63);
-        out[i] = k < r ? u[row * r + k] : 0.f;
-    }
 }
 
 // Target step of a Lagrange level (L_X^T v~ of eq. 8): v_i += sum_abc L_a(x_i) L_b(y_i) L_c(z_i) v~_a(abc),
@@ -1345,35 +994,19 @@ void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *a
         const int ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
         const size_t tblk = (size_t)F.n_trans * r * rk;
         const size_t vblk = (size_t)r * nrhs * p->bx[l].nb;
-        float *uts = nullptr;
-        const bool use_ts = F.ts_ok && F.Tsp && F.tune_tc == 2;
-        // all components in one launch
-        if (!use_ts && use_tc) lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
+        const bool use_ts = F.ts_ok && F.tune_tc == 2;
+        if (use_ts)
+            lag_targets(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
+        else if (use_tc)  // all components in one launch
+            lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
         for (int d = 0; d < ncomp; ++d) {
             const float *Td = F.T + d * tblk;
             float *vtd = (float *)vt + d * vblk;
-        if (use_ts) {
-            FFM_CUDA(cudaFuncSetAttribute(k_lag_gemm_ts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS_SMEM));
-            const float *u64 = (const float *)ut;
-            if (r < 64) {  // rows of 64 floats, once for all components
-                const int64_t nrow = (int64_t)p->by[l].nb * nrhs;
-                if (!uts) {
-                    uts = tmp.get<float>((size_t)nrow * 64);
-                    unsigned gs = (unsigned)std::min<int64_t>(cdiv(nrow * 64, 256), 152 * 16);
-                    FFM_LAUNCH(k_pad_rows64, gs, 256, 0, s, (const float *)ut, nrow, r, uts);
-                }
-                u64 = uts;
-            }
-            dim3 gts(cdiv(F.n_tgt, TS_M), nrhs);
-            FFM_LAUNCH(k_lag_gemm_ts, gts, TS_NP + 32, TS_SMEM, s, F.tgt, F.n_tgt, F.adm_off, F.adm_src, F.adm_t,
-                       F.n_trans, F.Tsp, r, nrhs, u64, vtd, p->dev_err, p->wait_tries);
-        } else if (!use_tc) {
-            FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, Td, r,
-                       rk, nrhs, (const float *)ut, vtd);
-        }
+            if (!use_ts && !use_tc)
+                FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, Td,
+                           r, rk, nrhs, (const float *)ut, vtd);
             lagrange_points_r1<false>(p, F, AX, cb, false, vtd, nrhs, accf + (size_t)d * nrhs * p->nx, s);
         }
-        if (uts) tmp.drop(uts);
     }
 }
 

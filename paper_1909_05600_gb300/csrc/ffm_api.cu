@@ -485,7 +485,7 @@ ffm_status ffm_plan_info(const ffm_plan_t *plan, ffm_info *info) {
         // the variant far_lagrange runs: ACA levels by their own choice, dense levels on tcgen05
         // unless the CUDA-core GEMM is forced or picked
         bool tc = F.aca ? F.aca_tc : (F.tune_tc != 0 && F.Th != nullptr);
-        bool ts = F.ts_ok && F.Tsp && F.tune_tc == 2;
+        bool ts = F.ts_ok && F.tune_tc == 2;
         info->tune_tc[l] = act && F.mode == 1 ? (ts ? 2 : tc ? 1 : 0) : 0;
         info->tune_pw[l][0] = act && F.mode == 2 ? F.pw_qpt : 0;
         info->tune_pw[l][1] = act && F.mode == 2 ? F.pw_ppt : 0;

@@ -166,10 +166,13 @@ struct FarLevel {
     int64_t n_src_chunks = 0, n_tgt_chunks = 0;
     uint2 *src_chunks = nullptr;    // (source box, first point): LAG_CHUNK-point pieces of the boxes
     uint2 *tgt_chunks = nullptr;    // likewise for the target boxes
-    bool ts_ok = false;             // target-stationary transfer possible (Laplace, r <= 64,
-                                    // partners sorted by translation within each target)
-    float *Tsp = nullptr;           // target-stationary transfer (r <= 64): T_t split into TF32
-                                    // hi and lo, 64 x 64 each, in the K-major core-matrix layout
+    // target-stationary transfer (Laplace, r <= 64): each 128-target tile's pairs by translation,
+    // made where the level runs it (transfer.cu)
+    bool ts_ok = false;
+    uint32_t *ts_src = nullptr;     // n_adm source boxes
+    uint8_t *ts_row = nullptr;      // n_adm target rows in the tile
+    uint32_t *ts_steps = nullptr;   // n_trans per tile: translation | first entry << 12
+    uint32_t *ts_n = nullptr;       // steps per tile
     // tensor-core transfer by translation: f16 hi / lo images of T_t (transfer.cu), h_bpc blocks of
     // h_nb rows per component, h_nk chunks of 32 columns, 1 / scale
     uint16_t *Th = nullptr;
@@ -272,8 +275,8 @@ namespace ffm {
 // tree.cu
 void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_dtype ydt, const void *w,
                 ffm_dtype wdt, Alloc &tmp);
-// tree.cu: partners sorted by translation and T pre-split for the target-stationary
-// transfer of Lagrange level l (on demand); tables.cu: the T split
+// transfer.cu: pairs of Lagrange level l by tile and translation, for the target-stationary
+// transfer (on demand)
 void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s);
 // tree.cu: pairs of Lagrange level l grouped by translation; column tiles of the CUDA-core
 // transfer and of the ACA factors (both on demand; no-ops if present)
@@ -282,10 +285,11 @@ void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s);
 // transfer.cu: operator images of a Lagrange level; v~ += T u~ over its pairs by translation
 void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, cudaStream_t s);
 void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
+// the same over each target's partners (target-stationary; ts_ok levels)
+void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
 // autotune.cu: the transfer variant stored for Lagrange level l in the plan's autotune
 // cache (0 CUDA cores, 1 tcgen05 per translation, 2 target-stationary), or -1
 int cached_lag_pick(const ffm_plan_s *p, int l);
-void launch_table_split(ffm_plan_s *p, int l, cudaStream_t s);
 
 // tree.cu: near-field work items with targets in chunks of tchunk and at most smax source
 // points per item, allocated from out_mem; returns their number.

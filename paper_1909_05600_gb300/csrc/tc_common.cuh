@@ -24,6 +24,16 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, 
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
+// this thread arrives on bar once all its earlier cp.async copies have landed (the barrier's count
+// includes the arrival)
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+// Shared-memory writes that this thread has observed (by a barrier wait) become visible to the tensor
+// cores' reads.  Run by the thread that issues the MMAs, not by the copying threads: there the
+// fence waits for every copy the thread still has in flight.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // bulk copy global -> shared, completion counted in bytes on an mbarrier
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -42,17 +52,25 @@ __device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 
+__device__ __forceinline__ uint32_t mbar_try(uint64_t *bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done)
+                 : "r"(smem_addr(bar)), "r"(parity)
+                 : "memory");
+    return done;
+}
+
 // Bounded wait for the completion of phase `parity` of an mbarrier: at most `tries`
 // try_wait attempts (none for tries <= 0); false if it gave up.
 // With `abort` (the launch's device error flag), the wait also gives up once another CTA has
 // raised the flag (checked every 1024 attempts), so one failure does not make every later
 // CTA spend its whole limit.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int tries, const int *abort = nullptr) {
+    if (tries > 0 && mbar_try(bar, parity)) return true;
     uint32_t done = 0;
-    for (int it = 0; it < tries && !done; ++it) {
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(smem_addr(bar)), "r"(parity));
+    for (int it = 1; it < tries && !done; ++it) {
+        done = mbar_try(bar, parity);
         if (!done && abort && (it & 1023) == 1023 && *reinterpret_cast<const volatile int *>(abort)) break;
     }
     return done != 0;
@@ -69,12 +87,14 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                  : "memory");
 }
 
-// D (+)= A B for f16 operands in shared memory, FP32 accumulator in tensor memory
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// D (+)= A B for f16 operands in shared memory, FP32 accumulator in tensor memory; the operand
+// descriptors as their low and high words (only the low one, with the address, changes)
+__device__ __forceinline__ void mma_f16(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                        uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+        "{\n.reg .pred p;\n.reg .b64 a, b;\nsetp.ne.b32 p, %6, 0;\nmov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate));
 }
 
 // instruction descriptor of kind::f16: f16 A and B (both K-major), FP32 accumulator, M = 128

@@ -23,6 +23,49 @@ constexpr int HK = 32;            // K values (source nodes) per chunk
 constexpr int HROW = 2 * HK;      // halves per row and chunk: hi part, then lo part (128 bytes)
 constexpr int HM = 128;           // rows (pairs times right-hand sides) per tile
 constexpr int H_LBO = 128, H_SBO = (HK / 8) * 128;
+constexpr uint32_t A_BYTES = HM * HROW * 2;  // a tile's rows, one chunk
+
+// The gathered rows lie in shared memory as 128-byte rows (hi, then lo) in the 128-byte swizzle:
+// 16-byte segment c of row i at 128 i + 16 (c ^ (i % 8)).  A warp's cp.async writes whole 128-byte
+// lines of it (4 wavefronts for 4 rows); in the no-swizzle core-matrix order the same copies, 64
+// bytes of a row spread over four lines, took 26 wavefronts.
+// Descriptor words: the high ones are constants (rows: 128-byte swizzle, 1024 bytes between 8-row
+// groups; operator: no swizzle, H_SBO), the low ones address / 16 and the K stride.
+constexpr uint32_t A_DHI = (1024u >> 4) | (1u << 14) | (2u << 29), B_DHI = ((uint32_t)H_SBO >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t a_dlo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
+__device__ __forceinline__ uint32_t b_dlo(uint32_t saddr) { return (saddr >> 4) | ((uint32_t)(H_LBO >> 4) << 16); }
+
+// The MMAs of one stage (CPS chunks of 32 K values: the chunks' rows, then the operator's chunks) into
+// accumulator d: hi hi + hi lo + lo hi per K step of 16.  alo, blo: low descriptor words of the stage's
+// first chunk.  STACK: the operator's hi and lo rows as one operand of 2 npad rows, so that hi hi and
+// hi lo are one MMA (lo hi joins hi lo in columns npad ..).  The issuing thread's own instructions
+// are what a small stage waits for (its 4 MMAs took 1200 cycles with 64-bit descriptors formed
+// for each and two barriers per chunk), so they are kept to an add and the MMA.
+template <int CPS, bool STACK>
+__device__ __forceinline__ void stage_mma(uint32_t d, uint32_t alo, uint32_t blo, uint32_t npad, uint32_t id1,
+                                          uint32_t id2, bool first) {
+#pragma unroll
+    for (int kc = 0; kc < CPS; ++kc) {
+#pragma unroll
+        for (int ks = 0; ks < HK / 16; ++ks) {
+            const uint32_t ah = alo + kc * (A_BYTES >> 4) + ks * 2, al = ah + (HK * 2 >> 4);
+            const uint32_t bh = blo + kc * npad * (HROW * 2 >> 4) + ks * (2 * H_LBO >> 4);
+            const uint32_t acc = kc > 0 || ks > 0 || !first;
+            mma_f16(d, ah, A_DHI, bh, B_DHI, id2, acc);
+            if constexpr (STACK) {
+                mma_f16(d + npad, al, A_DHI, bh, B_DHI, id1, 1u);
+            } else {
+                mma_f16(d, ah, A_DHI, bh + npad * (HK * 2 >> 4), B_DHI, id1, 1u);
+                mma_f16(d, al, A_DHI, bh, B_DHI, id1, 1u);
+            }
+        }
+    }
+}
+
+// dynamic shared memory from its first 1024-byte boundary (the swizzle repeats every 1024 bytes)
+__device__ __forceinline__ unsigned char *aligned_smem(unsigned char *p) {
+    return p + ((1024u - (smem_addr(p) & 1023u)) & 1023u);
+}
 
 // a power of two s with max s in [2^13, 2^14), and its inverse (both finite and normal)
 __device__ __forceinline__ void row_scale(float mx, float &s, float &inv) {
@@ -41,19 +84,25 @@ __device__ __forceinline__ void half_split(float x, __half &hi, __half &lo) {
 }
 
 // Rows of n floats as f16 hi / lo images, one warp per row: chunk kc of row i holds the hi
-// parts of values 32 kc .. + 31, then their lo parts (zero past n); inv[i] = 1 / scale.
+// parts of values 32 kc .. + 31, then their lo parts (zero past n).  The scale is the row's own
+// (its inverse in inv[i]), or with `common` the one of that largest value, for all rows.
 __global__ void __launch_bounds__(256) k_rows_split(const float *__restrict__ u, int64_t nrow, int n, int nk,
-                                                    __half *__restrict__ img, float *__restrict__ inv) {
+                                                    __half *__restrict__ img, float *__restrict__ inv,
+                                                    const uint32_t *__restrict__ common) {
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= nrow) return;
     const float *row = u + i * n;
     float mx = 0.f;
-    for (int k = lane; k < n; k += 32) mx = fmaxf(mx, fabsf(row[k]));
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (common) {
+        mx = __uint_as_float(*common);
+    } else {
+        for (int k = lane; k < n; k += 32) mx = fmaxf(mx, fabsf(row[k]));
+        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
     float s, si;
     row_scale(mx, s, si);
-    if (lane == 0) inv[i] = si;
+    if (lane == 0 && !common) inv[i] = si;
     __half *out = img + i * (int64_t)nk * HROW;
     for (int k = 2 * lane; k < nk * HK; k += 64) {
         __half h0, l0, h1, l1;
@@ -109,7 +158,6 @@ struct PairArgs {
     const __half *T;    // operator images
     float tinv;
     int nk, npad, tcols;
-    int stack;          // hi and lo rows of T in one MMA operand of 2 npad rows
     int ostride;        // floats between rows of v~
     int nout[PAIR_MAXBLK];
     int64_t ooff[PAIR_MAXBLK];  // first float of the block's columns in v~
@@ -126,39 +174,51 @@ struct PairArgs {
 // a row block of the operator (at most 256 rows), and the blocks of one persistent grid take
 // units in turn, so that neighbouring blocks read the same operator.  Per unit and chunk of 32 K
 // values:
+//   warps 9-12  fetch the row numbers (source, target, source scale) of coming units, one warp a unit,
+//               into a ring in shared memory: a chain of dependent loads that no copying or adding
+//               thread waits for
 //   warps 0-3   copy the tile's rows (hi and lo, 16 KB) with cp.async, rows past the tile's pairs
-//               zero-filled; the row numbers of the next unit are fetched while this one is copied
+//               zero-filled
 //   thread 0    also starts the bulk copy of the operator's chunk (128 npad bytes)
 //   warp 8      issues the MMAs into one of two TMEM accumulators
 //   warps 4-7   read the other accumulator, undo the scales and add it into v~: 32 columns at a
 //               time through shared memory, so that eight lanes add 128 consecutive bytes
 // The MMAs of a K step are hi [hi; lo] (one operand of 2 npad rows, accumulated apart) and lo hi
 // up to 128 operator rows, else three of npad rows into one accumulator.
-// NSTG chunks are in flight: 8 at npad = 64 (24 KB each), 4 at 224 (45 KB).
+// NSTG stages of CPS chunks are in flight: 4 of two at npad = 64 (48 KB each), 4 of one at 224 (45 KB).
 //
-// Measured on GB300, transfers of one apply, against the kernel before it (a block per 256-pair
+// Measured on GB300 (level 7 of clustered 10M, 68M pairs of r = 64): 11.7 ms with the row numbers fetched
+// by the copying and adding threads themselves, 9.85 with index warps, 6.98 with rows in the swizzled
+// layout, 6.14 with the lean MMA loop.  Transfers of one apply, against the kernel before it (a block per 256-pair
 // tile, which split its FP32 rows into TF32 for every pair, no overlap of tiles): gradient sphere 300k
 // (r = 216, three operators) 6.54 -> 3.12 ms, double layer 200k (K = 648) 2.16 -> 0.97, Laplace volume
 // 250k at 1e-4 (r = 216) 1.47 -> 0.79, 100k x 8 right-hand sides (r = 64) 1.68 -> 0.72, clustered
 // 10M (r = 64) 21.8 -> 14.0.  Complex operators (Helmholtz volume 120k at 1e-4, 432 real rows), on
 // CUDA cores before: 24.4 -> 2.4 ms.
-constexpr int PAIR_T = 288;
+constexpr int PAIR_T = 416;
+constexpr int PAIR_IXW = 4;  // index warps
+constexpr int PAIR_IX = 4;   // units whose row numbers are held
 constexpr int PAIR_ST = 36;  // floats per row of the epilogue's staging (conflict-free float4)
 
-static size_t pair_stage(int npad) { return (size_t)HM * HROW * 2 + (size_t)npad * HROW * 2; }
-static size_t pair_smem(int nstg, int npad, int n_trans) {
-    return nstg * pair_stage(npad) + 4 * 32 * PAIR_ST * sizeof(float) + sizeof(uint32_t) * ((size_t)n_trans + 1);
+static size_t pair_smem(int nchunk, int npad, int n_trans) {
+    return 1024 + nchunk * (A_BYTES + (size_t)npad * HROW * 2) + 4 * 32 * PAIR_ST * sizeof(float) + sizeof(uint32_t) * ((size_t)n_trans + 1);
 }
 
-template <int NSTG>
+template <int NSTG, int CPS, bool STACK>
 __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__ PairArgs A) {
-    constexpr int LOOK = NSTG - 1;  // chunks a copying thread runs ahead of the one it hands over
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t s_afull[NSTG], s_bfull[NSTG], s_empty[NSTG], s_accfull[2], s_accempty[2], s_done;
-    __shared__ uint32_t s_tmem, s_carry, s_w[PAIR_T / 32];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = aligned_smem(smem_raw);
+    __shared__ __align__(8) uint64_t s_full[NSTG], s_empty[NSTG], s_accfull[2], s_accempty[2], s_done;
+    __shared__ __align__(8) uint64_t s_ixfull[PAIR_IX], s_ixempty[PAIR_IX];
+    __shared__ uint32_t s_src[PAIR_IX][HM];  // row of the images, NONE past the tile's pairs
+    __shared__ uint32_t s_dst[PAIR_IX][HM];  // row of v~
+    __shared__ float s_inv[PAIR_IX][HM];
+    __shared__ int s_trans[PAIR_IX];
+    __shared__ uint32_t s_tmem, s_carry, s_cmax, s_w[PAIR_T / 32];
+    constexpr uint32_t NONE = 0xffffffffu;
     __shared__ int s_bad;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t stage = (uint32_t)(HM * HROW * 2 + A.npad * HROW * 2);
+    const uint32_t bbytes = (uint32_t)A.npad * HROW * 2 * CPS, stage = CPS * A_BYTES + bbytes;
     float *stag = reinterpret_cast<float *>(smem + (size_t)NSTG * stage);
     uint32_t *pre = reinterpret_cast<uint32_t *>(stag + 4 * 32 * PAIR_ST);  // tiles before translation t
     if (warp == 8) {
@@ -168,15 +228,19 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
     }
     if (tid == 0) {
         s_bad = 0;
+        s_cmax = 0;
         s_carry = 0;
         for (int i = 0; i < NSTG; ++i) {
-            mbar_init(&s_afull[i], 128);
-            mbar_init(&s_bfull[i], 1);
+            mbar_init(&s_full[i], 129);  // the copying threads, and the operator copy's byte count
             mbar_init(&s_empty[i], 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s_accfull[i], 1);
-            mbar_init(&s_accempty[i], 128);
+            mbar_init(&s_accempty[i], 4);
+        }
+        for (int i = 0; i < PAIR_IX; ++i) {
+            mbar_init(&s_ixfull[i], 1);
+            mbar_init(&s_ixempty[i], 8);
         }
         mbar_init(&s_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -225,80 +289,118 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         nrows = (int)min((uint64_t)HM, all - row0);
     };
     bool ok = true;
-    if (warp < 4) {
-        // ---- copies: lane handles rows 32 warp + 8 g + lane % 8 (g < 4), 16-byte segment lane / 8 of
-        // the hi and of the lo part: conflict-free core-matrix stores, 64 contiguous bytes per row
-        constexpr uint32_t NONE = 0xffffffffu;
-        const uint32_t dst0 = smem_addr(smem) + (uint32_t)((4 * warp) * H_SBO + (lane >> 3) * H_LBO + (lane & 7) * 16);
-        int t = 0, tn = 0;
-        uint32_t rows[4], rnext[4];
-        auto fetch = [&](int64_t un, int &tt, uint32_t (&out)[4]) {
+    if (warp > 8) {
+        // ---- row numbers: warp w takes units w - 9, w - 9 + PAIR_IXW, ... of this block
+        uint32_t i = warp - 9;
+        for (int64_t un = blockIdx.x + (int64_t)i * gridDim.x; un < units; un += (int64_t)PAIR_IXW * gridDim.x, i += PAIR_IXW) {
+            const uint32_t k = i % PAIR_IX;
+            int t, n;
             uint32_t p0;
             uint64_t row0;
-            int n;
-            locate(un, tt, p0, row0, n);
+            locate(un, t, p0, row0, n);
+            uint32_t src[4], dst[4];
+            float inv[4];
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
-                const int q = 32 * warp + 8 * g + (lane & 7);
-                out[g] = NONE;
+                const int q = 32 * g + lane;
+                src[g] = NONE;
+                dst[g] = 0u;
+                inv[g] = 0.f;
                 if (q < n) {
                     const uint64_t R = row0 + q;
                     const uint32_t pr = A.nrhs == 1 ? (uint32_t)R : (uint32_t)(R / (uint32_t)A.nrhs);
-                    out[g] = A.bt_src[p0 + pr] * (uint32_t)A.nrhs + (uint32_t)(R - (uint64_t)pr * A.nrhs);
+                    const uint32_t m = (uint32_t)(R - (uint64_t)pr * A.nrhs);
+                    src[g] = A.bt_src[p0 + pr] * (uint32_t)A.nrhs + m;
+                    dst[g] = A.bt_tgt[p0 + pr] * (uint32_t)A.nrhs + m;
                 }
             }
-        };
-        int64_t un = blockIdx.x;
-        if (un < units) fetch(un, t, rows);
-        uint32_t c = 0;
-        auto hand_over = [&](uint32_t done) {  // this thread's copies of chunk `done` have landed
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(&s_afull[done % NSTG]);
-        };
-        for (; un < units && ok; un += gridDim.x) {
-            if (un + gridDim.x < units) fetch(un + gridDim.x, tn, rnext);
-            const int blk = (int)(un % A.nblk);
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+                if (src[g] != NONE) inv[g] = A.uinv[src[g]];
+            const bool w_ok = i < PAIR_IX || mbar_wait(&s_ixempty[k], ((i / PAIR_IX) - 1) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, w_ok)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                s_src[k][32 * g + lane] = src[g];
+                s_dst[k][32 * g + lane] = dst[g];
+                s_inv[k][32 * g + lane] = inv[g];
+            }
+            if (lane == 0) s_trans[k] = t;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_ixfull[k]);
+        }
+    } else if (warp < 4) {
+        // ---- copies: lane handles 16-byte segment lane % 8 of rows 32 warp + 4 g + lane / 8 (g < 8)
+        const uint32_t r0 = 32 * warp + (lane >> 3), sg = lane & 7;
+        const uint32_t dst0 = smem_addr(smem) + r0 * 128, sw0 = (sg ^ (r0 & 7)) * 16, sw1 = (sg ^ ((r0 + 4) & 7)) * 16;
+        uint32_t c = 0, i = 0;
+        for (int64_t un = blockIdx.x; un < units && ok; un += gridDim.x, ++i) {
+            const uint32_t ix = i % PAIR_IX;
+            const bool i_ok = mbar_wait(&s_ixfull[ix], (i / PAIR_IX) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, i_ok)) {
+                ok = false;
+                break;
+            }
+            const int t = s_trans[ix], blk = (int)(un % A.nblk);
+            const __half *src[8];
+            uint32_t bytes[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const uint32_t row = s_src[ix][r0 + 4 * g];
+                bytes[g] = row != NONE ? 16u : 0u;
+                src[g] = A.u + (size_t)(row != NONE ? row : 0u) * A.nk * HROW + sg * 8;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_ixempty[ix]);
             const __half *Tb = A.T + ((size_t)t * A.nblk + blk) * A.nk * A.npad * HROW;
-            for (int kc = 0; kc < A.nk; ++kc, ++c) {
+            for (int kc = 0; kc < A.nk; kc += CPS, ++c) {
                 const uint32_t slot = c % NSTG;
-                if (c >= NSTG && !mbar_wait(&s_empty[slot], ((c / NSTG) - 1) & 1, A.tries, A.err)) {
+                const bool w_ok = c < NSTG || mbar_wait(&s_empty[slot], ((c / NSTG) - 1) & 1, A.tries, A.err);
+                if (!__all_sync(0xffffffffu, w_ok)) {
                     ok = false;
                     break;
                 }
                 if (tid == 0) {
-                    mbar_expect(&s_bfull[slot], (uint32_t)A.npad * HROW * 2);
-                    bulk_g2s(smem + (size_t)slot * stage + HM * HROW * 2, Tb + (size_t)kc * A.npad * HROW,
-                             (uint32_t)A.npad * HROW * 2, &s_bfull[slot]);
+                    mbar_expect(&s_full[slot], bbytes);
+                    bulk_g2s(smem + (size_t)slot * stage + CPS * A_BYTES, Tb + (size_t)kc * A.npad * HROW, bbytes,
+                             &s_full[slot]);
                 }
                 const uint32_t dst = dst0 + slot * stage;
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const bool have = rows[g] != NONE;
-                    const __half *src = A.u + ((size_t)(have ? rows[g] : 0u) * A.nk + kc) * HROW + (lane >> 3) * 8;
-                    cp_async16_zfill(dst + g * H_SBO, src, have ? 16u : 0u);
-                    cp_async16_zfill(dst + g * H_SBO + HM * HK * 2, src + HK, have ? 16u : 0u);
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-                asm volatile("cp.async.wait_group %0;" ::"n"(LOOK) : "memory");
-                if (c >= LOOK) hand_over(c - LOOK);
-            }
-            t = tn;
+                for (int g = 0; g < 8; ++g) {
 #pragma unroll
-            for (int g = 0; g < 4; ++g) rows[g] = rnext[g];
+                    for (int j = 0; j < CPS; ++j)
+                        cp_async16_zfill(dst + j * A_BYTES + g * 512 + ((g & 1) ? sw1 : sw0), src[g] + j * HROW, bytes[g]);
+                    src[g] += CPS * HROW;
+                }
+                cp_async_arrive(&s_full[slot]);
+            }
         }
+        // After a give-up some warps may have copied further than others: all arrive on every stage any of
+        // them started, so that the operator copies can be waited for.
+        if (!ok) atomicOr(&s_bad, 1);
         asm volatile("cp.async.wait_all;" ::: "memory");
-        if (ok)
-            for (uint32_t d = c > LOOK ? c - LOOK : 0; d < c; ++d) hand_over(d);
-        // the operator copies of the last chunks (all others have been consumed)
+        atomicMax(&s_cmax, c);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (s_bad) {
+            const uint32_t last = *reinterpret_cast<volatile uint32_t *>(&s_cmax);
+            for (; c < last; ++c) {
+                if (tid == 0) mbar_arrive(&s_full[c % NSTG]);
+                mbar_arrive(&s_full[c % NSTG]);
+            }
+        }
         if (tid == 0)
             for (uint32_t d = c > NSTG ? c - NSTG : 0; d < c; ++d)
-                mbar_wait(&s_bfull[d % NSTG], (d / NSTG) & 1, DRAIN_TRIES);
+                mbar_wait(&s_full[d % NSTG], (d / NSTG) & 1, DRAIN_TRIES);
     } else if (warp == 8) {
         if (lane == 0) {
             // ---- MMA thread
-            const uint32_t id1 = idesc_f16(A.npad), id2 = A.stack ? idesc_f16(2 * A.npad) : id1;
-            const uint32_t base = smem_addr(smem);
-            uint32_t c = 0, i = 0;
+            const uint32_t id1 = idesc_f16(A.npad), id2 = STACK ? idesc_f16(2 * A.npad) : id1;
+            const uint32_t alo = a_dlo(smem_addr(smem)), blo = b_dlo(smem_addr(smem) + CPS * A_BYTES);
+            uint32_t i = 0, slot = 0, par = 0;
             for (int64_t un = blockIdx.x; un < units && ok; un += gridDim.x, ++i) {
                 const uint32_t buf = i & 1;
                 if (i >= 2 && !mbar_wait(&s_accempty[buf], ((i >> 1) - 1) & 1, A.tries, A.err)) {
@@ -306,31 +408,20 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                     break;
                 }
                 const uint32_t d = tmem + buf * (uint32_t)A.tcols;
-                for (int kc = 0; kc < A.nk; ++kc, ++c) {
-                    const uint32_t slot = c % NSTG, par = (c / NSTG) & 1;
-                    if (!mbar_wait(&s_bfull[slot], par, A.tries, A.err) ||
-                        !mbar_wait(&s_afull[slot], par, A.tries, A.err)) {
+                for (int kc = 0; kc < A.nk; kc += CPS) {
+                    if (!mbar_wait(&s_full[slot], par, A.tries, A.err)) {
                         ok = false;
                         break;
                     }
+                    fence_proxy_async();  // the rows came by cp.async, through the generic proxy
                     tc_fence_after();
-                    const uint32_t ah = base + slot * stage, al = ah + HM * HK * 2, bh = ah + HM * HROW * 2;
-                    const uint32_t bl = bh + (uint32_t)A.npad * HK * 2;
-#pragma unroll
-                    for (int ks = 0; ks < HK / 16; ++ks) {
-                        const uint64_t dah = umma_desc(ah + ks * 2 * H_LBO, H_LBO, H_SBO);
-                        const uint64_t dal = umma_desc(al + ks * 2 * H_LBO, H_LBO, H_SBO);
-                        const uint64_t dbh = umma_desc(bh + ks * 2 * H_LBO, H_LBO, H_SBO);
-                        const uint32_t acc = kc > 0 || ks > 0;
-                        mma_f16(d, dah, dbh, id2, acc);
-                        if (A.stack) {
-                            mma_f16(d + (uint32_t)A.npad, dal, dbh, id1, 1u);
-                        } else {
-                            mma_f16(d, dah, umma_desc(bl + ks * 2 * H_LBO, H_LBO, H_SBO), id1, 1u);
-                            mma_f16(d, dal, dbh, id1, 1u);
-                        }
-                    }
+                    const uint32_t off = slot * (stage >> 4);
+                    stage_mma<CPS, STACK>(d, alo + off, blo + off, (uint32_t)A.npad, id1, id2, kc == 0);
                     tc_commit(&s_empty[slot]);
+                    if (++slot == NSTG) {
+                        slot = 0;
+                        par ^= 1;
+                    }
                 }
                 if (ok) tc_commit(&s_accfull[buf]);
             }
@@ -343,34 +434,20 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         const int q = warp - 4;
         float *st = stag + q * 32 * PAIR_ST;
         const bool vec = (A.ostride & 3) == 0;
-        // rows of this warp with pairs (<= 0: none), this lane's row of v~ and its source's scale;
-        // fetched one unit ahead, a chain of dependent loads
-        auto fetch = [&](int64_t un, int &mine, int64_t &drow, float &inv) {
-            int t, n;
-            uint32_t p0;
-            uint64_t row0;
-            locate(un, t, p0, row0, n);
-            mine = n - 32 * q;
-            if (lane < mine) {
-                const uint64_t R = row0 + 32 * q + lane;
-                const uint32_t pr = A.nrhs == 1 ? (uint32_t)R : (uint32_t)(R / (uint32_t)A.nrhs);
-                const uint32_t m = (uint32_t)(R - (uint64_t)pr * A.nrhs);
-                drow = (int64_t)A.bt_tgt[p0 + pr] * A.nrhs + m;
-                inv = A.uinv[(int64_t)A.bt_src[p0 + pr] * A.nrhs + m];
-            }
-        };
-        int mine = 0, mine_n = 0;
-        int64_t drow = 0, drow_n = 0;
-        float inv = 0.f, inv_n = 0.f;
         uint32_t i = 0;
-        if (blockIdx.x < units) fetch(blockIdx.x, mine_n, drow_n, inv_n);
         for (int64_t un = blockIdx.x; un < units; un += gridDim.x, ++i) {
-            mine = mine_n;
-            drow = drow_n;
-            inv = inv_n;
-            if (un + gridDim.x < units) fetch(un + gridDim.x, mine_n, drow_n, inv_n);
+            const uint32_t buf = i & 1, ix = i % PAIR_IX;
             const int blk = (int)(un % A.nblk), nout = A.nout[blk];
-            const uint32_t buf = i & 1;
+            const bool i_ok = mbar_wait(&s_ixfull[ix], (i / PAIR_IX) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, i_ok)) {
+                ok = false;
+                break;
+            }
+            const float inv = s_inv[ix][32 * q + lane];
+            const uint32_t drow = s_dst[ix][32 * q + lane];
+            // rows of this warp with pairs (a prefix)
+            const int mine = __popc(__ballot_sync(0xffffffffu, s_src[ix][32 * q + lane] != NONE));
+            if (lane == 0) mbar_arrive(&s_ixempty[ix]);
             const bool w_ok = mbar_wait(&s_accfull[buf], (i >> 1) & 1, A.tries, A.err);
             if (!__all_sync(0xffffffffu, w_ok)) {
                 ok = false;
@@ -387,7 +464,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                         if (cc >= A.npad) break;
                         uint32_t v[16], w[16];
                         tmem_ld16(v, d + (uint32_t)cc);
-                        if (A.stack) tmem_ld16(w, d + (uint32_t)(A.npad + cc));
+                        if constexpr (STACK) tmem_ld16(w, d + (uint32_t)(A.npad + cc));
                         tmem_wait_ld();
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
@@ -395,7 +472,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 float y = __uint_as_float(v[4 * k + j]);
-                                if (A.stack) y += __uint_as_float(w[4 * k + j]);
+                                if constexpr (STACK) y += __uint_as_float(w[4 * k + j]);
                                 x[j] = y * inv * A.tinv;
                             }
                             *reinterpret_cast<float4 *>(st + lane * PAIR_ST + 16 * h + 4 * k) =
@@ -408,25 +485,27 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
 #pragma unroll
                         for (int it = 0; it < 8; ++it) {
                             const int row = it * 4 + (lane >> 3);
-                            const int64_t dr = __shfl_sync(0xffffffffu, drow, row);
+                            const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
                             if (row < mine && col < nout)
-                                atomicAdd(reinterpret_cast<float4 *>(out + dr * A.ostride + col),
+                                atomicAdd(reinterpret_cast<float4 *>(out + (size_t)dr * A.ostride + col),
                                           *reinterpret_cast<const float4 *>(st + row * PAIR_ST + (lane & 7) * 4));
                         }
                     } else {
-                        for (int row = 0; row < min(mine, 32); ++row) {
-                            const int64_t dr = __shfl_sync(0xffffffffu, drow, row);
-                            if (c0 + lane < nout) atomicAdd(out + dr * A.ostride + c0 + lane, st[row * PAIR_ST + lane]);
+                        for (int row = 0; row < mine; ++row) {
+                            const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
+                            if (c0 + lane < nout)
+                                atomicAdd(out + (size_t)dr * A.ostride + c0 + lane, st[row * PAIR_ST + lane]);
                         }
                     }
                     __syncwarp();
                 }
             }
             tc_fence_before();
-            mbar_arrive(&s_accempty[buf]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_accempty[buf]);
         }
     }
-    if (!ok) s_bad = 1;
+    if (!ok) atomicOr(&s_bad, 1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -469,12 +548,12 @@ void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, 
         FFM_LAUNCH(k_op_image<false>, g, 256, 0, s, F.T, F.n_trans, r, rk, F.h_nb, F.h_bpc, F.h_nb, F.h_nk, sc, (__half *)F.Th);
 }
 
-template <int NSTG>
+template <int NSTG, int CPS, bool STACK>
 static void launch_pairs(const PairArgs &A, unsigned grid, cudaStream_t s) {
-    const size_t sm = pair_smem(NSTG, A.npad, A.n_trans);
+    const size_t sm = pair_smem(NSTG * CPS, A.npad, A.n_trans);
     // per device and cheap: set before every launch (plans may live on several devices)
-    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    FFM_LAUNCH_NAMED("k_lag_pairs", k_lag_pairs<NSTG>, grid, PAIR_T, sm, s, A);
+    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG, CPS, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    FFM_LAUNCH_NAMED("k_lag_pairs", (k_lag_pairs<NSTG, CPS, STACK>), grid, PAIR_T, sm, s, A);
 }
 
 // v~ += T u~ for all pairs of the level: u has rows of K floats per (source box, right-hand side),
@@ -488,7 +567,7 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     PairArgs A{};
     __half *img = tmp.get<__half>((size_t)nrow * F.h_nk * HROW);
     float *inv = tmp.get<float>(nrow);
-    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, K, F.h_nk, img, inv);
+    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, K, F.h_nk, img, inv, (const uint32_t *)nullptr);
     A.bt_off = F.bt_off;
     A.bt_src = F.bt_src;
     A.bt_tgt = F.bt_tgt;
@@ -501,9 +580,9 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.tinv = F.h_inv;
     A.nk = F.h_nk;
     A.npad = F.h_nb;
-    A.stack = F.h_nb <= 128;
+    const bool stack = A.npad <= 128;
     A.tcols = 32;
-    while (A.tcols < (A.stack ? 2 : 1) * A.npad) A.tcols <<= 1;
+    while (A.tcols < (stack ? 2 : 1) * A.npad) A.tcols <<= 1;
     A.ostride = rows;
     const int64_t vblk = (int64_t)rows * nrhs * p->bx[l].nb;
     for (int b = 0; b < A.nblk; ++b) {
@@ -516,13 +595,422 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.tries = p->wait_tries;
     const int64_t most = ((int64_t)F.n_trans + F.n_adm * nrhs / HM) * A.nblk;  // at least the number of units
     const unsigned grid = (unsigned)std::min<int64_t>(most, 152);
-    if (A.npad <= 64)
-        launch_pairs<8>(A, grid, s);
-    else if (A.npad <= 128)
-        launch_pairs<6>(A, grid, s);
+    // stages of two chunks where the K extent allows: half the barrier round trips
+    if (A.npad <= 64 && A.nk % 2 == 0)
+        launch_pairs<4, 2, true>(A, grid, s);
+    else if (A.npad <= 64)
+        launch_pairs<8, 1, true>(A, grid, s);
+    else if (stack)
+        launch_pairs<6, 1, true>(A, grid, s);
     else
-        launch_pairs<4>(A, grid, s);
+        launch_pairs<4, 1, false>(A, grid, s);
     tmp.drop(inv);
+    tmp.drop(img);
+}
+
+// ---- target-stationary transfer (real operators, r <= 64)
+//
+// For levels whose targets have many partners (volumes: 290-360 of 665 translations).  A block owns
+// TG_M = 128 consecutive target boxes (TMEM lane = box) and runs over the translations present
+// among their pairs; the products accumulate and each target's v~ is written once: no adds to
+// memory, no grouping of all pairs by translation.  k_tile_entries orders each tile's pairs by
+// translation once per plan.
+//
+// What bounds it: the gathered rows' and the operators' way from L2 (48 KB a step at most).  A step is
+// one translation: warps 9-12 fetch the steps' (row, source) entries in turn and lay them out by row
+// in a shared ring, so that no copying thread waits for a list; warps 0-3 copy the 128 source rows
+// (hi and lo images, 16-byte cp.async segments, rows without a partner zero-filled without a
+// read), thread 0 starts the bulk copy of T_t's image, warp 8 issues hi [hi; lo] (N = 2 npad) and
+// lo hi, 4 steps in flight (8 where K <= 32).  Nothing is converted on the way.
+// Rows of different sources meet in one accumulator, so the level shares one scale (k_level_max):
+// a value keeps its 22 bits down to 2^-15 of the level's largest, and below that an absolute
+// error of 2^-39 of it.
+//
+// One long tensor-core accumulation loses accuracy, so the block alternates between two TMEM
+// accumulators every TG_DRAIN translations; warps 4-7 add each finished one into FP32 registers
+// while the other fills.  Every wait is bounded as in k_lag_pairs.
+//
+// Measured on GB300, level 7 of clustered 10M (193k targets, 68M pairs): 3.52 ms, 0.53 us a step
+// (the kernel before it, FP32 rows split into TF32 by the copying warps: 7.9 ms).
+constexpr int TG_M = 128;
+constexpr int TG_DRAIN = 8;        // translations per accumulator fill
+constexpr int TG_MAXT = 4096;      // translation indices are below this
+constexpr int TG_T = 416;
+constexpr int TG_IX = 8;           // steps whose sources are held by row
+
+// The pairs of each tile of TG_M targets ordered by translation: entry e of the tile (at the tile's
+// first pair) holds a source box and the target's row in the tile; step k of the tile is its k-th
+// translation present, t | first entry << 12.  One block per tile: counts per translation in shared
+// memory, their prefix sums, then every pair takes the next place of its translation (the order
+// of a step's entries does not matter: their rows differ).
+__global__ void __launch_bounds__(256) k_tile_entries(const uint32_t *__restrict__ adm_off, int64_t n_tgt,
+                                                      const uint32_t *__restrict__ adm_src,
+                                                      const uint32_t *__restrict__ adm_t, int n_trans,
+                                                      uint32_t *__restrict__ ent_src, uint8_t *__restrict__ ent_row,
+                                                      uint32_t *__restrict__ steps, uint32_t *__restrict__ nsteps) {
+    __shared__ uint32_t cnt[TG_MAXT];
+    __shared__ uint32_t wsum[8], wstep[8];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t x0 = (int64_t)blockIdx.x * TG_M, x1 = min(n_tgt, x0 + TG_M);
+    for (int t = tid; t < TG_MAXT; t += 256) cnt[t] = 0u;
+    __syncthreads();
+    const uint32_t e0 = adm_off[x0], e1 = adm_off[x1];
+    for (uint32_t e = e0 + tid; e < e1; e += 256) atomicAdd(&cnt[adm_t[e]], 1u);
+    __syncthreads();
+    // thread i owns translations 16 i .. + 15: first entry and step number of each
+    constexpr int PER = TG_MAXT / 256;
+    uint32_t c[PER], sum = 0, st = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        c[j] = cnt[tid * PER + j];
+        sum += c[j];
+        st += c[j] > 0;
+    }
+    uint32_t isum = sum, ist = st;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t a = __shfl_up_sync(0xffffffffu, isum, o), b = __shfl_up_sync(0xffffffffu, ist, o);
+        if (lane >= o) {
+            isum += a;
+            ist += b;
+        }
+    }
+    if (lane == 31) {
+        wsum[warp] = isum;
+        wstep[warp] = ist;
+    }
+    __syncthreads();
+    uint32_t off = isum - sum, k = ist - st;
+    for (int w = 0; w < warp; ++w) {
+        off += wsum[w];
+        k += wstep[w];
+    }
+    uint32_t *out = steps + (size_t)blockIdx.x * n_trans;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        cnt[tid * PER + j] = off;
+        if (c[j] > 0) out[k++] = (uint32_t)(tid * PER + j) | (off << 12);
+        off += c[j];
+    }
+    if (tid == 255) nsteps[blockIdx.x] = k;
+    __syncthreads();
+    for (int64_t x = x0 + warp; x < x1; x += 8)
+        for (uint32_t e = adm_off[x] + lane; e < adm_off[x + 1]; e += 32) {
+            const uint32_t o = e0 + atomicAdd(&cnt[adm_t[e]], 1u);
+            ent_src[o] = adm_src[e];
+            ent_row[o] = (uint8_t)(x - x0);
+        }
+}
+
+// The target-stationary transfer of a Lagrange level made possible (ts_ok), where the plan's rule, the
+// option, the autotuner or its cache asks for it.
+void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s) {
+    FarLevel &F = p->far[l];
+    if (F.mode != 1 || F.n_adm == 0 || F.ts_ok || !F.Th || p->kind != FFM_LAPLACE || F.r1 > 4) return;
+    const int64_t nt = cdiv(F.n_tgt, TG_M);
+    F.ts_src = p->mem.get<uint32_t>(F.n_adm);
+    F.ts_row = p->mem.get<uint8_t>(F.n_adm);
+    F.ts_steps = p->mem.get<uint32_t>((size_t)nt * F.n_trans);
+    F.ts_n = p->mem.get<uint32_t>(nt);
+    FFM_LAUNCH(k_tile_entries, (unsigned)nt, 256, 0, s, F.adm_off, F.n_tgt, F.adm_src, F.adm_t, F.n_trans, F.ts_src,
+               F.ts_row, F.ts_steps, F.ts_n);
+    F.ts_ok = true;
+}
+
+// largest |u| of the level's rows, as float bits (0 for an all-zero level)
+__global__ void k_level_max(const float *__restrict__ u, int64_t n, uint32_t *__restrict__ out) {
+    float mx = 0.f;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        mx = fmaxf(mx, fabsf(u[i]));
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx > 0.f) atomicMax(out, __float_as_uint(mx));
+}
+
+struct TargetArgs {
+    const uint32_t *tgt, *adm_off, *ent_src, *steps, *nsteps;
+    const uint8_t *ent_row;
+    int64_t n_tgt;
+    int n_trans, nrhs, nk, npad, r, tcols;
+    const __half *u;        // row images of (source box, right-hand side), one scale for all
+    const uint32_t *umax;   // that scale's value (k_level_max)
+    const __half *T;
+    float tinv;
+    float *vt;
+    int *err;
+    int tries;
+};
+
+template <int NSTG, int CPS>
+__global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__ TargetArgs A) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = aligned_smem(smem_raw);
+    __shared__ __align__(8) uint64_t s_full[NSTG], s_empty[NSTG], s_accfull[2], s_accempty[2], s_done;
+    __shared__ __align__(8) uint64_t s_ixfull[TG_IX], s_ixempty[TG_IX];
+    __shared__ uint32_t s_src[TG_IX][TG_M];  // the step's source box by row, NONE without a partner
+    __shared__ uint32_t s_trans[TG_IX];
+    __shared__ uint32_t s_tmem, s_cmax;
+    __shared__ int s_bad;
+    constexpr uint32_t NONE = 0xffffffffu;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m = blockIdx.y;
+    const int64_t x0 = (int64_t)blockIdx.x * TG_M;
+    const uint32_t bbytes = (uint32_t)A.npad * HROW * 2 * CPS, stage = CPS * A_BYTES + bbytes;
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
+                     "r"(2 * A.tcols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        s_bad = 0;
+        s_cmax = 0;
+        for (int i = 0; i < NSTG; ++i) {
+            mbar_init(&s_full[i], 129);  // the copying threads, and the operator copy's byte count
+            mbar_init(&s_empty[i], 1);
+        }
+        for (int i = 0; i < TG_IX; ++i) {
+            mbar_init(&s_ixfull[i], 1);
+            mbar_init(&s_ixempty[i], 4);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&s_accfull[i], 1);
+            mbar_init(&s_accempty[i], 4);
+        }
+        mbar_init(&s_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    const uint32_t nsteps = A.nsteps[blockIdx.x];
+    bool ok = true;
+    if (warp > 8) {
+        // ---- sources: warp w lays out steps w - 9, w - 9 + 4, ...
+        const uint32_t e0 = A.adm_off[x0], ne = A.adm_off[min(A.n_tgt, x0 + TG_M)] - e0;
+        const uint32_t *steps = A.steps + (size_t)blockIdx.x * A.n_trans;
+        for (uint32_t s = warp - 9; s < nsteps; s += 4) {
+            const uint32_t ix = s % TG_IX, rec = steps[s], nxt = s + 1 < nsteps ? steps[s + 1] : 0u;
+            const uint32_t f0 = rec >> 12, f1 = s + 1 < nsteps ? nxt >> 12 : ne;
+            uint32_t src[4];
+            int row[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {  // at most TG_M entries
+                const uint32_t f = f0 + 32 * g + lane;
+                row[g] = -1;
+                if (f < f1) {
+                    src[g] = A.ent_src[e0 + f];
+                    row[g] = A.ent_row[e0 + f];
+                }
+            }
+            const bool w_ok = s < TG_IX || mbar_wait(&s_ixempty[ix], ((s / TG_IX) - 1) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, w_ok)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) s_src[ix][32 * g + lane] = NONE;
+            __syncwarp();
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+                if (row[g] >= 0) s_src[ix][row[g]] = src[g];
+            if (lane == 0) s_trans[ix] = rec & 4095u;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_ixfull[ix]);
+        }
+    } else if (warp < 4) {
+        // ---- copies: lane handles 16-byte segment lane % 8 of rows 32 warp + 4 g + lane / 8 (g < 8)
+        const uint32_t r0 = 32 * warp + (lane >> 3), sg = lane & 7;
+        const uint32_t dst0 = smem_addr(smem) + r0 * 128, sw0 = (sg ^ (r0 & 7)) * 16, sw1 = (sg ^ ((r0 + 4) & 7)) * 16;
+        uint32_t c = 0;
+        for (uint32_t s = 0; s < nsteps && ok; ++s) {
+            const uint32_t ix = s % TG_IX;
+            const bool i_ok = mbar_wait(&s_ixfull[ix], (s / TG_IX) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, i_ok)) {
+                ok = false;
+                break;
+            }
+            const uint32_t t = s_trans[ix];
+            const __half *p[8];
+            uint32_t n[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const uint32_t sb = s_src[ix][r0 + 4 * g];
+                n[g] = sb != NONE ? 16u : 0u;
+                p[g] = A.u + ((size_t)(sb != NONE ? sb : 0u) * A.nrhs + m) * (CPS * HROW) + sg * 8;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_ixempty[ix]);
+            const uint32_t slot = c % NSTG;
+            const bool w_ok = c < NSTG || mbar_wait(&s_empty[slot], ((c / NSTG) - 1) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, w_ok)) {
+                ok = false;
+                break;
+            }
+            if (tid == 0) {
+                mbar_expect(&s_full[slot], bbytes);
+                bulk_g2s(smem + (size_t)slot * stage + CPS * A_BYTES, A.T + (size_t)t * CPS * A.npad * HROW, bbytes,
+                         &s_full[slot]);
+            }
+            const uint32_t dst = dst0 + slot * stage;
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+#pragma unroll
+                for (int j = 0; j < CPS; ++j)
+                    cp_async16_zfill(dst + j * A_BYTES + g * 512 + ((g & 1) ? sw1 : sw0), p[g] + j * HROW, n[g]);
+            cp_async_arrive(&s_full[slot]);
+            ++c;
+        }
+        // After a give-up some warps may have copied further than others: all arrive on every stage any of
+        // them started, so that the operator copies can be waited for.
+        if (!ok) atomicOr(&s_bad, 1);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        atomicMax(&s_cmax, c);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (s_bad) {
+            const uint32_t last = *reinterpret_cast<volatile uint32_t *>(&s_cmax);
+            for (; c < last; ++c) {
+                if (tid == 0) mbar_arrive(&s_full[c % NSTG]);
+                mbar_arrive(&s_full[c % NSTG]);
+            }
+        }
+        if (tid == 0)
+            for (uint32_t d = c > NSTG ? c - NSTG : 0; d < c; ++d)
+                mbar_wait(&s_full[d % NSTG], (d / NSTG) & 1, DRAIN_TRIES);
+    } else if (warp == 8) {
+        if (lane == 0) {
+            // ---- MMA thread
+            const uint32_t id1 = idesc_f16(A.npad), id2 = idesc_f16(2 * A.npad);
+            const uint32_t alo = a_dlo(smem_addr(smem)), blo = b_dlo(smem_addr(smem) + CPS * A_BYTES);
+            uint32_t slot = 0, par = 0;
+            for (uint32_t s = 0; s < nsteps; ++s) {
+                const uint32_t fill = s / TG_DRAIN, buf = fill & 1;
+                if (s % TG_DRAIN == 0 && fill >= 2 &&
+                    !mbar_wait(&s_accempty[buf], ((fill >> 1) - 1) & 1, A.tries, A.err)) {
+                    ok = false;
+                    break;
+                }
+                if (!mbar_wait(&s_full[slot], par, A.tries, A.err)) {
+                    ok = false;
+                    break;
+                }
+                fence_proxy_async();  // the rows came by cp.async, through the generic proxy
+                tc_fence_after();
+                const uint32_t off = slot * (stage >> 4);
+                stage_mma<CPS, true>(tmem + buf * (uint32_t)A.tcols, alo + off, blo + off, (uint32_t)A.npad, id1, id2,
+                                     s % TG_DRAIN == 0);
+                tc_commit(&s_empty[slot]);
+                if (s % TG_DRAIN == TG_DRAIN - 1 || s + 1 == nsteps) tc_commit(&s_accfull[buf]);
+                if (++slot == NSTG) {
+                    slot = 0;
+                    par ^= 1;
+                }
+            }
+            // everything issued is done before the block gives up its shared memory and TMEM
+            tc_commit(&s_done);
+            mbar_wait(&s_done, 0, DRAIN_TRIES);
+        }
+    } else {
+        // ---- sums: warp w holds lanes 32 (w - 4) .. + 31
+        const int q = warp - 4;
+        float sum[64];
+#pragma unroll
+        for (int c = 0; c < 64; ++c) sum[c] = 0.f;
+        const uint32_t fills = (nsteps + TG_DRAIN - 1) / TG_DRAIN;
+        for (uint32_t f = 0; f < fills; ++f) {
+            const uint32_t buf = f & 1;
+            const bool w_ok = mbar_wait(&s_accfull[buf], (f >> 1) & 1, A.tries, A.err);
+            if (!__all_sync(0xffffffffu, w_ok)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem + buf * (uint32_t)A.tcols + ((uint32_t)(32 * q) << 16);
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += 16) {
+                if (c0 < A.npad) {
+                    uint32_t v[16], w[16];
+                    tmem_ld16(v, d + (uint32_t)c0);
+                    tmem_ld16(w, d + (uint32_t)(A.npad + c0));
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum[c0 + j] += __uint_as_float(v[j]) + __uint_as_float(w[j]);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_accempty[buf]);
+        }
+        const int64_t x = x0 + 32 * q + lane;
+        if (ok && x < A.n_tgt) {
+            float us, ui;
+            row_scale(__uint_as_float(*A.umax), us, ui);
+            float *dst = A.vt + ((size_t)A.tgt[x] * A.nrhs + m) * A.r;
+#pragma unroll
+            for (int c = 0; c < 64; ++c) sum[c] = sum[c] * ui * A.tinv;
+            if (A.r == 64) {
+#pragma unroll
+                for (int c = 0; c < 64; c += 4)
+                    *reinterpret_cast<float4 *>(dst + c) = make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 64; ++c)
+                    if (c < A.r) dst[c] = sum[c];
+            }
+        }
+    }
+    if (!ok) atomicOr(&s_bad, 1);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (tid == 0 && s_bad) atomicOr(A.err, 1);
+    if (warp == 8)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * A.tcols));
+}
+
+template <int NSTG, int CPS>
+static void launch_targets(const TargetArgs &A, dim3 grid, cudaStream_t s) {
+    const size_t sm = 1024 + (size_t)NSTG * CPS * (A_BYTES + A.npad * HROW * 2);
+    FFM_CUDA(cudaFuncSetAttribute(k_lag_targets<NSTG, CPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    FFM_LAUNCH_NAMED("k_lag_targets", (k_lag_targets<NSTG, CPS>), grid, TG_T, sm, s, A);
+}
+
+// v~ = sum over each target's partners of T u~ (rows of targets without partners untouched)
+void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s) {
+    const FarLevel &F = p->far[l];
+    const int r = F.r1 * F.r1 * F.r1;
+    const int64_t nrow = (int64_t)p->by[l].nb * nrhs;
+    TargetArgs A{};
+    __half *img = tmp.get<__half>((size_t)nrow * F.h_nk * HROW);
+    uint32_t *mx = tmp.get<uint32_t>(1);
+    FFM_CUDA(cudaMemsetAsync(mx, 0, sizeof(uint32_t), s));
+    FFM_LAUNCH(k_level_max, (unsigned)std::min<int64_t>(cdiv(nrow * r, 1024), 152 * 8), 256, 0, s, u, nrow * r, mx);
+    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, r, F.h_nk, img, (float *)nullptr, (const uint32_t *)mx);
+    A.tgt = F.tgt;
+    A.adm_off = F.adm_off;
+    A.ent_src = F.ts_src;
+    A.ent_row = F.ts_row;
+    A.steps = F.ts_steps;
+    A.nsteps = F.ts_n;
+    A.n_trans = F.n_trans;
+    A.n_tgt = F.n_tgt;
+    A.nrhs = nrhs;
+    A.nk = F.h_nk;
+    A.npad = F.h_nb;
+    A.r = r;
+    A.tcols = 32;
+    while (A.tcols < 2 * A.npad) A.tcols <<= 1;
+    A.u = img;
+    A.umax = mx;
+    A.T = (const __half *)F.Th;
+    A.tinv = F.h_inv;
+    A.vt = vt;
+    A.err = p->dev_err;
+    A.tries = p->wait_tries;
+    const dim3 grid(cdiv(F.n_tgt, TG_M), nrhs);
+    if (A.nk == 2)
+        launch_targets<4, 2>(A, grid, s);
+    else  // r <= 27
+        launch_targets<8, 1>(A, grid, s);
+    tmp.drop(mx);
     tmp.drop(img);
 }
 

@@ -1033,89 +1033,16 @@ static uint2 *build_chunks(ffm_plan_s *p, const uint32_t *list, int64_t n, const
     return out;
 }
 
-// Admissible partners of each target box sorted by translation index, one warp per target.
-// Translations are distinct within a target and below 4096, so the sort is a rank by
-// counting: the warp sets one bit per partner's translation in a 4096-bit map in shared
-// memory, prefix-counts the map's words, and each partner's rank is the number of set bits
-// below its own.  Targets with more than 512 partners are left as they are and flagged.
-constexpr int SP_MAX = 512;
-__global__ void __launch_bounds__(128) k_sort_partners(const uint32_t *__restrict__ off, int64_t n_tgt,
-                                                       uint32_t *__restrict__ src, uint32_t *__restrict__ tr,
-                                                       int *__restrict__ too_long) {
-    __shared__ uint32_t bm[4][128], pre[4][128];
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int64_t x = (int64_t)blockIdx.x * 4 + w;
-    if (x >= n_tgt) return;  // warp-level work only: no block barrier below
-    uint32_t e0 = off[x];
-    int n = (int)(off[x + 1] - e0);
-    if (n > SP_MAX) {
-        if (lane == 0) atomicOr(too_long, 1);
-        return;
-    }
-    uint32_t *b = bm[w], *pr = pre[w];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[lane * 4 + j] = 0u;
-    __syncwarp();
-    uint32_t t[SP_MAX / 32], sv[SP_MAX / 32];
-#pragma unroll
-    for (int k = 0; k < SP_MAX / 32; ++k) {
-        int i = lane + 32 * k;
-        if (i < n) {
-            t[k] = tr[e0 + i];
-            sv[k] = src[e0 + i];
-            atomicOr(&b[t[k] >> 5], 1u << (t[k] & 31));
-        }
-    }
-    __syncwarp();
-    uint32_t c[4], tot = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        c[j] = __popc(b[lane * 4 + j]);
-        tot += c[j];
-    }
-    uint32_t inc = tot;
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-    }
-    uint32_t run = inc - tot;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        pr[lane * 4 + j] = run;
-        run += c[j];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < SP_MAX / 32; ++k) {
-        int i = lane + 32 * k;
-        if (i < n) {
-            uint32_t q = t[k];
-            uint32_t rank = pr[q >> 5] + __popc(b[q >> 5] & ((1u << (q & 31)) - 1u));
-            tr[e0 + rank] = q;
-            src[e0 + rank] = sv[k];
-        }
-    }
-}
-
-// Data of the target-stationary transfer for Lagrange level l, made on demand (it is used
-// when forced or picked by the autotuner): partners sorted by translation within each
-// target (the sort keeps every other consumer of the CSR lists valid) and T_t pre-split.
-// Sets ts_ok if every target has at most 512 partners.
-void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s) {
-    FarLevel &F = p->far[l];
-    if (F.mode != 1 || F.n_adm == 0 || F.Tsp || p->kind != FFM_LAPLACE || F.r1 > 4) return;
-    Alloc tmp;
-    tmp.stream = s;
-    int *flag = tmp.get<int>(1);
-    FFM_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
-    FFM_LAUNCH(k_sort_partners, cdiv(F.n_tgt, 4), 128, 0, s, F.adm_off, F.n_tgt, F.adm_src, F.adm_t, flag);
-    launch_table_split(p, l, s);
-    int hflag = 1;
-    FFM_CUDA(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    FFM_CUDA(cudaStreamSynchronize(s));
-    F.ts_ok = hflag == 0;
-    // a level the target-stationary kernel cannot take runs the per-translation transfer
-    if (!F.ts_ok) build_translation_groups(p, l, s);
+// Whether a level runs the target-stationary transfer when nothing else decides.  Measured on GB300 at
+// r = 64: that transfer takes 0.53 us per translation of a 128-target tile, one tile per SM at a
+// time, whatever the tile's pairs; the one by translation 9.0e-5 us per pair (from 1.4M pairs on), and
+// grouping the pairs for it about as much again in the plan.  So it pays from about 3000 (one product)
+// to 5900 (many products) pairs per translation and wave of tiles.  Both sides, us: clustered 10M level 7
+// (68M pairs, 10 waves) 3520 / 6139, level 6 (11M, 2 waves) 709 / 1006, level 5 (1.4M, 1 wave)
+// 356 / 141; volume 2M level 5 (11.9M, 2 waves) 704 / 1087; sphere 2M level 7 (5.5M, 4 waves) 631 / 511.
+static bool target_stationary_pays(const FarLevel &F) {
+    const int64_t waves = (F.n_tgt + 128 * 152 - 1) / (128 * 152);
+    return F.n_adm >= 4000 * (int64_t)F.n_trans * waves;
 }
 
 // Column tiles of the per-translation transfer: tile i of translation t covers pairs
@@ -1243,10 +1170,11 @@ static void finish_far_level(ffm_plan_s *p, int l, uint32_t *aa, uint32_t *ab, i
         if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
         // pairs grouped by translation for the per-translation transfer kernels, unless the
         // level is to run the target-stationary transfer, which reads the per-target lists
-        // (forced, or the pick stored in the plan's autotune cache); ACA levels need them
+        // (forced, the pick stored in the plan's autotune cache, or the rule); ACA levels need them
         const int pick = p->lag_transfer == 0 ? cached_lag_pick(p, l) : -1;
-        const bool ts_first = (p->lag_transfer == 3 || pick == 2) && p->kind == FFM_LAPLACE && F.r1 <= 4 &&
-                              !(p->aca_eps > 0.0);
+        const bool ts_can = p->kind == FFM_LAPLACE && F.r1 <= 4 && !(p->aca_eps > 0.0);
+        if (ts_can && p->lag_transfer == 0 && pick < 0 && target_stationary_pays(F)) F.tune_tc = 2;
+        const bool ts_first = ts_can && (F.tune_tc == 2 || pick == 2);
         if (!ts_first) build_translation_groups(p, l, s);
         if (p->lag_transfer == 1 || pick == 0 || p->aca_eps > 0.0) build_group_tiles(p, l, s);
         F.src_chunks = build_chunks(p, F.src, F.n_src, p->by[l].start, &F.n_src_chunks, tmp, s);
@@ -1493,8 +1421,8 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
     }
     for (int l = 0; l <= ls; ++l)
         if (p->far[l].n_adm > 0) build_octants(p, l, tj);
-    if (p->lag_transfer == 3)
-        for (int l = 0; l <= ls; ++l) prepare_target_stationary(p, l, s);
+    for (int l = 0; l <= ls; ++l)
+        if (p->far[l].tune_tc == 2) prepare_target_stationary(p, l, s);
     // plane-wave levels whose F steps run as type-3 NUFFTs: FP32 levels with many directions
     // (the NUFFT's cost per box barely depends on nQ, the direct sums' grows with it), all
     // FP32 and compensated-FP32 levels when forced, none when direct sums are forced

@@ -1,4 +1,4 @@
-"""The f16 hi / lo tensor-core transfer by translation against the CUDA-core transfer of the same
+"""The f16 hi / lo tensor-core transfers (by translation, and target-stationary) against the CUDA-core transfer of the same
 plan constants, at the edges of its tiles: operator rows that pad (r1 = 2, 3, 5, 7), fill one, two and
 four row blocks, K chunks with remainders, tiles of one pair, rows of several right-hand sides that
 cross tiles, complex operators, stacked and component operators.
@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 TOL = 3e-6
 
 
-def _pair(kernel, r1, nrhs, n=3000, scale=1.0, spread=False):
+def _pair(kernel, r1, nrhs, n=3000, scale=1.0, spread=False, variant=ffm.LAG_TC_TRANSLATION):
     rng = np.random.default_rng(r1 + 10 * nrhs)
     X, Y = scale * W.cube_volume(n, 1), scale * W.cube_volume(n - 7, 2)
     k = 1.0 / scale if kernel == ffm.HELMHOLTZ else 0.0
@@ -30,7 +30,7 @@ def _pair(kernel, r1, nrhs, n=3000, scale=1.0, spread=False):
     u = torch.as_tensor(u.astype(np.complex64 if kernel == ffm.HELMHOLTZ else np.float32), device="cuda")
     t = lambda a: torch.as_tensor(a, device="cuda")
     out = []
-    for variant in (ffm.LAG_TC_TRANSLATION, ffm.LAG_CUDA_CORES):
+    for variant in (variant, ffm.LAG_CUDA_CORES):
         with ffm.Plan(t(X), t(Y), kernel, k, 1e-3, r1_override=r1, n_leaf=16, kappa_switch=1e9,
                       normals=t(Y) if kernel == ffm.LAPLACE_DL else None, lagrange_transfer=variant) as p:
             v = p.apply(u)
@@ -54,6 +54,31 @@ def test_matches_the_cuda_core_transfer(kernel, r1):
 def test_several_right_hand_sides(kernel, nrhs):
     a, b = _pair(kernel, 4, nrhs, n=1200)
     assert O.rel_l2(a, b) < TOL
+
+
+@pytest.mark.parametrize("nrhs,n", [(1, 3000), (3, 1200), (1, 12000)])
+@pytest.mark.parametrize("r1", [2, 3, 4])
+def test_target_stationary(r1, nrhs, n):
+    a, b = _pair(ffm.LAPLACE, r1, nrhs, n=n, variant=ffm.LAG_TC_TARGET)
+    assert O.rel_l2(a, b) < TOL
+
+
+def test_the_rule_takes_a_level_of_many_pairs_to_the_target_stationary_transfer():
+    n = 700_000
+    X, Y = (torch.as_tensor(W.cube_volume(n, s), device="cuda") for s in (1, 2))
+    u = torch.as_tensor(np.random.default_rng(3).standard_normal(n).astype(np.float32), device="cuda")
+    out = []
+    for variant in (ffm.LAG_DEFAULT, ffm.LAG_TC_TRANSLATION):
+        with ffm.Plan(X, Y, ffm.LAPLACE, 0.0, 1e-3, lagrange_transfer=variant) as p:
+            out.append(p.apply(u).double())
+            info = p.info()
+        assert info["device_errors"] == 0
+        many = [l for l in range(22) if info["n_adm"][l] >= 4000 * info["n_trans"][l] * -(-info["n_tgt_boxes"][l] // 19456) > 0]
+        assert many
+        for l in range(22):
+            if info["n_adm"][l]:
+                assert info["tune_tc"][l] == (2 if variant == ffm.LAG_DEFAULT and l in many else 1)
+    assert float((out[0] - out[1]).norm() / out[1].norm()) < TOL
 
 
 @pytest.mark.parametrize("scale", [1e-12, 1e12])
