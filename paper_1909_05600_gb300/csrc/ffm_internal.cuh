@@ -109,7 +109,6 @@ void scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total, A
 // Stable LSD radix sort of (key, val) by the key bits [0, nbits).  Buffers are
 // ping-ponged; the sorted data ends in (keys, vals) on return.
 void radix_sort_u64(uint64_t *keys, uint32_t *vals, int64_t n, int nbits, Alloc &al, cudaStream_t s);
-void radix_sort_u32(uint32_t *keys, uint32_t *vals, int64_t n, int nbits, Alloc &al, cudaStream_t s);
 
 // ----------------------------------------------------------- the plan
 
@@ -119,7 +118,7 @@ struct BoxLevel {
     int4 *g = nullptr;          // integer box coordinates at this level
     uint32_t *first_leaf = nullptr;  // nb+1: first leaf (stop-level box) of each box
     uint32_t *first_child = nullptr; // nb+1: first child in the next level (descent only)
-    uint32_t *fine = nullptr;   // nb: index of the first box of the deepest table
+    uint32_t *fine = nullptr;   // nb+1: index of the first box of the deepest table
 };
 
 // Type-3 NUFFT of a plane-wave level (nufft.cu): grids, direction windows, point blocks
@@ -292,9 +291,10 @@ void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt
 int cached_lag_pick(const ffm_plan_s *p, int l);
 
 // tree.cu: near-field work items with targets in chunks of tchunk and at most smax source
-// points per item, allocated from out_mem; returns their number.
+// points per item, allocated from out_mem; returns their number (and the near field's point
+// pairs in *pairs).
 int64_t build_p2p_items(ffm_plan_s *p, int tchunk, uint32_t smax, Alloc &out_mem, int4 **items, Alloc &tmp,
-                        cudaStream_t s);
+                        cudaStream_t s, int64_t *pairs = nullptr);
 
 // tables.cu
 // Host staging buffers that must outlive the asynchronous copies reading them.

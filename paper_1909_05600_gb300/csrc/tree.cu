@@ -333,9 +333,6 @@ static void radix_sort(K *keys, uint32_t *vals, int64_t n, int nbits, Alloc &al,
 void radix_sort_u64(uint64_t *keys, uint32_t *vals, int64_t n, int nbits, Alloc &al, cudaStream_t s) {
     radix_sort<unsigned long long>((unsigned long long *)keys, vals, n, nbits, al, s);
 }
-void radix_sort_u32(uint32_t *keys, uint32_t *vals, int64_t n, int nbits, Alloc &al, cudaStream_t s) {
-    radix_sort<uint32_t>(keys, vals, n, nbits, al, s);
-}
 
 // ========================================================== bounding cubes
 
@@ -443,66 +440,123 @@ __global__ void k_split_sorted(const uint64_t *__restrict__ keys, const uint32_t
     }
 }
 
-// First level at which point i and point i-1 lie in different boxes; counts per level.
-__global__ void k_levels(const uint64_t *__restrict__ key, int64_t n, uint8_t *__restrict__ f,
-                         unsigned long long *__restrict__ counts) {
-    __shared__ unsigned int c[LMAX + 1];
-    if (threadIdx.x <= LMAX) c[threadIdx.x] = 0;
+// ---- box tables of both sets, every level at once
+//
+// A point starts a box at every level from the first one at which it and its predecessor in Morton
+// order differ.  Pass 1 finds that level per point and counts, per tile of BT_TILE points, the
+// points that start a box at each level; pass 2 scans the tiles' counts level by level; pass 3
+// (k_box_emit) ranks the tile's points again and writes every level's tables: start, integer
+// coordinates, parent, first child, and rank in the deepest level.  Three launches for both sets and
+// all levels, where a flag, scan, compaction, coordinate and search launch per level and set made
+// about a hundred (20k points: 0.55 of 2.3 ms of kernels).
+constexpr int BT_TILE = 4096, BT_T = 256, BT_PER = BT_TILE / BT_T;
+
+struct SetPts {
+    const uint64_t *key;
+    int64_t n;
+    uint8_t *f;       // first level at which the point starts a box (LMAX + 1: none)
+    uint32_t *cnt;    // LMAX + 1 rows of ntile counts, then their exclusive scans
+    int64_t ntile;
+};
+struct SetPair {
+    SetPts s[2];
+};
+
+__global__ void __launch_bounds__(BT_T) k_level_marks(SetPair P) {
+    const SetPts S = P.s[blockIdx.y];
+    if (blockIdx.x >= S.ntile) return;
+    __shared__ uint32_t c[LMAX + 2];
+    if (threadIdx.x < LMAX + 2) c[threadIdx.x] = 0;
     __syncthreads();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        int lev = 0;
-        if (i > 0) {
-            uint64_t d = key[i] ^ key[i - 1];
-            lev = d ? LMAX - (63 - __clzll((long long)d)) / 3 : LMAX + 1;
+    const int64_t i0 = (int64_t)blockIdx.x * BT_TILE;
+    for (int j = 0; j < BT_PER; ++j) {
+        const int64_t i = i0 + j * BT_T + threadIdx.x;
+        int lev = LMAX + 1;
+        if (i < S.n) {
+            lev = 0;
+            if (i > 0) {
+                const uint64_t d = S.key[i] ^ S.key[i - 1];
+                lev = d ? LMAX - (63 - __clzll((long long)d)) / 3 : LMAX + 1;
+            }
+            S.f[i] = (uint8_t)lev;
         }
-        f[i] = (uint8_t)lev;
-        if (i > 0 && lev <= LMAX) atomicAdd(&c[lev], 1u);
+        const uint32_t peers = __match_any_sync(0xffffffffu, lev);
+        if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&c[lev], (uint32_t)__popc(peers));
     }
     __syncthreads();
-    if (threadIdx.x <= LMAX && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], (unsigned long long)c[threadIdx.x]);
-}
-
-__global__ void k_flag_le(const uint8_t *__restrict__ f, int64_t n, int l, uint32_t *__restrict__ flag) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = (f[i] <= l) ? 1u : 0u;
-}
-
-// Deepest box table: starts of boxes (points with f <= l) and each box's f value.
-__global__ void k_compact_pts(const uint8_t *__restrict__ f, const uint32_t *__restrict__ pos, int64_t n, int l,
-                              uint32_t *__restrict__ start, uint8_t *__restrict__ bf, int64_t nb) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && f[i] <= l) {
-        start[pos[i]] = (uint32_t)i;
-        bf[pos[i]] = f[i];
+    if (threadIdx.x <= LMAX) {
+        uint32_t sum = 0;
+        for (int l = 0; l <= (int)threadIdx.x; ++l) sum += c[l];
+        S.cnt[(int64_t)threadIdx.x * S.ntile + blockIdx.x] = sum;
     }
-    if (i == 0) start[nb] = (uint32_t)n;
 }
 
-// Coarser table from the deepest one: boxes of the deep table with f <= l.
-__global__ void k_compact_boxes(const uint8_t *__restrict__ bf, const uint32_t *__restrict__ dstart,
-                                const uint32_t *__restrict__ pos, int64_t nd, int l, int64_t n,
-                                uint32_t *__restrict__ start, uint32_t *__restrict__ fine, int64_t nb) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nd && bf[i] <= l) {
-        start[pos[i]] = dstart[i];
-        fine[pos[i]] = (uint32_t)i;
+// one block per (level, set): exclusive scan of the level's tile counts; total in tot[set][level]
+__global__ void __launch_bounds__(1024) k_level_scan(SetPair P, uint32_t *__restrict__ tot) {
+    const SetPts S = P.s[blockIdx.y];
+    uint32_t *row = S.cnt + (int64_t)blockIdx.x * S.ntile;
+    __shared__ uint32_t sw[32];
+    __shared__ uint32_t t;
+    uint32_t carry = 0;
+    for (int64_t b = 0; b < S.ntile; b += 1024) {
+        const int64_t i = b + threadIdx.x;
+        const uint32_t v = i < S.ntile ? row[i] : 0u;
+        const uint32_t e = block_excl_scan(v, sw, &t);
+        if (i < S.ntile) row[i] = e + carry;
+        carry += t;
+        __syncthreads();
     }
-    if (i == 0) start[nb] = (uint32_t)n;
+    if (threadIdx.x == 0) tot[blockIdx.y * (LMAX + 1) + blockIdx.x] = carry;
 }
 
-__global__ void k_iota(uint32_t *a, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = (uint32_t)i;
-}
+struct BoxOut {
+    uint32_t *start[LMAX + 1], *first_child[LMAX + 1], *fine[LMAX + 1], *parent[LMAX + 1];
+    int4 *g[LMAX + 1];
+    uint32_t nb[LMAX + 1];
+};
 
-__global__ void k_box_coords(const uint64_t *__restrict__ key, const uint32_t *__restrict__ start, int64_t nb,
-                             int l, int4 *__restrict__ g) {
-    int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    uint64_t k = key[start[b]];
-    int sh = LMAX - l;
-    g[b] = make_int4((int)(compact3(k >> 2) >> sh), (int)(compact3(k >> 1) >> sh), (int)(compact3(k) >> sh), 0);
+__global__ void __launch_bounds__(BT_T) k_box_emit(const __grid_constant__ SetPts S, const __grid_constant__ BoxOut O,
+                                                   int ldeep) {
+    __shared__ uint32_t run[LMAX + 1][BT_T];  // boxes before the thread's points, per level
+    __shared__ uint32_t sw[BT_T / 32], tot;
+    const int64_t i0 = (int64_t)blockIdx.x * BT_TILE + (int64_t)threadIdx.x * BT_PER;
+    uint8_t f[BT_PER];
+#pragma unroll
+    for (int j = 0; j < BT_PER; ++j) f[j] = i0 + j < S.n ? S.f[i0 + j] : (uint8_t)(LMAX + 1);
+    for (int l = 0; l <= ldeep; ++l) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < BT_PER; ++j) c += f[j] <= l;
+        const uint32_t e = block_excl_scan(c, sw, &tot);
+        run[l][threadIdx.x] = S.cnt[(int64_t)l * S.ntile + blockIdx.x] + e;
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (int j = 0; j < BT_PER; ++j) {
+        const int fl = f[j];
+        if (fl > ldeep) continue;
+        const int64_t i = i0 + j;
+        const uint64_t k = S.key[i];
+        const uint32_t cx = (uint32_t)compact3(k >> 2), cy = (uint32_t)compact3(k >> 1), cz = (uint32_t)compact3(k);
+        const uint32_t deep = run[ldeep][threadIdx.x];
+        uint32_t up = fl > 0 ? run[fl - 1][threadIdx.x] - 1u : 0u;  // the box of level fl - 1 that holds the point
+        for (int l = fl; l <= ldeep; ++l) {
+            const uint32_t r = run[l][threadIdx.x]++;
+            const int sh = LMAX - l;
+            O.start[l][r] = (uint32_t)i;
+            O.g[l][r] = make_int4((int)(cx >> sh), (int)(cy >> sh), (int)(cz >> sh), 0);
+            O.fine[l][r] = deep;
+            if (O.parent[l]) O.parent[l][r] = up;
+            if (l > fl) O.first_child[l - 1][up] = r;
+            up = r;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x <= ldeep) {
+        const int l = threadIdx.x;
+        O.start[l][O.nb[l]] = (uint32_t)S.n;
+        O.fine[l][O.nb[l]] = O.nb[ldeep];
+        if (l < ldeep) O.first_child[l][O.nb[l]] = O.nb[l + 1];
+    }
 }
 
 // out[b] = first index j in sorted `hay` (length nh) with hay[j] >= needle[b]; out[nb] = nh.
@@ -527,10 +581,6 @@ __global__ void k_lower_bound(const uint32_t *__restrict__ needle, int64_t nb, c
 }
 
 // ================================================================== descent
-
-// Two-pass expansion without candidate arrays: pass 1 counts the admissible children of
-// each near pair, pass 2 writes admissible and near child pairs at their scanned offsets.
-// Children of (a, b) are visited in the same order in both passes.
 
 // Admissibility of a child pair as integer comparisons.  The offset test |sigma + k| >= 2
 // (k = g_X - g_Y per axis, sigma the trees' shift in box units, FP64) depends on k through
@@ -563,200 +613,353 @@ static AdmK adm_thresholds(const D3 &sig) {
     return K;
 }
 
-// One warp per near pair (a, b) of level l: lane c takes child pair c and c + 32 of the at
-// most 8 x 8 children (a2 = first child of a + c / nb, b2 = first child of b + c % nb);
-// ballots count and place the admissible ones and the near ones, so a warp writes its
-// pairs contiguously.
-constexpr int EXP_W = 8;  // warps (near pairs) per block
+// One warp per target box a2 of the child level: its candidates are the children of the sources
+// near its parent (CSR near_off, near_src over the parents), four near sources of up to eight
+// children per round.  Both passes visit them in the same order and test them alike; the
+// first counts the admissible and the near ones (and marks the translations and source boxes
+// in use), the second writes them at the scanned offsets.  The lists come out in CSR order by
+// target with no sort, each target's sources in the order of its parent's list, the order that a
+// stable sort by target of the expanded pairs gives.
+//
+// What bounds it: the candidates' coordinate loads (16 bytes each from L2) and, at 1e8 points, the
+// lists' 24 bytes per pair.  Expanding pairs and sorting them by target per level (an iota, a radix
+// sort, gathers, run starts, scans: about forty launches and eight read-backs a level) took 2.3 ms of
+// kernels at 20k points and 330 ms at 1e8.
+//
+// Translation code of a pair: integer offset m = gX - gY relative to c = round(-sigma 2^l), 4 bits
+// per axis (the descent bounds |sigma 2^l + m| < 5).
+constexpr int DS_W = 8;  // warps (targets in flight) per block
+struct DescendArgs {
+    int64_t n;                    // target boxes of the child level
+    const uint32_t *parent;
+    const uint32_t *near_off, *near_src;
+    const uint32_t *fcy;          // first children of the source boxes
+    const int4 *gx, *gy;          // child level
+    AdmK K;
+    int4 c;
+    uint32_t *cadm, *cnear;       // pass 1: counts; pass 2: offsets
+    uint32_t *used;               // 4096 flags by code
+    uint8_t *src_used;
+    int *err;
+    const uint32_t *tpos;         // pass 2: translation index by code
+    uint32_t *adm_src, *adm_t, *near_out;
+};
 
-__global__ void __launch_bounds__(32 * EXP_W) k_expand_count(const uint32_t *__restrict__ na,
-                                                            const uint32_t *__restrict__ nbb, int64_t nnear,
-                                                            const uint32_t *__restrict__ fcx,
-                                                            const uint32_t *__restrict__ fcy,
-                                                            const int4 *__restrict__ gx, const int4 *__restrict__ gy,
-                                                            AdmK K, uint32_t *__restrict__ nadm,
-                                                            uint32_t *__restrict__ nnr) {
-    const int lane = threadIdx.x & 31;
-    const int64_t e = (int64_t)blockIdx.x * EXP_W + (threadIdx.x >> 5);
-    if (e >= nnear) return;
-    const uint32_t a = na[e], b = nbb[e];
-    const uint32_t a0 = fcx[a], b0 = fcy[b];
-    const int nax = (int)(fcx[a + 1] - a0), nby = (int)(fcy[b + 1] - b0), tot = nax * nby;
-    uint32_t c = 0;
-    for (int c0 = 0; c0 < tot; c0 += 32) {
-        const int ci = c0 + lane;
-        bool adm = false;
-        if (ci < tot) adm = child_adm_k(gx[a0 + ci / nby], gy[b0 + ci % nby], K);
-        c += __popc(__ballot_sync(0xffffffffu, adm));
+template <bool EMIT>
+__global__ void __launch_bounds__(32 * DS_W) k_descend(const __grid_constant__ DescendArgs A) {
+    __shared__ uint32_t bits[EMIT ? 1 : 128];
+    __shared__ uint16_t pos[EMIT ? 4096 : 1];
+    const int lane = threadIdx.x & 31, sub = lane >> 3, cb = lane & 7;
+    if constexpr (EMIT) {
+        for (int i = threadIdx.x; i < 4096; i += blockDim.x) pos[i] = (uint16_t)A.tpos[i];
+    } else {
+        if (threadIdx.x < 128) bits[threadIdx.x] = 0u;
     }
-    if (lane == 0) {
-        nadm[e] = c;
-        nnr[e] = (uint32_t)tot - c;
-    }
-}
-
-__global__ void __launch_bounds__(32 * EXP_W) k_expand_emit(const uint32_t *__restrict__ na,
-                                                           const uint32_t *__restrict__ nbb, int64_t nnear,
-                                                           const uint32_t *__restrict__ fcx,
-                                                           const uint32_t *__restrict__ fcy,
-                                                           const int4 *__restrict__ gx, const int4 *__restrict__ gy,
-                                                           AdmK K, const uint32_t *__restrict__ oadm,
-                                                           const uint32_t *__restrict__ onr, uint32_t *__restrict__ aa,
-                                                           uint32_t *__restrict__ ab, uint32_t *__restrict__ ea,
-                                                           uint32_t *__restrict__ eb) {
-    const int lane = threadIdx.x & 31;
-    const int64_t e = (int64_t)blockIdx.x * EXP_W + (threadIdx.x >> 5);
-    if (e >= nnear) return;
-    const uint32_t a = na[e], b = nbb[e];
-    const uint32_t a0 = fcx[a], b0 = fcy[b];
-    const int nax = (int)(fcx[a + 1] - a0), nby = (int)(fcy[b + 1] - b0), tot = nax * nby;
-    uint32_t ia = oadm[e], in = onr[e];
+    __syncthreads();
     const uint32_t below = (1u << lane) - 1u;
-    for (int c0 = 0; c0 < tot; c0 += 32) {
-        const int ci = c0 + lane;
-        const bool valid = ci < tot;
-        uint32_t a2 = 0, b2 = 0;
-        bool adm = false;
-        if (valid) {
-            a2 = a0 + (uint32_t)(ci / nby);
-            b2 = b0 + (uint32_t)(ci % nby);
-            adm = child_adm_k(gx[a2], gy[b2], K);
-        }
-        const uint32_t ma = __ballot_sync(0xffffffffu, valid && adm), mn = __ballot_sync(0xffffffffu, valid && !adm);
-        if (valid) {
-            if (adm) {
-                uint32_t o = ia + __popc(ma & below);
-                aa[o] = a2;
-                ab[o] = b2;
-            } else {
-                uint32_t o = in + __popc(mn & below);
-                ea[o] = a2;
-                eb[o] = b2;
+    for (int64_t x = (int64_t)blockIdx.x * DS_W + (threadIdx.x >> 5); x < A.n; x += (int64_t)gridDim.x * DS_W) {
+        const uint32_t par = A.parent[x], e0 = A.near_off[par], e1 = A.near_off[par + 1];
+        const int4 p = A.gx[x];
+        uint32_t ia = EMIT ? A.cadm[x] : 0u, in = EMIT ? A.cnear[x] : 0u;
+        for (uint32_t eb = e0; eb < e1; eb += 32) {
+            uint32_t b0 = 0, nb = 0;
+            if (eb + lane < e1) {
+                const uint32_t b = A.near_src[eb + lane];
+                b0 = A.fcy[b];
+                nb = A.fcy[b + 1] - b0;
+            }
+            const int ne = (int)min(32u, e1 - eb);
+            for (int j = 0; j < ne; j += 4) {
+                const uint32_t B0 = __shfl_sync(0xffffffffu, b0, j + sub), NB = __shfl_sync(0xffffffffu, nb, j + sub);
+                const bool valid = cb < (int)NB;  // lanes past the list have no children
+                const uint32_t b2 = B0 + cb;
+                bool adm = false;
+                uint32_t code = 0;
+                if (valid) {
+                    const int4 q = A.gy[b2];
+                    adm = child_adm_k(p, q, A.K);
+                    if (adm) {
+                        int mx = p.x - q.x - A.c.x + 8, my = p.y - q.y - A.c.y + 8, mz = p.z - q.z - A.c.z + 8;
+                        if (mx < 0 || mx > 15 || my < 0 || my > 15 || mz < 0 || mz > 15) {
+                            atomicOr(A.err, 1);
+                            mx = my = mz = 0;
+                        }
+                        code = (uint32_t)(mx | (my << 4) | (mz << 8));
+                    }
+                }
+                const uint32_t ma = __ballot_sync(0xffffffffu, adm), mn = __ballot_sync(0xffffffffu, valid && !adm);
+                if constexpr (EMIT) {
+                    if (adm) {
+                        const uint32_t o = ia + __popc(ma & below);
+                        A.adm_src[o] = b2;
+                        A.adm_t[o] = pos[code];
+                    } else if (valid) {
+                        A.near_out[in + __popc(mn & below)] = b2;
+                    }
+                } else if (adm) {
+                    const uint32_t bit = 1u << (code & 31);
+                    if (!(*reinterpret_cast<volatile uint32_t *>(&bits[code >> 5]) & bit)) atomicOr(&bits[code >> 5], bit);
+                    A.src_used[b2] = 1;
+                }
+                ia += __popc(ma);
+                in += __popc(mn);
             }
         }
-        ia += __popc(ma);
-        in += __popc(mn);
-    }
-}
-
-
-__global__ void k_gather_u32(const uint32_t *__restrict__ src, const uint32_t *__restrict__ idx, int64_t n,
-                             uint32_t *__restrict__ dst) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = src[idx[i]];
-}
-
-// Translation code of a pair: integer offset m = gX - gY relative to c = round(-sigma 2^l),
-// 4 bits per axis (the descent bounds |sigma 2^l + m| < 5).
-// Translation code of every pair; the codes in use are collected in a 4096-bit map per block
-// (shared atomics) and written once per block and code, not once per pair.
-__global__ void k_trans_code(const uint32_t *__restrict__ a, const uint32_t *__restrict__ b, int64_t n,
-                             const int4 *__restrict__ gx, const int4 *__restrict__ gy, int4 c,
-                             uint32_t *__restrict__ code, uint32_t *__restrict__ used, int *__restrict__ err) {
-    __shared__ uint32_t bits[128];
-    if (threadIdx.x < 128) bits[threadIdx.x] = 0u;
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int4 p = gx[a[i]], q = gy[b[i]];
-        int mx = p.x - q.x - c.x + 8, my = p.y - q.y - c.y + 8, mz = p.z - q.z - c.z + 8;
-        if (mx < 0 || mx > 15 || my < 0 || my > 15 || mz < 0 || mz > 15) {
-            atomicOr(err, 1);
-            mx = my = mz = 0;
+        if (!EMIT && lane == 0) {
+            A.cadm[x] = ia;
+            A.cnear[x] = in;
         }
-        uint32_t k = (uint32_t)(mx | (my << 4) | (mz << 8));
-        code[i] = k;
-        atomicOr(&bits[k >> 5], 1u << (k & 31));
+    }
+    if constexpr (!EMIT) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < 4096; k += blockDim.x)
+            if (bits[k >> 5] & (1u << (k & 31))) A.used[k] = 1u;
+    }
+}
+
+// ---- a level's lists from its counts: offsets of the admissible and near pairs by target, the
+// targets with admissible pairs and the sources in use, and both lists' point chunks (box, first
+// point) of at most ch points, so that the point-wise kernels spread large boxes over many blocks.
+// Tiles of LV_TILE boxes: sums per tile, a scan over the tiles in one block (which also numbers the
+// translations in use and leaves all totals in one place, the level's only read-back), then the lists.
+constexpr int LV_T = 256, LV_PER = 8, LV_TILE = LV_T * LV_PER;
+
+struct LevelTotals {
+    unsigned long long tgt_points, src_points;
+    uint32_t na, nn, ntgt, nsrc, tch, sch, ntrans, err;
+    uint32_t pw_sch, pw_tch;  // chunks of PW_TC_FCH source points and PW_TC_BCH target points
+    uint32_t bits[128];       // the translation codes in use
+};
+
+struct LevelArgsL {
+    int64_t nx, ny, ntx, nty;
+    uint32_t *cadm, *cnear;          // counts in, offsets out (nx + 1)
+    const uint8_t *src_used;
+    const uint32_t *xstart, *ystart;
+    uint32_t ch;
+    unsigned long long *ta, *tb;     // per tile: admissible << 32 | near (X); listed << 32 | chunks (X, then Y)
+    const uint32_t *used;
+    uint32_t *tpos;
+    LevelTotals *tot;
+    const int *err;
+    uint32_t *tgt, *adm_off, *src;
+    uint2 *tchunks, *schunks;
+};
+
+__device__ __forceinline__ unsigned long long warp_incl_scan64(unsigned long long v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// block-wide exclusive scan of one 64-bit value per thread
+__device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long long v, unsigned long long *sm,
+                                                                unsigned long long *tot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned long long inc = warp_incl_scan64(v);
+    if (lane == 31) sm[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long w = lane < nw ? sm[lane] : 0ull, wi = warp_incl_scan64(w);
+        if (lane < nw) sm[lane] = wi - w;
+        if (lane == nw - 1) *tot = wi;
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < 4096; k += blockDim.x)
-        if (bits[k >> 5] & (1u << (k & 31))) used[k] = 1u;
+    return inc - v + sm[warp];
 }
 
-__global__ void k_trans_list(const uint32_t *__restrict__ used, const uint32_t *__restrict__ pos, int4 c,
-                             int4 *__restrict__ m) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < 4096 && used[k]) m[pos[k]] = make_int4((k & 15) - 8 + c.x, ((k >> 4) & 15) - 8 + c.y, (k >> 8) - 8 + c.z, 0);
-}
-
-__global__ void k_map(const uint32_t *__restrict__ code, const uint32_t *__restrict__ pos, int64_t n,
-                      uint32_t *__restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = pos[code[i]];
-}
-
-__global__ void k_run_starts(const uint32_t *__restrict__ a, int64_t n, uint32_t *__restrict__ flag) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = (i == 0 || a[i] != a[i - 1]) ? 1u : 0u;
-}
-
-__global__ void k_run_list(const uint32_t *__restrict__ a, const uint32_t *__restrict__ flag,
-                           const uint32_t *__restrict__ pos, int64_t n, int64_t nruns, uint32_t *__restrict__ ids,
-                           uint32_t *__restrict__ off) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && flag[i]) {
-        ids[pos[i]] = a[i];
-        off[pos[i]] = (uint32_t)i;
+__global__ void __launch_bounds__(LV_T) k_level_sums(const __grid_constant__ LevelArgsL A) {
+    const bool X = blockIdx.x < A.ntx;
+    const int64_t tile = X ? blockIdx.x : blockIdx.x - A.ntx, n = X ? A.nx : A.ny;
+    const uint32_t *start = X ? A.xstart : A.ystart;
+    unsigned long long a = 0, b = 0, pts = 0;
+    uint32_t pw = 0;
+    for (int j = 0; j < LV_PER; ++j) {
+        const int64_t i = tile * LV_TILE + j * LV_T + threadIdx.x;
+        if (i >= n) break;
+        bool listed;
+        if (X) {
+            const uint32_t na = A.cadm[i];
+            a += ((unsigned long long)na << 32) | A.cnear[i];
+            listed = na > 0;
+        } else {
+            listed = A.src_used[i] != 0;
+        }
+        if (listed) {
+            const uint32_t sz = start[i + 1] - start[i];
+            b += (1ull << 32) | (A.ch ? (sz + A.ch - 1) / A.ch : 0u);
+            pts += sz;
+            pw += X ? (sz + PW_TC_BCH - 1) / PW_TC_BCH : (sz + PW_TC_FCH - 1) / PW_TC_FCH;
+        }
     }
-    if (i == 0) off[nruns] = (uint32_t)n;
+    __shared__ unsigned long long sm[32], t;
+    block_excl_scan64(a, sm, &t);
+    if (threadIdx.x == 0 && X) A.ta[tile] = t;
+    __syncthreads();
+    block_excl_scan64(b, sm, &t);
+    if (threadIdx.x == 0) A.tb[blockIdx.x] = t;
+    __syncthreads();
+    block_excl_scan64(pts, sm, &t);
+    if (threadIdx.x == 0 && t) atomicAdd(X ? &A.tot->tgt_points : &A.tot->src_points, t);
+    __syncthreads();
+    block_excl_scan64(pw, sm, &t);
+    if (threadIdx.x == 0 && t) atomicAdd(X ? &A.tot->pw_tch : &A.tot->pw_sch, (uint32_t)t);
 }
 
-__global__ void k_mark(const uint32_t *__restrict__ b, int64_t n, uint32_t *__restrict__ used) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) used[b[i]] = 1u;
-}
-
-__global__ void k_list_marked(const uint32_t *__restrict__ used, const uint32_t *__restrict__ pos, int64_t n,
-                              uint32_t *__restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && used[i]) out[pos[i]] = (uint32_t)i;
-}
-
-// sum over listed boxes of their point counts
-__global__ void k_sum_sizes(const uint32_t *__restrict__ list, int64_t n, const uint32_t *__restrict__ start,
-                            unsigned long long *__restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long v = 0;
-    if (i < n) v = start[list[i] + 1] - start[list[i]];
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(out, v);
-}
-
-// sum over pairs (a, b) of n_a * n_b
-__global__ void k_sum_pair_sizes(const uint32_t *__restrict__ a, const uint32_t *__restrict__ b, int64_t n,
-                                 const uint32_t *__restrict__ sa, const uint32_t *__restrict__ sb,
-                                 unsigned long long *__restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long v = 0;
-    if (i < n) v = (unsigned long long)(sa[a[i] + 1] - sa[a[i]]) * (sb[b[i] + 1] - sb[b[i]]);
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(out, v);
-}
-
-static int64_t read_u64(const unsigned long long *d, cudaStream_t s) {
-    unsigned long long h;
-    FFM_CUDA(cudaMemcpyAsync(&h, d, sizeof h, cudaMemcpyDeviceToHost, s));
-    FFM_CUDA(cudaStreamSynchronize(s));
-    return (int64_t)h;
-}
-
-__global__ void k_hist_u32(const uint32_t *__restrict__ a, int64_t n, uint32_t *__restrict__ cnt) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[a[i]], 1u);
-}
-
-// CSR offsets of a sorted key array: off[b] = first i with key[i] >= b, b = 0..nkeys.
-__global__ void k_csr_offsets(const uint32_t *__restrict__ key, int64_t n, int64_t nkeys, uint32_t *__restrict__ off) {
-    int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > nkeys) return;
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (key[mid] < (uint32_t)b)
-            lo = mid + 1;
-        else
-            hi = mid;
+__global__ void __launch_bounds__(1024) k_level_mid(const __grid_constant__ LevelArgsL A) {
+    __shared__ unsigned long long sm[32], t;
+    auto scan_row = [&](unsigned long long *row, int64_t n) {
+        unsigned long long carry = 0;
+        for (int64_t b = 0; b < n; b += 1024) {
+            const int64_t i = b + threadIdx.x;
+            const unsigned long long v = i < n ? row[i] : 0ull;
+            const unsigned long long e = block_excl_scan64(v, sm, &t);
+            if (i < n) row[i] = e + carry;
+            carry += t;
+            __syncthreads();
+        }
+        return carry;
+    };
+    const unsigned long long a = scan_row(A.ta, A.ntx), bx = scan_row(A.tb, A.ntx), by = scan_row(A.tb + A.ntx, A.nty);
+    uint32_t u[4], c = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        u[j] = c;
+        c += A.used[threadIdx.x * 4 + j];
     }
-    off[b] = (uint32_t)lo;
+    const uint32_t e = (uint32_t)block_excl_scan64(c, sm, &t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) A.tpos[threadIdx.x * 4 + j] = e + u[j];
+    if (threadIdx.x < 128) {
+        uint32_t w = 0;
+        for (int j = 0; j < 32; ++j) w |= (A.used[threadIdx.x * 32 + j] ? 1u : 0u) << j;
+        A.tot->bits[threadIdx.x] = w;
+    }
+    if (threadIdx.x == 0) {
+        A.tot->na = (uint32_t)(a >> 32);
+        A.tot->nn = (uint32_t)a;
+        A.tot->ntgt = (uint32_t)(bx >> 32);
+        A.tot->tch = (uint32_t)bx;
+        A.tot->nsrc = (uint32_t)(by >> 32);
+        A.tot->sch = (uint32_t)by;
+        A.tot->ntrans = (uint32_t)t;
+        A.tot->err = (uint32_t)*A.err;
+        A.cadm[A.nx] = (uint32_t)(a >> 32);
+        A.cnear[A.nx] = (uint32_t)a;
+        A.adm_off[bx >> 32] = (uint32_t)(a >> 32);
+    }
+}
+
+__global__ void __launch_bounds__(LV_T) k_level_lists(const __grid_constant__ LevelArgsL A) {
+    __shared__ unsigned long long sm[32], t;
+    __shared__ uint32_t cpos[LV_TILE + 1];  // first chunk of each box of the tile
+    const bool X = blockIdx.x < A.ntx;
+    const int64_t tile = X ? blockIdx.x : blockIdx.x - A.ntx, n = X ? A.nx : A.ny;
+    const int64_t i0 = tile * LV_TILE + (int64_t)threadIdx.x * LV_PER;
+    const uint32_t *start = X ? A.xstart : A.ystart;
+    unsigned long long a[LV_PER], b[LV_PER], sa = 0, sb = 0;
+#pragma unroll
+    for (int j = 0; j < LV_PER; ++j) {
+        const int64_t i = i0 + j;
+        a[j] = b[j] = 0;
+        if (i < n) {
+            bool listed;
+            if (X) {
+                const uint32_t na = A.cadm[i];
+                a[j] = ((unsigned long long)na << 32) | A.cnear[i];
+                listed = na > 0;
+            } else {
+                listed = A.src_used[i] != 0;
+            }
+            if (listed) {
+                const uint32_t sz = start[i + 1] - start[i];
+                b[j] = (1ull << 32) | (A.ch ? (sz + A.ch - 1) / A.ch : 0u);
+            }
+        }
+        sa += a[j];
+        sb += b[j];
+    }
+    unsigned long long ea = block_excl_scan64(sa, sm, &t);
+    if (X) ea += A.ta[tile];
+    __syncthreads();
+    unsigned long long eb = block_excl_scan64(sb, sm, &t) + A.tb[blockIdx.x];
+    const uint32_t c0 = (uint32_t)A.tb[blockIdx.x];
+#pragma unroll
+    for (int j = 0; j < LV_PER; ++j) {
+        const int64_t i = i0 + j;
+        cpos[threadIdx.x * LV_PER + j] = (uint32_t)eb - c0;
+        if (i < n) {
+            if (b[j]) {
+                const uint32_t r = (uint32_t)(eb >> 32);
+                if (X) {
+                    A.tgt[r] = (uint32_t)i;
+                    A.adm_off[r] = (uint32_t)(ea >> 32);
+                } else {
+                    A.src[r] = (uint32_t)i;
+                }
+            }
+            if (X) {
+                A.cadm[i] = (uint32_t)(ea >> 32);
+                A.cnear[i] = (uint32_t)ea;
+            }
+        }
+        ea += a[j];
+        eb += b[j];
+    }
+    if (threadIdx.x == LV_T - 1) cpos[LV_TILE] = (uint32_t)eb - c0;
+    __syncthreads();
+    if (!A.ch) return;
+    // the tile's chunks, consecutive in the list: each finds its box in the tile's positions
+    uint2 *out = (X ? A.tchunks : A.schunks) + c0;
+    const uint32_t m = cpos[LV_TILE];
+    for (uint32_t k = threadIdx.x; k < m; k += LV_T) {
+        int lo = 0, hi = LV_TILE;  // last box with cpos <= k
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (cpos[mid] <= k)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        const uint32_t box = (uint32_t)(tile * LV_TILE + lo);
+        out[k] = make_uint2(box, start[box] + (k - cpos[lo]) * A.ch);
+    }
+}
+
+// ---- pairs grouped by translation, for the transfers by translation: counts per translation, their
+// scan, then every block of GP_TGT targets reserves a range in each of its translations and places
+// its pairs there (the order within a translation decides nothing: the transfers add).
+constexpr int GP_TGT = 32, GP_MAXT = 4096;
+
+template <bool PLACE>
+__global__ void __launch_bounds__(256) k_group_pairs(const uint32_t *__restrict__ tgt, const uint32_t *__restrict__ off,
+                                                     int64_t n_tgt, const uint32_t *__restrict__ src,
+                                                     const uint32_t *__restrict__ tr, int n_trans,
+                                                     uint32_t *__restrict__ cursor, uint32_t *__restrict__ bt_src,
+                                                     uint32_t *__restrict__ bt_tgt) {
+    __shared__ uint32_t cnt[GP_MAXT];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t x0 = (int64_t)blockIdx.x * GP_TGT, x1 = min(n_tgt, x0 + GP_TGT);
+    for (int t = tid; t < n_trans; t += 256) cnt[t] = 0u;
+    __syncthreads();
+    const uint32_t e0 = off[x0], e1 = off[x1];
+    for (uint32_t e = e0 + tid; e < e1; e += 256) atomicAdd(&cnt[tr[e]], 1u);
+    __syncthreads();
+    for (int t = tid; t < n_trans; t += 256)
+        if (cnt[t]) cnt[t] = atomicAdd(&cursor[t], cnt[t]);
+    if constexpr (PLACE) {
+        __syncthreads();
+        for (int64_t x = x0 + warp; x < x1; x += 8)
+            for (uint32_t e = off[x] + lane; e < off[x + 1]; e += 32) {
+                const uint32_t o = atomicAdd(&cnt[tr[e]], 1u);
+                bt_src[o] = src[e];
+                bt_tgt[o] = tgt[x];
+            }
+    }
 }
 
 static uint32_t read_u32(const uint32_t *d, cudaStream_t s) {
@@ -769,11 +972,14 @@ static uint32_t read_u32(const uint32_t *d, cudaStream_t s) {
 // Near-field work items of one target leaf: its targets in chunks of tchunk times its
 // near pairs split into consecutive ranges of at most smax source points.
 __device__ __forceinline__ int p2p_ranges(const uint32_t *off, const uint32_t *src, const uint32_t *ystart, int64_t a,
-                                          int4 *out, int base, int tc, int tchunk, uint32_t smax) {
+                                          int4 *out, int base, int tc, int tchunk, uint32_t smax,
+                                          unsigned long long &sources) {
     int nr = 0;
     uint32_t e0 = off[a], acc = 0;
+    sources = 0;
     for (uint32_t e = off[a]; e < off[a + 1]; ++e) {
         uint32_t nb = ystart[src[e] + 1] - ystart[src[e]];
+        sources += nb;
         if (acc > 0 && acc + nb > smax) {
             if (out)
                 for (int c = 0; c < tc; ++c) out[base + nr * tc + c] = make_int4((int)a, c * tchunk, (int)e0, (int)e);
@@ -792,46 +998,49 @@ __device__ __forceinline__ int p2p_ranges(const uint32_t *off, const uint32_t *s
     return nr;
 }
 
+// Pass 1 (out null) counts the items per leaf and, with `pairs`, sums the point pairs n_a n_b.
 __global__ void k_p2p_items(const uint32_t *__restrict__ off, const uint32_t *__restrict__ src,
                             const uint32_t *__restrict__ xstart, const uint32_t *__restrict__ ystart, int64_t nleaf,
                             int tchunk, uint32_t smax, const uint32_t *__restrict__ pos, uint32_t *__restrict__ cnt,
-                            int4 *__restrict__ out) {
+                            int4 *__restrict__ out, unsigned long long *__restrict__ pairs) {
     int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= nleaf) return;
-    int np = (int)(xstart[a + 1] - xstart[a]);
-    int tc = (np + tchunk - 1) / tchunk;
-    if (!out) {
-        cnt[a] = (uint32_t)(p2p_ranges(off, src, ystart, a, nullptr, 0, tc, tchunk, smax) * tc);
-    } else {
-        p2p_ranges(off, src, ystart, a, out, (int)pos[a], tc, tchunk, smax);
+    unsigned long long v = 0;
+    if (a < nleaf) {
+        int np = (int)(xstart[a + 1] - xstart[a]);
+        int tc = (np + tchunk - 1) / tchunk;
+        if (!out) {
+            cnt[a] = (uint32_t)(p2p_ranges(off, src, ystart, a, nullptr, 0, tc, tchunk, smax, v) * tc);
+            v *= (unsigned long long)np;
+        } else {
+            p2p_ranges(off, src, ystart, a, out, (int)pos[a], tc, tchunk, smax, v);
+        }
     }
+    if (!pairs) return;
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(pairs, v);
 }
 
 // Work items for the near field with targets in chunks of tchunk (<= P2P_T) and at most
 // smax source points per item (a larger single leaf stays whole); returns the count.
 int64_t build_p2p_items(ffm_plan_s *p, int tchunk, uint32_t smax, Alloc &out_mem, int4 **items, Alloc &tmp,
-                        cudaStream_t s) {
+                        cudaStream_t s, int64_t *pairs) {
     int ls = p->l_stop;
     int64_t nleafX = p->bx[ls].nb;
     uint32_t *icnt = tmp.get<uint32_t>(nleafX + 1), *ipos = tmp.get<uint32_t>(nleafX + 1);
-    FFM_CUDA(cudaMemsetAsync(icnt, 0, sizeof(uint32_t) * (nleafX + 1), s));
+    unsigned long long *sums = tmp.get<unsigned long long>(2), h[2];  // point pairs, items
+    FFM_CUDA(cudaMemsetAsync(icnt + nleafX, 0, sizeof(uint32_t), s));
+    FFM_CUDA(cudaMemsetAsync(sums, 0, sizeof h, s));
     FFM_LAUNCH(k_p2p_items, cdiv(nleafX, 128), 128, 0, s, p->near_off, p->near_src, p->bx[ls].start, p->by[ls].start,
-               nleafX, tchunk, smax, (const uint32_t *)nullptr, icnt, (int4 *)nullptr);
-    uint32_t *itot = tmp.get<uint32_t>(1);
-    scan_u32(icnt, ipos, nleafX + 1, itot, tmp, s);
-    int64_t n = read_u32(itot, s);
+               nleafX, tchunk, smax, (const uint32_t *)nullptr, icnt, (int4 *)nullptr, pairs ? sums : nullptr);
+    scan_u32(icnt, ipos, nleafX + 1, (uint32_t *)(sums + 1), tmp, s);
+    FFM_CUDA(cudaMemcpyAsync(h, sums, sizeof h, cudaMemcpyDeviceToHost, s));
+    FFM_CUDA(cudaStreamSynchronize(s));
+    int64_t n = (int64_t)(uint32_t)h[1];
+    if (pairs) *pairs = (int64_t)h[0];
     *items = out_mem.get<int4>(n);
     FFM_LAUNCH(k_p2p_items, cdiv(nleafX, 128), 128, 0, s, p->near_off, p->near_src, p->bx[ls].start, p->by[ls].start,
-               nleafX, tchunk, smax, ipos, icnt, *items);
+               nleafX, tchunk, smax, ipos, icnt, *items, (unsigned long long *)nullptr);
     return n;
-}
-
-// Target box of every pair of a CSR list (pairs of listed target x: [off[x], off[x+1])).
-__global__ void k_expand_csr_targets(const uint32_t *__restrict__ tgt, const uint32_t *__restrict__ off, int64_t nt,
-                                     uint32_t *__restrict__ out) {
-    int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nt) return;
-    for (uint32_t e = off[x]; e < off[x + 1]; ++e) out[e] = tgt[x];
 }
 
 // ======================================================== leaf coordinates
@@ -886,12 +1095,6 @@ __global__ void k_sorted_normals(const T *__restrict__ nrm, const uint32_t *__re
 
 // ================================================================ host side
 
-static int bits_for(int64_t n) {
-    int b = 1;
-    while (b < 32 && ((int64_t)1 << b) < n) ++b;
-    return b;
-}
-
 static bool is_device_ptr(const void *p) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -931,67 +1134,23 @@ static void launch_leaf_eps(const void *P, const uint32_t *perm, const uint64_t 
 }
 
 
-// Box tables of one set for levels 0..ldeep (boxes at level l = runs of key >> 3(21-l)).
-static void build_boxes(ffm_plan_s *p, BoxLevel *bl, const uint64_t *key, int64_t n, const uint8_t *f,
-                        const int64_t *nb, int ldeep, Alloc &tmp, cudaStream_t s) {
+// Box tables of one set for levels 0..ldeep (boxes at level l = runs of key >> 3(21-l)); parents
+// only where asked for (the target boxes).
+static void build_boxes(ffm_plan_s *p, BoxLevel *bl, const SetPts &S, const int64_t *nb, int ldeep, uint32_t **parent,
+                        Alloc &tmp, cudaStream_t s) {
     Alloc &m = p->mem;
-    uint32_t *flag = tmp.get<uint32_t>(n), *pos = tmp.get<uint32_t>(n);
-    FFM_LAUNCH(k_flag_le, cdiv(n, 256), 256, 0, s, f, n, ldeep, flag);
-    scan_u32(flag, pos, n, nullptr, tmp, s);
-    int64_t nd = nb[ldeep];
-    BoxLevel &D = bl[ldeep];
-    D.nb = nd;
-    D.start = m.get<uint32_t>(nd + 1);
-    uint8_t *bf = tmp.get<uint8_t>(nd);
-    FFM_LAUNCH(k_compact_pts, cdiv(n, 256), 256, 0, s, f, pos, n, ldeep, D.start, bf, nd);
-    D.fine = m.get<uint32_t>(nd);
-    FFM_LAUNCH(k_iota, cdiv(nd, 256), 256, 0, s, D.fine, nd);
-    uint32_t *bflag = tmp.get<uint32_t>(nd), *bpos = tmp.get<uint32_t>(nd);
-    for (int l = 0; l < ldeep; ++l) {
-        BoxLevel &B = bl[l];
-        B.nb = nb[l];
-        B.start = m.get<uint32_t>(B.nb + 1);
-        B.fine = m.get<uint32_t>(B.nb);
-        FFM_LAUNCH(k_flag_le, cdiv(nd, 256), 256, 0, s, bf, nd, l, bflag);
-        scan_u32(bflag, bpos, nd, nullptr, tmp, s);
-        FFM_LAUNCH(k_compact_boxes, cdiv(nd, 256), 256, 0, s, bf, D.start, bpos, nd, l, n, B.start, B.fine, B.nb);
-    }
+    BoxOut O{};
     for (int l = 0; l <= ldeep; ++l) {
         BoxLevel &B = bl[l];
-        B.g = m.get<int4>(B.nb);
-        FFM_LAUNCH(k_box_coords, cdiv(B.nb, 256), 256, 0, s, key, B.start, B.nb, l, B.g);
-        if (l < ldeep) {
-            B.first_child = m.get<uint32_t>(B.nb + 1);
-            FFM_LAUNCH(k_lower_bound, cdiv(B.nb + 1, 256), 256, 0, s, B.fine, B.nb, bl[l + 1].fine, bl[l + 1].nb,
-                       B.first_child);
-        }
+        B.nb = nb[l];
+        O.nb[l] = (uint32_t)nb[l];
+        O.start[l] = B.start = m.get<uint32_t>(B.nb + 1);
+        O.fine[l] = B.fine = m.get<uint32_t>(B.nb + 1);
+        O.g[l] = B.g = m.get<int4>(B.nb);
+        if (l < ldeep) O.first_child[l] = B.first_child = m.get<uint32_t>(B.nb + 1);
+        if (parent) O.parent[l] = parent[l] = tmp.get<uint32_t>(B.nb);
     }
-}
-
-// Sort pairs (a, b) by a (stable), then CSR: list of distinct a (ids), offsets per id.
-struct Csr {
-    int64_t n = 0, nruns = 0;
-    uint32_t *a = nullptr, *b = nullptr, *ids = nullptr, *off = nullptr, *perm = nullptr;
-};
-
-static Csr group_by_target(uint32_t *a, uint32_t *b, int64_t n, int64_t nbx, Alloc &dst, Alloc &tmp,
-                           cudaStream_t s) {
-    Csr c;
-    c.n = n;
-    c.perm = tmp.get<uint32_t>(n);
-    FFM_LAUNCH(k_iota, cdiv(n, 256), 256, 0, s, c.perm, n);
-    radix_sort_u32(a, c.perm, n, bits_for(nbx), tmp, s);
-    c.a = a;
-    c.b = dst.get<uint32_t>(n);
-    FFM_LAUNCH(k_gather_u32, cdiv(n, 256), 256, 0, s, b, c.perm, n, c.b);
-    uint32_t *flag = tmp.get<uint32_t>(n), *pos = tmp.get<uint32_t>(n), *tot = tmp.get<uint32_t>(1);
-    FFM_LAUNCH(k_run_starts, cdiv(n, 256), 256, 0, s, a, n, flag);
-    scan_u32(flag, pos, n, tot, tmp, s);
-    c.nruns = read_u32(tot, s);
-    c.ids = dst.get<uint32_t>(c.nruns);
-    c.off = dst.get<uint32_t>(c.nruns + 1);
-    FFM_LAUNCH(k_run_list, cdiv(n, 256), 256, 0, s, a, flag, pos, n, c.nruns, c.ids, c.off);
-    return c;
+    FFM_LAUNCH(k_box_emit, (unsigned)S.ntile, BT_T, 0, s, S, O, ldeep);
 }
 
 static int oscillatory(const ffm_plan_s *p, int l) {
@@ -1004,9 +1163,7 @@ static int pw_rank(double k, double dl, double eps) {
     return L < 1 ? 1 : L;
 }
 
-// Record the admissible pairs of level l: CSR by target box, source list, translations.
-// Chunks of at most ch points of the listed boxes: (box, first point), so that the
-// point-wise kernels of a level spread large boxes over many blocks.
+// Chunks of at most ch points of the listed boxes (their number is known): (box, first point).
 __global__ void k_chunk_count(const uint32_t *__restrict__ list, int64_t n, const uint32_t *__restrict__ start,
                               uint32_t ch, uint32_t *__restrict__ cnt) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1022,13 +1179,12 @@ __global__ void k_chunk_emit(const uint32_t *__restrict__ list, int64_t n, const
     for (uint32_t q = start[b]; q < start[b + 1]; q += ch) out[k++] = make_uint2(b, q);
 }
 
-static uint2 *build_chunks(ffm_plan_s *p, const uint32_t *list, int64_t n, const uint32_t *start, int64_t *count,
-                           Alloc &tmp, cudaStream_t s, uint32_t ch = LAG_CHUNK) {
-    uint32_t *cnt = tmp.get<uint32_t>(n), *pos = tmp.get<uint32_t>(n), *tot = tmp.get<uint32_t>(1);
+static uint2 *build_chunks(ffm_plan_s *p, const uint32_t *list, int64_t n, const uint32_t *start, int64_t count,
+                           Alloc &tmp, cudaStream_t s, uint32_t ch) {
+    uint32_t *cnt = tmp.get<uint32_t>(n), *pos = tmp.get<uint32_t>(n);
     FFM_LAUNCH(k_chunk_count, cdiv(n, 256), 256, 0, s, list, n, start, ch, cnt);
-    scan_u32(cnt, pos, n, tot, tmp, s);
-    *count = read_u32(tot, s);
-    uint2 *out = p->mem.get<uint2>(*count);
+    scan_u32(cnt, pos, n, nullptr, tmp, s);
+    uint2 *out = p->mem.get<uint2>(count);
     FFM_LAUNCH(k_chunk_emit, cdiv(n, 256), 256, 0, s, list, n, start, ch, pos, out);
     return out;
 }
@@ -1080,22 +1236,20 @@ static int64_t build_tiles(ffm_plan_s *p, const FarLevel &F, uint32_t bn, uint32
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
     if (F.mode != 1 || F.n_adm == 0 || F.bt_off) return;
-    const int64_t na = F.n_adm;
     Alloc tmp;
     tmp.stream = s;
-    uint32_t *tk = tmp.get<uint32_t>(na), *pidx = tmp.get<uint32_t>(na);
-    FFM_CUDA(cudaMemcpyAsync(tk, F.adm_t, sizeof(uint32_t) * na, cudaMemcpyDeviceToDevice, s));
-    FFM_LAUNCH(k_iota, cdiv(na, 256), 256, 0, s, pidx, na);
-    radix_sort_u32(tk, pidx, na, bits_for(F.n_trans), tmp, s);
-    // target of every pair in CSR order
-    uint32_t *ptgt = tmp.get<uint32_t>(na);
-    FFM_LAUNCH(k_expand_csr_targets, cdiv(F.n_tgt, 128), 128, 0, s, F.tgt, F.adm_off, F.n_tgt, ptgt);
-    F.bt_src = p->mem.get<uint32_t>(na);
-    F.bt_tgt = p->mem.get<uint32_t>(na);
-    FFM_LAUNCH(k_gather_u32, cdiv(na, 256), 256, 0, s, F.adm_src, pidx, na, F.bt_src);
-    FFM_LAUNCH(k_gather_u32, cdiv(na, 256), 256, 0, s, ptgt, pidx, na, F.bt_tgt);
+    F.bt_src = p->mem.get<uint32_t>(F.n_adm);
+    F.bt_tgt = p->mem.get<uint32_t>(F.n_adm);
     F.bt_off = p->mem.get<uint32_t>(F.n_trans + 1);
-    FFM_LAUNCH(k_csr_offsets, cdiv(F.n_trans + 1, 256), 256, 0, s, tk, na, F.n_trans, F.bt_off);
+    uint32_t *cursor = tmp.get<uint32_t>(F.n_trans + 1);
+    const unsigned g = cdiv(F.n_tgt, GP_TGT);
+    FFM_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * (F.n_trans + 1), s));
+    FFM_LAUNCH(k_group_pairs<false>, g, 256, 0, s, F.tgt, F.adm_off, F.n_tgt, F.adm_src, F.adm_t, F.n_trans, cursor,
+               (uint32_t *)nullptr, (uint32_t *)nullptr);
+    scan_u32(cursor, F.bt_off, F.n_trans + 1, nullptr, tmp, s);
+    FFM_CUDA(cudaMemcpyAsync(cursor, F.bt_off, sizeof(uint32_t) * F.n_trans, cudaMemcpyDeviceToDevice, s));
+    FFM_LAUNCH(k_group_pairs<true>, g, 256, 0, s, F.tgt, F.adm_off, F.n_tgt, F.adm_src, F.adm_t, F.n_trans, cursor,
+               F.bt_src, F.bt_tgt);
     tmp.release();
 }
 
@@ -1112,59 +1266,134 @@ void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s) {
     tmp.release();
 }
 
-static void finish_far_level(ffm_plan_s *p, int l, uint32_t *aa, uint32_t *ab, int64_t na, Alloc &tmp,
+// Level l of the descent (its temporaries in tmp): counts, lists, the read-back of their sizes, the pairs.  D holds
+// the geometry and the parents' near lists; at l = 0 (root cubes already far apart) the one pair is
+// given.  The near pairs of the level go to near_off / near_src, in the plan's memory when the
+// descent stops here (stop(near pairs)).  Returns the number of near pairs.
+struct NearLists {
+    uint32_t *off = nullptr, *src = nullptr;
+};
+
+template <class Stop>
+static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, NearLists &near, int64_t pw[2], Alloc &tmp,
                              cudaStream_t s) {
     FarLevel &F = p->far[l];
+    const int64_t nx = p->bx[l].nb, ny = p->by[l].nb;
+    const bool root = l == 0;
+    D.n = nx;
+    D.gx = p->bx[l].g;
+    D.gy = p->by[l].g;
+    D.c.x = (int)std::floor(-std::ldexp(p->sigma[0], l) + 0.5);
+    D.c.y = (int)std::floor(-std::ldexp(p->sigma[1], l) + 0.5);
+    D.c.z = (int)std::floor(-std::ldexp(p->sigma[2], l) + 0.5);
+    D.c.w = 0;
+    if (root) D.c = make_int4(0, 0, 0, 0);  // the single root pair has m = 0
+    // zeroed scratch: totals, translation flags, error flag, source flags
+    struct Scratch {
+        LevelTotals tot;
+        uint32_t used[4096];
+        int err;
+    };
+    unsigned char *scr = static_cast<unsigned char *>(tmp.raw(sizeof(Scratch) + (size_t)ny));
+    Scratch *S = reinterpret_cast<Scratch *>(scr);
+    FFM_CUDA(cudaMemsetAsync(scr, 0, sizeof(Scratch) + (size_t)ny, s));
+    D.used = S->used;
+    D.err = &S->err;
+    D.src_used = scr + sizeof(Scratch);
+    D.cadm = tmp.get<uint32_t>(nx + 1);
+    D.cnear = tmp.get<uint32_t>(nx + 1);
+    uint32_t *tpos = tmp.get<uint32_t>(4096);
+    D.tpos = tpos;
+    const unsigned dg = std::min<unsigned>(cdiv(nx, DS_W), 152u * 32u);
+    if (root) {
+        static const uint32_t one = 1, zero = 0;
+        FFM_CUDA(cudaMemcpyAsync(D.cadm, &one, sizeof one, cudaMemcpyHostToDevice, s));
+        FFM_CUDA(cudaMemcpyAsync(D.cnear, &zero, sizeof zero, cudaMemcpyHostToDevice, s));
+        FFM_CUDA(cudaMemcpyAsync(D.used + (8 | 8 << 4 | 8 << 8), &one, sizeof one, cudaMemcpyHostToDevice, s));
+        FFM_CUDA(cudaMemsetAsync(D.src_used, 1, 1, s));
+    } else {
+        FFM_LAUNCH(k_descend<false>, dg, 32 * DS_W, 0, s, D);
+    }
+    // Lagrange levels take point chunks; the lists are sized by their upper bounds
+    const bool lag = !oscillatory(p, l);
+    LevelArgsL L{};
+    L.nx = nx;
+    L.ny = ny;
+    L.ntx = cdiv(nx, LV_TILE);
+    L.nty = cdiv(ny, LV_TILE);
+    L.cadm = D.cadm;
+    L.cnear = D.cnear;
+    L.src_used = D.src_used;
+    L.xstart = p->bx[l].start;
+    L.ystart = p->by[l].start;
+    L.ch = lag ? LAG_CHUNK : 0;
+    L.ta = tmp.get<unsigned long long>(L.ntx);
+    L.tb = tmp.get<unsigned long long>(L.ntx + L.nty);
+    L.used = D.used;
+    L.tpos = tpos;
+    L.tot = &S->tot;
+    L.err = D.err;
+    L.tgt = p->mem.get<uint32_t>(nx);
+    L.adm_off = p->mem.get<uint32_t>(nx + 1);
+    L.src = p->mem.get<uint32_t>(ny);
+    if (lag) {
+        L.tchunks = p->mem.get<uint2>(nx + p->nx / LAG_CHUNK);
+        L.schunks = p->mem.get<uint2>(ny + p->ny / LAG_CHUNK);
+    }
+    const unsigned lg = (unsigned)(L.ntx + L.nty);
+    FFM_LAUNCH(k_level_sums, lg, LV_T, 0, s, L);
+    FFM_LAUNCH(k_level_mid, 1, 1024, 0, s, L);
+    FFM_LAUNCH(k_level_lists, lg, LV_T, 0, s, L);
+    LevelTotals h;
+    FFM_CUDA(cudaMemcpyAsync(&h, &S->tot, sizeof h, cudaMemcpyDeviceToHost, s));
+    FFM_CUDA(cudaStreamSynchronize(s));
+    if (h.err) fail(FFM_ECUDA, "box translation outside the expected range");
+    const int64_t na = h.na, nn = h.nn;
     F.n_adm = na;
     p->info.n_adm[l] = na;
-    if (na == 0) return;
-    F.mode = oscillatory(p, l) ? 2 : 1;
-    Csr c = group_by_target(aa, ab, na, p->bx[l].nb, p->mem, tmp, s);
-    F.n_tgt = c.nruns;
-    F.tgt = c.ids;
-    F.adm_off = c.off;
-    F.adm_src = c.b;
-    // translations
-    int4 cc;
-    cc.x = (int)std::floor(-std::ldexp(p->sigma[0], l) + 0.5);
-    cc.y = (int)std::floor(-std::ldexp(p->sigma[1], l) + 0.5);
-    cc.z = (int)std::floor(-std::ldexp(p->sigma[2], l) + 0.5);
-    cc.w = 0;
-    if (l == 0) cc = make_int4(0, 0, 0, 0);  // the single root pair has m = 0
-    uint32_t *code = tmp.get<uint32_t>(na), *used = tmp.get<uint32_t>(4096), *upos = tmp.get<uint32_t>(4096);
-    uint32_t *tot = tmp.get<uint32_t>(1);
-    int *err = tmp.get<int>(1);
-    FFM_CUDA(cudaMemsetAsync(used, 0, 4096 * sizeof(uint32_t), s));
-    FFM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    FFM_LAUNCH(k_trans_code, std::min<unsigned>(cdiv(na, 256), 152u * 8u), 256, 0, s, c.a, c.b, na, p->bx[l].g,
-               p->by[l].g, cc, code, used, err);
-    scan_u32(used, upos, 4096, tot, tmp, s);
-    F.adm_t = p->mem.get<uint32_t>(na);
-    FFM_LAUNCH(k_map, cdiv(na, 256), 256, 0, s, code, upos, na, F.adm_t);
-    int herr = 0;
-    FFM_CUDA(cudaMemcpyAsync(&herr, err, sizeof herr, cudaMemcpyDeviceToHost, s));
-    F.n_trans = (int)read_u32(tot, s);
-    if (herr) fail(FFM_ECUDA, "box translation outside the expected range");
+    const bool last = stop(nn);
+    if (na > 0) {
+        F.adm_src = p->mem.get<uint32_t>(na);
+        F.adm_t = p->mem.get<uint32_t>(na);
+    }
+    near.src = last ? p->mem.get<uint32_t>(nn) : tmp.get<uint32_t>(nn);
+    near.off = D.cnear;
+    if (last) {
+        near.off = p->mem.get<uint32_t>(nx + 1);
+        FFM_CUDA(cudaMemcpyAsync(near.off, D.cnear, sizeof(uint32_t) * (nx + 1), cudaMemcpyDeviceToDevice, s));
+    }
+    D.adm_src = F.adm_src;
+    D.adm_t = F.adm_t;
+    D.near_out = near.src;
+    if (root) {
+        FFM_CUDA(cudaMemsetAsync(F.adm_src, 0, sizeof(uint32_t), s));
+        FFM_CUDA(cudaMemsetAsync(F.adm_t, 0, sizeof(uint32_t), s));
+    } else {
+        FFM_LAUNCH(k_descend<true>, dg, 32 * DS_W, 0, s, D);
+    }
+    if (na == 0) return nn;
+    F.mode = lag ? 1 : 2;
+    F.n_tgt = h.ntgt;
+    F.tgt = L.tgt;
+    F.adm_off = L.adm_off;
+    F.n_src = h.nsrc;
+    F.src = L.src;
+    F.tgt_chunks = L.tchunks;
+    F.src_chunks = L.schunks;
+    F.n_tgt_chunks = h.tch;
+    F.n_src_chunks = h.sch;
+    pw[0] = h.pw_sch;
+    pw[1] = h.pw_tch;
+    F.n_trans = (int)h.ntrans;
+    F.h_trans_m.clear();
+    for (int k = 0; k < 4096; ++k)
+        if (h.bits[k >> 5] >> (k & 31) & 1u)
+            F.h_trans_m.push_back(make_int4((k & 15) - 8 + D.c.x, ((k >> 4) & 15) - 8 + D.c.y, (k >> 8) - 8 + D.c.z, 0));
     F.trans_m = p->mem.get<int4>(F.n_trans);
-    FFM_LAUNCH(k_trans_list, 16, 256, 0, s, used, upos, cc, F.trans_m);
-    F.h_trans_m.resize(F.n_trans);
-    FFM_CUDA(cudaMemcpyAsync(F.h_trans_m.data(), F.trans_m, sizeof(int4) * F.n_trans, cudaMemcpyDeviceToHost, s));
+    FFM_CUDA(cudaMemcpyAsync(F.trans_m, F.h_trans_m.data(), sizeof(int4) * F.n_trans, cudaMemcpyHostToDevice, s));
     p->info.n_trans[l] = F.n_trans;
-    // source boxes in use
-    int64_t nby = p->by[l].nb;
-    uint32_t *su = tmp.get<uint32_t>(nby), *spos = tmp.get<uint32_t>(nby);
-    FFM_CUDA(cudaMemsetAsync(su, 0, sizeof(uint32_t) * nby, s));
-    FFM_LAUNCH(k_mark, cdiv(na, 256), 256, 0, s, F.adm_src, na, su);
-    scan_u32(su, spos, nby, tot, tmp, s);
-    F.n_src = read_u32(tot, s);
-    F.src = p->mem.get<uint32_t>(F.n_src);
-    FFM_LAUNCH(k_list_marked, cdiv(nby, 256), 256, 0, s, su, spos, nby, F.src);
-    unsigned long long *sums = tmp.get<unsigned long long>(2);
-    FFM_CUDA(cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), s));
-    FFM_LAUNCH(k_sum_sizes, cdiv(F.n_src, 256), 256, 0, s, F.src, F.n_src, p->by[l].start, sums);
-    FFM_LAUNCH(k_sum_sizes, cdiv(F.n_tgt, 256), 256, 0, s, F.tgt, F.n_tgt, p->bx[l].start, sums + 1);
-    p->info.src_points[l] = read_u64(sums, s);
-    p->info.tgt_points[l] = read_u64(sums + 1, s);
+    p->info.src_points[l] = (int64_t)h.src_points;
+    p->info.tgt_points[l] = (int64_t)h.tgt_points;
     if (F.mode == 1) {
         F.r1 = p->r1_override > 0 ? p->r1_override : r1_rule(p->kind, p->eps);
         if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
@@ -1177,19 +1406,16 @@ static void finish_far_level(ffm_plan_s *p, int l, uint32_t *aa, uint32_t *ab, i
         const bool ts_first = ts_can && (F.tune_tc == 2 || pick == 2);
         if (!ts_first) build_translation_groups(p, l, s);
         if (p->lag_transfer == 1 || pick == 0 || p->aca_eps > 0.0) build_group_tiles(p, l, s);
-        F.src_chunks = build_chunks(p, F.src, F.n_src, p->by[l].start, &F.n_src_chunks, tmp, s);
-        F.tgt_chunks = build_chunks(p, F.tgt, F.n_tgt, p->bx[l].start, &F.n_tgt_chunks, tmp, s);
+        p->info.r1[l] = F.r1;
     }
     p->info.mode[l] = F.mode;
-    if (F.mode == 1) {
-        F.r1 = p->r1_override > 0 ? p->r1_override : r1_rule(p->kind, p->eps);
-        p->info.r1[l] = F.r1;
-    } else {
+    if (F.mode == 2) {
         F.L = pw_rank(p->k, std::ldexp(p->d0, -l), p->eps);
         F.nQ = 2 * F.L * (F.L + 1);
         p->info.L[l] = F.L;
         p->info.nQ[l] = F.nQ;
     }
+    return nn;
 }
 
 void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_dtype ydt, const void *w,
@@ -1276,25 +1502,32 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
     sortmem.release();
 
     // ---- boxes per level
-    uint8_t *fX = tmp.get<uint8_t>(nx), *fY = tmp.get<uint8_t>(ny);
-    unsigned long long *cnt = tmp.get<unsigned long long>(2 * (LMAX + 1));
-    FFM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 2 * (LMAX + 1), s));
-    FFM_LAUNCH(k_levels, cdiv(nx, 256), 256, 0, s, p->keyX, nx, fX, cnt);
-    FFM_LAUNCH(k_levels, cdiv(ny, 256), 256, 0, s, p->keyY, ny, fY, cnt + LMAX + 1);
-    unsigned long long hc[2 * (LMAX + 1)];
-    FFM_CUDA(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s));
+    SetPair sp;
+    uint32_t *lvtot = tmp.get<uint32_t>(2 * (LMAX + 1));
+    for (int i = 0; i < 2; ++i) {
+        SetPts &S = sp.s[i];
+        S.key = i == 0 ? p->keyX : p->keyY;
+        S.n = i == 0 ? nx : ny;
+        S.ntile = cdiv(S.n, BT_TILE);
+        S.f = tmp.get<uint8_t>(S.n);
+        S.cnt = tmp.get<uint32_t>((size_t)S.ntile * (LMAX + 1));
+    }
+    FFM_LAUNCH(k_level_marks, dim3((unsigned)std::max(sp.s[0].ntile, sp.s[1].ntile), 2), BT_T, 0, s, sp);
+    FFM_LAUNCH(k_level_scan, dim3(LMAX + 1, 2), 1024, 0, s, sp, lvtot);
+    uint32_t hc[2 * (LMAX + 1)];
+    FFM_CUDA(cudaMemcpyAsync(hc, lvtot, sizeof hc, cudaMemcpyDeviceToHost, s));
     FFM_CUDA(cudaStreamSynchronize(s));
     int64_t nbx[LMAX + 1], nby[LMAX + 1];
-    nbx[0] = nby[0] = 1;
-    for (int l = 1; l <= LMAX; ++l) {
-        nbx[l] = nbx[l - 1] + (int64_t)hc[l];
-        nby[l] = nby[l - 1] + (int64_t)hc[LMAX + 1 + l];
+    for (int l = 0; l <= LMAX; ++l) {
+        nbx[l] = hc[l];
+        nby[l] = hc[LMAX + 1 + l];
     }
     // deepest level the occupancy rule can reach
     int ldeep = 0;
     while (ldeep < p->l_cap && !(n < (int64_t)p->n_leaf * (nbx[ldeep] + nby[ldeep]))) ++ldeep;
-    build_boxes(p, p->bx, p->keyX, nx, fX, nbx, ldeep, tmp, s);
-    build_boxes(p, p->by, p->keyY, ny, fY, nby, ldeep, tmp, s);
+    uint32_t *parent[LMAX + 1] = {};
+    build_boxes(p, p->bx, sp.s[0], nbx, ldeep, parent, tmp, s);
+    build_boxes(p, p->by, sp.s[1], nby, ldeep, nullptr, tmp, s);
     for (int l = 0; l <= ldeep; ++l) {
         p->info.nboxX[l] = nbx[l];
         p->info.nboxY[l] = nby[l];
@@ -1306,81 +1539,63 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
         if (std::fabs(p->sigma[d]) >= 2.0) root_adm = true;
     Alloc levels[LMAX + 2];  // per-level temporaries of the descent, released level by level
     TableJob tj(s);
-    uint32_t *nearA = tmp.get<uint32_t>(1), *nearB = tmp.get<uint32_t>(1);
-    FFM_CUDA(cudaMemsetAsync(nearA, 0, sizeof(uint32_t), s));
-    FFM_CUDA(cudaMemsetAsync(nearB, 0, sizeof(uint32_t), s));
-    int64_t nnear = 1;
+    NearLists near;  // at the root: box 0 with box 0
+    near.off = p->mem.get<uint32_t>(2);
+    near.src = p->mem.get<uint32_t>(1);
+    static const uint32_t root_off[2] = {0, 1};
+    FFM_CUDA(cudaMemcpyAsync(near.off, root_off, sizeof root_off, cudaMemcpyHostToDevice, s));
+    FFM_CUDA(cudaMemsetAsync(near.src, 0, sizeof(uint32_t), s));
+    int64_t nnear = 1, pwc[LMAX + 1][2] = {};
+    auto stops = [&](int l, int64_t nn) {
+        return nn == 0 || n < (int64_t)p->n_leaf * (nbx[l] + nby[l]) || l >= p->l_cap;
+    };
     p->l_stop = 0;
     if (root_adm) {
         p->root_adm = 1;
         p->info.root_admissible = 1;
-        finish_far_level(p, 0, nearA, nearB, 1, tmp, s);
-        if (p->far[0].n_adm > 0) build_tables(p, 0, tj);
-        nnear = 0;
+        levels[0].stream = s;
+        nnear = descend_level(p, 0, DescendArgs{}, [](int64_t) { return true; }, near, pwc[0], levels[0], s);
+        build_tables(p, 0, tj);
     } else {
         p->info.n_near[0] = 1;
-        for (int l = 0;; ++l) {
-            bool stop = nnear == 0 || n < (int64_t)p->n_leaf * (nbx[l] + nby[l]) || l >= p->l_cap;
-            if (stop) {
-                p->l_stop = l;
-                break;
-            }
-            int lc = l + 1;
+        int l = 0;
+        for (; !stops(l, nnear); ++l) {
+            const int lc = l + 1;
             D3 sg{{std::ldexp(p->sigma[0], lc), std::ldexp(p->sigma[1], lc), std::ldexp(p->sigma[2], lc)}};
-            Alloc &lvl = levels[lc];
-            lvl.stream = s;
-            uint32_t *nadm = lvl.get<uint32_t>(nnear), *nnr = lvl.get<uint32_t>(nnear);
-            uint32_t *oadm = lvl.get<uint32_t>(nnear), *onr = lvl.get<uint32_t>(nnear);
-            uint32_t *tot = lvl.get<uint32_t>(2);
-            const AdmK K = adm_thresholds(sg);
-            FFM_LAUNCH(k_expand_count, cdiv(nnear, EXP_W), 32 * EXP_W, 0, s, nearA, nearB, nnear,
-                       p->bx[l].first_child, p->by[l].first_child, p->bx[lc].g, p->by[lc].g, K, nadm, nnr);
-            scan_u32(nadm, oadm, nnear, tot, lvl, s);
-            scan_u32(nnr, onr, nnear, tot + 1, lvl, s);
-            uint32_t htot[2];
-            FFM_CUDA(cudaMemcpyAsync(htot, tot, sizeof htot, cudaMemcpyDeviceToHost, s));
-            FFM_CUDA(cudaStreamSynchronize(s));
-            int64_t na = htot[0], nn = htot[1];
-            uint32_t *aa = lvl.get<uint32_t>(na), *ab = lvl.get<uint32_t>(na);
-            uint32_t *ea = lvl.get<uint32_t>(nn), *eb = lvl.get<uint32_t>(nn);
-            FFM_LAUNCH(k_expand_emit, cdiv(nnear, EXP_W), 32 * EXP_W, 0, s, nearA, nearB, nnear,
-                       p->bx[l].first_child, p->by[l].first_child, p->bx[lc].g, p->by[lc].g, K, oadm, onr, aa, ab,
-                       ea, eb);
-            // the previous level's near list is no longer needed
+            DescendArgs D{};
+            D.parent = parent[lc];
+            D.near_off = near.off;
+            D.near_src = near.src;
+            D.fcy = p->by[l].first_child;
+            D.K = adm_thresholds(sg);
+            levels[lc].stream = s;
+            nnear = descend_level(p, lc, D, [&](int64_t nn) { return stops(lc, nn); }, near, pwc[lc], levels[lc], s);
+            // the previous level's near lists are no longer needed
             if (l >= 1) levels[l].release();
-            finish_far_level(p, lc, aa, ab, na, lvl, s);
             if (p->far[lc].n_adm > 0) build_tables(p, lc, tj);
-            nearA = ea;
-            nearB = eb;
-            nnear = nn;
-            p->info.n_near[lc] = nn;
+            p->info.n_near[lc] = nnear;
         }
+        p->l_stop = l;
     }
     int ls = p->l_stop;
     p->info.l_stop = ls;
 
     // ---- near pairs at the stop level: CSR over all target leaves
     p->n_near = nnear;
-    int64_t nleafX = p->bx[ls].nb;
-    p->near_off = p->mem.get<uint32_t>(nleafX + 1);
+    p->near_off = near.off;
     if (nnear > 0) {
-        Csr c = group_by_target(nearA, nearB, nnear, nleafX, p->mem, tmp, s);
-        p->near_src = c.b;
-        FFM_LAUNCH(k_csr_offsets, cdiv(nleafX + 1, 256), 256, 0, s, c.a, nnear, nleafX, p->near_off);
+        p->near_src = near.src;
         // work items: target chunks x bounded source ranges
-        p->n_items = build_p2p_items(p, p->p2p_tchunk, p->p2p_smax, p->mem, &p->items, tmp, s);
-        unsigned long long *pp = tmp.get<unsigned long long>(1);
-        FFM_CUDA(cudaMemsetAsync(pp, 0, sizeof(unsigned long long), s));
-        FFM_LAUNCH(k_sum_pair_sizes, cdiv(nnear, 256), 256, 0, s, c.a, c.b, nnear, p->bx[ls].start, p->by[ls].start,
-                   pp);
-        p->info.p2p_pairs = read_u64(pp, s);
-    } else {
-        FFM_CUDA(cudaMemsetAsync(p->near_off, 0, sizeof(uint32_t) * (nleafX + 1), s));
+        p->n_items = build_p2p_items(p, p->p2p_tchunk, p->p2p_smax, p->mem, &p->items, tmp, s, &p->info.p2p_pairs);
     }
 
     // ---- leaf links and leaf-relative coordinates
     for (int l = 0; l <= ls; ++l) {
         for (BoxLevel *B : {&p->bx[l], &p->by[l]}) {
+            if (ls == ldeep) {  // the leaves are the deepest boxes: their ranks are in the tables
+                B->first_leaf = B->fine;
+                continue;
+            }
             BoxLevel &Lf = (B == &p->bx[l]) ? p->bx[ls] : p->by[ls];
             B->first_leaf = p->mem.get<uint32_t>(B->nb + 1);
             FFM_LAUNCH(k_lower_bound, cdiv(B->nb + 1, 256), 256, 0, s, B->fine, B->nb, Lf.fine, Lf.nb, B->first_leaf);
@@ -1442,8 +1657,10 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
             FarLevel &F = p->far[l];
             if (F.mode != 2 || F.n_adm == 0 || F.nufft || (F.prec != FFM_PREC_F32 && F.prec != FFM_PREC_F32C))
                 continue;
-            F.pw_chunks = build_chunks(p, F.src, F.n_src, p->by[l].start, &F.n_pw_chunks, tmp, s, PW_TC_FCH);
-            F.pw_tchunks = build_chunks(p, F.tgt, F.n_tgt, p->bx[l].start, &F.n_pw_tchunks, tmp, s, PW_TC_BCH);
+            F.n_pw_chunks = pwc[l][0];
+            F.n_pw_tchunks = pwc[l][1];
+            F.pw_chunks = build_chunks(p, F.src, F.n_src, p->by[l].start, pwc[l][0], tmp, s, PW_TC_FCH);
+            F.pw_tchunks = build_chunks(p, F.tgt, F.n_tgt, p->bx[l].start, pwc[l][1], tmp, s, PW_TC_BCH);
         }
     FFM_CUDA(cudaStreamSynchronize(s));
 }
