@@ -203,8 +203,6 @@ void autotune(ffm_plan_s *p, int nrhs, const char *cache_path, cudaStream_t s) {
     size_t nout = (size_t)nrhs * (p->kind == FFM_LAPLACE_GRAD ? 3 : 1);
     double2 *acc = tmp.get<double2>((size_t)p->nx * nout);
     FFM_CUDA(cudaMemsetAsync(acc, 0, sizeof(double2) * (size_t)p->nx * nout, s));
-    float2 *accf = tmp.get<float2>((size_t)p->nx * nout);
-    FFM_CUDA(cudaMemsetAsync(accf, 0, sizeof(float2) * (size_t)p->nx * nout, s));
     Timer T(s);
 
     // ---- near field: work-item shape
@@ -236,11 +234,22 @@ void autotune(ffm_plan_s *p, int nrhs, const char *cache_path, cudaStream_t s) {
     for (int l = 0; l <= p->l_stop; ++l) {
         FarLevel &F = p->far[l];
         if (F.n_adm == 0) continue;
+        Alloc lm;  // a Lagrange level's coefficients
+        lm.stream = s;
+        void *ut = nullptr, *vt = nullptr;
+        if (F.mode == 1) {
+            size_t ub, vb;
+            lagrange_bytes(p, l, nrhs, &ub, &vb);
+            ut = lm.raw(ub);
+            vt = lm.raw(vb);
+            FFM_CUDA(cudaMemsetAsync(ut, 0, ub, s));
+            FFM_CUDA(cudaMemsetAsync(vt, 0, vb, s));
+        }
         auto run_level = [&] {
             Alloc lt;
             lt.stream = s;
             if (F.mode == 1)
-                far_lagrange(p, l, q, nrhs, accf, lt, s);
+                lagrange_transfer(p, l, ut, nrhs, vt, lt, s);
             else
                 far_planewave(p, l, (const float2 *)q, nrhs, acc, lt, s);
         };

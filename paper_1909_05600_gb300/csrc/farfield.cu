@@ -619,7 +619,7 @@ __device__ __forceinline__ void tmem_st8(uint32_t ta, const uint32_t (&v)[8]) {
 }
 
 // Target step of a Lagrange level (L_X^T v~ of eq. 8): v_i += sum_abc L_a(x_i) L_b(y_i) L_c(z_i) v~_a(abc),
-// one block per chunk of at most LAG_CHUNK points of a target box, added in FP32 into accf.
+// one block per chunk of at most LAG_CHUNK points of a target box, written in FP32 to accf.
 template <bool CPLX, int R1>
 __global__ void __launch_bounds__(128) k_lag_interp(LevelArgs A, const uint2 *__restrict__ chunks, Cheb cb,
                                                     const typename QT<CPLX>::T *__restrict__ vt, int nrhs,
@@ -661,9 +661,7 @@ __global__ void __launch_bounds__(128) k_lag_interp(LevelArgs A, const uint2 *__
                 sr = fmaf(lab, pr, sr);
                 if constexpr (CPLX) si = fmaf(lab, pi, si);
             }
-        float2 &dst = accf[(int64_t)m * nx + i];
-        dst.x += sr;
-        if constexpr (CPLX) dst.y += si;
+        accf[(int64_t)m * nx + i] = make_float2(sr, si);
     }
 }
 
@@ -825,9 +823,7 @@ __global__ void __launch_bounds__(32 * LAG_WC) k_lag_interp_w(LevelArgs A, const
                 sr = fmaf(lab, pr, sr);
                 if constexpr (CPLX) si = fmaf(lab, pi, si);
             }
-        float2 &dst = accf[(int64_t)m * nx + i];
-        dst.x += sr;
-        if constexpr (CPLX) dst.y += si;
+        accf[(int64_t)m * nx + i] = make_float2(sr, si);
     }
 }
 
@@ -929,85 +925,369 @@ static void tc_transfer(const FarLevel &F, const uint32_t *src, const uint32_t *
     }
 }
 
-void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s) {
-    const FarLevel &F = p->far[l];
-    int ls = p->l_stop;
-    int r = F.r1 * F.r1 * F.r1;
-    Cheb cb = make_cheb(F.r1);
-    LevelArgs AY = level_args(p, p->by[l], p->by[ls], p->epsY, l);
-    LevelArgs AX = level_args(p, p->bx[l], p->bx[ls], p->epsX, l);
-    bool cplx = p->kind == FFM_HELMHOLTZ;
-    int rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;  // K extent of the transfer
-    size_t esz = cplx ? sizeof(float2) : sizeof(float);
-    size_t ub = esz * rk * nrhs * (size_t)p->by[l].nb,
-           vb = esz * r * nrhs * (size_t)p->bx[l].nb * (p->kind == FFM_LAPLACE_GRAD ? 3 : 1);
-    void *ut = tmp.raw(ub);
-    void *vt = tmp.raw(vb);
-    dim3 gg((unsigned)F.n_tiles, cdiv(r, LG_BM), nrhs);
-    // the transfer by translation runs on the tensor cores (transfer.cu) unless the CUDA-core GEMM is
-    // forced or picked by the autotuner
-    const bool use_tc = F.tune_tc != 0 && F.Th;
-    FFM_CUDA(cudaMemsetAsync(ut, 0, ub, s));
-    FFM_CUDA(cudaMemsetAsync(vt, 0, vb, s));
-    if (cplx) {
-        lagrange_points_r1<true>(p, F, AY, cb, true, q, nrhs, ut, s);
-        if (use_tc)
-            lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
-        else
-            FFM_LAUNCH(k_lag_gemm<true>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, F.T, r, rk,
-                       nrhs, (const float2 *)ut, (float2 *)vt);
-        lagrange_points_r1<true>(p, F, AX, cb, false, vt, nrhs, accf, s);
-    } else {
-        if (p->kind == FFM_LAPLACE_DL)
-            lagrange_anterp_dl_r1(p, F, AY, cb, q, nrhs, ut, s);
-        else
-            lagrange_points_r1<false>(p, F, AY, cb, true, q, nrhs, ut, s);
-        int npad = (r + 15) / 16 * 16;
-        if (F.aca) {
-            // ACA factors (eq. 11): w_p = B_t^T u~_src(p) for every pair p of translation t
-            // (rows of w indexed by pair), then v~_tgt(p) += A_t w_p
-            const int rp = F.aca_rp;
-            float *w = tmp.get<float>((size_t)F.n_adm * nrhs * rp);
-            FFM_CUDA(cudaMemsetAsync(w, 0, sizeof(float) * (size_t)F.n_adm * nrhs * rp, s));
-            if (F.aca_tc) {
-                int64_t nrow = (int64_t)p->by[l].nb * nrhs;
-                float *upad = tmp.get<float>((size_t)nrow * F.rkp);
-                split_pad((const float *)ut, 1, (int)nrow, r, (int)nrow, F.rkp, upad, nullptr, s);
-                tc_transfer(F, F.bt_src, F.pair_id, F.Bca, (int64_t)rp * F.rkp, rp, F.rkp, rp, nrhs, upad, w,
-                            p->dev_err, p->wait_tries, s);
-                tc_transfer(F, F.pair_id, F.bt_tgt, F.Aca, (int64_t)npad * rp, r, rp, r, nrhs, w, (float *)vt,
-                            p->dev_err, p->wait_tries, s);
-                tmp.drop(upad);
-            } else {
-                dim3 g1((unsigned)F.n_tiles, cdiv(rp, LG_BM), nrhs);
-                FFM_LAUNCH(k_lag_gemm<false>, g1, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.pair_id,
-                           F.Bca, rp, r, nrhs, (const float *)ut, w);
-                FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.pair_id, F.bt_tgt,
-                           F.Aca, r, rp, nrhs, (const float *)w, (float *)vt);
+// ---- coefficients between the levels
+//
+// The Lagrange basis of a box is made of polynomials of degree r1 - 1 per axis, which the basis of a
+// child box reproduces exactly: L_alpha(y) = sum_beta L_alpha(y_beta) L^child_beta(y) for y in the
+// child.  So u~ of a box is the sum over its children of M u~_child, M the tensor product of the 1-D
+// matrices M_h[a][b] = L_a((t_b +- 1) / 2), h the child's half, and v~ of a box goes to its children by
+// the transposes: only the finest Lagrange level touches the points.  Forming every level's sums from
+// the points read 20 bytes and did r multiply-adds per point, level and direction (1e8 clustered:
+// 24.4 + 22.1 ms over eight levels, gradient 300k: 0.28 + 0.81 ms).
+//
+// The three 1-D steps run in FP32 pairs (error-free products and sums): their rounding is shared by all
+// points of a box, where that of the point-wise sums averages out, and in plain FP32 it took
+// the Helmholtz parity case (cube surface, k = 12) from 3.1e-7 to 1.0e-6 of the oracle's FFM.
+struct Halves {
+    float2 m[2][R1MAX][R1MAX];  // [half][parent node][child node], as unevaluated pairs
+};
+
+// (h, l) += x m for pairs x and m: leading product split exactly, its sum into h with the rounding error
+// (Knuth's TwoSum) and all residuals collected in l
+__device__ __forceinline__ void pair_fma(float &h, float &l, float2 x, float2 m) {
+    const float p = __fmul_rn(x.x, m.x);
+    float e = fmaf(x.x, m.x, -p);
+    e = fmaf(x.y, m.x, e);
+    e = fmaf(x.x, m.y, e);
+    const float s = __fadd_rn(h, p), bb = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb)), e));
+    h = s;
+}
+// normalised pair
+__device__ __forceinline__ float2 pair_norm(float h, float l) {
+    const float s = __fadd_rn(h, l);
+    return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+
+static Halves make_halves(int r1) {
+    Halves H{};
+    double t[R1MAX];
+    for (int a = 0; a < r1; ++a) t[a] = std::cos((2.0 * a + 1.0) * PI / (2.0 * r1));
+    for (int h = 0; h < 2; ++h)
+        for (int b = 0; b < r1; ++b) {
+            const double x = 0.5 * (t[b] + (h ? 1.0 : -1.0));
+            for (int a = 0; a < r1; ++a) {
+                double v = 1.0;
+                for (int c = 0; c < r1; ++c)
+                    if (c != a) v *= (x - t[c]) / (t[a] - t[c]);
+                    H.m[h][a][b] = make_float2((float)v, (float)(v - (double)(float)v));
             }
-            tmp.drop(w);
-            lagrange_points_r1<false>(p, F, AX, cb, false, vt, nrhs, accf, s);
-            return;
         }
-        // the gradient has three operator blocks (component-major) and three outputs per
-        // target; v~ and the FP32 accumulators are component-major too
-        const int ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
-        const size_t tblk = (size_t)F.n_trans * r * rk;
-        const size_t vblk = (size_t)r * nrhs * p->bx[l].nb;
-        const bool use_ts = F.ts_ok && F.tune_tc == 2;
-        if (use_ts)
-            lag_targets(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
-        else if (use_tc)  // all components in one launch
-            lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
-        for (int d = 0; d < ncomp; ++d) {
-            const float *Td = F.T + d * tblk;
-            float *vtd = (float *)vt + d * vblk;
-            if (!use_ts && !use_tc)
-                FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, Td,
-                           r, rk, nrhs, (const float *)ut, vtd);
-            lagrange_points_r1<false>(p, F, AX, cb, false, vtd, nrhs, accf + (size_t)d * nrhs * p->nx, s);
+    return H;
+}
+
+struct LinkArgs {
+    int64_t n;                    // parent boxes
+    const uint32_t *first_child;
+    const int4 *gc;               // children's coordinates (low bits: octant)
+    int nrhs, rowlen, es;         // floats between rows, between values of a row
+    int coff;                     // floats between components within a row
+    int64_t pbase, cbase;         // floats between components of the parents', the children's array
+};
+
+// One parent per warp up to r = 64, per block of 128 threads above.  Three 1-D steps, shared by the
+// children as far as their halves agree: 8 along x, 4 along y, 2 along z.
+template <int R1>
+struct LinkShape {
+    static constexpr int r = R1 * R1 * R1, T = R1 <= 4 ? 32 : 128, NB = R1 <= 4 ? 8 : 1, NV = (r + T - 1) / T;
+};
+
+template <int R1>
+__device__ __forceinline__ void link_sync() {
+    if constexpr (R1 <= 4)
+        __syncwarp();
+    else
+        __syncthreads();
+}
+
+template <int R1>
+__global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
+    k_lag_up(const __grid_constant__ LinkArgs A, const __grid_constant__ Halves H, const float *__restrict__ uc,
+             float *__restrict__ up) {
+    typedef LinkShape<R1> S;
+    constexpr int r = S::r, T = S::T, NV = S::NV;
+    __shared__ float2 mat[2][R1][R1];
+    __shared__ float2 buf[S::NB][4][r];
+    for (int i = threadIdx.x; i < 2 * R1 * R1; i += T * S::NB)
+        mat[i / (R1 * R1)][i / R1 % R1][i % R1] = H.m[i / (R1 * R1)][i / R1 % R1][i % R1];
+    const int grp = threadIdx.x / T, th = threadIdx.x % T, m = blockIdx.y, comp = blockIdx.z;
+    const int64_t p = (int64_t)blockIdx.x * S::NB + grp;
+    float2(*B)[r] = buf[grp];
+    for (int i = th; i < 4 * r; i += T) B[i / r][i % r] = make_float2(0.f, 0.f);
+    __syncthreads();
+    if (p >= A.n) return;  // whole warps (or the block): no block barrier below for R1 <= 4
+    const float *src = uc + comp * A.cbase + (int64_t)comp * A.coff;
+    // x step: the children's sums by their (y, z) half; every thread owns its values of buf
+    const uint32_t c0 = A.first_child[p], c1 = A.first_child[p + 1];
+    for (uint32_t c = c0; c < c1; ++c) {
+        const int4 g = A.gc[c];
+        const int hx = g.x & 1, hyz = (g.y & 1) * 2 + (g.z & 1);
+        const float *row = src + ((int64_t)c * A.nrhs + m) * A.rowlen;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int i = th + v * T;
+            if (i < r) {
+                const int a = i / (R1 * R1), rest = i % (R1 * R1);
+                float2 o = B[hyz][i];
+#pragma unroll
+                for (int b = 0; b < R1; ++b)
+                    pair_fma(o.x, o.y, make_float2(__ldg(row + (int64_t)(b * R1 * R1 + rest) * A.es), 0.f), mat[hx][a][b]);
+                B[hyz][i] = o;
+            }
         }
     }
+    link_sync<R1>();
+    float2 acc[2][NV];
+#pragma unroll
+    for (int hz = 0; hz < 2; ++hz)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int i = th + v * T;
+            float h = 0.f, l = 0.f;
+            if (i < r) {
+                const int a = i / (R1 * R1), y = i / R1 % R1, z = i % R1;
+#pragma unroll
+                for (int hy = 0; hy < 2; ++hy)
+#pragma unroll
+                    for (int b = 0; b < R1; ++b) pair_fma(h, l, B[hy * 2 + hz][(a * R1 + b) * R1 + z], mat[hy][y][b]);
+            }
+            acc[hz][v] = pair_norm(h, l);
+        }
+    link_sync<R1>();
+#pragma unroll
+    for (int hz = 0; hz < 2; ++hz)
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            if (th + v * T < r) B[hz][th + v * T] = acc[hz][v];
+    link_sync<R1>();
+    float *out = up + comp * A.pbase + (int64_t)comp * A.coff + (p * A.nrhs + m) * (int64_t)A.rowlen;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const int i = th + v * T;
+        if (i < r) {
+            const int z = i % R1, ab = i - z;
+            float h = 0.f, l = 0.f;
+#pragma unroll
+            for (int hz = 0; hz < 2; ++hz)
+#pragma unroll
+                for (int b = 0; b < R1; ++b) pair_fma(h, l, B[hz][ab + b], mat[hz][z][b]);
+            out[(int64_t)i * A.es] = h + l;
+        }
+    }
+}
+
+template <int R1>
+__global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
+    k_lag_down(const __grid_constant__ LinkArgs A, const __grid_constant__ Halves H, const float *__restrict__ vp,
+               float *__restrict__ vc) {
+    typedef LinkShape<R1> S;
+    constexpr int r = S::r, T = S::T, NV = S::NV;
+    __shared__ float2 mat[2][R1][R1];
+    __shared__ float2 buf[S::NB][4][r], first[S::NB][2][r];
+    for (int i = threadIdx.x; i < 2 * R1 * R1; i += T * S::NB)
+        mat[i / (R1 * R1)][i / R1 % R1][i % R1] = H.m[i / (R1 * R1)][i / R1 % R1][i % R1];
+    __syncthreads();
+    const int grp = threadIdx.x / T, th = threadIdx.x % T, m = blockIdx.y, comp = blockIdx.z;
+    const int64_t p = (int64_t)blockIdx.x * S::NB + grp;
+    if (p >= A.n) return;
+    float2(*B)[r] = buf[grp], (*Z)[r] = first[grp];
+    const float *row = vp + comp * A.pbase + (int64_t)comp * A.coff + (p * A.nrhs + m) * (int64_t)A.rowlen;
+    for (int i = th; i < r; i += T) B[0][i] = make_float2(row[(int64_t)i * A.es], 0.f);
+    link_sync<R1>();
+#pragma unroll
+    for (int hz = 0; hz < 2; ++hz)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int i = th + v * T;
+            if (i < r) {
+                const int z = i % R1, ab = i - z;
+                float h = 0.f, l = 0.f;
+#pragma unroll
+                for (int a = 0; a < R1; ++a) pair_fma(h, l, B[0][ab + a], mat[hz][a][z]);
+                Z[hz][i] = pair_norm(h, l);
+            }
+        }
+    link_sync<R1>();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int i = th + v * T;
+            if (i < r) {
+                const int x = i / (R1 * R1), y = i / R1 % R1, z = i % R1;
+                float h = 0.f, l = 0.f;
+#pragma unroll
+                for (int a = 0; a < R1; ++a) pair_fma(h, l, Z[k & 1][(x * R1 + a) * R1 + z], mat[k >> 1][a][y]);
+                B[k][i] = pair_norm(h, l);
+            }
+        }
+    link_sync<R1>();
+    float *dst = vc + comp * A.cbase + (int64_t)comp * A.coff;
+    const uint32_t c0 = A.first_child[p], c1 = A.first_child[p + 1];
+    for (uint32_t c = c0; c < c1; ++c) {
+        const int4 g = A.gc[c];
+        const int hx = g.x & 1, hyz = (g.y & 1) * 2 + (g.z & 1);
+        float *out = dst + ((int64_t)c * A.nrhs + m) * A.rowlen;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int i = th + v * T;
+            if (i < r) {
+                const int x = i / (R1 * R1), rest = i % (R1 * R1);
+                float h = out[(int64_t)i * A.es], l = 0.f;
+#pragma unroll
+                for (int a = 0; a < R1; ++a) pair_fma(h, l, B[hyz][a * R1 * R1 + rest], mat[hx][a][x]);
+                out[(int64_t)i * A.es] = h + l;
+            }
+        }
+    }
+}
+
+template <int R1>
+static void lag_link(const LinkArgs &A, int ncomp, const Halves &H, bool up, const float *in, float *out, cudaStream_t s) {
+    typedef LinkShape<R1> S;
+    const dim3 g(cdiv(A.n, S::NB), A.nrhs, ncomp);
+    if (up)
+        FFM_LAUNCH_NAMED("k_lag_up", k_lag_up<R1>, g, S::T * S::NB, 0, s, A, H, in, out);
+    else
+        FFM_LAUNCH_NAMED("k_lag_down", k_lag_down<R1>, g, S::T * S::NB, 0, s, A, H, in, out);
+}
+
+static void lag_link_r1(int r1, const LinkArgs &A, int ncomp, const Halves &H, bool up, const float *in, float *out,
+                        cudaStream_t s) {
+    switch (r1) {
+        case 2: lag_link<2>(A, ncomp, H, up, in, out, s); break;
+        case 3: lag_link<3>(A, ncomp, H, up, in, out, s); break;
+        case 4: lag_link<4>(A, ncomp, H, up, in, out, s); break;
+        case 5: lag_link<5>(A, ncomp, H, up, in, out, s); break;
+        case 6: lag_link<6>(A, ncomp, H, up, in, out, s); break;
+        case 7: lag_link<7>(A, ncomp, H, up, in, out, s); break;
+        case 8: lag_link<8>(A, ncomp, H, up, in, out, s); break;
+        default: fail(FFM_EUNSUPPORTED, "Chebyshev nodes per axis outside 2..8");
+    }
+}
+
+// Bytes of a Lagrange level's u~ and v~ for nrhs right-hand sides.
+void lagrange_bytes(const ffm_plan_s *p, int l, int nrhs, size_t *ub, size_t *vb) {
+    const FarLevel &F = p->far[l];
+    const size_t r = (size_t)F.r1 * F.r1 * F.r1, esz = p->kind == FFM_HELMHOLTZ ? sizeof(float2) : sizeof(float);
+    *ub = esz * (p->kind == FFM_LAPLACE_DL ? 3 * r : r) * nrhs * (size_t)p->by[l].nb;
+    *vb = esz * r * nrhs * (size_t)p->bx[l].nb * (p->kind == FFM_LAPLACE_GRAD ? 3 : 1);
+}
+
+// The transfer of one Lagrange level: v~ (zeroed by the caller) += T u~ over its pairs.
+void lagrange_transfer(const ffm_plan_s *p, int l, const void *ut, int nrhs, void *vt, Alloc &tmp, cudaStream_t s) {
+    const FarLevel &F = p->far[l];
+    const int r = F.r1 * F.r1 * F.r1;
+    const bool cplx = p->kind == FFM_HELMHOLTZ;
+    const int rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;  // K extent of the transfer
+    dim3 gg((unsigned)F.n_tiles, cdiv(r, LG_BM), nrhs);
+    // by translation on the tensor cores (transfer.cu) unless the target-stationary form is prepared or
+    // the CUDA-core GEMM is forced or picked by the autotuner
+    const bool use_tc = F.tune_tc != 0 && F.Th;
+    if (F.aca) {
+        // ACA factors (eq. 11): w_p = B_t^T u~_src(p) for every pair p of translation t
+        // (rows of w indexed by pair), then v~_tgt(p) += A_t w_p
+        const int npad = (r + 15) / 16 * 16, rp = F.aca_rp;
+        float *w = tmp.get<float>((size_t)F.n_adm * nrhs * rp);
+        FFM_CUDA(cudaMemsetAsync(w, 0, sizeof(float) * (size_t)F.n_adm * nrhs * rp, s));
+        if (F.aca_tc) {
+            int64_t nrow = (int64_t)p->by[l].nb * nrhs;
+            float *upad = tmp.get<float>((size_t)nrow * F.rkp);
+            split_pad((const float *)ut, 1, (int)nrow, r, (int)nrow, F.rkp, upad, nullptr, s);
+            tc_transfer(F, F.bt_src, F.pair_id, F.Bca, (int64_t)rp * F.rkp, rp, F.rkp, rp, nrhs, upad, w, p->dev_err,
+                        p->wait_tries, s);
+            tc_transfer(F, F.pair_id, F.bt_tgt, F.Aca, (int64_t)npad * rp, r, rp, r, nrhs, w, (float *)vt, p->dev_err,
+                        p->wait_tries, s);
+            tmp.drop(upad);
+        } else {
+            dim3 g1((unsigned)F.n_tiles, cdiv(rp, LG_BM), nrhs);
+            FFM_LAUNCH(k_lag_gemm<false>, g1, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.pair_id, F.Bca,
+                       rp, r, nrhs, (const float *)ut, w);
+            FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.pair_id, F.bt_tgt, F.Aca, r,
+                       rp, nrhs, (const float *)w, (float *)vt);
+        }
+        tmp.drop(w);
+    } else if (F.ts_ok && F.tune_tc == 2) {
+        lag_targets(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
+    } else if (use_tc) {
+        lag_pairs(p, l, (const float *)ut, nrhs, (float *)vt, tmp, s);
+    } else if (cplx) {
+        FFM_LAUNCH(k_lag_gemm<true>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt, F.T, r, rk,
+                   nrhs, (const float2 *)ut, (float2 *)vt);
+    } else {
+        // the gradient has three operator blocks and three outputs per target, component-major
+        for (int d = 0; d < (p->kind == FFM_LAPLACE_GRAD ? 3 : 1); ++d)
+            FFM_LAUNCH(k_lag_gemm<false>, gg, LG_T, 0, s, F.tile_t, F.tile_p0, F.bt_off, F.bt_src, F.bt_tgt,
+                       F.T + (size_t)d * F.n_trans * r * rk, r, rk, nrhs, (const float *)ut,
+                       (float *)vt + (size_t)d * r * nrhs * p->bx[l].nb);
+    }
+}
+
+// All Lagrange levels of an apply, coarsest lo to finest hi: u~ of level hi from the points, up to lo
+// through the children, every level's transfer, v~ down to hi, and from there to the points
+// (every target's accf is written).  False if the plan has no Lagrange level.
+bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s) {
+    int lo = -1, hi = -1;
+    for (int l = 0; l <= p->l_stop; ++l)
+        if (p->far[l].mode == 1 && p->far[l].n_adm > 0) {
+            if (lo < 0) lo = l;
+            hi = l;
+        }
+    if (lo < 0) return false;
+    const FarLevel &F = p->far[hi];
+    const int ls = p->l_stop, r = F.r1 * F.r1 * F.r1;
+    const bool cplx = p->kind == FFM_HELMHOLTZ, dl = p->kind == FFM_LAPLACE_DL, grad = p->kind == FFM_LAPLACE_GRAD;
+    const Cheb cb = make_cheb(F.r1);
+    void *ut[LMAX + 1], *vt[LMAX + 1];
+    const size_t val = sizeof(float) * (cplx ? 2 : 1);
+    for (int l = lo; l <= hi; ++l) {
+        const size_t ub = val * (dl ? 3 : 1) * r * nrhs * (size_t)p->by[l].nb,
+                     vb = val * (grad ? 3 : 1) * r * nrhs * (size_t)p->bx[l].nb;
+        ut[l] = tmp.raw(ub);
+        vt[l] = tmp.raw(vb);
+        if (l == hi) FFM_CUDA(cudaMemsetAsync(ut[l], 0, ub, s));
+        FFM_CUDA(cudaMemsetAsync(vt[l], 0, vb, s));
+    }
+    const LevelArgs AY = level_args(p, p->by[hi], p->by[ls], p->epsY, hi), AX = level_args(p, p->bx[hi], p->bx[ls], p->epsX, hi);
+    if (cplx)
+        lagrange_points_r1<true>(p, F, AY, cb, true, q, nrhs, ut[hi], s);
+    else if (dl)
+        lagrange_anterp_dl_r1(p, F, AY, cb, q, nrhs, ut[hi], s);
+    else
+        lagrange_points_r1<false>(p, F, AY, cb, true, q, nrhs, ut[hi], s);
+    const Halves H = make_halves(F.r1);
+    LinkArgs A{};
+    A.nrhs = nrhs;
+    A.es = cplx ? 2 : 1;
+    for (int l = hi - 1; l >= lo; --l) {
+        A.n = p->by[l].nb;
+        A.first_child = p->by[l].first_child;
+        A.gc = p->by[l + 1].g;
+        A.rowlen = r * (dl ? 3 : cplx ? 2 : 1);
+        A.coff = dl ? r : cplx ? 1 : 0;
+        lag_link_r1(F.r1, A, dl ? 3 : cplx ? 2 : 1, H, true, (const float *)ut[l + 1], (float *)ut[l], s);
+    }
+    for (int l = lo; l <= hi; ++l)
+        if (p->far[l].mode == 1 && p->far[l].n_adm > 0) lagrange_transfer(p, l, ut[l], nrhs, vt[l], tmp, s);
+    for (int l = lo; l < hi; ++l) {
+        A.n = p->bx[l].nb;
+        A.first_child = p->bx[l].first_child;
+        A.gc = p->bx[l + 1].g;
+        A.rowlen = r * (cplx ? 2 : 1);
+        A.coff = cplx ? 1 : 0;
+        A.pbase = grad ? (int64_t)r * nrhs * p->bx[l].nb : 0;
+        A.cbase = grad ? (int64_t)r * nrhs * p->bx[l + 1].nb : 0;
+        lag_link_r1(F.r1, A, grad ? 3 : cplx ? 2 : 1, H, false, (const float *)vt[l], (float *)vt[l + 1], s);
+    }
+    // the gradient's three outputs per target, component-major like its accumulators
+    for (int d = 0; d < (grad ? 3 : 1); ++d) {
+        float2 *out = accf + (size_t)d * nrhs * p->nx;
+        if (cplx)
+            lagrange_points_r1<true>(p, F, AX, cb, false, vt[hi], nrhs, out, s);
+        else
+            lagrange_points_r1<false>(p, F, AX, cb, false, (float *)vt[hi] + (size_t)d * r * nrhs * p->bx[hi].nb, nrhs, out, s);
+    }
+    return true;
 }
 
 // ======================================================= plane-wave kernels

@@ -228,7 +228,6 @@ static void apply_impl(ffm_plan_s *p, const void *u, ffm_dtype udt, int nrhs, vo
     double2 *acc = tmp.get<double2>((size_t)nx * nout);
     FFM_CUDA(cudaMemsetAsync(acc, 0, sizeof(double2) * (size_t)nx * nout, s));
     float2 *accf = tmp.get<float2>((size_t)nx * nout);
-    FFM_CUDA(cudaMemsetAsync(accf, 0, sizeof(float2) * (size_t)nx * nout, s));
     dim3 gy(cdiv(ny, 256), nrhs), gx(cdiv(nx, 256), nout);
     if (dl) {
         if (udt == FFM_F64)
@@ -243,14 +242,10 @@ static void apply_impl(ffm_plan_s *p, const void *u, ffm_dtype udt, int nrhs, vo
         case FFM_C64: FFM_LAUNCH((k_gather_q<float, true>), gy, 256, 0, s, (const float *)du, p->permY, p->wY, ny, nrhs, q); break;
         case FFM_C128: FFM_LAUNCH((k_gather_q<double, true>), gy, 256, 0, s, (const double *)du, p->permY, p->wY, ny, nrhs, q); break;
     }
-    for (int l = 0; l <= p->l_stop; ++l) {
-        const FarLevel &F = p->far[l];
-        if (F.n_adm == 0) continue;
-        if (F.mode == 1)
-            far_lagrange(p, l, q, nrhs, accf, tmp, s);
-        else
-            far_planewave(p, l, (const float2 *)q, nrhs, acc, tmp, s);
-    }
+    if (!far_lagrange(p, q, nrhs, accf, tmp, s))
+        FFM_CUDA(cudaMemsetAsync(accf, 0, sizeof(float2) * (size_t)nx * nout, s));
+    for (int l = 0; l <= p->l_stop; ++l)
+        if (p->far[l].mode == 2 && p->far[l].n_adm > 0) far_planewave(p, l, (const float2 *)q, nrhs, acc, tmp, s);
     near_field(p, q, nrhs, acc, s);
     switch (udt) {
         case FFM_F32: FFM_LAUNCH((k_scatter_v<float, false>), gx, 256, 0, s, acc, accf, p->permX, nx, nrhs, ncomp, (float *)dv); break;

@@ -163,8 +163,8 @@ struct FarLevel {
     uint32_t *tile_t = nullptr;     // per tile: translation
     uint32_t *tile_p0 = nullptr;    // per tile: first pair (index into bt_*)
     int64_t n_src_chunks = 0, n_tgt_chunks = 0;
-    uint2 *src_chunks = nullptr;    // (source box, first point): LAG_CHUNK-point pieces of the boxes
-    uint2 *tgt_chunks = nullptr;    // likewise for the target boxes
+    uint2 *src_chunks = nullptr;    // (box, first point): LAG_CHUNK-point pieces of all source boxes
+    uint2 *tgt_chunks = nullptr;    // likewise of all target boxes
     // target-stationary transfer (Laplace, r <= 64): each 128-target tile's pairs by translation,
     // made where the level runs it (transfer.cu)
     bool ts_ok = false;
@@ -323,9 +323,12 @@ void build_tables(ffm_plan_s *p, int l, TableJob &tj);   // once level l's trans
 void build_octants(ffm_plan_s *p, int l, TableJob &tj);  // once the stop level is known
 int r1_rule(int kind, double eps);
 // farfield.cu / nearfield.cu
-// Lagrange levels add their contributions in FP32 into accf (float2 per target and RHS);
-// the apply adds accf into the FP64 accumulators once, at the end.
-void far_lagrange(const ffm_plan_s *p, int l, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s);
+// All Lagrange levels: their sum in FP32 into accf (float2 per target and RHS, written; false and
+// untouched without such a level); the apply adds accf into the FP64 accumulators at the end.
+bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s);
+// one level's transfer alone, and the bytes of its u~ and v~ (v~ zeroed by the caller)
+void lagrange_transfer(const ffm_plan_s *p, int l, const void *ut, int nrhs, void *vt, Alloc &tmp, cudaStream_t s);
+void lagrange_bytes(const ffm_plan_s *p, int l, int nrhs, size_t *ub, size_t *vb);
 // nmat row-major matrices written with padded rows and columns (zeros): as TF32 hi / lo parts,
 // or (lo == nullptr) as a plain copy into hi
 void split_pad(const float *src, int64_t nmat, int rows, int cols, int rows_pad, int cols_pad, float *hi, float *lo,

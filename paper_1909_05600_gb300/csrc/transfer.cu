@@ -158,6 +158,7 @@ struct PairArgs {
     const __half *T;    // operator images
     float tinv;
     int nk, npad, tcols;
+    int parts;          // K parts of a unit's product, each added to v~ by itself
     int ostride;        // floats between rows of v~
     int nout[PAIR_MAXBLK];
     int64_t ooff[PAIR_MAXBLK];  // first float of the block's columns in v~
@@ -270,10 +271,15 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
     if (tid == 0) pre[A.n_trans] = s_carry;
     __syncthreads();
     const uint32_t tmem = s_tmem;
-    const int64_t units = (int64_t)s_carry * A.nblk;
+    const int per = A.nblk * A.parts;  // units of a tile: (row block, K part)
+    const int64_t units = (int64_t)s_carry * per;
+    // row block, first and end chunk of unit un
+    auto block_of = [&](int64_t un) { return (int)(un % per) / A.parts; };
+    auto k_first = [&](int64_t un) { return (int)(un % A.parts) * A.nk / A.parts; };
+    auto k_end = [&](int64_t un) { return ((int)(un % A.parts) + 1) * A.nk / A.parts; };
     // translation, first row and row count of the tile of unit un
     auto locate = [&](int64_t un, int &t, uint32_t &p0, uint64_t &row0, int &nrows) {
-        const uint32_t tile = (uint32_t)(un / A.nblk);
+        const uint32_t tile = (uint32_t)(un / per);
         int lo = 0, hi = A.n_trans;  // last t with pre[t] <= tile
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -344,19 +350,19 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                 ok = false;
                 break;
             }
-            const int t = s_trans[ix], blk = (int)(un % A.nblk);
+            const int t = s_trans[ix], blk = block_of(un), k0 = k_first(un), k1 = k_end(un);
             const __half *src[8];
             uint32_t bytes[8];
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 const uint32_t row = s_src[ix][r0 + 4 * g];
                 bytes[g] = row != NONE ? 16u : 0u;
-                src[g] = A.u + (size_t)(row != NONE ? row : 0u) * A.nk * HROW + sg * 8;
+                src[g] = A.u + ((size_t)(row != NONE ? row : 0u) * A.nk + k0) * HROW + sg * 8;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_ixempty[ix]);
             const __half *Tb = A.T + ((size_t)t * A.nblk + blk) * A.nk * A.npad * HROW;
-            for (int kc = 0; kc < A.nk; kc += CPS, ++c) {
+            for (int kc = k0; kc < k1; kc += CPS, ++c) {
                 const uint32_t slot = c % NSTG;
                 const bool w_ok = c < NSTG || mbar_wait(&s_empty[slot], ((c / NSTG) - 1) & 1, A.tries, A.err);
                 if (!__all_sync(0xffffffffu, w_ok)) {
@@ -408,7 +414,8 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                     break;
                 }
                 const uint32_t d = tmem + buf * (uint32_t)A.tcols;
-                for (int kc = 0; kc < A.nk; kc += CPS) {
+                const int k0 = k_first(un), k1 = k_end(un);
+                for (int kc = k0; kc < k1; kc += CPS) {
                     if (!mbar_wait(&s_full[slot], par, A.tries, A.err)) {
                         ok = false;
                         break;
@@ -416,7 +423,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                     fence_proxy_async();  // the rows came by cp.async, through the generic proxy
                     tc_fence_after();
                     const uint32_t off = slot * (stage >> 4);
-                    stage_mma<CPS, STACK>(d, alo + off, blo + off, (uint32_t)A.npad, id1, id2, kc == 0);
+                    stage_mma<CPS, STACK>(d, alo + off, blo + off, (uint32_t)A.npad, id1, id2, kc == k0);
                     tc_commit(&s_empty[slot]);
                     if (++slot == NSTG) {
                         slot = 0;
@@ -437,7 +444,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         uint32_t i = 0;
         for (int64_t un = blockIdx.x; un < units; un += gridDim.x, ++i) {
             const uint32_t buf = i & 1, ix = i % PAIR_IX;
-            const int blk = (int)(un % A.nblk), nout = A.nout[blk];
+            const int blk = block_of(un), nout = A.nout[blk];
             const bool i_ok = mbar_wait(&s_ixfull[ix], (i / PAIR_IX) & 1, A.tries, A.err);
             if (!__all_sync(0xffffffffu, i_ok)) {
                 ok = false;
@@ -522,7 +529,11 @@ void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, 
     const bool cplx = p->kind == FFM_HELMHOLTZ;
     const int r = F.r1 * F.r1 * F.r1, rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;
     const int rows = cplx ? 2 * r : r, K = cplx ? 2 * rk : rk, ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
-    F.h_bpc = cdiv(rows, 256);
+    // Complex levels: at most 128 rows, so that hi hi has an accumulator of its own, and K parts of at most
+    // eight chunks (lag_pairs).  A tensor-core accumulation truncates at every step; with one accumulator
+    // for the three products over the whole K = 432 the Helmholtz parity case (cube surface, k = 12) went from 3.1e-7
+    // (FP32 multiply-adds) to 1.03e-6 of the oracle's FFM.
+    F.h_bpc = cdiv(rows, cplx ? 128 : 256);
     F.h_nb = ((int)cdiv(rows, F.h_bpc) + 15) / 16 * 16;
     F.h_nk = cdiv(K, HK);
     const int nblk = F.h_bpc * ncomp;
@@ -579,6 +590,7 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.T = (const __half *)F.Th;
     A.tinv = F.h_inv;
     A.nk = F.h_nk;
+    A.parts = cplx ? cdiv(F.h_nk, 8) : 1;
     A.npad = F.h_nb;
     const bool stack = A.npad <= 128;
     A.tcols = 32;
@@ -593,7 +605,7 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.vt = vt;
     A.err = p->dev_err;
     A.tries = p->wait_tries;
-    const int64_t most = ((int64_t)F.n_trans + F.n_adm * nrhs / HM) * A.nblk;  // at least the number of units
+    const int64_t most = ((int64_t)F.n_trans + F.n_adm * nrhs / HM) * A.nblk * A.parts;  // at least the number of units
     const unsigned grid = (unsigned)std::min<int64_t>(most, 152);
     // stages of two chunks where the K extent allows: half the barrier round trips
     if (A.npad <= 64 && A.nk % 2 == 0)

@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(32 * DS_W) k_descend(const __grid_constant__ D
 }
 
 // ---- a level's lists from its counts: offsets of the admissible and near pairs by target, the
-// targets with admissible pairs and the sources in use, and both lists' point chunks (box, first
+// targets with admissible pairs and the sources in use, and all boxes' point chunks (box, first
 // point) of at most ch points, so that the point-wise kernels spread large boxes over many blocks.
 // Tiles of LV_TILE boxes: sums per tile, a scan over the tiles in one block (which also numbers the
 // translations in use and leaves all totals in one place, the level's only read-back), then the lists.
@@ -789,9 +789,10 @@ __global__ void __launch_bounds__(LV_T) k_level_sums(const __grid_constant__ Lev
         } else {
             listed = A.src_used[i] != 0;
         }
+        const uint32_t sz = start[i + 1] - start[i];
+        if (A.ch) b += (sz + A.ch - 1) / A.ch;
         if (listed) {
-            const uint32_t sz = start[i + 1] - start[i];
-            b += (1ull << 32) | (A.ch ? (sz + A.ch - 1) / A.ch : 0u);
+            b += 1ull << 32;
             pts += sz;
             pw += X ? (sz + PW_TC_BCH - 1) / PW_TC_BCH : (sz + PW_TC_FCH - 1) / PW_TC_FCH;
         }
@@ -875,10 +876,8 @@ __global__ void __launch_bounds__(LV_T) k_level_lists(const __grid_constant__ Le
             } else {
                 listed = A.src_used[i] != 0;
             }
-            if (listed) {
-                const uint32_t sz = start[i + 1] - start[i];
-                b[j] = (1ull << 32) | (A.ch ? (sz + A.ch - 1) / A.ch : 0u);
-            }
+            const uint32_t sz = start[i + 1] - start[i];
+            b[j] = ((unsigned long long)listed << 32) | (A.ch ? (sz + A.ch - 1) / A.ch : 0u);
         }
         sa += a[j];
         sb += b[j];
@@ -893,7 +892,7 @@ __global__ void __launch_bounds__(LV_T) k_level_lists(const __grid_constant__ Le
         const int64_t i = i0 + j;
         cpos[threadIdx.x * LV_PER + j] = (uint32_t)eb - c0;
         if (i < n) {
-            if (b[j]) {
+            if (b[j] >> 32) {
                 const uint32_t r = (uint32_t)(eb >> 32);
                 if (X) {
                     A.tgt[r] = (uint32_t)i;
