@@ -521,7 +521,14 @@ ffm_status ffm_plan_export(const ffm_plan_t *plan, int what, int level, void *ho
             if (!host_out || F.n_adm == 0) return;
             auto tgt = to_host(F.tgt, F.n_tgt, s);
             auto off = to_host(F.adm_off, F.n_tgt + 1, s);
-            auto src = to_host(F.adm_src, F.n_adm, s);
+            Alloc tmp;  // a level without pair lists gets them for this call
+            tmp.stream = s;
+            uint32_t *adm = F.adm_src;
+            if (!adm) {
+                adm = tmp.get<uint32_t>(F.n_adm);
+                fill_pair_lists(plan, level, adm, tmp.get<uint32_t>(F.n_adm), s);
+            }
+            auto src = to_host(adm, F.n_adm, s);
             auto gx = to_host(plan->bx[level].g, plan->bx[level].nb, s);
             auto gy = to_host(plan->by[level].g, plan->by[level].nb, s);
             FFM_CUDA(cudaStreamSynchronize(s));

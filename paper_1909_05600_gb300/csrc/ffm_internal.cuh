@@ -150,7 +150,7 @@ struct FarLevel {
     uint32_t *tgt = nullptr;        // n_tgt target box indices
     uint32_t *src = nullptr;        // n_src source box indices
     uint32_t *adm_off = nullptr;    // n_tgt+1 CSR offsets (per listed target)
-    uint32_t *adm_src = nullptr;    // n_adm source box per pair
+    uint32_t *adm_src = nullptr;    // n_adm source box per pair (null on target-stationary levels)
     uint32_t *adm_t = nullptr;      // n_adm translation index per pair
     int4 *trans_m = nullptr;        // n_trans integer offsets gX - gY
     std::vector<int4> h_trans_m;
@@ -165,13 +165,11 @@ struct FarLevel {
     int64_t n_src_chunks = 0, n_tgt_chunks = 0;
     uint2 *src_chunks = nullptr;    // (box, first point): LAG_CHUNK-point pieces of all source boxes
     uint2 *tgt_chunks = nullptr;    // likewise of all target boxes
-    // target-stationary transfer (Laplace, r <= 64): each 128-target tile's pairs by translation,
-    // made where the level runs it (transfer.cu)
+    // target-stationary transfer (Laplace, r <= 64): the parents' near tables (64 entries of first
+    // child, child mask), made where the level runs it (transfer.cu); such a level has no pair lists
+    // (adm_src, adm_t) unless something else asks for them
     bool ts_ok = false;
-    uint32_t *ts_src = nullptr;     // n_adm source boxes
-    uint8_t *ts_row = nullptr;      // n_adm target rows in the tile
-    uint32_t *ts_steps = nullptr;   // n_trans per tile: translation | first entry << 12
-    uint32_t *ts_n = nullptr;       // steps per tile
+    uint2 *ts_near = nullptr;
     // tensor-core transfer by translation: f16 hi / lo images of T_t (transfer.cu), h_bpc blocks of
     // h_nb rows per component, h_nk chunks of 32 columns, 1 / scale
     uint16_t *Th = nullptr;
@@ -255,6 +253,10 @@ struct ffm_plan_s {
     double *wY = nullptr;                          // sorted weights (or null)
     uint64_t *keyX = nullptr, *keyY = nullptr;     // sorted Morton keys (exports)
     ffm::BoxLevel bx[ffm::LMAX + 1], by[ffm::LMAX + 1];
+    uint32_t *parent[ffm::LMAX + 1] = {};         // parent of each target box
+    // near source boxes of each target box, per level (CSR); kept where a finer level can run the
+    // target-stationary transfer
+    uint32_t *nr_off[ffm::LMAX + 1] = {}, *nr_src[ffm::LMAX + 1] = {};
     ffm::FarLevel far[ffm::LMAX + 1];
     int64_t n_near = 0;
     uint32_t *near_off = nullptr;   // nbx(l_stop)+1 CSR over all target leaves
@@ -274,8 +276,11 @@ namespace ffm {
 // tree.cu
 void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_dtype ydt, const void *w,
                 ffm_dtype wdt, Alloc &tmp);
-// transfer.cu: pairs of Lagrange level l by tile and translation, for the target-stationary
-// transfer (on demand)
+// tree.cu: smallest offset g_X - g_Y per axis of a near pair of level l; the admissible pairs of a
+// level without lists, from its parents' near lists, into src and t (n_adm entries)
+int3 near_base(const ffm_plan_s *p, int l);
+void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cudaStream_t s);
+// transfer.cu: near tables of Lagrange level l for the target-stationary transfer (on demand)
 void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s);
 // tree.cu: pairs of Lagrange level l grouped by translation; column tiles of the CUDA-core
 // transfer and of the ACA factors (both on demand; no-ops if present)

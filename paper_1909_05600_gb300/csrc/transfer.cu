@@ -623,17 +623,18 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
 // ---- target-stationary transfer (real operators, r <= 64)
 //
 // For levels whose targets have many partners (volumes: 290-360 of 665 translations).  A block owns
-// TG_M = 128 consecutive target boxes (TMEM lane = box) and runs over the translations present
-// among their pairs; the products accumulate and each target's v~ is written once: no adds to
-// memory, no grouping of all pairs by translation.  k_tile_entries orders each tile's pairs by
-// translation once per plan.
+// TG_M = 128 consecutive target boxes (TMEM lane = box) and runs over the level's translations; the
+// products accumulate and each target's v~ is written once: no adds to memory, no grouping of the
+// pairs, and no pair lists at all.  The source box of a target at a translation is found from its
+// parent's near table (k_near_table): the near source boxes of the parent level by their offset (at
+// most 4 per axis), each with its first child and the mask of its children's octants.
 //
 // What bounds it: the gathered rows' and the operators' way from L2 (48 KB a step at most).  A step is
-// one translation: warps 9-12 fetch the steps' (row, source) entries in turn and lay them out by row
-// in a shared ring, so that no copying thread waits for a list; warps 0-3 copy the 128 source rows
-// (hi and lo images, 16-byte cp.async segments, rows without a partner zero-filled without a
-// read), thread 0 starts the bulk copy of T_t's image, warp 8 issues hi [hi; lo] (N = 2 npad) and
-// lo hi, 4 steps in flight (8 where K <= 32).  Nothing is converted on the way.
+// one translation: warps 9-12 look up the step's 128 sources in turn and leave them in a shared ring, so
+// that no copying thread waits for a lookup; warps 0-3 copy the source rows (hi and lo images,
+// 16-byte cp.async segments, rows without a partner zero-filled without a read), thread 0 starts
+// the bulk copy of T_t's image, warp 8 issues hi [hi; lo] (N = 2 npad) and lo hi, 4 steps in flight (8
+// where K <= 32).  Nothing is converted on the way.
 // Rows of different sources meet in one accumulator, so the level shares one scale (k_level_max):
 // a value keeps its 22 bits down to 2^-15 of the level's largest, and below that an absolute
 // error of 2^-39 of it.
@@ -643,88 +644,65 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
 // while the other fills.  Every wait is bounded as in k_lag_pairs.
 //
 // Measured on GB300, level 7 of clustered 10M (193k targets, 68M pairs): 3.52 ms, 0.53 us a step
-// (the kernel before it, FP32 rows split into TF32 by the copying warps: 7.9 ms).
+// (the kernel before it, FP32 rows split into TF32 by the copying warps: 7.9 ms).  Lists of the
+// pairs by tile and translation instead of the near tables cost 64 ms of plan at 1e8 points.
 constexpr int TG_M = 128;
 constexpr int TG_DRAIN = 8;        // translations per accumulator fill
-constexpr int TG_MAXT = 4096;      // translation indices are below this
 constexpr int TG_T = 416;
-constexpr int TG_IX = 8;           // steps whose sources are held by row
+constexpr int TG_IX = 8;           // steps whose sources are held
 
-// The pairs of each tile of TG_M targets ordered by translation: entry e of the tile (at the tile's
-// first pair) holds a source box and the target's row in the tile; step k of the tile is its k-th
-// translation present, t | first entry << 12.  One block per tile: counts per translation in shared
-// memory, their prefix sums, then every pair takes the next place of its translation (the order
-// of a step's entries does not matter: their rows differ).
-__global__ void __launch_bounds__(256) k_tile_entries(const uint32_t *__restrict__ adm_off, int64_t n_tgt,
-                                                      const uint32_t *__restrict__ adm_src,
-                                                      const uint32_t *__restrict__ adm_t, int n_trans,
-                                                      uint32_t *__restrict__ ent_src, uint8_t *__restrict__ ent_row,
-                                                      uint32_t *__restrict__ steps, uint32_t *__restrict__ nsteps) {
-    __shared__ uint32_t cnt[TG_MAXT];
-    __shared__ uint32_t wsum[8], wstep[8];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t x0 = (int64_t)blockIdx.x * TG_M, x1 = min(n_tgt, x0 + TG_M);
-    for (int t = tid; t < TG_MAXT; t += 256) cnt[t] = 0u;
-    __syncthreads();
-    const uint32_t e0 = adm_off[x0], e1 = adm_off[x1];
-    for (uint32_t e = e0 + tid; e < e1; e += 256) atomicAdd(&cnt[adm_t[e]], 1u);
-    __syncthreads();
-    // thread i owns translations 16 i .. + 15: first entry and step number of each
-    constexpr int PER = TG_MAXT / 256;
-    uint32_t c[PER], sum = 0, st = 0;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        c[j] = cnt[tid * PER + j];
-        sum += c[j];
-        st += c[j] > 0;
+// octants of each box's children, one bit each (children are in octant order)
+__global__ void k_child_masks(const uint32_t *__restrict__ first_child, const int4 *__restrict__ gc, int64_t n,
+                              uint8_t *__restrict__ mask) {
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= n) return;
+    uint32_t m = 0;
+    for (uint32_t c = first_child[b]; c < first_child[b + 1]; ++c) {
+        const int4 g = gc[c];
+        m |= 1u << ((g.x & 1) << 2 | (g.y & 1) << 1 | (g.z & 1));
     }
-    uint32_t isum = sum, ist = st;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t a = __shfl_up_sync(0xffffffffu, isum, o), b = __shfl_up_sync(0xffffffffu, ist, o);
-        if (lane >= o) {
-            isum += a;
-            ist += b;
-        }
+    mask[b] = (uint8_t)m;
+}
+
+// Near table of every target box of a level, one warp per box: entry (kx, ky, kz) - base of the offset
+// k = g_X - g_Y of a near source box holds its first child and child mask (mask 0: no such box).
+__global__ void __launch_bounds__(256) k_near_table(int64_t n, const uint32_t *__restrict__ off,
+                                                    const uint32_t *__restrict__ src, const int4 *__restrict__ gx,
+                                                    const int4 *__restrict__ gy, const uint32_t *__restrict__ fcy,
+                                                    const uint8_t *__restrict__ mask, int3 base, int *__restrict__ err,
+                                                    uint2 *__restrict__ table) {
+    const int64_t a = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (a >= n) return;
+    uint2 *t = table + a * 64;
+    t[lane] = t[32 + lane] = make_uint2(0u, 0u);
+    __syncwarp();
+    const int4 p = gx[a];
+    for (uint32_t e = off[a] + lane; e < off[a + 1]; e += 32) {
+        const uint32_t b = src[e];
+        const int4 q = gy[b];
+        const unsigned kx = p.x - q.x - base.x, ky = p.y - q.y - base.y, kz = p.z - q.z - base.z;
+        if (kx < 4u && ky < 4u && kz < 4u)
+            t[(kx * 4 + ky) * 4 + kz] = make_uint2(fcy[b], mask[b]);
+        else
+            atomicOr(err, 1);  // not possible: |sigma + k| < 2 holds for at most four integers k
     }
-    if (lane == 31) {
-        wsum[warp] = isum;
-        wstep[warp] = ist;
-    }
-    __syncthreads();
-    uint32_t off = isum - sum, k = ist - st;
-    for (int w = 0; w < warp; ++w) {
-        off += wsum[w];
-        k += wstep[w];
-    }
-    uint32_t *out = steps + (size_t)blockIdx.x * n_trans;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        cnt[tid * PER + j] = off;
-        if (c[j] > 0) out[k++] = (uint32_t)(tid * PER + j) | (off << 12);
-        off += c[j];
-    }
-    if (tid == 255) nsteps[blockIdx.x] = k;
-    __syncthreads();
-    for (int64_t x = x0 + warp; x < x1; x += 8)
-        for (uint32_t e = adm_off[x] + lane; e < adm_off[x + 1]; e += 32) {
-            const uint32_t o = e0 + atomicAdd(&cnt[adm_t[e]], 1u);
-            ent_src[o] = adm_src[e];
-            ent_row[o] = (uint8_t)(x - x0);
-        }
 }
 
 // The target-stationary transfer of a Lagrange level made possible (ts_ok), where the plan's rule, the
 // option, the autotuner or its cache asks for it.
 void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
-    if (F.mode != 1 || F.n_adm == 0 || F.ts_ok || !F.Th || p->kind != FFM_LAPLACE || F.r1 > 4) return;
-    const int64_t nt = cdiv(F.n_tgt, TG_M);
-    F.ts_src = p->mem.get<uint32_t>(F.n_adm);
-    F.ts_row = p->mem.get<uint8_t>(F.n_adm);
-    F.ts_steps = p->mem.get<uint32_t>((size_t)nt * F.n_trans);
-    F.ts_n = p->mem.get<uint32_t>(nt);
-    FFM_LAUNCH(k_tile_entries, (unsigned)nt, 256, 0, s, F.adm_off, F.n_tgt, F.adm_src, F.adm_t, F.n_trans, F.ts_src,
-               F.ts_row, F.ts_steps, F.ts_n);
+    if (F.mode != 1 || F.n_adm == 0 || F.ts_ok || !F.Th || p->kind != FFM_LAPLACE || F.r1 > 4 || l == 0 || !p->nr_off[l - 1])
+        return;
+    const int64_t nx = p->bx[l - 1].nb, ny = p->by[l - 1].nb;
+    Alloc tmp;
+    tmp.stream = s;
+    uint8_t *mask = tmp.get<uint8_t>(ny);
+    FFM_LAUNCH(k_child_masks, cdiv(ny, 256), 256, 0, s, p->by[l - 1].first_child, p->by[l].g, ny, mask);
+    F.ts_near = p->mem.get<uint2>(nx * 64);
+    FFM_LAUNCH(k_near_table, cdiv(nx, 8), 256, 0, s, nx, p->nr_off[l - 1], p->nr_src[l - 1], p->bx[l - 1].g, p->by[l - 1].g,
+               p->by[l - 1].first_child, mask, near_base(p, l - 1), p->dev_err, F.ts_near);
     F.ts_ok = true;
 }
 
@@ -738,8 +716,10 @@ __global__ void k_level_max(const float *__restrict__ u, int64_t n, uint32_t *__
 }
 
 struct TargetArgs {
-    const uint32_t *tgt, *adm_off, *ent_src, *steps, *nsteps;
-    const uint8_t *ent_row;
+    const uint32_t *tgt, *parent;
+    const int4 *g, *trans;  // coordinates of the target boxes, translations
+    const uint2 *near;      // near tables of the parents
+    int3 base;
     int64_t n_tgt;
     int n_trans, nrhs, nk, npad, r, tcols;
     const __half *u;        // row images of (source box, right-hand side), one scale for all
@@ -758,7 +738,6 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
     __shared__ __align__(8) uint64_t s_full[NSTG], s_empty[NSTG], s_accfull[2], s_accempty[2], s_done;
     __shared__ __align__(8) uint64_t s_ixfull[TG_IX], s_ixempty[TG_IX];
     __shared__ uint32_t s_src[TG_IX][TG_M];  // the step's source box by row, NONE without a partner
-    __shared__ uint32_t s_trans[TG_IX];
     __shared__ uint32_t s_tmem, s_cmax;
     __shared__ int s_bad;
     constexpr uint32_t NONE = 0xffffffffu;
@@ -793,24 +772,37 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t nsteps = A.nsteps[blockIdx.x];
+    const uint32_t nsteps = (uint32_t)A.n_trans;
     bool ok = true;
     if (warp > 8) {
-        // ---- sources: warp w lays out steps w - 9, w - 9 + 4, ...
-        const uint32_t e0 = A.adm_off[x0], ne = A.adm_off[min(A.n_tgt, x0 + TG_M)] - e0;
-        const uint32_t *steps = A.steps + (size_t)blockIdx.x * A.n_trans;
-        for (uint32_t s = warp - 9; s < nsteps; s += 4) {
-            const uint32_t ix = s % TG_IX, rec = steps[s], nxt = s + 1 < nsteps ? steps[s + 1] : 0u;
-            const uint32_t f0 = rec >> 12, f1 = s + 1 < nsteps ? nxt >> 12 : ne;
-            uint32_t src[4];
-            int row[4];
+        // ---- sources: warp w looks up steps w - 9, w - 9 + 4, ...; lane: rows lane, lane + 32, ...
+        int4 g[4];
+        const uint2 *near[4];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {  // at most TG_M entries
-                const uint32_t f = f0 + 32 * g + lane;
-                row[g] = -1;
-                if (f < f1) {
-                    src[g] = A.ent_src[e0 + f];
-                    row[g] = A.ent_row[e0 + f];
+        for (int k = 0; k < 4; ++k) {
+            const int64_t x = x0 + 32 * k + lane;
+            near[k] = nullptr;
+            if (x < A.n_tgt) {
+                const uint32_t box = A.tgt[x];
+                g[k] = A.g[box];
+                near[k] = A.near + (size_t)A.parent[box] * 64;
+            }
+        }
+        for (uint32_t s = warp - 9; s < nsteps; s += 4) {
+            const uint32_t ix = s % TG_IX;
+            const int4 m4 = A.trans[s];
+            uint2 e[4];
+            uint32_t oct[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                e[k] = make_uint2(0u, 0u);
+                oct[k] = 0;
+                if (near[k]) {
+                    const int qx = g[k].x - m4.x, qy = g[k].y - m4.y, qz = g[k].z - m4.z;
+                    const unsigned kx = (g[k].x >> 1) - (qx >> 1) - A.base.x, ky = (g[k].y >> 1) - (qy >> 1) - A.base.y,
+                                   kz = (g[k].z >> 1) - (qz >> 1) - A.base.z;
+                    oct[k] = (qx & 1) << 2 | (qy & 1) << 1 | (qz & 1);
+                    if (kx < 4u && ky < 4u && kz < 4u) e[k] = __ldg(near[k] + (kx * 4 + ky) * 4 + kz);
                 }
             }
             const bool w_ok = s < TG_IX || mbar_wait(&s_ixempty[ix], ((s / TG_IX) - 1) & 1, A.tries, A.err);
@@ -819,12 +811,9 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
                 break;
             }
 #pragma unroll
-            for (int g = 0; g < 4; ++g) s_src[ix][32 * g + lane] = NONE;
-            __syncwarp();
-#pragma unroll
-            for (int g = 0; g < 4; ++g)
-                if (row[g] >= 0) s_src[ix][row[g]] = src[g];
-            if (lane == 0) s_trans[ix] = rec & 4095u;
+            for (int k = 0; k < 4; ++k)
+                s_src[ix][32 * k + lane] =
+                    (e[k].y >> oct[k] & 1u) ? e[k].x + __popc(e[k].y & ((1u << oct[k]) - 1u)) : NONE;
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_ixfull[ix]);
         }
@@ -840,7 +829,6 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
                 ok = false;
                 break;
             }
-            const uint32_t t = s_trans[ix];
             const __half *p[8];
             uint32_t n[8];
 #pragma unroll
@@ -859,7 +847,7 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
             }
             if (tid == 0) {
                 mbar_expect(&s_full[slot], bbytes);
-                bulk_g2s(smem + (size_t)slot * stage + CPS * A_BYTES, A.T + (size_t)t * CPS * A.npad * HROW, bbytes,
+                bulk_g2s(smem + (size_t)slot * stage + CPS * A_BYTES, A.T + (size_t)s * CPS * A.npad * HROW, bbytes,
                          &s_full[slot]);
             }
             const uint32_t dst = dst0 + slot * stage;
@@ -997,11 +985,11 @@ void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt
     FFM_LAUNCH(k_level_max, (unsigned)std::min<int64_t>(cdiv(nrow * r, 1024), 152 * 8), 256, 0, s, u, nrow * r, mx);
     FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, r, F.h_nk, img, (float *)nullptr, (const uint32_t *)mx);
     A.tgt = F.tgt;
-    A.adm_off = F.adm_off;
-    A.ent_src = F.ts_src;
-    A.ent_row = F.ts_row;
-    A.steps = F.ts_steps;
-    A.nsteps = F.ts_n;
+    A.parent = p->parent[l];
+    A.g = p->bx[l].g;
+    A.trans = F.trans_m;
+    A.near = F.ts_near;
+    A.base = near_base(p, l - 1);
     A.n_trans = F.n_trans;
     A.n_tgt = F.n_tgt;
     A.nrhs = nrhs;

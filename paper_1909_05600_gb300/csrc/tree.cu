@@ -642,7 +642,7 @@ struct DescendArgs {
     uint8_t *src_used;
     int *err;
     const uint32_t *tpos;         // pass 2: translation index by code
-    uint32_t *adm_src, *adm_t, *near_out;
+    uint32_t *adm_src, *adm_t, *near_out;  // pass 2: null where not wanted
 };
 
 template <bool EMIT>
@@ -690,10 +690,12 @@ __global__ void __launch_bounds__(32 * DS_W) k_descend(const __grid_constant__ D
                 const uint32_t ma = __ballot_sync(0xffffffffu, adm), mn = __ballot_sync(0xffffffffu, valid && !adm);
                 if constexpr (EMIT) {
                     if (adm) {
-                        const uint32_t o = ia + __popc(ma & below);
-                        A.adm_src[o] = b2;
-                        A.adm_t[o] = pos[code];
-                    } else if (valid) {
+                        if (A.adm_src) {
+                            const uint32_t o = ia + __popc(ma & below);
+                            A.adm_src[o] = b2;
+                            A.adm_t[o] = pos[code];
+                        }
+                    } else if (valid && A.near_out) {
                         A.near_out[in + __popc(mn & below)] = b2;
                     }
                 } else if (adm) {
@@ -1136,7 +1138,7 @@ static void launch_leaf_eps(const void *P, const uint32_t *perm, const uint64_t 
 // Box tables of one set for levels 0..ldeep (boxes at level l = runs of key >> 3(21-l)); parents
 // only where asked for (the target boxes).
 static void build_boxes(ffm_plan_s *p, BoxLevel *bl, const SetPts &S, const int64_t *nb, int ldeep, uint32_t **parent,
-                        Alloc &tmp, cudaStream_t s) {
+                        cudaStream_t s) {
     Alloc &m = p->mem;
     BoxOut O{};
     for (int l = 0; l <= ldeep; ++l) {
@@ -1147,7 +1149,7 @@ static void build_boxes(ffm_plan_s *p, BoxLevel *bl, const SetPts &S, const int6
         O.fine[l] = B.fine = m.get<uint32_t>(B.nb + 1);
         O.g[l] = B.g = m.get<int4>(B.nb);
         if (l < ldeep) O.first_child[l] = B.first_child = m.get<uint32_t>(B.nb + 1);
-        if (parent) O.parent[l] = parent[l] = tmp.get<uint32_t>(B.nb);
+        if (parent) O.parent[l] = parent[l] = m.get<uint32_t>(B.nb);
     }
     FFM_LAUNCH(k_box_emit, (unsigned)S.ntile, BT_T, 0, s, S, O, ldeep);
 }
@@ -1228,6 +1230,65 @@ static int64_t build_tiles(ffm_plan_s *p, const FarLevel &F, uint32_t bn, uint32
     return n;
 }
 
+static D3 level_shift(const ffm_plan_s *p, int l) {
+    return D3{{std::ldexp(p->sigma[0], l), std::ldexp(p->sigma[1], l), std::ldexp(p->sigma[2], l)}};
+}
+
+int3 near_base(const ffm_plan_s *p, int l) {
+    const AdmK K = adm_thresholds(level_shift(p, l));
+    return make_int3(K.hi[0] + 1, K.hi[1] + 1, K.hi[2] + 1);
+}
+
+static int4 trans_centre(const ffm_plan_s *p, int l) {
+    if (l == 0) return make_int4(0, 0, 0, 0);  // the single root pair has m = 0
+    return make_int4((int)std::floor(-std::ldexp(p->sigma[0], l) + 0.5), (int)std::floor(-std::ldexp(p->sigma[1], l) + 0.5),
+                     (int)std::floor(-std::ldexp(p->sigma[2], l) + 0.5), 0);
+}
+
+__global__ void k_trans_codes(const int4 *__restrict__ m, int n, int4 c, uint32_t *__restrict__ tpos) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const int4 v = m[t];
+    tpos[(v.x - c.x + 8) | (v.y - c.y + 8) << 4 | (v.z - c.z + 8) << 8] = (uint32_t)t;
+}
+
+// The descent's second pass again, for the admissible pairs alone; the offsets per box come from the
+// listed targets' offsets.
+__global__ void k_box_offsets(const uint32_t *__restrict__ tgt, const uint32_t *__restrict__ off, int64_t n,
+                              uint32_t *__restrict__ out) {
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x < n) out[tgt[x]] = off[x];
+}
+
+void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cudaStream_t s) {
+    const FarLevel &F = p->far[l];
+    Alloc tmp;
+    tmp.stream = s;
+    DescendArgs D{};
+    D.n = p->bx[l].nb;
+    D.parent = p->parent[l];
+    D.near_off = p->nr_off[l - 1];
+    D.near_src = p->nr_src[l - 1];
+    D.fcy = p->by[l - 1].first_child;
+    D.gx = p->bx[l].g;
+    D.gy = p->by[l].g;
+    D.K = adm_thresholds(level_shift(p, l));
+    D.c = trans_centre(p, l);
+    D.cadm = tmp.get<uint32_t>(D.n);
+    D.cnear = tmp.get<uint32_t>(D.n);
+    uint32_t *tpos = tmp.get<uint32_t>(4096);
+    D.tpos = tpos;
+    D.err = p->dev_err;
+    D.adm_src = src;
+    D.adm_t = t;
+    FFM_CUDA(cudaMemsetAsync(D.cadm, 0, sizeof(uint32_t) * D.n, s));
+    FFM_CUDA(cudaMemsetAsync(D.cnear, 0, sizeof(uint32_t) * D.n, s));
+    FFM_CUDA(cudaMemsetAsync(tpos, 0, sizeof(uint32_t) * 4096, s));
+    FFM_LAUNCH(k_trans_codes, cdiv(F.n_trans, 256), 256, 0, s, F.trans_m, F.n_trans, D.c, tpos);
+    FFM_LAUNCH(k_box_offsets, cdiv(F.n_tgt, 256), 256, 0, s, F.tgt, F.adm_off, F.n_tgt, D.cadm);
+    FFM_LAUNCH(k_descend<true>, std::min<unsigned>(cdiv(D.n, DS_W), 152u * 32u), 32 * DS_W, 0, s, D);
+}
+
 // Pairs of Lagrange level l grouped by translation (CSR bt_off over translations, with each
 // pair's source and target box).  Made while the plan is built, or later by the autotuner or
 // when the target-stationary transfer cannot take the level; a level that runs the
@@ -1237,6 +1298,11 @@ void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     if (F.mode != 1 || F.n_adm == 0 || F.bt_off) return;
     Alloc tmp;
     tmp.stream = s;
+    if (!F.adm_src) {
+        F.adm_src = p->mem.get<uint32_t>(F.n_adm);
+        F.adm_t = p->mem.get<uint32_t>(F.n_adm);
+        fill_pair_lists(p, l, F.adm_src, F.adm_t, s);
+    }
     F.bt_src = p->mem.get<uint32_t>(F.n_adm);
     F.bt_tgt = p->mem.get<uint32_t>(F.n_adm);
     F.bt_off = p->mem.get<uint32_t>(F.n_trans + 1);
@@ -1282,11 +1348,7 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     D.n = nx;
     D.gx = p->bx[l].g;
     D.gy = p->by[l].g;
-    D.c.x = (int)std::floor(-std::ldexp(p->sigma[0], l) + 0.5);
-    D.c.y = (int)std::floor(-std::ldexp(p->sigma[1], l) + 0.5);
-    D.c.z = (int)std::floor(-std::ldexp(p->sigma[2], l) + 0.5);
-    D.c.w = 0;
-    if (root) D.c = make_int4(0, 0, 0, 0);  // the single root pair has m = 0
+    D.c = trans_centre(p, l);
     // zeroed scratch: totals, translation flags, error flag, source flags
     struct Scratch {
         LevelTotals tot;
@@ -1351,15 +1413,32 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     F.n_adm = na;
     p->info.n_adm[l] = na;
     const bool last = stop(nn);
-    if (na > 0) {
+    F.n_trans = (int)h.ntrans;
+    F.n_tgt = h.ntgt;
+    F.r1 = p->r1_override > 0 ? p->r1_override : r1_rule(p->kind, p->eps);
+    // a level that is to run the target-stationary transfer (the option, the pick stored in the plan's
+    // autotune cache, or the rule) takes no pair lists
+    const bool ts_able = p->kind == FFM_LAPLACE && F.r1 <= 4 && !(p->aca_eps > 0.0);
+    const int pick = lag && na > 0 && p->lag_transfer == 0 ? cached_lag_pick(p, l) : -1;
+    bool ts_first = false;
+    if (lag && na > 0) {
+        if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
+        if (ts_able && !root && p->lag_transfer == 0 && pick < 0 && target_stationary_pays(F)) F.tune_tc = 2;
+        ts_first = ts_able && !root && (F.tune_tc == 2 || pick == 2);
+    }
+    if (na > 0 && !ts_first) {
         F.adm_src = p->mem.get<uint32_t>(na);
         F.adm_t = p->mem.get<uint32_t>(na);
     }
-    near.src = last ? p->mem.get<uint32_t>(nn) : tmp.get<uint32_t>(nn);
+    // the near lists outlive the descent where it stops and where the next level may look into them
+    const bool keep = last || ts_able;
+    near.src = keep ? p->mem.get<uint32_t>(nn) : tmp.get<uint32_t>(nn);
     near.off = D.cnear;
-    if (last) {
+    if (keep) {
         near.off = p->mem.get<uint32_t>(nx + 1);
         FFM_CUDA(cudaMemcpyAsync(near.off, D.cnear, sizeof(uint32_t) * (nx + 1), cudaMemcpyDeviceToDevice, s));
+        p->nr_off[l] = near.off;
+        p->nr_src[l] = near.src;
     }
     D.adm_src = F.adm_src;
     D.adm_t = F.adm_t;
@@ -1372,7 +1451,6 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     }
     if (na == 0) return nn;
     F.mode = lag ? 1 : 2;
-    F.n_tgt = h.ntgt;
     F.tgt = L.tgt;
     F.adm_off = L.adm_off;
     F.n_src = h.nsrc;
@@ -1383,7 +1461,6 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     F.n_src_chunks = h.sch;
     pw[0] = h.pw_sch;
     pw[1] = h.pw_tch;
-    F.n_trans = (int)h.ntrans;
     F.h_trans_m.clear();
     for (int k = 0; k < 4096; ++k)
         if (h.bits[k >> 5] >> (k & 31) & 1u)
@@ -1394,15 +1471,7 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     p->info.src_points[l] = (int64_t)h.src_points;
     p->info.tgt_points[l] = (int64_t)h.tgt_points;
     if (F.mode == 1) {
-        F.r1 = p->r1_override > 0 ? p->r1_override : r1_rule(p->kind, p->eps);
-        if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
-        // pairs grouped by translation for the per-translation transfer kernels, unless the
-        // level is to run the target-stationary transfer, which reads the per-target lists
-        // (forced, the pick stored in the plan's autotune cache, or the rule); ACA levels need them
-        const int pick = p->lag_transfer == 0 ? cached_lag_pick(p, l) : -1;
-        const bool ts_can = p->kind == FFM_LAPLACE && F.r1 <= 4 && !(p->aca_eps > 0.0);
-        if (ts_can && p->lag_transfer == 0 && pick < 0 && target_stationary_pays(F)) F.tune_tc = 2;
-        const bool ts_first = ts_can && (F.tune_tc == 2 || pick == 2);
+        // pairs grouped by translation for the transfers by translation (ACA levels need them)
         if (!ts_first) build_translation_groups(p, l, s);
         if (p->lag_transfer == 1 || pick == 0 || p->aca_eps > 0.0) build_group_tiles(p, l, s);
         p->info.r1[l] = F.r1;
@@ -1524,9 +1593,8 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
     // deepest level the occupancy rule can reach
     int ldeep = 0;
     while (ldeep < p->l_cap && !(n < (int64_t)p->n_leaf * (nbx[ldeep] + nby[ldeep]))) ++ldeep;
-    uint32_t *parent[LMAX + 1] = {};
-    build_boxes(p, p->bx, sp.s[0], nbx, ldeep, parent, tmp, s);
-    build_boxes(p, p->by, sp.s[1], nby, ldeep, nullptr, tmp, s);
+    build_boxes(p, p->bx, sp.s[0], nbx, ldeep, p->parent, s);
+    build_boxes(p, p->by, sp.s[1], nby, ldeep, nullptr, s);
     for (int l = 0; l <= ldeep; ++l) {
         p->info.nboxX[l] = nbx[l];
         p->info.nboxY[l] = nby[l];
@@ -1539,8 +1607,8 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
     Alloc levels[LMAX + 2];  // per-level temporaries of the descent, released level by level
     TableJob tj(s);
     NearLists near;  // at the root: box 0 with box 0
-    near.off = p->mem.get<uint32_t>(2);
-    near.src = p->mem.get<uint32_t>(1);
+    p->nr_off[0] = near.off = p->mem.get<uint32_t>(2);
+    p->nr_src[0] = near.src = p->mem.get<uint32_t>(1);
     static const uint32_t root_off[2] = {0, 1};
     FFM_CUDA(cudaMemcpyAsync(near.off, root_off, sizeof root_off, cudaMemcpyHostToDevice, s));
     FFM_CUDA(cudaMemsetAsync(near.src, 0, sizeof(uint32_t), s));
@@ -1560,13 +1628,12 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
         int l = 0;
         for (; !stops(l, nnear); ++l) {
             const int lc = l + 1;
-            D3 sg{{std::ldexp(p->sigma[0], lc), std::ldexp(p->sigma[1], lc), std::ldexp(p->sigma[2], lc)}};
             DescendArgs D{};
-            D.parent = parent[lc];
+            D.parent = p->parent[lc];
             D.near_off = near.off;
             D.near_src = near.src;
             D.fcy = p->by[l].first_child;
-            D.K = adm_thresholds(sg);
+            D.K = adm_thresholds(level_shift(p, lc));
             levels[lc].stream = s;
             nnear = descend_level(p, lc, D, [&](int64_t nn) { return stops(lc, nn); }, near, pwc[lc], levels[lc], s);
             // the previous level's near lists are no longer needed

@@ -107,3 +107,27 @@ def test_wait_give_up_of_a_complex_level():
     with ffm.Plan(X, X, ffm.HELMHOLTZ, 1.0, 1e-3, n_leaf=16) as p:
         p.apply(u)
         assert p.info()["device_errors"] == 0
+
+
+@pytest.mark.parametrize("shift", [0.0, 0.3, 1.7])
+def test_pair_lists_of_a_target_stationary_level_come_back_on_request(shift):
+    """Such a level keeps no pair lists: the export makes them from the near lists, the autotuner (which
+    times the transfers by translation) makes and keeps them; both equal the other plan's."""
+    X = torch.as_tensor(W.gaussian_mixture(20000, 1), device="cuda")
+    Y = torch.as_tensor(W.gaussian_mixture(15000, 2) + shift, device="cuda")
+    u = torch.ones(15000, device="cuda")
+    with ffm.Plan(X, Y, ffm.LAPLACE, 0.0, 1e-3, lagrange_transfer=ffm.LAG_TC_TARGET) as p, \
+            ffm.Plan(X, Y, ffm.LAPLACE, 0.0, 1e-3, lagrange_transfer=ffm.LAG_TC_TRANSLATION) as q:
+        info = q.info()
+        levels = [l for l in range(info["l_stop"] + 1) if info["n_adm"][l]]
+        assert levels and p.info()["n_adm"] == info["n_adm"]
+        assert any(p.info()["tune_tc"][l] == 2 for l in levels)
+        for l in levels:
+            np.testing.assert_array_equal(p.pairs(l, "adm"), q.pairs(l, "adm"))
+        a, b = p.apply(u).double(), q.apply(u).double()
+        assert float((a - b).norm() / b.norm()) < TOL
+        p.autotune()
+        for l in levels:
+            np.testing.assert_array_equal(p.pairs(l, "adm"), q.pairs(l, "adm"))
+        assert float((p.apply(u).double() - b).norm() / b.norm()) < TOL
+        assert p.info()["device_errors"] == 0
