@@ -54,6 +54,33 @@ using ::fma;
 __device__ __forceinline__ dd fma(dd a, dd b, dd c) { return a * b + c; }
 __device__ __forceinline__ dd fma(dd a, float b, dd c) { return a * b + c; }
 
+// c + a b into an accumulator that is normalised only now and then: the leading product split exactly, its
+// sum into c.hi with the rounding error (TwoSum), everything else collected in c.lo.  12 FP32
+// operations (11 for an FP32 b) where a product and an addition with their normalisations take
+// 18 (17).  Eight terms between normalisations (acc_norm) let |c.lo| grow to about eight ulps of
+// c.hi, whose own rounding is then 2^-45 of c.hi: the accuracy of the normalised form.
+constexpr int DD_TERMS = 8;
+__device__ __forceinline__ dd dd_acc(dd c, float p, float e) {
+    float s = __fadd_rn(c.hi, p), bb = __fsub_rn(s, c.hi);
+    float err = __fadd_rn(__fsub_rn(c.hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    return dd(s, __fadd_rn(c.lo, __fadd_rn(err, e)));
+}
+__device__ __forceinline__ dd acc_fma(dd a, dd b, dd c) {
+    float p = __fmul_rn(a.hi, b.hi), e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, e);
+    return dd_acc(c, p, fmaf(a.lo, b.hi, e));
+}
+__device__ __forceinline__ dd acc_fma(dd a, float b, dd c) {
+    float p = __fmul_rn(a.hi, b), e = fmaf(a.hi, b, -p);
+    return dd_acc(c, p, fmaf(a.lo, b, e));
+}
+__device__ __forceinline__ void acc_norm(dd &c) { c = dd_two_sum(c.hi, c.lo); }
+// the other arithmetics' accumulators have nothing to normalise
+__device__ __forceinline__ float acc_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double acc_fma(double a, double b, double c) { return ::fma(a, b, c); }
+__device__ __forceinline__ void acc_norm(float &) {}
+__device__ __forceinline__ void acc_norm(double &) {}
+
 struct dd2 {
     dd x, y;
 };

@@ -1512,10 +1512,16 @@ __global__ void __launch_bounds__(128) k_pw_forward(PwArgs<R> P, const uint32_t 
                     R ph = fma(kx[t], e.x, fma(ky[t], e.y, kz[t] * e.z));
                     R sn, cs;
                     phase_sincos<PH>(ph, sn, cs, P.sctab);
-                    Pc[t].x = fma(cs, (R)w.x, Pc[t].x);
-                    Pc[t].y = fma(cs, (R)w.y, Pc[t].y);
-                    Qs[t].x = fma(sn, (R)w.x, Qs[t].x);
-                    Qs[t].y = fma(sn, (R)w.y, Qs[t].y);
+                    Pc[t].x = acc_fma(cs, w.x, Pc[t].x);
+                    Pc[t].y = acc_fma(cs, w.y, Pc[t].y);
+                    Qs[t].x = acc_fma(sn, w.x, Qs[t].x);
+                    Qs[t].y = acc_fma(sn, w.y, Qs[t].y);
+                    if (j % DD_TERMS == DD_TERMS - 1 || j == cnt - 1) {
+                        acc_norm(Pc[t].x);
+                        acc_norm(Pc[t].y);
+                        acc_norm(Qs[t].x);
+                        acc_norm(Qs[t].y);
+                    }
                 }
             }
         }
@@ -1574,8 +1580,12 @@ __global__ void k_pw_transfer(const uint32_t *__restrict__ tgt, const uint32_t *
                         two_sum_acc(a[m].x, al[m].x, fma(d.x, u.x, -d.y * u.y));
                         two_sum_acc(a[m].y, al[m].y, fma(d.x, u.y, d.y * u.x));
                     } else {
-                        a[m].x = fma(d.x, u.x, fma(-d.y, u.y, a[m].x));
-                        a[m].y = fma(d.x, u.y, fma(d.y, u.x, a[m].y));
+                        a[m].x = acc_fma(d.x, u.x, acc_fma(-d.y, u.y, a[m].x));
+                        a[m].y = acc_fma(d.x, u.y, acc_fma(d.y, u.x, a[m].y));
+                        if (((e - off[x]) * 2) % DD_TERMS == DD_TERMS - 2 || e + 1 == off[x + 1]) {
+                            acc_norm(a[m].x);
+                            acc_norm(a[m].y);
+                        }
                     }
                 }
         }
@@ -1683,8 +1693,12 @@ __global__ void __launch_bounds__(128) k_pw_backward(PwArgs<R> P, const uint32_t
                             two_sum_acc(sr[u], lr[u], fma(cs, A.x, sn * B.x));
                             two_sum_acc(si[u], li[u], fma(cs, A.y, sn * B.y));
                         } else {
-                            sr[u] = fma(cs, A.x, fma(sn, B.x, sr[u]));
-                            si[u] = fma(cs, A.y, fma(sn, B.y, si[u]));
+                            sr[u] = acc_fma(cs, A.x, acc_fma(sn, B.x, sr[u]));
+                            si[u] = acc_fma(cs, A.y, acc_fma(sn, B.y, si[u]));
+                            if (((j - j0) * 2) % DD_TERMS == DD_TERMS - 2 || j == j1 - 1) {
+                                acc_norm(sr[u]);
+                                acc_norm(si[u]);
+                            }
                         }
                     }
                 }
@@ -1779,15 +1793,23 @@ __global__ void __launch_bounds__(128) k_pw_forward_mr(PwArgs<R> P, const uint32
                 for (int m2 = 0; m2 < MC / 2; ++m2) {
                     float4 w2 = sq4[m2];
                     int m = 2 * m2;
-                    Pc[m].x = fma(er, (R)w2.x, Pc[m].x);
-                    Pc[m].y = fma(er, (R)w2.y, Pc[m].y);
-                    Qs[m].x = fma(ei, (R)w2.x, Qs[m].x);
-                    Qs[m].y = fma(ei, (R)w2.y, Qs[m].y);
-                    Pc[m + 1].x = fma(er, (R)w2.z, Pc[m + 1].x);
-                    Pc[m + 1].y = fma(er, (R)w2.w, Pc[m + 1].y);
-                    Qs[m + 1].x = fma(ei, (R)w2.z, Qs[m + 1].x);
-                    Qs[m + 1].y = fma(ei, (R)w2.w, Qs[m + 1].y);
+                    Pc[m].x = acc_fma(er, w2.x, Pc[m].x);
+                    Pc[m].y = acc_fma(er, w2.y, Pc[m].y);
+                    Qs[m].x = acc_fma(ei, w2.x, Qs[m].x);
+                    Qs[m].y = acc_fma(ei, w2.y, Qs[m].y);
+                    Pc[m + 1].x = acc_fma(er, w2.z, Pc[m + 1].x);
+                    Pc[m + 1].y = acc_fma(er, w2.w, Pc[m + 1].y);
+                    Qs[m + 1].x = acc_fma(ei, w2.z, Qs[m + 1].x);
+                    Qs[m + 1].y = acc_fma(ei, w2.w, Qs[m + 1].y);
                 }
+                if (j % DD_TERMS == DD_TERMS - 1 || j == cnt - 1)
+#pragma unroll
+                    for (int m = 0; m < MC; ++m) {
+                        acc_norm(Pc[m].x);
+                        acc_norm(Pc[m].y);
+                        acc_norm(Qs[m].x);
+                        acc_norm(Qs[m].y);
+                    }
             }
         }
     }
@@ -1879,9 +1901,17 @@ __global__ void __launch_bounds__(128) k_pw_backward_mr(PwArgs<R> P, const uint3
                             two_sum_acc(o[m].x, ol[m].x, fma(cs, A.x, sn * B.x));
                             two_sum_acc(o[m].y, ol[m].y, fma(cs, A.y, sn * B.y));
                         } else {
-                            o[m].x = fma(cs, A.x, fma(sn, B.x, o[m].x));
-                            o[m].y = fma(cs, A.y, fma(sn, B.y, o[m].y));
+                            o[m].x = acc_fma(cs, A.x, acc_fma(sn, B.x, o[m].x));
+                            o[m].y = acc_fma(cs, A.y, acc_fma(sn, B.y, o[m].y));
                         }
+                    }
+                    if constexpr (!COMP) {
+                        if ((j * 2) % DD_TERMS == DD_TERMS - 2 || j == qc - 1)
+#pragma unroll
+                            for (int m = 0; m < MC; ++m) {
+                                acc_norm(o[m].x);
+                                acc_norm(o[m].y);
+                            }
                     }
                 }
             }
