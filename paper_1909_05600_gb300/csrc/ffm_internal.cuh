@@ -96,6 +96,15 @@ __host__ __device__ inline uint32_t kmajor_index(int row, int k, int KT) {
     return (uint32_t)((((row >> 3) * (KT >> 2) + (k >> 2)) << 5) + ((row & 7) << 2) + (k & 3));
 }
 
+struct LagGeo {
+    double oxy[3];  // oX - oY
+    double dl;
+    float k;
+    int r1;
+    int kind;
+    float hnode[R1MAX];  // (d_l / 2) cos((2a+1) pi / (2 r1))
+};
+
 struct alignas(32) D4 {
     double x, y, z, w;
 };
@@ -155,7 +164,8 @@ struct FarLevel {
     int4 *trans_m = nullptr;        // n_trans integer offsets gX - gY
     std::vector<int4> h_trans_m;
     // Lagrange
-    float *T = nullptr;             // n_trans * r * r (real) or float2 (complex), [t][i][j]
+    float *T = nullptr;             // n_trans * r * r (real) or float2 (complex), [t][i][j]; only for
+                                    // the CUDA-core transfer
     uint32_t *bt_off = nullptr;     // n_trans+1: pairs grouped by translation (CSR)
     uint32_t *bt_src = nullptr;     // n_adm source box per pair, grouped by translation
     uint32_t *bt_tgt = nullptr;     // n_adm target box per pair, grouped by translation
@@ -287,7 +297,10 @@ void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s);
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s);
 void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s);
 // transfer.cu: operator images of a Lagrange level; v~ += T u~ over its pairs by translation
-void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, cudaStream_t s);
+void build_operator_image(ffm_plan_s *p, int l, const LagGeo &geo, cudaStream_t s);
+// tables.cu: geometry of Lagrange level l's operators; their FP32 form for the CUDA-core transfer
+LagGeo lag_geo(const ffm_plan_s *p, int l);
+void build_lag_table(ffm_plan_s *p, int l, cudaStream_t s);
 void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
 // the same over each target's partners (target-stationary; ts_ok levels)
 void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);

@@ -34,15 +34,6 @@ int r1_rule(int kind, double eps) {
     return 10;
 }
 
-struct LagGeo {
-    double oxy[3];  // oX - oY
-    double dl;
-    float k;
-    int r1;
-    int kind;
-    float hnode[R1MAX];  // (d_l / 2) cos((2a+1) pi / (2 r1))
-};
-
 // T stored as [t][i][j] (source node j innermost): rows of T are K-major operands of the
 // transfer GEMMs.
 // The translation r0 is formed in FP64 and rounded once; node differences, the distance
@@ -580,6 +571,28 @@ static void build_aca(ffm_plan_s *p, int l, const double oxy[3], double dl, Tabl
     FFM_LAUNCH(k_aca_pair_id, cdiv(F.n_adm, 256), 256, 0, s, F.pair_id, F.n_adm);
 }
 
+LagGeo lag_geo(const ffm_plan_s *p, int l) {
+    const FarLevel &F = p->far[l];
+    LagGeo g{};
+    for (int d = 0; d < 3; ++d) g.oxy[d] = p->oX[d] - p->oY[d];
+    g.dl = std::ldexp(p->d0, -l);
+    g.k = (float)p->k;
+    g.r1 = F.r1;
+    g.kind = p->kind;
+    for (int a = 0; a < F.r1; ++a) g.hnode[a] = (float)(0.5 * g.dl * std::cos((2.0 * a + 1.0) * PI / (2.0 * F.r1)));
+    return g;
+}
+
+// FP32 operators of a Lagrange level, for the CUDA-core transfer (no-op if present).
+void build_lag_table(ffm_plan_s *p, int l, cudaStream_t s) {
+    FarLevel &F = p->far[l];
+    if (F.T) return;
+    const size_t r = (size_t)F.r1 * F.r1 * F.r1;
+    const int per = p->kind == FFM_HELMHOLTZ ? 2 : p->kind == FFM_LAPLACE ? 1 : 3;
+    F.T = p->mem.get<float>(F.n_trans * r * r * per);
+    FFM_LAUNCH(k_lag_table, F.n_trans, 256, 0, s, F.trans_m, F.n_trans, lag_geo(p, l), F.T);
+}
+
 void build_tables(ffm_plan_s *p, int l, TableJob &tj) {
     FarLevel &F = p->far[l];
     cudaStream_t s = tj.side;
@@ -588,23 +601,12 @@ void build_tables(ffm_plan_s *p, int l, TableJob &tj) {
     double dl = std::ldexp(p->d0, -l);
     double oxy[3] = {p->oX[0] - p->oY[0], p->oX[1] - p->oY[1], p->oX[2] - p->oY[2]};
     if (F.mode == 1) {
-        int r = F.r1 * F.r1 * F.r1;
-        bool cplx = p->kind == FFM_HELMHOLTZ;
-        bool three = p->kind == FFM_LAPLACE_DL || p->kind == FFM_LAPLACE_GRAD;
-        F.T = p->mem.get<float>((size_t)F.n_trans * r * r * (cplx ? 2 : three ? 3 : 1));
-            LagGeo g{};
-        for (int d = 0; d < 3; ++d) g.oxy[d] = oxy[d];
-        g.dl = dl;
-        g.k = (float)p->k;
-        g.r1 = F.r1;
-        g.kind = p->kind;
-        for (int a = 0; a < F.r1; ++a) g.hnode[a] = (float)(0.5 * dl * std::cos((2.0 * a + 1.0) * PI / (2.0 * F.r1)));
-        FFM_LAUNCH(k_lag_table, F.n_trans, 256, 0, s, F.trans_m, F.n_trans, g, F.T);
+        const int r = F.r1 * F.r1 * F.r1;
         if (p->aca_eps > 0.0 && p->kind == FFM_LAPLACE) {
             F.rkp = (r + 15) / 16 * 16;
             build_aca(p, l, oxy, dl, tj);
         } else {
-            build_operator_image(p, l, oxy, dl, s);
+            build_operator_image(p, l, lag_geo(p, l), s);
         }
         return;
     }

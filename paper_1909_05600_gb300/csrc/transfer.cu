@@ -114,38 +114,81 @@ __global__ void __launch_bounds__(256) k_rows_split(const float *__restrict__ u,
     }
 }
 
-// Operators as the images the transfer copies: per translation t and row block blk, nk chunks of
+// Operators as the images the transfers copy: per translation t and row block blk, nk chunks of
 // the hi parts of npad rows x 32 values in K-major core matrices, then the lo parts.  Block blk
 // holds rows (blk % bpc) nb .. of component blk / bpc.  A complex operator is the real matrix
 // of its action on interleaved (re, im) rows: rows 2i, 2i + 1 = (Re, -Im), (Im, Re) of T(i, j) at
-// columns 2j, 2j + 1.
-template <bool CPLX>
-__global__ void __launch_bounds__(256) k_op_image(const float *__restrict__ T, int n_trans, int r, int rk, int nb,
+// columns 2j, 2j + 1.  The values are k_lag_table's (the same FP32 expressions), formed here so that no
+// FP32 operator is written and read back; with the node count a template parameter the index
+// arithmetic is free of divisions (volume 250k at 1e-4: table and image 0.54 + 0.34 -> 0.36 ms).
+template <int KIND, int R1>
+__global__ void __launch_bounds__(256) k_op_image(const int4 *__restrict__ m, const __grid_constant__ LagGeo geo, int nb,
                                                   int bpc, int npad, int nk, float scale, __half *__restrict__ img) {
+    constexpr int r = R1 * R1 * R1;
+    constexpr bool CPLX = KIND == FFM_HELMHOLTZ;
+    constexpr int rows = CPLX ? 2 * r : r, cols = CPLX ? 2 * r : KIND == FFM_LAPLACE_DL ? 3 * r : r;
+    __shared__ float node[R1];
+    if (threadIdx.x < R1) node[threadIdx.x] = geo.hnode[threadIdx.x];
+    __syncthreads();
     const int t = blockIdx.x, blk = blockIdx.y, nblk = gridDim.y;
     const int comp = blk / bpc, row0 = (blk % bpc) * nb;
-    const int rows = CPLX ? 2 * r : r, cols = CPLX ? 2 * rk : rk;
-    const float *Tt = T + ((size_t)comp * n_trans + t) * r * rk * (CPLX ? 2 : 1);
+    const int4 mt = m[t];
+    const float r0x = (float)(geo.oxy[0] + mt.x * geo.dl), r0y = (float)(geo.oxy[1] + mt.y * geo.dl),
+                r0z = (float)(geo.oxy[2] + mt.z * geo.dl);
+    const float c4pi = 0.07957747154594767f;  // 1 / (4 pi)
+    auto diff = [&](int i, int j, float (&d)[3]) {
+        d[0] = r0x + (node[i / (R1 * R1)] - node[j / (R1 * R1)]);
+        d[1] = r0y + (node[i / R1 % R1] - node[j / R1 % R1]);
+        d[2] = r0z + (node[i % R1] - node[j % R1]);
+    };
+    auto value = [&](int i, int j, int c) {  // component c of the derivative kernels
+        float d[3];
+        diff(i, j, d);
+        const float r2 = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2])), rr = sqrtf(r2);
+        if constexpr (KIND == FFM_LAPLACE) return c4pi / rr;
+        const float dc = c == 0 ? d[0] : c == 1 ? d[1] : d[2];
+        return (KIND == FFM_LAPLACE_GRAD ? -c4pi : c4pi) * dc / (r2 * rr);
+    };
     __half *out = img + ((size_t)t * nblk + blk) * nk * npad * HROW;
     const int per = npad * HK;  // values per chunk
-    for (int e = threadIdx.x; e < nk * per; e += blockDim.x) {
-        const int kc = e / per, o = e - kc * per;
+    for (int e = threadIdx.x; e < nk * per / 2; e += blockDim.x) {  // two columns each
+        const int kc = 2 * e / per, o = 2 * e - kc * per;
         const int k = kc * HK + ((o >> 6) & 3) * 8 + (o & 7), i = ((o >> 8) << 3) + ((o >> 3) & 7), ri = row0 + i;
-        float v = 0.f;
-        if (i < nb && ri < rows && k < cols) {
+        float v0 = 0.f, v1 = 0.f;
+        if (i < nb && ri < rows) {
             if constexpr (CPLX) {
-                const float *z = Tt + 2 * ((size_t)(ri >> 1) * rk + (k >> 1));
-                const int ci = ri & 1, cj = k & 1;
-                v = ci == cj ? z[0] : (cj ? -z[1] : z[1]);
+                if (k < cols) {
+                    float d[3], sn, cs;
+                    diff(ri >> 1, k >> 1, d);
+                    const float rr = sqrtf(fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]))), a = c4pi / rr;
+                    sincosf(geo.k * rr, &sn, &cs);
+                    const float re = a * cs, im = a * sn;
+                    v0 = ri & 1 ? im : re;
+                    v1 = ri & 1 ? re : -im;
+                }
             } else {
-                v = Tt[(size_t)ri * rk + k];
+                if (k < cols) v0 = value(ri, k % r, KIND == FFM_LAPLACE_DL ? k / r : comp);
+                if (k + 1 < cols) v1 = value(ri, (k + 1) % r, KIND == FFM_LAPLACE_DL ? (k + 1) / r : comp);
             }
         }
-        __half h, l;
-        half_split(v * scale, h, l);
+        __half h0, l0, h1, l1;
+        half_split(v0 * scale, h0, l0);
+        half_split(v1 * scale, h1, l1);
         __half *c = out + (size_t)kc * npad * HROW;
-        c[o] = h;
-        c[per + o] = l;
+        *reinterpret_cast<__half2 *>(c + o) = __halves2half2(h0, h1);
+        *reinterpret_cast<__half2 *>(c + per + o) = __halves2half2(l0, l1);
+    }
+}
+
+template <int R1>
+static void launch_op_image(int kind, dim3 g, const int4 *m, const LagGeo &geo, int nb, int bpc, int nk, float sc,
+                            __half *img, cudaStream_t s) {
+    auto run = [&](auto k) { FFM_LAUNCH_NAMED("k_op_image", k, g, 256, 0, s, m, geo, nb, bpc, nb, nk, sc, img); };
+    switch (kind) {
+        case FFM_HELMHOLTZ: run(k_op_image<FFM_HELMHOLTZ, R1>); break;
+        case FFM_LAPLACE_DL: run(k_op_image<FFM_LAPLACE_DL, R1>); break;
+        case FFM_LAPLACE_GRAD: run(k_op_image<FFM_LAPLACE_GRAD, R1>); break;
+        default: run(k_op_image<FFM_LAPLACE, R1>); break;
     }
 }
 
@@ -521,10 +564,11 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * A.tcols));
 }
 
-// Operator images of a Lagrange level (F.T is in place).  The scale is common to the level's
+// Operator images of a Lagrange level.  The scale is common to the level's
 // translations: the kernels decay at most as 1/R^2 and the distances of a level's node pairs
 // differ by at most a factor of about ten, so every translation keeps its bits.
-void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, cudaStream_t s) {
+void build_operator_image(ffm_plan_s *p, int l, const LagGeo &geo, cudaStream_t s) {
+    const double *oxy = geo.oxy, dl = geo.dl;
     FarLevel &F = p->far[l];
     const bool cplx = p->kind == FFM_HELMHOLTZ;
     const int r = F.r1 * F.r1 * F.r1, rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;
@@ -553,10 +597,16 @@ void build_operator_image(ffm_plan_s *p, int l, const double oxy[3], double dl, 
     F.Th = p->mem.get<uint16_t>(n);
     dim3 g(F.n_trans, nblk);
     const float sc = (float)std::ldexp(1.0, e);
-    if (cplx)
-        FFM_LAUNCH(k_op_image<true>, g, 256, 0, s, F.T, F.n_trans, r, rk, F.h_nb, F.h_bpc, F.h_nb, F.h_nk, sc, (__half *)F.Th);
-    else
-        FFM_LAUNCH(k_op_image<false>, g, 256, 0, s, F.T, F.n_trans, r, rk, F.h_nb, F.h_bpc, F.h_nb, F.h_nk, sc, (__half *)F.Th);
+    switch (F.r1) {
+        case 2: launch_op_image<2>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 3: launch_op_image<3>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 4: launch_op_image<4>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 5: launch_op_image<5>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 6: launch_op_image<6>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 7: launch_op_image<7>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        case 8: launch_op_image<8>(p->kind, g, F.trans_m, geo, F.h_nb, F.h_bpc, F.h_nk, sc, (__half *)F.Th, s); break;
+        default: fail(FFM_EUNSUPPORTED, "Chebyshev nodes per axis outside 2..8");
+    }
 }
 
 template <int NSTG, int CPS, bool STACK>

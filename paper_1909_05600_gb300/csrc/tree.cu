@@ -98,8 +98,9 @@ __global__ void k_scan_down(const uint32_t *in, uint32_t *out, int64_t n, const 
 }
 
 // The whole scan in one block, tile after tile with a running carry: one launch instead
-// of three for the many small scans of a plan.
-constexpr int64_t SCAN_SMALL = 16 * SCAN_TILE;
+// of three for the small scans of a plan.  A tile takes about 1.3 us in one block, the three
+// launches about 8 us together, so up to six tiles.
+constexpr int64_t SCAN_SMALL = 6 * SCAN_TILE;
 __global__ void __launch_bounds__(SCAN_T) k_scan_small(const uint32_t *in, uint32_t *out, int64_t n,
                                                        uint32_t *d_total) {
     __shared__ uint32_t tile[SCAN_TILE];
@@ -347,34 +348,53 @@ static double ord_dec(unsigned long long k) {
     return d;
 }
 
-// out[0..2] = encoded min, out[3..5] = encoded max, out[6] = non-finite flag.
+// out[0..2] = encoded min, out[3..5] = encoded max, out[6] = non-finite flag.  Minima and maxima in
+// the points' own type (this part's FP64 rate is a small fraction of its FP32 rate), reduced over the
+// block first: one atomic per block and bound on the seven words (one per warp took 44 us at 250k points).
 template <class T>
-__global__ void k_bbox(const T *__restrict__ P, int64_t n, unsigned long long *out) {
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    unsigned long long bad = 0;
+__global__ void __launch_bounds__(256) k_bbox(const T *__restrict__ P, int64_t n, unsigned long long *out) {
+    T lo[3] = {(T)INFINITY, (T)INFINITY, (T)INFINITY}, hi[3] = {-(T)INFINITY, -(T)INFINITY, -(T)INFINITY};
+    bool bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            double x = (double)P[3 * i + d];
-            if (!isfinite(x)) bad = 1;
-            lo[d] = fmin(lo[d], x);
-            hi[d] = fmax(hi[d], x);
+            const T x = P[3 * i + d];
+            bad |= !isfinite(x);
+            lo[d] = x < lo[d] ? x : lo[d];
+            hi[d] = x > hi[d] ? x : hi[d];
         }
     }
+    __shared__ T s[6][8];
+    __shared__ int sbad;
+    if (threadIdx.x == 0) sbad = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
+    for (int d = 0; d < 3; ++d) {
         for (int off = 16; off; off >>= 1) {
-            lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], off));
-            hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], off));
+            const T a = __shfl_xor_sync(0xffffffffu, lo[d], off), c = __shfl_xor_sync(0xffffffffu, hi[d], off);
+            lo[d] = a < lo[d] ? a : lo[d];
+            hi[d] = c > hi[d] ? c : hi[d];
         }
-    bad = __any_sync(0xffffffffu, bad != 0);
-    if ((threadIdx.x & 31) == 0) {
-        for (int d = 0; d < 3; ++d) {
-            atomicMin(&out[d], ord_enc(lo[d]));
-            atomicMax(&out[3 + d], ord_enc(hi[d]));
+        if (lane == 0) {
+            s[d][warp] = lo[d];
+            s[3 + d][warp] = hi[d];
         }
-        if (bad) atomicOr(&out[6], 1ull);
     }
+    if (bad) sbad = 1;
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        T v = s[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) {
+            const T o = s[threadIdx.x][w];
+            v = threadIdx.x < 3 ? (o < v ? o : v) : (o > v ? o : v);
+        }
+        if (threadIdx.x < 3)
+            atomicMin(&out[threadIdx.x], ord_enc((double)v));
+        else
+            atomicMax(&out[threadIdx.x], ord_enc((double)v));
+    }
+    if (threadIdx.x == 0 && sbad) atomicOr(&out[6], 1ull);
 }
 
 // =================================================================== keys
@@ -399,13 +419,18 @@ __host__ __device__ __forceinline__ uint64_t compact3(uint64_t x) {
 }
 
 // Finest-grid coordinate floor(((x - o)/d0) * 2^21), clamped to [0, 2^21 - 1]; the
-// subtraction and the division are IEEE FP64 operations, the scaling is exact.
-__device__ __forceinline__ uint64_t fine_coord(double x, double o, double d0) {
-    double t = __ddiv_rn(__dsub_rn(x, o), d0);
-    double f = floor(t * 2097152.0);
+// subtraction and the division are IEEE FP64 operations, the scaling is exact.  The quotient is
+// first formed as a product with scale = 2^21 / d0 (rounded), which is off by at most two roundings, 2^-30
+// of a grid cell here; only when it lies within 2^-26 of a cell boundary, where the floor could
+// differ, is the division done (16.4 -> 11.0 ms for 2e8 points: an FP64 division is about twenty FP64 operations).
+__device__ __forceinline__ uint64_t fine_coord(double x, double o, double d0, double scale) {
+    const double y = __dsub_rn(x, o);
+    double t = __dmul_rn(y, scale), f = floor(t);
+    const double r = t - f;
+    if (!(r > 1.4901161193847656e-08 && r < 1.0 - 1.4901161193847656e-08)) f = floor(__ddiv_rn(y, d0) * 2097152.0);
     f = fmax(f, 0.0);
     f = fmin(f, 2097151.0);
-    return (uint64_t)f;
+    return (uint64_t)(uint32_t)f;
 }
 
 struct D3 {
@@ -413,13 +438,13 @@ struct D3 {
 };
 
 template <class T>
-__global__ void k_keys(const T *__restrict__ P, int64_t n, D3 o, double d0, uint64_t setbit, uint32_t idx0,
+__global__ void k_keys(const T *__restrict__ P, int64_t n, D3 o, double d0, double scale, uint64_t setbit, uint32_t idx0,
                        uint64_t *__restrict__ keys, uint32_t *__restrict__ idx) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    uint64_t g0 = fine_coord((double)P[3 * i], o.v[0], d0);
-    uint64_t g1 = fine_coord((double)P[3 * i + 1], o.v[1], d0);
-    uint64_t g2 = fine_coord((double)P[3 * i + 2], o.v[2], d0);
+    uint64_t g0 = fine_coord((double)P[3 * i], o.v[0], d0, scale);
+    uint64_t g1 = fine_coord((double)P[3 * i + 1], o.v[1], d0, scale);
+    uint64_t g2 = fine_coord((double)P[3 * i + 2], o.v[2], d0, scale);
     keys[i] = setbit | (spread3(g0) << 2) | (spread3(g1) << 1) | spread3(g2);
     idx[i] = idx0 + (uint32_t)i;
 }
@@ -1117,12 +1142,13 @@ template <class T>
 static void launch_keys(const void *P, int64_t n, const double o[3], double d0, uint64_t setbit, uint32_t idx0,
                         uint64_t *keys, uint32_t *idx, cudaStream_t s) {
     D3 oo{{o[0], o[1], o[2]}};
-    FFM_LAUNCH(k_keys<T>, cdiv(n, 256), 256, 0, s, (const T *)P, n, oo, d0, setbit, idx0, keys, idx);
+    FFM_LAUNCH(k_keys<T>, cdiv(n, 256), 256, 0, s, (const T *)P, n, oo, d0, 2097152.0 / d0, setbit, idx0, keys,
+               idx);
 }
 
 template <class T>
 static void launch_bbox(const void *P, int64_t n, unsigned long long *out, cudaStream_t s) {
-    FFM_LAUNCH(k_bbox<T>, std::min<unsigned>(cdiv(n, 256), 2048u), 256, 0, s, (const T *)P, n, out);
+    FFM_LAUNCH(k_bbox<T>, std::min<unsigned>(cdiv(n, 1024), 152u * 8u), 256, 0, s, (const T *)P, n, out);
 }
 
 template <class T>
@@ -1324,6 +1350,7 @@ void build_group_tiles(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
     if (F.mode != 1 || F.n_adm == 0 || F.tile_t) return;
     build_translation_groups(p, l, s);
+    if (!(p->aca_eps > 0.0)) build_lag_table(p, l, s);
     Alloc tmp;
     tmp.stream = s;
     F.n_tiles = build_tiles(p, F, LAG_GEMM_BN, &F.tile_t, &F.tile_p0, tmp, s);
