@@ -303,7 +303,9 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
     return r;
 }
 
-constexpr int LAP_SB = 512;         // staged sources per batch (a multiple of 4)
+// staged sources per batch (a multiple of 4): 1024 against 512 is 190.2 -> 188.7 ms at 1e8 clustered
+// points, 65.7 -> 65.5 at 10M (fewer batch boundaries; 35 KB of shared memory do not cost a block)
+constexpr int LAP_SB = 1024;
 constexpr float LAP_FAR = 1.0e15f;  // coordinate of the padding sources (weight 0)
 
 // a target: hi and lo parts of each coordinate, duplicated in both halves
@@ -503,16 +505,27 @@ __global__ void __launch_bounds__(P2P_T) k_p2p_lap(NearArgs N, const float *__re
         red[threadIdx.x * PT + t] = u0 + u1;
     }
     __syncthreads();
-    if (active && grp == 0) {
-        const double c = 0.079577471545947667884;  // 1 / (4 pi)
-#pragma unroll
-        for (int t = 0; t < PT; ++t) {
-            int i = pi + t * pr;
-            if (i >= np) continue;
-            float tr = 0.f;
-            for (int g = 0; g < G; ++g) tr += red[(g * pr + pi) * PT + t];
-            atomicAdd(&acc[p0 + i].x, (double)tr * c);
-        }
+    // target i's sums: group g's at red[(g pr + i % pr) PT + i / pr].  All threads add, each a slice of the
+    // groups: leaves of fifteen points have 32 groups, which four threads summed alone before (1e8
+    // clustered 195.6 -> 190.2 ms, 10M 66.4 -> 65.7)
+    const int nt = pr * PT, ns = P2P_T / nt > 0 ? P2P_T / nt : 1;
+    __shared__ float part[P2P_T];
+    if (ns > 1) {
+        const int i = threadIdx.x % nt, sl = threadIdx.x / nt;
+        float tr = 0.f;
+        if (sl < ns)
+            for (int g = sl; g < G; g += ns) tr += red[(g * pr + i % pr) * PT + i / pr];
+        part[threadIdx.x] = tr;
+        __syncthreads();
+    }
+    const double c = 0.079577471545947667884;  // 1 / (4 pi)
+    for (int i = threadIdx.x; i < np; i += P2P_T) {
+        float tr = 0.f;
+        if (ns > 1)
+            for (int sl = 0; sl < ns; ++sl) tr += part[sl * nt + i];
+        else
+            for (int g = 0; g < G; ++g) tr += red[(g * pr + i % pr) * PT + i / pr];
+        atomicAdd(&acc[p0 + i].x, (double)tr * c);
     }
 }
 

@@ -233,12 +233,11 @@ struct PairArgs {
 //
 // Measured on GB300 (level 7 of clustered 10M, 68M pairs of r = 64): 11.7 ms with the row numbers fetched
 // by the copying and adding threads themselves, 9.85 with index warps, 6.98 with rows in the swizzled
-// layout, 6.14 with the lean MMA loop.  Transfers of one apply, against the kernel before it (a block per 256-pair
-// tile, which split its FP32 rows into TF32 for every pair, no overlap of tiles): gradient sphere 300k
-// (r = 216, three operators) 6.54 -> 3.12 ms, double layer 200k (K = 648) 2.16 -> 0.97, Laplace volume
-// 250k at 1e-4 (r = 216) 1.47 -> 0.79, 100k x 8 right-hand sides (r = 64) 1.68 -> 0.72, clustered
-// 10M (r = 64) 21.8 -> 14.0.  Complex operators (Helmholtz volume 120k at 1e-4, 432 real rows), on
-// CUDA cores before: 24.4 -> 2.4 ms.
+// layout, 6.14 with the lean MMA loop.  Transfers of one apply, against the kernel before it (a block per
+// 256-pair tile, which split its FP32 rows into TF32 for every pair, no overlap of tiles): gradient
+// sphere 300k (r = 216, three operators) 6.54 -> 1.78 ms, Laplace volume 250k at 1e-4 (r = 216) 1.47 ->
+// 0.45, 100k x 8 right-hand sides (r = 64) 1.68 -> 0.41.  Complex operators (Helmholtz volume 120k at
+// 1e-4, 432 real rows), on CUDA cores before: 24.4 -> 1.9 ms.
 constexpr int PAIR_T = 416;
 constexpr int PAIR_IXW = 4;  // index warps
 constexpr int PAIR_IX = 4;   // units whose row numbers are held
