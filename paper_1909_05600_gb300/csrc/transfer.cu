@@ -85,17 +85,18 @@ __device__ __forceinline__ void half_split(float x, __half &hi, __half &lo) {
 
 // Rows of n floats as f16 hi / lo images, one warp per row: chunk kc of row i holds the hi
 // parts of values 32 kc .. + 31, then their lo parts (zero past n).  The scale is the row's own
-// (its inverse in inv[i]), or with `common` the one of that largest value, for all rows.
+// (its inverse in inv[i]), or with `common` that of the largest value of the row's column (right-hand side
+// i % nrhs): never one of several columns, whose magnitudes have nothing to do with each other.
 __global__ void __launch_bounds__(256) k_rows_split(const float *__restrict__ u, int64_t nrow, int n, int nk,
                                                     __half *__restrict__ img, float *__restrict__ inv,
-                                                    const uint32_t *__restrict__ common) {
+                                                    const uint32_t *__restrict__ common, int nrhs) {
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= nrow) return;
     const float *row = u + i * n;
     float mx = 0.f;
     if (common) {
-        mx = __uint_as_float(*common);
+        mx = __uint_as_float(common[nrhs == 1 ? 0 : i % nrhs]);
     } else {
         for (int k = lane; k < n; k += 32) mx = fmaxf(mx, fabsf(row[k]));
         for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -627,7 +628,7 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     PairArgs A{};
     __half *img = tmp.get<__half>((size_t)nrow * F.h_nk * HROW);
     float *inv = tmp.get<float>(nrow);
-    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, K, F.h_nk, img, inv, (const uint32_t *)nullptr);
+    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, K, F.h_nk, img, inv, (const uint32_t *)nullptr, nrhs);
     A.bt_off = F.bt_off;
     A.bt_src = F.bt_src;
     A.bt_tgt = F.bt_tgt;
@@ -684,9 +685,10 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
 // 16-byte cp.async segments, rows without a partner zero-filled without a read), thread 0 starts
 // the bulk copy of T_t's image, warp 8 issues hi [hi; lo] (N = 2 npad) and lo hi, 4 steps in flight (8
 // where K <= 32).  Nothing is converted on the way.
-// Rows of different sources meet in one accumulator, so the level shares one scale (k_level_max):
-// a value keeps its 22 bits down to 2^-15 of the level's largest, and below that an absolute
-// error of 2^-39 of it.
+// Rows of different sources meet in one accumulator, so all rows of a right-hand side share one scale
+// (k_level_max; a block works on one right-hand side, and the others have scales of their own): a
+// value keeps its 22 bits down to 2^-15 of its column's largest, and below that an absolute error of 2^-38
+// of it, which is lost beside that source's own potential at every target.
 //
 // One long tensor-core accumulation loses accuracy, so the block alternates between two TMEM
 // accumulators every TG_DRAIN translations; warps 4-7 add each finished one into FP32 registers
@@ -755,13 +757,22 @@ void prepare_target_stationary(ffm_plan_s *p, int l, cudaStream_t s) {
     F.ts_ok = true;
 }
 
-// largest |u| of the level's rows, as float bits (0 for an all-zero level)
-__global__ void k_level_max(const float *__restrict__ u, int64_t n, uint32_t *__restrict__ out) {
+// largest |u| of right-hand side blockIdx.y over the level's nb rows of r values, as float bits (0 for an all-zero
+// column)
+__global__ void k_level_max(const float *__restrict__ u, int64_t nb, int r, int nrhs, uint32_t *__restrict__ out) {
+    const int m = blockIdx.y;
+    const int64_t n = nb * r;
     float mx = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        mx = fmaxf(mx, fabsf(u[i]));
+    if (nrhs == 1) {
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+            mx = fmaxf(mx, fabsf(u[i]));
+    } else {  // one row per warp and turn
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int64_t b = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5); b < nb; b += (int64_t)gridDim.x * nw)
+            for (int k = lane; k < r; k += 32) mx = fmaxf(mx, fabsf(u[(b * nrhs + m) * r + k]));
+    }
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && mx > 0.f) atomicMax(out, __float_as_uint(mx));
+    if ((threadIdx.x & 31) == 0 && mx > 0.f) atomicMax(out + m, __float_as_uint(mx));
 }
 
 struct TargetArgs {
@@ -771,8 +782,8 @@ struct TargetArgs {
     int3 base;
     int64_t n_tgt;
     int n_trans, nrhs, nk, npad, r, tcols;
-    const __half *u;        // row images of (source box, right-hand side), one scale for all
-    const uint32_t *umax;   // that scale's value (k_level_max)
+    const __half *u;        // row images of (source box, right-hand side), one scale per right-hand side
+    const uint32_t *umax;   // the scales' values (k_level_max)
     const __half *T;
     float tinv;
     float *vt;
@@ -991,7 +1002,7 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
         const int64_t x = x0 + 32 * q + lane;
         if (ok && x < A.n_tgt) {
             float us, ui;
-            row_scale(__uint_as_float(*A.umax), us, ui);
+            row_scale(__uint_as_float(A.umax[m]), us, ui);
             float *dst = A.vt + ((size_t)A.tgt[x] * A.nrhs + m) * A.r;
 #pragma unroll
             for (int c = 0; c < 64; ++c) sum[c] = sum[c] * ui * A.tinv;
@@ -1029,10 +1040,12 @@ void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt
     const int64_t nrow = (int64_t)p->by[l].nb * nrhs;
     TargetArgs A{};
     __half *img = tmp.get<__half>((size_t)nrow * F.h_nk * HROW);
-    uint32_t *mx = tmp.get<uint32_t>(1);
-    FFM_CUDA(cudaMemsetAsync(mx, 0, sizeof(uint32_t), s));
-    FFM_LAUNCH(k_level_max, (unsigned)std::min<int64_t>(cdiv(nrow * r, 1024), 152 * 8), 256, 0, s, u, nrow * r, mx);
-    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, r, F.h_nk, img, (float *)nullptr, (const uint32_t *)mx);
+    uint32_t *mx = tmp.get<uint32_t>(nrhs);
+    FFM_CUDA(cudaMemsetAsync(mx, 0, sizeof(uint32_t) * nrhs, s));
+    const int64_t nb = p->by[l].nb;
+    const dim3 gm((unsigned)std::min<int64_t>(cdiv(nb * r, 1024), std::max(1, 152 * 8 / nrhs)), nrhs);
+    FFM_LAUNCH(k_level_max, gm, 256, 0, s, u, nb, r, nrhs, mx);
+    FFM_LAUNCH(k_rows_split, cdiv(nrow, 8), 256, 0, s, u, nrow, r, F.h_nk, img, (float *)nullptr, (const uint32_t *)mx, nrhs);
     A.tgt = F.tgt;
     A.parent = p->parent[l];
     A.g = p->bx[l].g;
