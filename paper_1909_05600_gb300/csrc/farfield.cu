@@ -1436,6 +1436,10 @@ struct PwArgs {
     const float4 *sctab;          // double-float sin/cos table (double-float levels)
 };
 
+// points per turn of the forward sums: double-float sums are normalised once for two terms
+template <class R>
+constexpr int DD_STEP = std::is_same<R, dd>::value ? 2 : 1;
+
 // Octant path of a leaf: oct[d] = octant of its ancestor at depth l+1+d within its parent.
 __device__ __forceinline__ int leaf_octant(int4 gl, int shift, int d) {
     int sh = shift - 1 - d;  // depth l+1+d sits sh levels above the leaf
@@ -1465,6 +1469,7 @@ __global__ void __launch_bounds__(128) k_pw_forward(PwArgs<R> P, const uint32_t 
                                                     const float2 *__restrict__ q, int64_t ny, int nrhs,
                                                     typename PwT<R>::C *__restrict__ ut) {
     typedef typename PwT<R>::C C2;
+    constexpr int STEP = DD_STEP<R>;
     __shared__ float4 se[PW_CHUNK];
     __shared__ float4 sl[sizeof(R) == 8 ? PW_CHUNK : 1];
     __shared__ float2 sq[PW_CHUNK];
@@ -1504,23 +1509,33 @@ __global__ void __launch_bounds__(128) k_pw_forward(PwArgs<R> P, const uint32_t 
             if (base == p0 && threadIdx.x < P.A.shift) soct[threadIdx.x] = leaf_octant(P.A.leaf_g[leaf], P.A.shift, threadIdx.x);
             __syncthreads();
 #pragma unroll 2
-            for (int j = 0; j < cnt; ++j) {
+            for (int j = 0; j < cnt; j += STEP) {
                 auto e = Coord<R>::get(se[j], sl, (uint32_t)j);
                 float2 w = sq[j];
+                if constexpr (STEP == 2) {  // a lone last point is paired with itself at weight zero
+                    const int j1 = min(j + 1, cnt - 1);
+                    auto e1 = Coord<R>::get(se[j1], sl, (uint32_t)j1);
+                    const float2 w1 = j1 > j ? sq[j1] : make_float2(0.f, 0.f);
 #pragma unroll
-                for (int t = 0; t < QPT; ++t) {
-                    R ph = fma(kx[t], e.x, fma(ky[t], e.y, kz[t] * e.z));
-                    R sn, cs;
-                    phase_sincos<PH>(ph, sn, cs, P.sctab);
-                    Pc[t].x = acc_fma(cs, w.x, Pc[t].x);
-                    Pc[t].y = acc_fma(cs, w.y, Pc[t].y);
-                    Qs[t].x = acc_fma(sn, w.x, Qs[t].x);
-                    Qs[t].y = acc_fma(sn, w.y, Qs[t].y);
-                    if (j % DD_TERMS == DD_TERMS - 1 || j == cnt - 1) {
-                        acc_norm(Pc[t].x);
-                        acc_norm(Pc[t].y);
-                        acc_norm(Qs[t].x);
-                        acc_norm(Qs[t].y);
+                    for (int t = 0; t < QPT; ++t) {
+                        R sn, cs, sn1, cs1;
+                        phase_sincos<PH>(fma(kx[t], e.x, fma(ky[t], e.y, kz[t] * e.z)), sn, cs, P.sctab);
+                        phase_sincos<PH>(fma(kx[t], e1.x, fma(ky[t], e1.y, kz[t] * e1.z)), sn1, cs1, P.sctab);
+                        Pc[t].x = acc_fma2(cs, w.x, cs1, w1.x, Pc[t].x);
+                        Pc[t].y = acc_fma2(cs, w.y, cs1, w1.y, Pc[t].y);
+                        Qs[t].x = acc_fma2(sn, w.x, sn1, w1.x, Qs[t].x);
+                        Qs[t].y = acc_fma2(sn, w.y, sn1, w1.y, Qs[t].y);
+                    }
+                } else {
+#pragma unroll
+                    for (int t = 0; t < QPT; ++t) {
+                        R ph = fma(kx[t], e.x, fma(ky[t], e.y, kz[t] * e.z));
+                        R sn, cs;
+                        phase_sincos<PH>(ph, sn, cs, P.sctab);
+                        Pc[t].x = fma(cs, (R)w.x, Pc[t].x);
+                        Pc[t].y = fma(cs, (R)w.y, Pc[t].y);
+                        Qs[t].x = fma(sn, (R)w.x, Qs[t].x);
+                        Qs[t].y = fma(sn, (R)w.y, Qs[t].y);
                     }
                 }
             }
@@ -1580,12 +1595,8 @@ __global__ void k_pw_transfer(const uint32_t *__restrict__ tgt, const uint32_t *
                         two_sum_acc(a[m].x, al[m].x, fma(d.x, u.x, -d.y * u.y));
                         two_sum_acc(a[m].y, al[m].y, fma(d.x, u.y, d.y * u.x));
                     } else {
-                        a[m].x = acc_fma(d.x, u.x, acc_fma(-d.y, u.y, a[m].x));
-                        a[m].y = acc_fma(d.x, u.y, acc_fma(d.y, u.x, a[m].y));
-                        if (((e - off[x]) * 2) % DD_TERMS == DD_TERMS - 2 || e + 1 == off[x + 1]) {
-                            acc_norm(a[m].x);
-                            acc_norm(a[m].y);
-                        }
+                        a[m].x = acc_fma2(d.x, u.x, -d.y, u.y, a[m].x);
+                        a[m].y = acc_fma2(d.x, u.y, d.y, u.x, a[m].y);
                     }
                 }
         }
@@ -1693,12 +1704,8 @@ __global__ void __launch_bounds__(128) k_pw_backward(PwArgs<R> P, const uint32_t
                             two_sum_acc(sr[u], lr[u], fma(cs, A.x, sn * B.x));
                             two_sum_acc(si[u], li[u], fma(cs, A.y, sn * B.y));
                         } else {
-                            sr[u] = acc_fma(cs, A.x, acc_fma(sn, B.x, sr[u]));
-                            si[u] = acc_fma(cs, A.y, acc_fma(sn, B.y, si[u]));
-                            if (((j - j0) * 2) % DD_TERMS == DD_TERMS - 2 || j == j1 - 1) {
-                                acc_norm(sr[u]);
-                                acc_norm(si[u]);
-                            }
+                            sr[u] = acc_fma2(cs, A.x, sn, B.x, sr[u]);
+                            si[u] = acc_fma2(cs, A.y, sn, B.y, si[u]);
                         }
                     }
                 }
@@ -1747,7 +1754,7 @@ __global__ void __launch_bounds__(128) k_pw_forward_mr(PwArgs<R> P, const uint32
                                                        const float2 *__restrict__ q, int64_t ny, int nrhs,
                                                        typename PwT<R>::C *__restrict__ ut) {
     typedef typename PwT<R>::C C2;
-    constexpr int CH = 128;
+    constexpr int CH = 128, STEP = DD_STEP<R>;
     __shared__ float4 se[CH];
     __shared__ float4 sl[sizeof(R) == 8 ? CH : 1];
     __shared__ __align__(16) float2 sq[CH][MC];
@@ -1780,36 +1787,53 @@ __global__ void __launch_bounds__(128) k_pw_forward_mr(PwArgs<R> P, const uint32
             if (base == p0 && threadIdx.x < P.A.shift) soct[threadIdx.x] = leaf_octant(P.A.leaf_g[leaf], P.A.shift, threadIdx.x);
             __syncthreads();
             if (base == p0) f = leaf_factor<false>(P, soct, hc);
-            for (int j = 0; j < cnt; ++j) {
+            // e = f e^{-i ph} of point j
+            auto factor = [&](int j, R &er, R &ei) {
                 auto e3 = Coord<R>::get(se[j], sl, (uint32_t)j);
                 R ph = fma(kx, e3.x, fma(ky, e3.y, kz * e3.z));
                 R sn, cs;
                 phase_sincos<PH>(ph, sn, cs, P.sctab);
-                // e = f e^{-i ph}
-                R er = fma(f.x, cs, f.y * sn), ei = fma(f.y, cs, -f.x * sn);
+                er = fma(f.x, cs, f.y * sn);
+                ei = fma(f.y, cs, -f.x * sn);
+            };
+            for (int j = 0; j < cnt; j += STEP) {
+                R er, ei;
+                factor(j, er, ei);
                 // densities of two right-hand sides per 16-byte read
                 const float4 *sq4 = reinterpret_cast<const float4 *>(&sq[j][0]);
+                if constexpr (STEP == 2) {  // a lone last point is paired with itself at weight zero
+                    const int j1 = min(j + 1, cnt - 1);
+                    R er1, ei1;
+                    factor(j1, er1, ei1);
+                    const float4 *sr4 = reinterpret_cast<const float4 *>(&sq[j1][0]);
 #pragma unroll
-                for (int m2 = 0; m2 < MC / 2; ++m2) {
-                    float4 w2 = sq4[m2];
-                    int m = 2 * m2;
-                    Pc[m].x = acc_fma(er, w2.x, Pc[m].x);
-                    Pc[m].y = acc_fma(er, w2.y, Pc[m].y);
-                    Qs[m].x = acc_fma(ei, w2.x, Qs[m].x);
-                    Qs[m].y = acc_fma(ei, w2.y, Qs[m].y);
-                    Pc[m + 1].x = acc_fma(er, w2.z, Pc[m + 1].x);
-                    Pc[m + 1].y = acc_fma(er, w2.w, Pc[m + 1].y);
-                    Qs[m + 1].x = acc_fma(ei, w2.z, Qs[m + 1].x);
-                    Qs[m + 1].y = acc_fma(ei, w2.w, Qs[m + 1].y);
-                }
-                if (j % DD_TERMS == DD_TERMS - 1 || j == cnt - 1)
-#pragma unroll
-                    for (int m = 0; m < MC; ++m) {
-                        acc_norm(Pc[m].x);
-                        acc_norm(Pc[m].y);
-                        acc_norm(Qs[m].x);
-                        acc_norm(Qs[m].y);
+                    for (int m2 = 0; m2 < MC / 2; ++m2) {
+                        const float4 w2 = sq4[m2], v2 = j1 > j ? sr4[m2] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const int m = 2 * m2;
+                        Pc[m].x = acc_fma2(er, w2.x, er1, v2.x, Pc[m].x);
+                        Pc[m].y = acc_fma2(er, w2.y, er1, v2.y, Pc[m].y);
+                        Qs[m].x = acc_fma2(ei, w2.x, ei1, v2.x, Qs[m].x);
+                        Qs[m].y = acc_fma2(ei, w2.y, ei1, v2.y, Qs[m].y);
+                        Pc[m + 1].x = acc_fma2(er, w2.z, er1, v2.z, Pc[m + 1].x);
+                        Pc[m + 1].y = acc_fma2(er, w2.w, er1, v2.w, Pc[m + 1].y);
+                        Qs[m + 1].x = acc_fma2(ei, w2.z, ei1, v2.z, Qs[m + 1].x);
+                        Qs[m + 1].y = acc_fma2(ei, w2.w, ei1, v2.w, Qs[m + 1].y);
                     }
+                } else {
+#pragma unroll
+                    for (int m2 = 0; m2 < MC / 2; ++m2) {
+                        float4 w2 = sq4[m2];
+                        int m = 2 * m2;
+                        Pc[m].x = fma(er, (R)w2.x, Pc[m].x);
+                        Pc[m].y = fma(er, (R)w2.y, Pc[m].y);
+                        Qs[m].x = fma(ei, (R)w2.x, Qs[m].x);
+                        Qs[m].y = fma(ei, (R)w2.y, Qs[m].y);
+                        Pc[m + 1].x = fma(er, (R)w2.z, Pc[m + 1].x);
+                        Pc[m + 1].y = fma(er, (R)w2.w, Pc[m + 1].y);
+                        Qs[m + 1].x = fma(ei, (R)w2.z, Qs[m + 1].x);
+                        Qs[m + 1].y = fma(ei, (R)w2.w, Qs[m + 1].y);
+                    }
+                }
             }
         }
     }
@@ -1901,17 +1925,9 @@ __global__ void __launch_bounds__(128) k_pw_backward_mr(PwArgs<R> P, const uint3
                             two_sum_acc(o[m].x, ol[m].x, fma(cs, A.x, sn * B.x));
                             two_sum_acc(o[m].y, ol[m].y, fma(cs, A.y, sn * B.y));
                         } else {
-                            o[m].x = acc_fma(cs, A.x, acc_fma(sn, B.x, o[m].x));
-                            o[m].y = acc_fma(cs, A.y, acc_fma(sn, B.y, o[m].y));
+                            o[m].x = acc_fma2(cs, A.x, sn, B.x, o[m].x);
+                            o[m].y = acc_fma2(cs, A.y, sn, B.y, o[m].y);
                         }
-                    }
-                    if constexpr (!COMP) {
-                        if ((j * 2) % DD_TERMS == DD_TERMS - 2 || j == qc - 1)
-#pragma unroll
-                            for (int m = 0; m < MC; ++m) {
-                                acc_norm(o[m].x);
-                                acc_norm(o[m].y);
-                            }
                     }
                 }
             }
