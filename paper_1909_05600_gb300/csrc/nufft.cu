@@ -39,6 +39,7 @@ constexpr int NU_CHUNK_S = 256;  // points per spreading block (source side)
 constexpr int NU_CHUNK_T = 1024; // points per interpolation block (target side)
 constexpr int NU_TILE = 8;      // FFT-grid tile edge of the backward spread
 constexpr int NU_EMAX = 24;     // largest bin subgrid edge (E^3 float2 in shared memory)
+constexpr int NU_SMEM = (int)sizeof(float2) * NU_EMAX * NU_EMAX * NU_EMAX;
 constexpr int NU_PB = 64;       // points staged per round of the spreading kernel
 constexpr int NU_GL = 32;       // Gauss-Legendre nodes of the kernel's Fourier transform
 constexpr int NU_IB = 1;        // boxes per forward-interpolation block
@@ -738,7 +739,8 @@ void launch_forward(const ffm_plan_s *p, int l, const float2 *q, int nrhs, float
     float2 *grid = tmp.get<float2>(ns * nrhs * N1);
     FFM_CUDA(cudaMemsetAsync(grid, 0, sizeof(float2) * ns * nrhs * N1, s));
     size_t smem = sizeof(float2) * N.E * N.E * N.E;
-    FFM_CUDA(cudaFuncSetAttribute(k_nu_spread<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the largest size (E <= NU_EMAX), not this launch's: the attribute is shared by all threads and plans
+    FFM_CUDA(cudaFuncSetAttribute(k_nu_spread<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, NU_SMEM));
     FFM_LAUNCH(k_nu_spread<W>, dim3((unsigned)N.n_ych, nrhs), NU_T, smem, s, G, P, N.ych, q, p->ny, ns, grid);
     float2 *fine = tmp.get<float2>(ns * nrhs * N2);
     FFM_LAUNCH(k_nu_pad, dim3((unsigned)(ns * nrhs), N.n2), 256, 0, s, (const float2 *)grid, N.cinv, N.n1,
@@ -768,7 +770,7 @@ void launch_backward(const ffm_plan_s *p, int l, const float2 *vt, int nrhs, dou
                N.tile_q, N.dirU, N.dirW, F.nQ, F.tgt, nt, nrhs, vt, fine);
     exec_fft(N.fft_tgt, N.work_tgt, fine, nt * N2, nrhs, CUFFT_INVERSE, tmp, s);
     size_t smem = sizeof(float2) * N.E * N.E * N.E;
-    FFM_CUDA(cudaFuncSetAttribute(k_nu_binterp<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FFM_CUDA(cudaFuncSetAttribute(k_nu_binterp<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, NU_SMEM));
     FFM_LAUNCH(k_nu_binterp<W>, dim3((unsigned)N.n_xch, nrhs), NU_T, smem, s, G, P, N.xch, (const float2 *)fine,
                N.cinv, nt, p->nx, acc);
     tmp.drop(fine);

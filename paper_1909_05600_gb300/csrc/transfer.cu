@@ -240,6 +240,9 @@ struct PairArgs {
 // 0.45, 100k x 8 right-hand sides (r = 64) 1.68 -> 0.41.  Complex operators (Helmholtz volume 120k at
 // 1e-4, 432 real rows), on CUDA cores before: 24.4 -> 1.9 ms.
 constexpr int PAIR_T = 416;
+// Most translations of a level: the near offsets of the parents take at most four values per axis, their children's
+// at most nine, and the 64 offsets that stay near are none of them.
+constexpr int MAX_TRANS = 9 * 9 * 9 - 4 * 4 * 4;
 constexpr int PAIR_IXW = 4;  // index warps
 constexpr int PAIR_IX = 4;   // units whose row numbers are held
 constexpr int PAIR_ST = 36;  // floats per row of the epilogue's staging (conflict-free float4)
@@ -609,12 +612,16 @@ void build_operator_image(ffm_plan_s *p, int l, const LagGeo &geo, cudaStream_t 
     }
 }
 
-template <int NSTG, int CPS, bool STACK>
+// The dynamic shared memory that an instance may use is a property of the function, shared by all threads and
+// plans: it is set to the largest size of the instance (operator rows NPAD, translations MAX_TRANS), so
+// that no thread lowers it between another's setting and launch.  Per device and cheap: set before every
+// launch (plans may live on several devices).
+template <int NSTG, int CPS, bool STACK, int NPAD>
 static void launch_pairs(const PairArgs &A, unsigned grid, cudaStream_t s) {
-    const size_t sm = pair_smem(NSTG * CPS, A.npad, A.n_trans);
-    // per device and cheap: set before every launch (plans may live on several devices)
-    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG, CPS, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    FFM_LAUNCH_NAMED("k_lag_pairs", (k_lag_pairs<NSTG, CPS, STACK>), grid, PAIR_T, sm, s, A);
+    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG, CPS, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)pair_smem(NSTG * CPS, NPAD, MAX_TRANS)));
+    FFM_LAUNCH_NAMED("k_lag_pairs", (k_lag_pairs<NSTG, CPS, STACK>), grid, PAIR_T,
+                     pair_smem(NSTG * CPS, A.npad, A.n_trans), s, A);
 }
 
 // v~ += T u~ for all pairs of the level: u has rows of K floats per (source box, right-hand side),
@@ -659,13 +666,13 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     const unsigned grid = (unsigned)std::min<int64_t>(most, 152);
     // stages of two chunks where the K extent allows: half the barrier round trips
     if (A.npad <= 64 && A.nk % 2 == 0)
-        launch_pairs<4, 2, true>(A, grid, s);
+        launch_pairs<4, 2, true, 64>(A, grid, s);
     else if (A.npad <= 64)
-        launch_pairs<8, 1, true>(A, grid, s);
+        launch_pairs<8, 1, true, 64>(A, grid, s);
     else if (stack)
-        launch_pairs<6, 1, true>(A, grid, s);
+        launch_pairs<6, 1, true, 128>(A, grid, s);
     else
-        launch_pairs<4, 1, false>(A, grid, s);
+        launch_pairs<4, 1, false, 256>(A, grid, s);
     tmp.drop(inv);
     tmp.drop(img);
 }
@@ -1026,11 +1033,14 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * A.tcols));
 }
 
+static size_t target_smem(int nchunk, int npad) { return 1024 + (size_t)nchunk * (A_BYTES + npad * HROW * 2); }
+
+// (the attribute as in launch_pairs: the instance's largest size, 64 operator rows)
 template <int NSTG, int CPS>
 static void launch_targets(const TargetArgs &A, dim3 grid, cudaStream_t s) {
-    const size_t sm = 1024 + (size_t)NSTG * CPS * (A_BYTES + A.npad * HROW * 2);
-    FFM_CUDA(cudaFuncSetAttribute(k_lag_targets<NSTG, CPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    FFM_LAUNCH_NAMED("k_lag_targets", (k_lag_targets<NSTG, CPS>), grid, TG_T, sm, s, A);
+    FFM_CUDA(cudaFuncSetAttribute(k_lag_targets<NSTG, CPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)target_smem(NSTG * CPS, 64)));
+    FFM_LAUNCH_NAMED("k_lag_targets", (k_lag_targets<NSTG, CPS>), grid, TG_T, target_smem(NSTG * CPS, A.npad), s, A);
 }
 
 // v~ = sum over each target's partners of T u~ (rows of targets without partners untouched)
