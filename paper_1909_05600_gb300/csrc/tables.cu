@@ -597,7 +597,6 @@ void build_tables(ffm_plan_s *p, int l, TableJob &tj) {
     FarLevel &F = p->far[l];
     cudaStream_t s = tj.side;
     Alloc &tmp = tj.tmp;
-    if (F.mode == 1 && F.r1 > R1MAX) fail(FFM_EUNSUPPORTED, "eps needs more than 8 Chebyshev nodes per axis");
     double dl = std::ldexp(p->d0, -l);
     double oxy[3] = {p->oX[0] - p->oY[0], p->oX[1] - p->oY[1], p->oX[2] - p->oY[2]};
     if (F.mode == 1) {

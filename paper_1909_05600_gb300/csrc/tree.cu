@@ -1443,6 +1443,8 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     F.n_trans = (int)h.ntrans;
     F.n_tgt = h.ntgt;
     F.r1 = p->r1_override > 0 ? p->r1_override : r1_rule(p->kind, p->eps);
+    // before anything is sized or indexed by it
+    if (lag && na > 0 && F.r1 > R1MAX) fail(FFM_EUNSUPPORTED, "eps needs more than 8 Chebyshev nodes per axis");
     // a level that is to run the target-stationary transfer (the option, the pick stored in the plan's
     // autotune cache, or the rule) takes no pair lists
     const bool ts_able = p->kind == FFM_LAPLACE && F.r1 <= 4 && !(p->aca_eps > 0.0);
