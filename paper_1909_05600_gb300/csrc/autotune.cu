@@ -66,25 +66,22 @@ std::string device_tag() {
     return n + "_" + std::to_string(pr.multiProcessorCount) + "sm";
 }
 
-// "key value..." lines; the last line of a key wins
+bool find_pick(const TunePicks &kv, const std::string &k, std::string &v) {
+    auto it = kv.find(k);
+    if (it == kv.end()) return false;
+    v = it->second;
+    return true;
+}
+
+// the picks of a file, and new ones appended to it
 class Cache {
   public:
     explicit Cache(const char *path) {
         if (!path) return;
         path_ = path;
-        std::ifstream f(path_);
-        std::string line;
-        while (std::getline(f, line)) {
-            size_t sp = line.find(" = ");
-            if (sp != std::string::npos) kv_[line.substr(0, sp)] = line.substr(sp + 3);
-        }
+        kv_ = read_tune_picks(path);
     }
-    bool get(const std::string &k, std::string &v) const {
-        auto it = kv_.find(k);
-        if (it == kv_.end()) return false;
-        v = it->second;
-        return true;
-    }
+    bool get(const std::string &k, std::string &v) const { return find_pick(kv_, k, v); }
     void put(const std::string &k, const std::string &v) {
         kv_[k] = v;
         if (path_.empty()) return;
@@ -94,7 +91,7 @@ class Cache {
 
   private:
     std::string path_;
-    std::map<std::string, std::string> kv_;
+    TunePicks kv_;
 };
 
 std::string near_key(const ffm_plan_s *p, const std::string &dev, int rhsb) {
@@ -147,17 +144,31 @@ void set_items(ffm_plan_s *p, int tch, unsigned smax, Alloc &tmp, cudaStream_t s
 
 }  // namespace
 
+// "key = value" lines; the last line of a key wins
+TunePicks read_tune_picks(const char *path) {
+    TunePicks kv;
+    std::ifstream f(path);
+    std::string line;
+    while (std::getline(f, line)) {
+        size_t sp = line.find(" = ");
+        if (sp != std::string::npos) kv[line.substr(0, sp)] = line.substr(sp + 3);
+    }
+    return kv;
+}
+
 int cached_lag_pick(const ffm_plan_s *p, int l) {
-    if (p->tune_cache.empty()) return -1;
-    Cache cache(p->tune_cache.c_str());
+    if (p->tune_picks.empty()) return -1;
     std::string v;
     int a = -1;
-    if (cache.get(lag_key(p, l, device_tag(), 1), v) && parse_lag(v, a)) return a;
+    if (find_pick(p->tune_picks, lag_key(p, l, device_tag(), 1), v) && parse_lag(v, a)) return a;
     return -1;
 }
 
-void apply_cached_picks(ffm_plan_s *p, const char *cache_path, cudaStream_t s) {
-    Cache cache(cache_path);
+void apply_cached_picks(ffm_plan_s *p, cudaStream_t s) {
+    struct {
+        const TunePicks &kv;
+        bool get(const std::string &k, std::string &v) const { return find_pick(kv, k, v); }
+    } cache{p->tune_picks};
     const std::string dev = device_tag();
     Alloc tmp;
     tmp.stream = s;

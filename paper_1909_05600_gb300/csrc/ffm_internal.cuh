@@ -6,6 +6,7 @@
 
 #include <atomic>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -233,6 +234,7 @@ struct FarLevel {
 
 struct ffm_plan_s;
 namespace ffm {
+typedef std::map<std::string, std::string> TunePicks;  // autotune picks by key (autotune.cu)
 void nufft_release(ffm_plan_s *p);  // nufft.cu: cuFFT handles
 }
 
@@ -278,7 +280,7 @@ struct ffm_plan_s {
     int4 *items = nullptr;          // (target leaf, first target in the leaf, first pair, end pair)
     int *dev_err = nullptr;         // device-side error flags (bounded waits that gave up)
     int wait_tries = 1 << 24;       // try_wait attempts per bounded device-side wait (ffm_opts.wait_tries)
-    std::string tune_cache;         // ffm_opts.autotune_cache (empty: none)
+    ffm::TunePicks tune_picks;      // the contents of ffm_opts.autotune_cache, read once per plan
     ffm_info info{};
 };
 
@@ -304,8 +306,9 @@ void build_lag_table(ffm_plan_s *p, int l, cudaStream_t s);
 void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
 // the same over each target's partners (target-stationary; ts_ok levels)
 void lag_targets(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s);
-// autotune.cu: the transfer variant stored for Lagrange level l in the plan's autotune
-// cache (0 CUDA cores, 1 tcgen05 per translation, 2 target-stationary), or -1
+// autotune.cu: the contents of a cache file; the transfer variant stored for Lagrange level l in the plan's
+// picks (0 CUDA cores, 1 tcgen05 per translation, 2 target-stationary), or -1
+TunePicks read_tune_picks(const char *path);
 int cached_lag_pick(const ffm_plan_s *p, int l);
 
 // tree.cu: near-field work items with targets in chunks of tchunk and at most smax source
@@ -365,8 +368,8 @@ void nufft_backward(const ffm_plan_s *p, int l, const float2 *vt, int nrhs, doub
 void gauss_legendre_nodes(int n, std::vector<double> &x, std::vector<double> &w);  // tables.cu
 // autotune.cu: pick kernel variants by timing them on the plan (ffm_autotune)
 void autotune(ffm_plan_s *p, int nrhs, const char *cache_path, cudaStream_t s);
-// take the picks a cache file holds for this plan's sizes (no timing); at plan creation
-void apply_cached_picks(ffm_plan_s *p, const char *cache_path, cudaStream_t s);
+// take the plan's stored picks for its sizes (no timing); at plan creation
+void apply_cached_picks(ffm_plan_s *p, cudaStream_t s);
 // The same with explicit work items (the autotuner times candidate item shapes).
 void near_field_items(const ffm_plan_s *p, const int4 *items, int64_t n_items, int tchunk, const void *q, int nrhs,
                       double2 *acc, cudaStream_t s);

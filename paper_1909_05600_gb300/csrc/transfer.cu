@@ -628,6 +628,7 @@ static void launch_pairs(const PairArgs &A, unsigned grid, cudaStream_t s) {
 // v~ rows of `rows` floats per (target box, right-hand side) and component
 void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, Alloc &tmp, cudaStream_t s) {
     const FarLevel &F = p->far[l];
+    if (!F.bt_off) fail(FFM_ECUDA, "transfer by translation on a level without grouped pairs");
     const bool cplx = p->kind == FFM_HELMHOLTZ;
     const int r = F.r1 * F.r1 * F.r1, rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;
     const int rows = cplx ? 2 * r : r, K = cplx ? 2 * rk : rk, ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;

@@ -1453,7 +1453,8 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     if (lag && na > 0) {
         if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
         if (ts_able && !root && p->lag_transfer == 0 && pick < 0 && target_stationary_pays(F)) F.tune_tc = 2;
-        ts_first = ts_able && !root && (F.tune_tc == 2 || pick == 2);
+        if (ts_able && !root && pick == 2) F.tune_tc = 2;
+        ts_first = ts_able && !root && F.tune_tc == 2;
     }
     if (na > 0 && !ts_first) {
         F.adm_src = p->mem.get<uint32_t>(na);
@@ -1731,8 +1732,12 @@ void build_plan(ffm_plan_s *p, const void *X, ffm_dtype xdt, const void *Y, ffm_
     }
     for (int l = 0; l <= ls; ++l)
         if (p->far[l].n_adm > 0) build_octants(p, l, tj);
-    for (int l = 0; l <= ls; ++l)
-        if (p->far[l].tune_tc == 2) prepare_target_stationary(p, l, s);
+    // every dense Lagrange level leaves here with what its transfer reads: near tables or grouped pairs
+    for (int l = 0; l <= ls; ++l) {
+        FarLevel &F = p->far[l];
+        if (F.tune_tc == 2) prepare_target_stationary(p, l, s);
+        if (F.mode == 1 && F.n_adm > 0 && !F.ts_ok) build_translation_groups(p, l, s);
+    }
     // plane-wave levels whose F steps run as type-3 NUFFTs: FP32 levels with many directions
     // (the NUFFT's cost per box barely depends on nQ, the direct sums' grows with it), all
     // FP32 and compensated-FP32 levels when forced, none when direct sums are forced
