@@ -78,6 +78,15 @@ __device__ __forceinline__ void row_scale(float mx, float &s, float &inv) {
     inv = __int_as_float((127 - e) << 23);
 }
 
+// The two scales' inverses (powers of two) as factors f1 f2 = a b of about equal size: a value times f1, then f2,
+// stays between the value and the result, so it leaves FP32's range only where the result does
+// (densities of 1e34 and more did, with a and b one after the other).
+__device__ __forceinline__ void even_factors(float a, float b, float &f1, float &f2) {
+    const int e = (__float_as_int(a) >> 23) + (__float_as_int(b) >> 23) - 254, h = e >> 1;  // |e| <= 240
+    f1 = __int_as_float((127 + h) << 23);
+    f2 = __int_as_float((127 + e - h) << 23);
+}
+
 __device__ __forceinline__ void half_split(float x, __half &hi, __half &lo) {
     hi = __float2half_rn(x);
     lo = __float2half_rn(x - __half2float(hi));
@@ -496,7 +505,8 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                 ok = false;
                 break;
             }
-            const float inv = s_inv[ix][32 * q + lane];
+            float f1, f2;
+            even_factors(s_inv[ix][32 * q + lane], A.tinv, f1, f2);
             const uint32_t drow = s_dst[ix][32 * q + lane];
             // rows of this warp with pairs (a prefix)
             const int mine = __popc(__ballot_sync(0xffffffffu, s_src[ix][32 * q + lane] != NONE));
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                             for (int j = 0; j < 4; ++j) {
                                 float y = __uint_as_float(v[4 * k + j]);
                                 if constexpr (STACK) y += __uint_as_float(w[4 * k + j]);
-                                x[j] = y * inv * A.tinv;
+                                x[j] = y * f1 * f2;
                             }
                             *reinterpret_cast<float4 *>(st + lane * PAIR_ST + 16 * h + 4 * k) =
                                 make_float4(x[0], x[1], x[2], x[3]);
@@ -1009,11 +1019,12 @@ __global__ void __launch_bounds__(TG_T, 1) k_lag_targets(const __grid_constant__
         }
         const int64_t x = x0 + 32 * q + lane;
         if (ok && x < A.n_tgt) {
-            float us, ui;
+            float us, ui, f1, f2;
             row_scale(__uint_as_float(A.umax[m]), us, ui);
+            even_factors(ui, A.tinv, f1, f2);
             float *dst = A.vt + ((size_t)A.tgt[x] * A.nrhs + m) * A.r;
 #pragma unroll
-            for (int c = 0; c < 64; ++c) sum[c] = sum[c] * ui * A.tinv;
+            for (int c = 0; c < 64; ++c) sum[c] = sum[c] * f1 * f2;
             if (A.r == 64) {
 #pragma unroll
                 for (int c = 0; c < 64; c += 4)
