@@ -181,6 +181,7 @@ void apply_cached_picks(ffm_plan_s *p, cudaStream_t s) {
         if (F.n_adm == 0) continue;
         int a, b, c;
         if (F.mode == 1) {
+            if (F.n_adm > MAX_LISTED) continue;  // keeps the only transfer that can take it
             if (p->kind != FFM_HELMHOLTZ && !F.aca && cache.get(lag_key(p, l, dev, 1), v) && parse_lag(v, a)) {
                 if (a == 2) prepare_target_stationary(p, l, s);
                 if (a != 2 || !F.ts_ok) build_translation_groups(p, l, s);
@@ -266,7 +267,7 @@ void autotune(ffm_plan_s *p, int nrhs, const char *cache_path, cudaStream_t s) {
         };
         std::string v;
         if (F.mode == 1) {
-            if (helm || F.aca) continue;
+            if (helm || F.aca || F.n_adm > MAX_LISTED) continue;
             build_group_tiles(p, l, s);  // the per-translation candidates
             std::string key = lag_key(p, l, dev, rhs_bucket(nrhs));
             int pick = -1;

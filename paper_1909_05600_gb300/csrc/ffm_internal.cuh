@@ -17,6 +17,7 @@ namespace ffm {
 
 constexpr int LMAX = 21;         // finest level of the Morton keys (3 x 21 bits)
 constexpr int R1MAX = 8;         // largest Chebyshev node count per axis
+constexpr int64_t MAX_LISTED = 0xffffffffll;  // pairs of a level that a list with 32-bit offsets holds
 constexpr int LAG_GEMM_BN = 32;  // pairs (GEMM columns) per tile of the Lagrange transfer
 constexpr int P2P_T = 128;        // threads per near-field block (the largest target chunk)
 constexpr int LAG_CHUNK = 512;    // points per block of the Lagrange point-wise kernels
@@ -159,7 +160,7 @@ struct FarLevel {
     int64_t n_tgt = 0, n_src = 0;   // boxes with at least one admissible pair
     uint32_t *tgt = nullptr;        // n_tgt target box indices
     uint32_t *src = nullptr;        // n_src source box indices
-    uint32_t *adm_off = nullptr;    // n_tgt+1 CSR offsets (per listed target)
+    uint32_t *adm_off = nullptr;    // n_tgt+1 CSR offsets (per listed target; no use past MAX_LISTED pairs)
     uint32_t *adm_src = nullptr;    // n_adm source box per pair (null on target-stationary levels)
     uint32_t *adm_t = nullptr;      // n_adm translation index per pair
     int4 *trans_m = nullptr;        // n_trans integer offsets gX - gY

@@ -751,9 +751,12 @@ __global__ void __launch_bounds__(32 * DS_W) k_descend(const __grid_constant__ D
 // translations in use and leaves all totals in one place, the level's only read-back), then the lists.
 constexpr int LV_T = 256, LV_PER = 8, LV_TILE = LV_T * LV_PER;
 
+// Pairs are counted in 64 bits (a tile's in 32: LV_TILE boxes of at most 665 admissible and 64 near ones), their lists
+// and offsets have 32: the host refuses what does not fit before anything is written through them.
 struct LevelTotals {
     unsigned long long tgt_points, src_points;
-    uint32_t na, nn, ntgt, nsrc, tch, sch, ntrans, err;
+    unsigned long long na, nn;
+    uint32_t ntgt, nsrc, tch, sch, ntrans, err;
     uint32_t pw_sch, pw_tch;  // chunks of PW_TC_FCH source points and PW_TC_BCH target points
     uint32_t bits[128];       // the translation codes in use
 };
@@ -852,6 +855,18 @@ __global__ void __launch_bounds__(1024) k_level_mid(const __grid_constant__ Leve
         }
         return carry;
     };
+    // the pairs of all tiles, each kind by itself: the packed sums of the scan hold only 32 bits of each
+    unsigned long long na = 0, nn = 0;
+    for (int64_t i = threadIdx.x; i < A.ntx; i += 1024) {
+        na += A.ta[i] >> 32;
+        nn += A.ta[i] & 0xffffffffull;
+    }
+    block_excl_scan64(na, sm, &t);
+    if (threadIdx.x == 0) A.tot->na = t;
+    __syncthreads();
+    block_excl_scan64(nn, sm, &t);
+    if (threadIdx.x == 0) A.tot->nn = t;
+    __syncthreads();
     const unsigned long long a = scan_row(A.ta, A.ntx), bx = scan_row(A.tb, A.ntx), by = scan_row(A.tb + A.ntx, A.nty);
     uint32_t u[4], c = 0;
 #pragma unroll
@@ -868,8 +883,6 @@ __global__ void __launch_bounds__(1024) k_level_mid(const __grid_constant__ Leve
         A.tot->bits[threadIdx.x] = w;
     }
     if (threadIdx.x == 0) {
-        A.tot->na = (uint32_t)(a >> 32);
-        A.tot->nn = (uint32_t)a;
         A.tot->ntgt = (uint32_t)(bx >> 32);
         A.tot->tch = (uint32_t)bx;
         A.tot->nsrc = (uint32_t)(by >> 32);
@@ -1288,6 +1301,7 @@ __global__ void k_box_offsets(const uint32_t *__restrict__ tgt, const uint32_t *
 
 void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cudaStream_t s) {
     const FarLevel &F = p->far[l];
+    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs: the level has no list of them");
     Alloc tmp;
     tmp.stream = s;
     DescendArgs D{};
@@ -1322,6 +1336,7 @@ void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cud
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
     if (F.mode != 1 || F.n_adm == 0 || F.bt_off) return;
+    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs: the level has no list of them");
     Alloc tmp;
     tmp.stream = s;
     if (!F.adm_src) {
@@ -1436,7 +1451,8 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     FFM_CUDA(cudaMemcpyAsync(&h, &S->tot, sizeof h, cudaMemcpyDeviceToHost, s));
     FFM_CUDA(cudaStreamSynchronize(s));
     if (h.err) fail(FFM_ECUDA, "box translation outside the expected range");
-    const int64_t na = h.na, nn = h.nn;
+    const int64_t na = (int64_t)h.na, nn = (int64_t)h.nn;
+    if (nn > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 near pairs at one level");
     F.n_adm = na;
     p->info.n_adm[l] = na;
     const bool last = stop(nn);
@@ -1453,9 +1469,13 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     if (lag && na > 0) {
         if (p->lag_transfer > 0) F.tune_tc = p->lag_transfer - 1;  // forced variant
         if (ts_able && !root && p->lag_transfer == 0 && pick < 0 && target_stationary_pays(F)) F.tune_tc = 2;
-        if (ts_able && !root && pick == 2) F.tune_tc = 2;
+        // (the only transfer for more pairs than a list can hold)
+        if (ts_able && !root && (pick == 2 || (p->lag_transfer == 0 && na > MAX_LISTED))) F.tune_tc = 2;
         ts_first = ts_able && !root && F.tune_tc == 2;
     }
+    if (na > MAX_LISTED && !ts_first)
+        fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs at one level (only the target-stationary transfer "
+                               "of the Laplace single layer does without a list of them)");
     if (na > 0 && !ts_first) {
         F.adm_src = p->mem.get<uint32_t>(na);
         F.adm_t = p->mem.get<uint32_t>(na);
