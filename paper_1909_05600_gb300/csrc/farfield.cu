@@ -24,7 +24,7 @@ namespace ffm {
 // ----------------------------------------------------------- helpers
 
 struct Cheb {
-    float t[R1MAX];  // Chebyshev nodes cos((2a+1) pi / (2 r1))
+    float t[R1MAX];  // Chebyshev nodes (cheb_node)
     float w[R1MAX];  // 1 / prod_{b != a} (t_a - t_b)
     int r1;
 };
@@ -33,7 +33,7 @@ static Cheb make_cheb(int r1) {
     Cheb c{};
     c.r1 = r1;
     double t[R1MAX];
-    for (int a = 0; a < r1; ++a) t[a] = std::cos((2.0 * a + 1.0) * PI / (2.0 * r1));
+    for (int a = 0; a < r1; ++a) t[a] = cheb_node(r1, a);
     for (int a = 0; a < r1; ++a) {
         double d = 1.0;
         for (int b = 0; b < r1; ++b)
@@ -962,7 +962,7 @@ __device__ __forceinline__ float2 pair_norm(float h, float l) {
 static Halves make_halves(int r1) {
     Halves H{};
     double t[R1MAX];
-    for (int a = 0; a < r1; ++a) t[a] = std::cos((2.0 * a + 1.0) * PI / (2.0 * r1));
+    for (int a = 0; a < r1; ++a) t[a] = cheb_node(r1, a);
     for (int h = 0; h < 2; ++h)
         for (int b = 0; b < r1; ++b) {
             const double x = 0.5 * (t[b] + (h ? 1.0 : -1.0));
@@ -970,7 +970,7 @@ static Halves make_halves(int r1) {
                 double v = 1.0;
                 for (int c = 0; c < r1; ++c)
                     if (c != a) v *= (x - t[c]) / (t[a] - t[c]);
-                    H.m[h][a][b] = make_float2((float)v, (float)(v - (double)(float)v));
+                H.m[h][a][b] = make_float2((float)v, (float)(v - (double)(float)v));
             }
         }
     return H;

@@ -394,7 +394,7 @@ struct AcaGeo {
     double oxy[3];
     double dl;
     int r1;
-    double hnode[R1MAX];  // (d_l / 2) cos((2a+1) pi / (2 r1))
+    double hnode[R1MAX];  // (d_l / 2) cheb_node(r1, a)
 };
 
 // Magnitudes are compared as the bit patterns of non-negative doubles (their order is the
@@ -529,7 +529,7 @@ static void build_aca(ffm_plan_s *p, int l, const double oxy[3], double dl, Tabl
     for (int d = 0; d < 3; ++d) g.oxy[d] = oxy[d];
     g.dl = dl;
     g.r1 = F.r1;
-    for (int a = 0; a < F.r1; ++a) g.hnode[a] = 0.5 * dl * std::cos((2.0 * a + 1.0) * PI / (2.0 * F.r1));
+    for (int a = 0; a < F.r1; ++a) g.hnode[a] = 0.5 * dl * cheb_node(F.r1, a);
     const size_t rbytes = sizeof(double) * (size_t)r * r;
     const int in_smem = rbytes <= 125 * 1024;
     double *R = in_smem ? nullptr : tmp.get<double>((size_t)nt * r * r);
@@ -579,7 +579,7 @@ LagGeo lag_geo(const ffm_plan_s *p, int l) {
     g.k = (float)p->k;
     g.r1 = F.r1;
     g.kind = p->kind;
-    for (int a = 0; a < F.r1; ++a) g.hnode[a] = (float)(0.5 * g.dl * std::cos((2.0 * a + 1.0) * PI / (2.0 * F.r1)));
+    for (int a = 0; a < F.r1; ++a) g.hnode[a] = (float)(0.5 * g.dl * cheb_node(F.r1, a));
     return g;
 }
 
