@@ -619,11 +619,12 @@ __device__ __forceinline__ void tmem_st8(uint32_t ta, const uint32_t (&v)[8]) {
 }
 
 // Target step of a Lagrange level (L_X^T v~ of eq. 8): v_i += sum_abc L_a(x_i) L_b(y_i) L_c(z_i) v~_a(abc),
-// one block per chunk of at most LAG_CHUNK points of a target box, written in FP32 to accf.
+// one block per chunk of at most LAG_CHUNK points of a target box, in FP32 to accf: written, or (add) added
+// to what an earlier level wrote.
 template <bool CPLX, int R1>
 __global__ void __launch_bounds__(128) k_lag_interp(LevelArgs A, const uint2 *__restrict__ chunks, Cheb cb,
                                                     const typename QT<CPLX>::T *__restrict__ vt, int nrhs,
-                                                    int64_t nx, float2 *__restrict__ accf) {
+                                                    int64_t nx, bool add, float2 *__restrict__ accf) {
     typedef typename QT<CPLX>::T Q;
     constexpr int r = R1 * R1 * R1;
     __shared__ Q sv[r];
@@ -661,6 +662,11 @@ __global__ void __launch_bounds__(128) k_lag_interp(LevelArgs A, const uint2 *__
                 sr = fmaf(lab, pr, sr);
                 if constexpr (CPLX) si = fmaf(lab, pi, si);
             }
+        if (CPLX && add) {
+            const float2 f = accf[(int64_t)m * nx + i];
+            sr += f.x;
+            si += f.y;
+        }
         accf[(int64_t)m * nx + i] = make_float2(sr, si);
     }
 }
@@ -780,7 +786,7 @@ template <bool CPLX, int R1>
 __global__ void __launch_bounds__(32 * LAG_WC) k_lag_interp_w(LevelArgs A, const uint2 *__restrict__ chunks,
                                                              int64_t nchunks, Cheb cb,
                                                              const typename QT<CPLX>::T *__restrict__ vt, int nrhs,
-                                                             int64_t nx, float2 *__restrict__ accf) {
+                                                             int64_t nx, bool add, float2 *__restrict__ accf) {
     typedef typename QT<CPLX>::T Q;
     constexpr int r = R1 * R1 * R1;
     __shared__ Q sv[LAG_WC][r];
@@ -823,13 +829,18 @@ __global__ void __launch_bounds__(32 * LAG_WC) k_lag_interp_w(LevelArgs A, const
                 sr = fmaf(lab, pr, sr);
                 if constexpr (CPLX) si = fmaf(lab, pi, si);
             }
+        if (CPLX && add) {
+            const float2 f = accf[(int64_t)m * nx + i];
+            sr += f.x;
+            si += f.y;
+        }
         accf[(int64_t)m * nx + i] = make_float2(sr, si);
     }
 }
 
 template <bool CPLX, int R1>
 static void lagrange_points(const ffm_plan_s *p, const FarLevel &F, const LevelArgs &A, const Cheb &cb, bool anterp,
-                            const void *in, int nrhs, void *out, cudaStream_t s) {
+                            const void *in, int nrhs, void *out, cudaStream_t s, bool add) {
     typedef typename QT<CPLX>::T Q;
     // warp per chunk up to r = 64 (the ranks of eps >= 1e-4 for the single layer); the block
     // forms keep the larger bases, whose per-point sums need more registers per thread
@@ -841,7 +852,7 @@ static void lagrange_points(const ffm_plan_s *p, const FarLevel &F, const LevelA
         } else {
             dim3 g(cdiv(F.n_tgt_chunks, LAG_WC), nrhs);
             FFM_LAUNCH((k_lag_interp_w<CPLX, R1>), g, 32 * LAG_WC, 0, s, A, F.tgt_chunks, F.n_tgt_chunks, cb,
-                       (const Q *)in, nrhs, p->nx, (float2 *)out);
+                       (const Q *)in, nrhs, p->nx, add, (float2 *)out);
         }
         return;
     }
@@ -852,7 +863,7 @@ static void lagrange_points(const ffm_plan_s *p, const FarLevel &F, const LevelA
     } else {
         dim3 g((unsigned)F.n_tgt_chunks, nrhs);
         FFM_LAUNCH((k_lag_interp<CPLX, R1>), g, 128, 0, s, A, F.tgt_chunks, cb, (const Q *)in, nrhs, p->nx,
-                   (float2 *)out);
+                   add, (float2 *)out);
     }
 }
 
@@ -879,15 +890,15 @@ static void lagrange_anterp_dl_r1(const ffm_plan_s *p, const FarLevel &F, const 
 
 template <bool CPLX>
 static void lagrange_points_r1(const ffm_plan_s *p, const FarLevel &F, const LevelArgs &A, const Cheb &cb,
-                               bool anterp, const void *in, int nrhs, void *out, cudaStream_t s) {
+                               bool anterp, const void *in, int nrhs, void *out, cudaStream_t s, bool add = false) {
     switch (F.r1) {
-        case 2: lagrange_points<CPLX, 2>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 3: lagrange_points<CPLX, 3>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 4: lagrange_points<CPLX, 4>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 5: lagrange_points<CPLX, 5>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 6: lagrange_points<CPLX, 6>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 7: lagrange_points<CPLX, 7>(p, F, A, cb, anterp, in, nrhs, out, s); break;
-        case 8: lagrange_points<CPLX, 8>(p, F, A, cb, anterp, in, nrhs, out, s); break;
+        case 2: lagrange_points<CPLX, 2>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 3: lagrange_points<CPLX, 3>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 4: lagrange_points<CPLX, 4>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 5: lagrange_points<CPLX, 5>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 6: lagrange_points<CPLX, 6>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 7: lagrange_points<CPLX, 7>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
+        case 8: lagrange_points<CPLX, 8>(p, F, A, cb, anterp, in, nrhs, out, s, add); break;
         default: fail(FFM_EUNSUPPORTED, "Chebyshev nodes per axis outside 2..8");
     }
 }
@@ -936,8 +947,7 @@ static void tc_transfer(const FarLevel &F, const uint32_t *src, const uint32_t *
 // 24.4 + 22.1 ms over eight levels, gradient 300k: 0.28 + 0.81 ms).
 //
 // The three 1-D steps run in FP32 pairs (error-free products and sums): their rounding is shared by all
-// points of a box, where that of the point-wise sums averages out, and in plain FP32 it took
-// the Helmholtz parity case (cube surface, k = 12) from 3.1e-7 to 1.0e-6 of the oracle's FFM.
+// points of a box, where that of the point-wise sums averages out.  Real kernels only (far_lagrange_complex).
 struct Halves {
     float2 m[2][R1MAX][R1MAX];  // [half][parent node][child node], as unevaluated pairs
 };
@@ -980,7 +990,7 @@ struct LinkArgs {
     int64_t n;                    // parent boxes
     const uint32_t *first_child;
     const int4 *gc;               // children's coordinates (low bits: octant)
-    int nrhs, rowlen, es;         // floats between rows, between values of a row
+    int nrhs, rowlen;             // floats between rows
     int coff;                     // floats between components within a row
     int64_t pbase, cbase;         // floats between components of the parents', the children's array
 };
@@ -1031,7 +1041,7 @@ __global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
                 float2 o = B[hyz][i];
 #pragma unroll
                 for (int b = 0; b < R1; ++b)
-                    pair_fma(o.x, o.y, make_float2(__ldg(row + (int64_t)(b * R1 * R1 + rest) * A.es), 0.f), mat[hx][a][b]);
+                    pair_fma(o.x, o.y, make_float2(__ldg(row + b * R1 * R1 + rest), 0.f), mat[hx][a][b]);
                 B[hyz][i] = o;
             }
         }
@@ -1071,7 +1081,7 @@ __global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
             for (int hz = 0; hz < 2; ++hz)
 #pragma unroll
                 for (int b = 0; b < R1; ++b) pair_fma(h, l, B[hz][ab + b], mat[hz][z][b]);
-            out[(int64_t)i * A.es] = h + l;
+            out[i] = h + l;
         }
     }
 }
@@ -1092,7 +1102,7 @@ __global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
     if (p >= A.n) return;
     float2(*B)[r] = buf[grp], (*Z)[r] = first[grp];
     const float *row = vp + comp * A.pbase + (int64_t)comp * A.coff + (p * A.nrhs + m) * (int64_t)A.rowlen;
-    for (int i = th; i < r; i += T) B[0][i] = make_float2(row[(int64_t)i * A.es], 0.f);
+    for (int i = th; i < r; i += T) B[0][i] = make_float2(row[i], 0.f);
     link_sync<R1>();
 #pragma unroll
     for (int hz = 0; hz < 2; ++hz)
@@ -1133,10 +1143,10 @@ __global__ void __launch_bounds__(LinkShape<R1>::T *LinkShape<R1>::NB)
             const int i = th + v * T;
             if (i < r) {
                 const int x = i / (R1 * R1), rest = i % (R1 * R1);
-                float h = out[(int64_t)i * A.es], l = 0.f;
+                float h = out[i], l = 0.f;
 #pragma unroll
                 for (int a = 0; a < R1; ++a) pair_fma(h, l, B[hyz][a * R1 * R1 + rest], mat[hx][a][x]);
-                out[(int64_t)i * A.es] = h + l;
+                out[i] = h + l;
             }
         }
     }
@@ -1223,10 +1233,36 @@ void lagrange_transfer(const ffm_plan_s *p, int l, const void *ut, int nrhs, voi
     }
 }
 
-// All Lagrange levels of an apply, coarsest lo to finest hi: u~ of level hi from the points, up to lo
+// Complex Lagrange levels: every level's sums from and to the points.  Coefficients that go up and down between the
+// levels hand one level's rounding on to all coarser ones, where levels formed apart have errors of their own
+// (Helmholtz parity case, cube surface k = 12, FP32 multiply-adds: 3.1e-7 of the oracle's FFM apart, 3.7e-7 through the
+// links), and such a plan has only two or three Lagrange levels to form (volume 120k: 0.08 + 0.03 ms in all).
+static bool far_lagrange_complex(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s) {
+    bool any = false;
+    for (int l = 0; l <= p->l_stop; ++l) {
+        const FarLevel &F = p->far[l];
+        if (F.mode != 1 || F.n_adm == 0) continue;
+        size_t ub, vb;
+        lagrange_bytes(p, l, nrhs, &ub, &vb);
+        void *ut = tmp.raw(ub), *vt = tmp.raw(vb);
+        FFM_CUDA(cudaMemsetAsync(ut, 0, ub, s));
+        FFM_CUDA(cudaMemsetAsync(vt, 0, vb, s));
+        const Cheb cb = make_cheb(F.r1);
+        lagrange_points_r1<true>(p, F, level_args(p, p->by[l], p->by[p->l_stop], p->epsY, l), cb, true, q, nrhs, ut, s);
+        lagrange_transfer(p, l, ut, nrhs, vt, tmp, s);
+        lagrange_points_r1<true>(p, F, level_args(p, p->bx[l], p->bx[p->l_stop], p->epsX, l), cb, false, vt, nrhs, accf, s, any);
+        tmp.drop(vt);
+        tmp.drop(ut);
+        any = true;
+    }
+    return any;
+}
+
+// All Lagrange levels of an apply, coarsest lo to finest hi.  Real kernels: u~ of level hi from the points, up to lo
 // through the children, every level's transfer, v~ down to hi, and from there to the points
 // (every target's accf is written).  False if the plan has no Lagrange level.
 bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Alloc &tmp, cudaStream_t s) {
+    if (p->kind == FFM_HELMHOLTZ) return far_lagrange_complex(p, q, nrhs, accf, tmp, s);
     int lo = -1, hi = -1;
     for (int l = 0; l <= p->l_stop; ++l)
         if (p->far[l].mode == 1 && p->far[l].n_adm > 0) {
@@ -1236,36 +1272,32 @@ bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Al
     if (lo < 0) return false;
     const FarLevel &F = p->far[hi];
     const int ls = p->l_stop, r = F.r1 * F.r1 * F.r1;
-    const bool cplx = p->kind == FFM_HELMHOLTZ, dl = p->kind == FFM_LAPLACE_DL, grad = p->kind == FFM_LAPLACE_GRAD;
+    const bool dl = p->kind == FFM_LAPLACE_DL, grad = p->kind == FFM_LAPLACE_GRAD;
     const Cheb cb = make_cheb(F.r1);
     void *ut[LMAX + 1], *vt[LMAX + 1];
-    const size_t val = sizeof(float) * (cplx ? 2 : 1);
     for (int l = lo; l <= hi; ++l) {
-        const size_t ub = val * (dl ? 3 : 1) * r * nrhs * (size_t)p->by[l].nb,
-                     vb = val * (grad ? 3 : 1) * r * nrhs * (size_t)p->bx[l].nb;
+        const size_t ub = sizeof(float) * (dl ? 3 : 1) * r * nrhs * (size_t)p->by[l].nb,
+                     vb = sizeof(float) * (grad ? 3 : 1) * r * nrhs * (size_t)p->bx[l].nb;
         ut[l] = tmp.raw(ub);
         vt[l] = tmp.raw(vb);
         if (l == hi) FFM_CUDA(cudaMemsetAsync(ut[l], 0, ub, s));
         FFM_CUDA(cudaMemsetAsync(vt[l], 0, vb, s));
     }
     const LevelArgs AY = level_args(p, p->by[hi], p->by[ls], p->epsY, hi), AX = level_args(p, p->bx[hi], p->bx[ls], p->epsX, hi);
-    if (cplx)
-        lagrange_points_r1<true>(p, F, AY, cb, true, q, nrhs, ut[hi], s);
-    else if (dl)
+    if (dl)
         lagrange_anterp_dl_r1(p, F, AY, cb, q, nrhs, ut[hi], s);
     else
         lagrange_points_r1<false>(p, F, AY, cb, true, q, nrhs, ut[hi], s);
     const Halves H = make_halves(F.r1);
     LinkArgs A{};
     A.nrhs = nrhs;
-    A.es = cplx ? 2 : 1;
     for (int l = hi - 1; l >= lo; --l) {
         A.n = p->by[l].nb;
         A.first_child = p->by[l].first_child;
         A.gc = p->by[l + 1].g;
-        A.rowlen = r * (dl ? 3 : cplx ? 2 : 1);
-        A.coff = dl ? r : cplx ? 1 : 0;
-        lag_link_r1(F.r1, A, dl ? 3 : cplx ? 2 : 1, H, true, (const float *)ut[l + 1], (float *)ut[l], s);
+        A.rowlen = r * (dl ? 3 : 1);
+        A.coff = dl ? r : 0;
+        lag_link_r1(F.r1, A, dl ? 3 : 1, H, true, (const float *)ut[l + 1], (float *)ut[l], s);
     }
     for (int l = lo; l <= hi; ++l)
         if (p->far[l].mode == 1 && p->far[l].n_adm > 0) lagrange_transfer(p, l, ut[l], nrhs, vt[l], tmp, s);
@@ -1273,20 +1305,16 @@ bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Al
         A.n = p->bx[l].nb;
         A.first_child = p->bx[l].first_child;
         A.gc = p->bx[l + 1].g;
-        A.rowlen = r * (cplx ? 2 : 1);
-        A.coff = cplx ? 1 : 0;
+        A.rowlen = r;
+        A.coff = 0;
         A.pbase = grad ? (int64_t)r * nrhs * p->bx[l].nb : 0;
         A.cbase = grad ? (int64_t)r * nrhs * p->bx[l + 1].nb : 0;
-        lag_link_r1(F.r1, A, grad ? 3 : cplx ? 2 : 1, H, false, (const float *)vt[l], (float *)vt[l + 1], s);
+        lag_link_r1(F.r1, A, grad ? 3 : 1, H, false, (const float *)vt[l], (float *)vt[l + 1], s);
     }
     // the gradient's three outputs per target, component-major like its accumulators
-    for (int d = 0; d < (grad ? 3 : 1); ++d) {
-        float2 *out = accf + (size_t)d * nrhs * p->nx;
-        if (cplx)
-            lagrange_points_r1<true>(p, F, AX, cb, false, vt[hi], nrhs, out, s);
-        else
-            lagrange_points_r1<false>(p, F, AX, cb, false, (float *)vt[hi] + (size_t)d * r * nrhs * p->bx[hi].nb, nrhs, out, s);
-    }
+    for (int d = 0; d < (grad ? 3 : 1); ++d)
+        lagrange_points_r1<false>(p, F, AX, cb, false, (float *)vt[hi] + (size_t)d * r * nrhs * p->bx[hi].nb, nrhs,
+                                  accf + (size_t)d * nrhs * p->nx, s);
     return true;
 }
 
@@ -2407,7 +2435,8 @@ __global__ void __launch_bounds__(PWB_NP + 32, 1) k_pw_backward_tc(PwArgs<float>
         for (int s = 0; s < nsteps && ok; ++s) {
             if (s >= PWB_NA) {
                 // the MMAs of step s - PWB_NA are done: its A and B stages are free; fill k is
-                // drained once the first step of fill k + 1 is done (see k_lag_gemm_ts)
+                // drained once the first step of fill k + 1 is done: the fill is then final, and the
+                // MMA thread has passed its wait for the drain of fill k - 1
                 const int sb = s - PWB_NA;
                 bool w_ok = mbar_wait(&s_empty[sb % PWB_NB], (uint32_t)((sb / PWB_NB) & 1), tries, err);
                 if (!__all_sync(0xffffffffu, w_ok)) {

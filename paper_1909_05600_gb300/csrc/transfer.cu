@@ -211,7 +211,7 @@ struct PairArgs {
     const __half *T;    // operator images
     float tinv;
     int nk, npad, tcols;
-    int parts;          // K parts of a unit's product, each added to v~ by itself
+    int part;           // chunks per accumulator fill (all of them but for complex operators)
     int ostride;        // floats between rows of v~
     int nout[PAIR_MAXBLK];
     int64_t ooff[PAIR_MAXBLK];  // first float of the block's columns in v~
@@ -237,6 +237,7 @@ struct PairArgs {
 //   warp 8      issues the MMAs into one of two TMEM accumulators
 //   warps 4-7   read the other accumulator, undo the scales and add it into v~: 32 columns at a
 //               time through shared memory, so that eight lanes add 128 consecutive bytes
+//               (complex operators: also warps 13-16, see SUM)
 // The MMAs of a K step are hi [hi; lo] (one operand of 2 npad rows, accumulated apart) and lo hi
 // up to 128 operator rows, else three of npad rows into one accumulator.
 // NSTG stages of CPS chunks are in flight: 4 of two at npad = 64 (48 KB each), 4 of one at 224 (45 KB).
@@ -247,8 +248,13 @@ struct PairArgs {
 // 256-pair tile, which split its FP32 rows into TF32 for every pair, no overlap of tiles): gradient
 // sphere 300k (r = 216, three operators) 6.54 -> 1.78 ms, Laplace volume 250k at 1e-4 (r = 216) 1.47 ->
 // 0.45, 100k x 8 right-hand sides (r = 64) 1.68 -> 0.41.  Complex operators (Helmholtz volume 120k at
-// 1e-4, 432 real rows), on CUDA cores before: 24.4 -> 1.9 ms.
-constexpr int PAIR_T = 416;
+// 1e-4, 432 real rows), on CUDA cores before: 24.4 -> 1.77 ms (1.91 with both halves of K scattered).
+constexpr int PAIR_T = 416, PAIR_TS = PAIR_T + 128;  // threads; with SUM
+// Chunks per accumulator fill of a complex operator.  With 1, 2, 4, 8 and 14 (all of K) the transfer of the Helmholtz
+// volume 120k at 1e-4 takes 3.02, 2.27, 1.77, 1.69 and 1.64 ms; the product of a plane-wave density in a volume of
+// 40k points (k = 3, 1e-4) is 2.7, 2.9, 3.7 and 5.1e-7 of the oracle's FFM for the first four.  FP32
+// multiply-adds on CUDA cores, with the basis constants of their time, took 24.4 ms and gave 6.1e-7.
+constexpr int PAIR_PART = 4;
 // Most translations of a level: the near offsets of the parents take at most four values per axis, their children's
 // at most nine, and the 64 offsets that stay near are none of them.
 constexpr int MAX_TRANS = 9 * 9 * 9 - 4 * 4 * 4;
@@ -256,12 +262,17 @@ constexpr int PAIR_IXW = 4;  // index warps
 constexpr int PAIR_IX = 4;   // units whose row numbers are held
 constexpr int PAIR_ST = 36;  // floats per row of the epilogue's staging (conflict-free float4)
 
-static size_t pair_smem(int nchunk, int npad, int n_trans) {
-    return 1024 + nchunk * (A_BYTES + (size_t)npad * HROW * 2) + 4 * 32 * PAIR_ST * sizeof(float) + sizeof(uint32_t) * ((size_t)n_trans + 1);
+static size_t pair_smem(int nchunk, int npad, int n_trans, bool sum) {
+    return 1024 + nchunk * (A_BYTES + (size_t)npad * HROW * 2) + (sum ? 8 : 4) * 32 * PAIR_ST * sizeof(float) +
+           sizeof(uint32_t) * ((size_t)n_trans + 1);
 }
 
-template <int NSTG, int CPS, bool STACK>
-__global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__ PairArgs A) {
+// SUM (complex operators): a tensor-core accumulation truncates at every step, so hi hi is accumulated over
+// A.part chunks only; the epilogue adds the fills of a unit in FP32 registers, rounded to nearest, and
+// scatters the unit once.  Two warps per lane quarter (4-7 and 13-16) then take half of the columns each.
+template <int NSTG, int CPS, bool STACK, bool SUM>
+__global__ void __launch_bounds__(SUM ? PAIR_TS : PAIR_T, 1) k_lag_pairs(const __grid_constant__ PairArgs A) {
+    constexpr int T = SUM ? PAIR_TS : PAIR_T, EPW = SUM ? 8 : 4;  // threads, epilogue warps
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = aligned_smem(smem_raw);
     __shared__ __align__(8) uint64_t s_full[NSTG], s_empty[NSTG], s_accfull[2], s_accempty[2], s_done;
@@ -270,13 +281,13 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
     __shared__ uint32_t s_dst[PAIR_IX][HM];  // row of v~
     __shared__ float s_inv[PAIR_IX][HM];
     __shared__ int s_trans[PAIR_IX];
-    __shared__ uint32_t s_tmem, s_carry, s_cmax, s_w[PAIR_T / 32];
+    __shared__ uint32_t s_tmem, s_carry, s_cmax, s_w[T / 32];
     constexpr uint32_t NONE = 0xffffffffu;
     __shared__ int s_bad;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t bbytes = (uint32_t)A.npad * HROW * 2 * CPS, stage = CPS * A_BYTES + bbytes;
     float *stag = reinterpret_cast<float *>(smem + (size_t)NSTG * stage);
-    uint32_t *pre = reinterpret_cast<uint32_t *>(stag + 4 * 32 * PAIR_ST);  // tiles before translation t
+    uint32_t *pre = reinterpret_cast<uint32_t *>(stag + EPW * 32 * PAIR_ST);  // tiles before translation t
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
                      "r"(2 * A.tcols));
@@ -292,11 +303,11 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s_accfull[i], 1);
-            mbar_init(&s_accempty[i], 4);
+            mbar_init(&s_accempty[i], EPW);
         }
         for (int i = 0; i < PAIR_IX; ++i) {
             mbar_init(&s_ixfull[i], 1);
-            mbar_init(&s_ixempty[i], 8);
+            mbar_init(&s_ixempty[i], 4 + EPW);
         }
         mbar_init(&s_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -305,7 +316,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
     __syncthreads();
     tc_fence_after();
     // tiles of every translation, prefix sums
-    for (int t0 = 0; t0 < A.n_trans; t0 += PAIR_T) {
+    for (int t0 = 0; t0 < A.n_trans; t0 += T) {
         const int t = t0 + tid;
         uint32_t c = 0;
         if (t < A.n_trans) c = (uint32_t)(((uint64_t)(A.bt_off[t + 1] - A.bt_off[t]) * A.nrhs + HM - 1) / HM);
@@ -320,21 +331,17 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         for (int w = 0; w < warp; ++w) before += s_w[w];
         if (t < A.n_trans) pre[t] = before + inc - c;
         __syncthreads();
-        if (tid == PAIR_T - 1) s_carry = before + inc;
+        if (tid == T - 1) s_carry = before + inc;
         __syncthreads();
     }
     if (tid == 0) pre[A.n_trans] = s_carry;
     __syncthreads();
     const uint32_t tmem = s_tmem;
-    const int per = A.nblk * A.parts;  // units of a tile: (row block, K part)
-    const int64_t units = (int64_t)s_carry * per;
-    // row block, first and end chunk of unit un
-    auto block_of = [&](int64_t un) { return (int)(un % per) / A.parts; };
-    auto k_first = [&](int64_t un) { return (int)(un % A.parts) * A.nk / A.parts; };
-    auto k_end = [&](int64_t un) { return ((int)(un % A.parts) + 1) * A.nk / A.parts; };
+    const int64_t units = (int64_t)s_carry * A.nblk;
+    auto block_of = [&](int64_t un) { return (int)(un % A.nblk); };  // row block of unit un
     // translation, first row and row count of the tile of unit un
     auto locate = [&](int64_t un, int &t, uint32_t &p0, uint64_t &row0, int &nrows) {
-        const uint32_t tile = (uint32_t)(un / per);
+        const uint32_t tile = (uint32_t)(un / A.nblk);
         int lo = 0, hi = A.n_trans;  // last t with pre[t] <= tile
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -350,7 +357,7 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
         nrows = (int)min((uint64_t)HM, all - row0);
     };
     bool ok = true;
-    if (warp > 8) {
+    if (warp > 8 && warp < 9 + PAIR_IXW) {
         // ---- row numbers: warp w takes units w - 9, w - 9 + PAIR_IXW, ... of this block
         uint32_t i = warp - 9;
         for (int64_t un = blockIdx.x + (int64_t)i * gridDim.x; un < units; un += (int64_t)PAIR_IXW * gridDim.x, i += PAIR_IXW) {
@@ -405,19 +412,19 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
                 ok = false;
                 break;
             }
-            const int t = s_trans[ix], blk = block_of(un), k0 = k_first(un), k1 = k_end(un);
+            const int t = s_trans[ix], blk = block_of(un);
             const __half *src[8];
             uint32_t bytes[8];
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 const uint32_t row = s_src[ix][r0 + 4 * g];
                 bytes[g] = row != NONE ? 16u : 0u;
-                src[g] = A.u + ((size_t)(row != NONE ? row : 0u) * A.nk + k0) * HROW + sg * 8;
+                src[g] = A.u + (size_t)(row != NONE ? row : 0u) * A.nk * HROW + sg * 8;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_ixempty[ix]);
             const __half *Tb = A.T + ((size_t)t * A.nblk + blk) * A.nk * A.npad * HROW;
-            for (int kc = k0; kc < k1; kc += CPS, ++c) {
+            for (int kc = 0; kc < A.nk; kc += CPS, ++c) {
                 const uint32_t slot = c % NSTG;
                 const bool w_ok = c < NSTG || mbar_wait(&s_empty[slot], ((c / NSTG) - 1) & 1, A.tries, A.err);
                 if (!__all_sync(0xffffffffu, w_ok)) {
@@ -461,44 +468,46 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
             // ---- MMA thread
             const uint32_t id1 = idesc_f16(A.npad), id2 = STACK ? idesc_f16(2 * A.npad) : id1;
             const uint32_t alo = a_dlo(smem_addr(smem)), blo = b_dlo(smem_addr(smem) + CPS * A_BYTES);
-            uint32_t i = 0, slot = 0, par = 0;
-            for (int64_t un = blockIdx.x; un < units && ok; un += gridDim.x, ++i) {
-                const uint32_t buf = i & 1;
-                if (i >= 2 && !mbar_wait(&s_accempty[buf], ((i >> 1) - 1) & 1, A.tries, A.err)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t d = tmem + buf * (uint32_t)A.tcols;
-                const int k0 = k_first(un), k1 = k_end(un);
-                for (int kc = k0; kc < k1; kc += CPS) {
-                    if (!mbar_wait(&s_full[slot], par, A.tries, A.err)) {
+            uint32_t f = 0, slot = 0, par = 0;  // accumulator fills
+            for (int64_t un = blockIdx.x; un < units && ok; un += gridDim.x) {
+                for (int k0 = 0; k0 < A.nk && ok; k0 += A.part, ++f) {
+                    const uint32_t buf = f & 1;
+                    if (f >= 2 && !mbar_wait(&s_accempty[buf], ((f >> 1) - 1) & 1, A.tries, A.err)) {
                         ok = false;
                         break;
                     }
-                    fence_proxy_async();  // the rows came by cp.async, through the generic proxy
-                    tc_fence_after();
-                    const uint32_t off = slot * (stage >> 4);
-                    stage_mma<CPS, STACK>(d, alo + off, blo + off, (uint32_t)A.npad, id1, id2, kc == k0);
-                    tc_commit(&s_empty[slot]);
-                    if (++slot == NSTG) {
-                        slot = 0;
-                        par ^= 1;
+                    const uint32_t d = tmem + buf * (uint32_t)A.tcols;
+                    const int k1 = min(k0 + A.part, A.nk);
+                    for (int kc = k0; kc < k1; kc += CPS) {
+                        if (!mbar_wait(&s_full[slot], par, A.tries, A.err)) {
+                            ok = false;
+                            break;
+                        }
+                        fence_proxy_async();  // the rows came by cp.async, through the generic proxy
+                        tc_fence_after();
+                        const uint32_t off = slot * (stage >> 4);
+                        stage_mma<CPS, STACK>(d, alo + off, blo + off, (uint32_t)A.npad, id1, id2, kc == k0);
+                        tc_commit(&s_empty[slot]);
+                        if (++slot == NSTG) {
+                            slot = 0;
+                            par ^= 1;
+                        }
                     }
+                    if (ok) tc_commit(&s_accfull[buf]);
                 }
-                if (ok) tc_commit(&s_accfull[buf]);
             }
             // everything issued is done before the block gives up its shared memory and TMEM
             tc_commit(&s_done);
             mbar_wait(&s_done, 0, DRAIN_TRIES);
         }
     } else {
-        // ---- epilogue: warp w reads lanes 32 (w - 4) .. + 31
-        const int q = warp - 4;
-        float *st = stag + q * 32 * PAIR_ST;
+        // ---- epilogue: warp w reads lanes 32 (w % 4) .. + 31
+        const int q = warp & 3;
+        float *st = stag + (q + (warp > 8 ? 4 : 0)) * 32 * PAIR_ST;
         const bool vec = (A.ostride & 3) == 0;
-        uint32_t i = 0;
-        for (int64_t un = blockIdx.x; un < units; un += gridDim.x, ++i) {
-            const uint32_t buf = i & 1, ix = i % PAIR_IX;
+        uint32_t i = 0, f = 0;  // units, accumulator fills
+        for (int64_t un = blockIdx.x; un < units && ok; un += gridDim.x, ++i) {
+            const uint32_t ix = i % PAIR_IX;
             const int blk = block_of(un), nout = A.nout[blk];
             const bool i_ok = mbar_wait(&s_ixfull[ix], (i / PAIR_IX) & 1, A.tries, A.err);
             if (!__all_sync(0xffffffffu, i_ok)) {
@@ -511,61 +520,106 @@ __global__ void __launch_bounds__(PAIR_T, 1) k_lag_pairs(const __grid_constant__
             // rows of this warp with pairs (a prefix)
             const int mine = __popc(__ballot_sync(0xffffffffu, s_src[ix][32 * q + lane] != NONE));
             if (lane == 0) mbar_arrive(&s_ixempty[ix]);
-            const bool w_ok = mbar_wait(&s_accfull[buf], (i >> 1) & 1, A.tries, A.err);
-            if (!__all_sync(0xffffffffu, w_ok)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t d = tmem + buf * (uint32_t)A.tcols + ((uint32_t)(32 * q) << 16);
             float *out = A.vt + A.ooff[blk];
-            if (mine > 0) {
-                for (int c0 = 0; c0 < nout; c0 += 32) {
+            // the staged columns c0 .. c0 + 31 of the block into v~
+            auto scatter = [&](int c0) {
+                __syncwarp();
+                if (vec) {
+                    const int col = c0 + (lane & 7) * 4;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int cc = c0 + 16 * h;
-                        if (cc >= A.npad) break;
-                        uint32_t v[16], w[16];
-                        tmem_ld16(v, d + (uint32_t)cc);
-                        if constexpr (STACK) tmem_ld16(w, d + (uint32_t)(A.npad + cc));
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            float x[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                float y = __uint_as_float(v[4 * k + j]);
-                                if constexpr (STACK) y += __uint_as_float(w[4 * k + j]);
-                                x[j] = y * f1 * f2;
-                            }
-                            *reinterpret_cast<float4 *>(st + lane * PAIR_ST + 16 * h + 4 * k) =
-                                make_float4(x[0], x[1], x[2], x[3]);
-                        }
+                    for (int it = 0; it < 8; ++it) {
+                        const int row = it * 4 + (lane >> 3);
+                        const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
+                        if (row < mine && col < nout)
+                            atomicAdd(reinterpret_cast<float4 *>(out + (size_t)dr * A.ostride + col),
+                                      *reinterpret_cast<const float4 *>(st + row * PAIR_ST + (lane & 7) * 4));
                     }
-                    __syncwarp();
-                    if (vec) {
-                        const int col = c0 + (lane & 7) * 4;
-#pragma unroll
-                        for (int it = 0; it < 8; ++it) {
-                            const int row = it * 4 + (lane >> 3);
-                            const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
-                            if (row < mine && col < nout)
-                                atomicAdd(reinterpret_cast<float4 *>(out + (size_t)dr * A.ostride + col),
-                                          *reinterpret_cast<const float4 *>(st + row * PAIR_ST + (lane & 7) * 4));
-                        }
-                    } else {
-                        for (int row = 0; row < mine; ++row) {
-                            const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
-                            if (c0 + lane < nout)
-                                atomicAdd(out + (size_t)dr * A.ostride + c0 + lane, st[row * PAIR_ST + lane]);
-                        }
+                } else {
+                    for (int row = 0; row < mine; ++row) {
+                        const uint32_t dr = __shfl_sync(0xffffffffu, drow, row);
+                        if (c0 + lane < nout)
+                            atomicAdd(out + (size_t)dr * A.ostride + c0 + lane, st[row * PAIR_ST + lane]);
                     }
-                    __syncwarp();
                 }
+                __syncwarp();
+            };
+            auto fill_ready = [&] {
+                const bool w_ok = mbar_wait(&s_accfull[f & 1], (f >> 1) & 1, A.tries, A.err);
+                ok = __all_sync(0xffffffffu, w_ok);
+                tc_fence_after();
+                return ok;
+            };
+            auto fill_done = [&] {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&s_accempty[f & 1]);
+                ++f;
+            };
+            if constexpr (SUM) {
+                const int cb = warp > 8 ? 64 : 0;  // first column of this warp
+                float sum[64];
+#pragma unroll
+                for (int c = 0; c < 64; ++c) sum[c] = 0.f;
+                for (int k0 = 0; k0 < A.nk; k0 += A.part) {
+                    if (!fill_ready()) break;
+                    const uint32_t d = tmem + (f & 1) * (uint32_t)A.tcols + ((uint32_t)(32 * q) << 16) + (uint32_t)cb;
+                    if (mine > 0) {
+#pragma unroll
+                        for (int c0 = 0; c0 < 64; c0 += 16) {
+                            if (cb + c0 < A.npad) {
+                                uint32_t v[16], w[16];
+                                tmem_ld16(v, d + (uint32_t)c0);
+                                tmem_ld16(w, d + (uint32_t)(A.npad + c0));
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) sum[c0 + j] += __uint_as_float(v[j]) + __uint_as_float(w[j]);
+                            }
+                        }
+                    }
+                    fill_done();
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += 32)
+                    if (mine > 0 && cb + c0 < nout) {
+#pragma unroll
+                        for (int k = 0; k < 32; k += 4)
+                            *reinterpret_cast<float4 *>(st + lane * PAIR_ST + k) =
+                                make_float4(sum[c0 + k] * f1 * f2, sum[c0 + k + 1] * f1 * f2, sum[c0 + k + 2] * f1 * f2,
+                                            sum[c0 + k + 3] * f1 * f2);
+                        scatter(cb + c0);
+                    }
+            } else {
+                if (!fill_ready()) break;
+                const uint32_t d = tmem + (f & 1) * (uint32_t)A.tcols + ((uint32_t)(32 * q) << 16);
+                if (mine > 0) {
+                    for (int c0 = 0; c0 < nout; c0 += 32) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int cc = c0 + 16 * h;
+                            if (cc >= A.npad) break;
+                            uint32_t v[16], w[16];
+                            tmem_ld16(v, d + (uint32_t)cc);
+                            if constexpr (STACK) tmem_ld16(w, d + (uint32_t)(A.npad + cc));
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                float x[4];
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    float y = __uint_as_float(v[4 * k + j]);
+                                    if constexpr (STACK) y += __uint_as_float(w[4 * k + j]);
+                                    x[j] = y * f1 * f2;
+                                }
+                                *reinterpret_cast<float4 *>(st + lane * PAIR_ST + 16 * h + 4 * k) =
+                                    make_float4(x[0], x[1], x[2], x[3]);
+                            }
+                        }
+                        scatter(c0);
+                    }
+                }
+                fill_done();
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&s_accempty[buf]);
         }
     }
     if (!ok) atomicOr(&s_bad, 1);
@@ -586,10 +640,7 @@ void build_operator_image(ffm_plan_s *p, int l, const LagGeo &geo, cudaStream_t 
     const bool cplx = p->kind == FFM_HELMHOLTZ;
     const int r = F.r1 * F.r1 * F.r1, rk = p->kind == FFM_LAPLACE_DL ? 3 * r : r;
     const int rows = cplx ? 2 * r : r, K = cplx ? 2 * rk : rk, ncomp = p->kind == FFM_LAPLACE_GRAD ? 3 : 1;
-    // Complex levels: at most 128 rows, so that hi hi has an accumulator of its own, and K parts of at most
-    // eight chunks (lag_pairs).  A tensor-core accumulation truncates at every step; with one accumulator
-    // for the three products over the whole K = 432 the Helmholtz parity case (cube surface, k = 12) went from 3.1e-7
-    // (FP32 multiply-adds) to 1.03e-6 of the oracle's FFM.
+    // Complex levels: at most 128 rows, so that hi hi has an accumulator of its own (k_lag_pairs, SUM).
     F.h_bpc = cdiv(rows, cplx ? 128 : 256);
     F.h_nb = ((int)cdiv(rows, F.h_bpc) + 15) / 16 * 16;
     F.h_nk = cdiv(K, HK);
@@ -626,12 +677,12 @@ void build_operator_image(ffm_plan_s *p, int l, const LagGeo &geo, cudaStream_t 
 // plans: it is set to the largest size of the instance (operator rows NPAD, translations MAX_TRANS), so
 // that no thread lowers it between another's setting and launch.  Per device and cheap: set before every
 // launch (plans may live on several devices).
-template <int NSTG, int CPS, bool STACK, int NPAD>
+template <int NSTG, int CPS, bool STACK, int NPAD, bool SUM = false>
 static void launch_pairs(const PairArgs &A, unsigned grid, cudaStream_t s) {
-    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG, CPS, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)pair_smem(NSTG * CPS, NPAD, MAX_TRANS)));
-    FFM_LAUNCH_NAMED("k_lag_pairs", (k_lag_pairs<NSTG, CPS, STACK>), grid, PAIR_T,
-                     pair_smem(NSTG * CPS, A.npad, A.n_trans), s, A);
+    FFM_CUDA(cudaFuncSetAttribute(k_lag_pairs<NSTG, CPS, STACK, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)pair_smem(NSTG * CPS, NPAD, MAX_TRANS, SUM)));
+    FFM_LAUNCH_NAMED("k_lag_pairs", (k_lag_pairs<NSTG, CPS, STACK, SUM>), grid, SUM ? PAIR_TS : PAIR_T,
+                     pair_smem(NSTG * CPS, A.npad, A.n_trans, SUM), s, A);
 }
 
 // v~ += T u~ for all pairs of the level: u has rows of K floats per (source box, right-hand side),
@@ -658,7 +709,7 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.T = (const __half *)F.Th;
     A.tinv = F.h_inv;
     A.nk = F.h_nk;
-    A.parts = cplx ? cdiv(F.h_nk, 8) : 1;
+    A.part = cplx ? PAIR_PART : F.h_nk;
     A.npad = F.h_nb;
     const bool stack = A.npad <= 128;
     A.tcols = 32;
@@ -673,10 +724,12 @@ void lag_pairs(const ffm_plan_s *p, int l, const float *u, int nrhs, float *vt, 
     A.vt = vt;
     A.err = p->dev_err;
     A.tries = p->wait_tries;
-    const int64_t most = ((int64_t)F.n_trans + F.n_adm * nrhs / HM) * A.nblk * A.parts;  // at least the number of units
+    const int64_t most = ((int64_t)F.n_trans + F.n_adm * nrhs / HM) * A.nblk;  // at least the number of units
     const unsigned grid = (unsigned)std::min<int64_t>(most, 152);
     // stages of two chunks where the K extent allows: half the barrier round trips
-    if (A.npad <= 64 && A.nk % 2 == 0)
+    if (cplx)
+        launch_pairs<5, 1, true, 128, true>(A, grid, s);
+    else if (A.npad <= 64 && A.nk % 2 == 0)
         launch_pairs<4, 2, true, 64>(A, grid, s);
     else if (A.npad <= 64)
         launch_pairs<8, 1, true, 64>(A, grid, s);
