@@ -13,7 +13,8 @@
  * test of Sec. 2.2.2, far fields by Chebyshev-Lagrange interpolation (Sec. 2.2.2) or by
  * the Gegenbauer plane-wave expansion (Sec. 2.2.3), and a dense near field at the level
  * where the stopping criterion of Sec. 2.2.4 holds.  Pairs of coincident points
- * (|x-y| = 0) contribute nothing.
+ * (|x-y| = 0) contribute nothing.  Where the two sets' root cubes differ, that goes for pairs closer than the
+ * arithmetic resolves: 4 (2^-52 (d0 + largest coordinate) + 2^-46 (offset of the cubes + leaf edge)).
  *
  * Every step runs in CUDA kernels on the current device; no CPU fallback exists.
  *

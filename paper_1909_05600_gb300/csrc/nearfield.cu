@@ -29,7 +29,26 @@ struct NearArgs {
     float dls_h, dls_l;                   // leaf edge as an unevaluated FP32 pair
     float oyx_h[3], oyx_l[3];             // oY - oX, likewise
     float k;
+    float mtau2;                          // -tau^2, see coincidence_radius
 };
+
+constexpr float FLT_NORMAL = 1.17549435e-38f;  // the smallest normal number: below it rsqrt_hw gives +inf
+
+// Radius within which two points count as coincident, 0 where the two root cubes are the same.  A point of both sets then
+// lies in the same leaf of the same grid twice, and its difference is an exact zero.  With cubes that
+// differ it is the difference of two leaf-relative pairs with different roundings: FP64 roundings of the points' offsets
+// (2^-53 of the coordinates and of the cube's edge) and of the offset between the cubes and the leaves in FP32 pairs
+// (about 2^-47 of it).  tau is four times that (the largest of 8e6 random coincident pairs was 0.28 tau);
+// distances below it are rounding errors, and 1 / them counted as a pair of 1e14.
+static double coincidence_radius(const ffm_plan_s *p, double dls) {
+    double a = 0, m = 0;
+    for (int d = 0; d < 3; ++d) {
+        a = std::max(a, std::fabs(p->oY[d] - p->oX[d]));
+        for (double o : {p->oX[d], p->oY[d]}) m = std::max(m, std::max(std::fabs(o), std::fabs(o + p->d0)));
+    }
+    if (a == 0) return 0;
+    return 4 * (std::ldexp(p->d0 + m, -52) + std::ldexp(a + dls, -46));
+}
 
 // y (hi + lo, own leaf frame) plus the leaf-centre offset (oh + ol): an FP32 TwoSum of the
 // hi parts, the lo parts added to the rounding error.
@@ -108,8 +127,8 @@ __device__ __forceinline__ float dot_pair(float4 xh, float4 xl, float4 yh, float
 
 template <int KIND, int PT>
 __device__ __forceinline__ void interact(const float4 *sA, const float4 *sB, const float4 *sC, int j0, int j1,
-                                         const float4 *xh, const float4 *xl, float k, float *sr, float *si,
-                                         float *sz) {
+                                         const float4 *xh, const float4 *xl, float k, float mtau2, float *sr,
+                                         float *si, float *sz) {
 #pragma unroll 2
     for (int j = j0; j < j1; ++j) {
         float4 y = sA[j];
@@ -119,8 +138,8 @@ __device__ __forceinline__ void interact(const float4 *sA, const float4 *sB, con
             float dx = (xh[t].x - y.x) + (xl[t].x - yl.x);
             float dy = (xh[t].y - y.y) + (xl[t].y - yl.y);
             float dz = (xh[t].z - y.z) + (xl[t].z - yl.z);
-            float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            float inv = r2 > 0.f ? rsqrt_hw(r2) : 0.f;  // coincident points contribute nothing
+            float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, mtau2)));
+            float inv = r2 >= FLT_NORMAL ? rsqrt_hw(r2) : 0.f;  // coincident points contribute nothing
             if constexpr (KIND == NF_DOUBLE_LAYER) {
                 // (w u n) . (x - y) / |x - y|^3; for points of one surface the dot product
                 // is second order in |x - y|, so it is formed from x - y and q as FP32 pairs
@@ -220,14 +239,14 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(NearArgs N, const void *__restric
             if (fill == P2P_SB) {
                 __syncthreads();
                 if (active)
-                    interact<KIND, PT>(sA, sB, sC, grp * fill / G, (grp + 1) * fill / G, xh, xl, N.k, sr, si, sz);
+                    interact<KIND, PT>(sA, sB, sC, grp * fill / G, (grp + 1) * fill / G, xh, xl, N.k, N.mtau2, sr, si, sz);
                 __syncthreads();
                 fill = 0;
             }
         }
     }
     __syncthreads();
-    if (active) interact<KIND, PT>(sA, sB, sC, grp * fill / G, (grp + 1) * fill / G, xh, xl, N.k, sr, si, sz);
+    if (active) interact<KIND, PT>(sA, sB, sC, grp * fill / G, (grp + 1) * fill / G, xh, xl, N.k, N.mtau2, sr, si, sz);
 #pragma unroll
     for (int t = 0; t < PT; ++t) red[threadIdx.x * PT + t] = make_float4(sr[t], si[t], sz[t], 0.f);
     __syncthreads();
@@ -269,9 +288,10 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(NearArgs N, const void *__restric
 // target's accumulator pair: 6.5 issue slots of FP32 arithmetic (13 FP32 operations) and one
 // special-function result per pair, against about 17 issue slots in the generic kernel.
 //
-// Coincident points: rsqrt of 0 is +inf, which makes the target's accumulator non-finite.
-// Each thread checks its accumulators after every batch and recomputes that batch for the
-// affected target with the pair test (pairs with |x - y|^2 below the smallest normal FP32
+// Coincident points: -tau^2 in the innermost multiply-add (where a multiply stood) leaves 0 or less, whose rsqrt
+// is +inf or NaN and makes the target's accumulator non-finite.  It changes no other pair: tau is at most 4e-9
+// of a leaf's edge at level 15.  (The third operand takes the kernel from 65.5 to 66.1 ms at 10M clustered points.)  Each thread checks its accumulators after every batch and recomputes that batch for the
+// affected target with the pair test (pairs with |x - y|^2 - tau^2 below the smallest normal FP32
 // number contribute nothing, as in the generic kernel), starting again from the value it
 // had before the batch.
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
@@ -290,11 +310,6 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
 __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
     uint64_t r;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
 __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
@@ -320,24 +335,24 @@ struct LapStage {
 // Two pairs (sources a, b of one quad half) for one target: acc += w / |x - y| in both halves.
 template <bool GUARD>
 __device__ __forceinline__ uint64_t lap_two(const Tgt2 &x, const uint64_t *yh, const uint64_t *yl, uint64_t w,
-                                            uint64_t acc) {
+                                            uint64_t mtau2, uint64_t acc) {
     uint64_t d[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) d[c] = f2_add(f2_sub(x.h[c], yh[c]), f2_sub(x.l[c], yl[c]));
-    uint64_t r2 = f2_fma(d[2], d[2], f2_fma(d[1], d[1], f2_mul(d[0], d[0])));
+    uint64_t r2 = f2_fma(d[2], d[2], f2_fma(d[1], d[1], f2_fma(d[0], d[0], mtau2)));
     float ra, rb;
     f2_unpack(r2, ra, rb);
     float ia = rsqrt_hw(ra), ib = rsqrt_hw(rb);
     if constexpr (GUARD) {
-        ia = ra >= 1.17549435e-38f ? ia : 0.f;
-        ib = rb >= 1.17549435e-38f ? ib : 0.f;
+        ia = ra >= FLT_NORMAL ? ia : 0.f;
+        ib = rb >= FLT_NORMAL ? ib : 0.f;
     }
     return f2_fma(w, f2_pack(ia, ib), acc);
 }
 
 template <bool GUARD, int PT>
 __device__ __forceinline__ void lap_quads(const LapStage &S, int q0, int q1, int qstep, const Tgt2 *X,
-                                          uint64_t *acc) {
+                                          uint64_t mtau2, uint64_t *acc) {
 #pragma unroll 1
     for (int q = q0; q < q1; q += qstep) {
         float4 v[7];
@@ -354,8 +369,8 @@ __device__ __forceinline__ void lap_quads(const LapStage &S, int q0, int q1, int
         uint64_t wa = f2_pack(v[6].x, v[6].y), wb = f2_pack(v[6].z, v[6].w);
 #pragma unroll
         for (int t = 0; t < PT; ++t) {
-            acc[t] = lap_two<GUARD>(X[t], ha, la, wa, acc[t]);
-            acc[t] = lap_two<GUARD>(X[t], hb, lb, wb, acc[t]);
+            acc[t] = lap_two<GUARD>(X[t], ha, la, wa, mtau2, acc[t]);
+            acc[t] = lap_two<GUARD>(X[t], hb, lb, wb, mtau2, acc[t]);
         }
     }
 }
@@ -377,6 +392,7 @@ __global__ void __launch_bounds__(P2P_T) k_p2p_lap(NearArgs N, const float *__re
     int4 ga = N.xl_g[a];
     Tgt2 X[PT];
     uint64_t A[PT];
+    const uint64_t mtau2 = f2_pack(N.mtau2, N.mtau2);
 #pragma unroll
     for (int t = 0; t < PT; ++t) {
         int i = pi + t * pr;
@@ -410,14 +426,14 @@ __global__ void __launch_bounds__(P2P_T) k_p2p_lap(NearArgs N, const float *__re
             uint64_t save[PT];
 #pragma unroll
             for (int t = 0; t < PT; ++t) save[t] = A[t];
-            lap_quads<false, PT>(S, grp, nq, G, X, A);
+            lap_quads<false, PT>(S, grp, nq, G, X, mtau2, A);
 #pragma unroll
             for (int t = 0; t < PT; ++t) {
                 float u0, u1;
                 f2_unpack(A[t], u0, u1);
                 if (!isfinite(u0 + u1)) {  // a coincident pair: this batch again with the pair test
                     uint64_t one[1] = {save[t]};
-                    lap_quads<true, 1>(S, grp, nq, G, &X[t], one);
+                    lap_quads<true, 1>(S, grp, nq, G, &X[t], mtau2, one);
                     A[t] = one[0];
                 }
             }
@@ -586,8 +602,8 @@ __global__ void __launch_bounds__(P2P_T) k_p2p_mr(NearArgs N, const void *__rest
                         float dx = (x.x - y.x) + (xl.x - y.w);
                         float dy = (x.y - y.y) + (xl.y - yl2.x);
                         float dz = (x.z - y.z) + (xl.z - yl2.y);
-                        float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        float inv = r2 > 0.f ? rsqrt_hw(r2) : 0.f;
+                        float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, N.mtau2)));
+                        float inv = r2 >= FLT_NORMAL ? rsqrt_hw(r2) : 0.f;
                         float gr = inv, gi = 0.f;
                         if constexpr (HELM) {
                             float ph = N.k * (r2 * inv);
@@ -656,6 +672,8 @@ void near_field_items(const ffm_plan_s *p, const int4 *items, int64_t n_items, i
         N.oyx_l[d] = (float)(o - (double)N.oyx_h[d]);
     }
     N.k = (float)p->k;
+    const double tau = coincidence_radius(p, dls);
+    N.mtau2 = -(float)(tau * tau);
     if (p->kind == FFM_LAPLACE_DL) {
         dim3 g((unsigned)n_items, nrhs);
         FFM_LAUNCH(k_p2p<NF_DOUBLE_LAYER>, g, P2P_T, 0, s, N, q, p->ny, nrhs, p->nx, acc);
