@@ -101,11 +101,14 @@ std::string near_key(const ffm_plan_s *p, const std::string &dev, int rhsb) {
     return key;
 }
 
+// The kernel's kind decides the operators' shape (K = 3 r for the double layer, three operators for the gradient), and
+// LAG_GENERATION which kernels the times are of: raised when a candidate is replaced (2: f16 operands).
+constexpr int LAG_GENERATION = 2;
 std::string lag_key(const ffm_plan_s *p, int l, const std::string &dev, int rhsb) {
     const FarLevel &F = p->far[l];
     char key[320];
-    snprintf(key, sizeof key, "lag %s r1=%d rhs=%d adm=%d trans=%d", dev.c_str(), F.r1, rhsb, lg2((double)F.n_adm),
-             lg2((double)F.n_trans));
+    snprintf(key, sizeof key, "lag %s gen=%d kind=%d r1=%d rhs=%d adm=%d trans=%d", dev.c_str(), LAG_GENERATION, p->kind,
+             F.r1, rhsb, lg2((double)F.n_adm), lg2((double)F.n_trans));
     return key;
 }
 
@@ -157,7 +160,7 @@ TunePicks read_tune_picks(const char *path) {
 }
 
 int cached_lag_pick(const ffm_plan_s *p, int l) {
-    if (p->tune_picks.empty()) return -1;
+    if (p->tune_picks.empty() || p->kind == FFM_HELMHOLTZ) return -1;  // complex levels have nothing to pick
     std::string v;
     int a = -1;
     if (find_pick(p->tune_picks, lag_key(p, l, device_tag(), 1), v) && parse_lag(v, a)) return a;

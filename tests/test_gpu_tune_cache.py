@@ -1,6 +1,7 @@
 """A plan reads its autotune cache once, so that all its decisions rest on the same contents whatever happens to
 the file meanwhile: here a named pipe, whose first reader gets the picks and every later one nothing."""
 import os
+import re
 import threading
 import time
 
@@ -25,6 +26,32 @@ def _tuned(X, kernel, u, path, pick, **kw):
     assert any(ln.startswith("lag ") for ln in lines)
     path.write_text("\n".join(lines) + "\n")
     return v.double()
+
+
+def test_picks_belong_to_a_kernel_and_to_its_kernels_generation(tmp_path):
+    X = torch.as_tensor(W.cube_volume(20000, 1), device="cuda")
+    u = torch.ones(20000, device="cuda")
+    path = tmp_path / "picks"
+    _tuned(X, ffm.LAPLACE, u, path, 0, r1_override=4)
+    lines = path.read_text()
+    levels = lambda p: [p.info()["tune_tc"][l] for l in range(22) if p.info()["n_adm"][l]]
+    with ffm.Plan(X, X, ffm.LAPLACE, 0.0, 1e-3, r1_override=4, autotune_cache=str(path)) as p:
+        assert levels(p) and not any(levels(p))
+    for kernel, kw in ((ffm.LAPLACE_GRAD, {}), (ffm.LAPLACE_DL, dict(normals=X))):
+        with ffm.Plan(X, X, kernel, 0.0, 1e-3, r1_override=4, autotune_cache=str(path), **kw) as p:
+            assert levels(p) and all(levels(p))
+    # a pick timed on earlier kernels (keys without kind and generation)
+    path.write_text(re.sub(r" gen=\d+ kind=\d+", "", lines))
+    with ffm.Plan(X, X, ffm.LAPLACE, 0.0, 1e-3, r1_override=4, autotune_cache=str(path)) as p:
+        assert all(levels(p))
+    # complex levels have no pick, and build nothing for one
+    path.write_text("".join(ln.replace("kind=0", "kind=1") + "\n" for ln in lines.splitlines() if ln.startswith("lag ")))
+    size = []
+    for cache in (None, str(path)):
+        with ffm.Plan(X, X, ffm.HELMHOLTZ, 1.0, 1e-3, r1_override=4, kappa_switch=1e9, autotune_cache=cache) as p:
+            size.append(p.bytes())
+            assert all(levels(p))
+    assert size[0] == size[1]
 
 
 @pytest.mark.parametrize("pick", [0, 1, 2])
