@@ -829,7 +829,12 @@ __global__ void __launch_bounds__(LV_T) k_level_sums(const __grid_constant__ Lev
     }
     __shared__ unsigned long long sm[32], t;
     block_excl_scan64(a, sm, &t);
-    if (threadIdx.x == 0 && X) A.ta[tile] = t;
+    if (threadIdx.x == 0 && X) {
+        A.ta[tile] = t;
+        // the totals, each kind by itself: the scan's packed sums hold only 32 bits of each
+        atomicAdd(&A.tot->na, t >> 32);
+        atomicAdd(&A.tot->nn, t & 0xffffffffull);
+    }
     __syncthreads();
     block_excl_scan64(b, sm, &t);
     if (threadIdx.x == 0) A.tb[blockIdx.x] = t;
@@ -855,18 +860,6 @@ __global__ void __launch_bounds__(1024) k_level_mid(const __grid_constant__ Leve
         }
         return carry;
     };
-    // the pairs of all tiles, each kind by itself: the packed sums of the scan hold only 32 bits of each
-    unsigned long long na = 0, nn = 0;
-    for (int64_t i = threadIdx.x; i < A.ntx; i += 1024) {
-        na += A.ta[i] >> 32;
-        nn += A.ta[i] & 0xffffffffull;
-    }
-    block_excl_scan64(na, sm, &t);
-    if (threadIdx.x == 0) A.tot->na = t;
-    __syncthreads();
-    block_excl_scan64(nn, sm, &t);
-    if (threadIdx.x == 0) A.tot->nn = t;
-    __syncthreads();
     const unsigned long long a = scan_row(A.ta, A.ntx), bx = scan_row(A.tb, A.ntx), by = scan_row(A.tb + A.ntx, A.nty);
     uint32_t u[4], c = 0;
 #pragma unroll
