@@ -590,24 +590,13 @@ __global__ void __launch_bounds__(256) k_lag_gemm_tc(const uint32_t *__restrict_
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * tcols));
 }
 
-// nmat row-major matrices (rows x cols) copied with rows_pad rows of cols_pad floats each
-// (padding zero); with lo != nullptr the TF32 hi part goes to out and the lo part to lo.
-__global__ void k_split_pad(const float *__restrict__ src, int64_t nmat, int rows, int cols, int rows_pad,
-                            int cols_pad, float *__restrict__ out, float *__restrict__ lo) {
-    int64_t n = nmat * rows_pad * (int64_t)cols_pad;
+// rows of cols floats copied into rows of cols_pad (padding zero)
+__global__ void k_pad_rows(const float *__restrict__ src, int64_t rows, int cols, int cols_pad, float *__restrict__ out) {
+    const int64_t n = rows * cols_pad;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t mat = i / ((int64_t)rows_pad * cols_pad);
-        int rem = (int)(i - mat * rows_pad * (int64_t)cols_pad);
-        int row = rem / cols_pad, col = rem - row * cols_pad;
-        float x = row < rows && col < cols ? src[(mat * rows + row) * (int64_t)cols + col] : 0.f;
-        if (lo) {
-            float h, l;
-            tf32_split(x, h, l);
-            out[i] = h;
-            lo[i] = l;
-        } else {
-            out[i] = x;
-        }
+        const int64_t row = i / cols_pad;
+        const int col = (int)(i - row * cols_pad);
+        out[i] = col < cols ? src[row * cols + col] : 0.f;
     }
 }
 
@@ -903,13 +892,6 @@ static void lagrange_points_r1(const ffm_plan_s *p, const FarLevel &F, const Lev
     }
 }
 
-void split_pad(const float *src, int64_t nmat, int rows, int cols, int rows_pad, int cols_pad, float *hi, float *lo,
-               cudaStream_t s) {  // lo == nullptr: padded copy into hi
-    int64_t n = nmat * rows_pad * (int64_t)cols_pad;
-    unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 16);
-    FFM_LAUNCH(k_split_pad, g, 256, 0, s, src, nmat, rows, cols, rows_pad, cols_pad, hi, lo);
-}
-
 // The tcgen05 transfer over row blocks of the operator: every launch takes rows [row0, row0 +
 // nb) of each T_t (nb <= 224, a multiple of 16, the blocks as even as possible) with the
 // whole K, and adds output columns row0 .. of v~.  T_t starts every tstride floats with rows
@@ -1203,7 +1185,8 @@ void lagrange_transfer(const ffm_plan_s *p, int l, const void *ut, int nrhs, voi
         if (F.aca_tc) {
             int64_t nrow = (int64_t)p->by[l].nb * nrhs;
             float *upad = tmp.get<float>((size_t)nrow * F.rkp);
-            split_pad((const float *)ut, 1, (int)nrow, r, (int)nrow, F.rkp, upad, nullptr, s);
+            const unsigned gp = (unsigned)std::min<int64_t>((nrow * F.rkp + 255) / 256, 152 * 16);
+            FFM_LAUNCH(k_pad_rows, gp, 256, 0, s, (const float *)ut, nrow, r, F.rkp, upad);
             tc_transfer(F, F.bt_src, F.pair_id, F.Bca, (int64_t)rp * F.rkp, rp, F.rkp, rp, nrhs, upad, w, p->dev_err,
                         p->wait_tries, s);
             tc_transfer(F, F.pair_id, F.bt_tgt, F.Aca, (int64_t)npad * rp, r, rp, r, nrhs, w, (float *)vt, p->dev_err,

@@ -357,10 +357,6 @@ bool far_lagrange(const ffm_plan_s *p, const void *q, int nrhs, float2 *accf, Al
 // one level's transfer alone, and the bytes of its u~ and v~ (v~ zeroed by the caller)
 void lagrange_transfer(const ffm_plan_s *p, int l, const void *ut, int nrhs, void *vt, Alloc &tmp, cudaStream_t s);
 void lagrange_bytes(const ffm_plan_s *p, int l, int nrhs, size_t *ub, size_t *vb);
-// nmat row-major matrices written with padded rows and columns (zeros): as TF32 hi / lo parts,
-// or (lo == nullptr) as a plain copy into hi
-void split_pad(const float *src, int64_t nmat, int rows, int cols, int rows_pad, int cols_pad, float *hi, float *lo,
-               cudaStream_t s);
 // true for the kinds whose transfer operators are the real Laplace G (Laplace, double layer)
 inline bool real_kernel(int kind) { return kind != FFM_HELMHOLTZ; }
 void far_planewave(const ffm_plan_s *p, int l, const float2 *q, int nrhs, double2 *acc, Alloc &tmp,

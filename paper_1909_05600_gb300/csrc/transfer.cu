@@ -3,11 +3,13 @@
 //
 // Split.  Every operand value x is written as hi + lo with hi = f16(x s) and lo = f16(x s - hi),
 // s a power of two, and a product is hi hi + hi lo + lo hi in FP32 accumulators.  Both
-// roundings are to nearest, so hi + lo carries 22 bits plus sign and the dropped lo lo term
-// is below 2^-24 of the product; the TF32 split used before truncated (hi: 11 bits, lo: 11 bits of
-// the rest), which is four to eight times coarser, and f16 runs at twice the TF32 rate.  The
-// scale keeps the largest value of a row between 2^13 and 2^14, so a value keeps its 22 bits
-// down to 2^-15 of its row's largest, and below that an absolute error of 2^-39 of it.
+// roundings are to nearest: |lo| is at most 2^-11 of the value, hi + lo is within 2^-22 of it, and the
+// dropped lo lo term is at most 2^-22 of the product (x = y = 1 + 2^-11 reach it; over random operands each of the
+// three is 2^-24.3 in the root mean square, and a row's sum of 216 products is off by 1e-8).  The TF32 split used
+// before truncated (hi: 11 bits, lo: 11 bits of the rest), which is four to eight times coarser, and f16
+// runs at twice the TF32 rate.  The scale keeps the largest value of a row between 2^13 and 2^14, so a
+// value keeps its 22 bits down to 2^-15 of its row's largest, and below that an absolute error of at most 2^-38
+// of it.
 //
 // Rows are split once per box (k_rows_split), the operators once per plan (k_op_image); both
 // are stored in the order in which the kernels copy them, so the transfer itself converts

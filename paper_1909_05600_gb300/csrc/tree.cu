@@ -1229,6 +1229,10 @@ static uint2 *build_chunks(ffm_plan_s *p, const uint32_t *list, int64_t n, const
 // to 5900 (many products) pairs per translation and wave of tiles.  Both sides, us: clustered 10M level 7
 // (68M pairs, 10 waves) 3520 / 6139, level 6 (11M, 2 waves) 709 / 1006, level 5 (1.4M, 1 wave)
 // 356 / 141; volume 2M level 5 (11.9M, 2 waves) 704 / 1087; sphere 2M level 7 (5.5M, 4 waves) 631 / 511.
+// Lower ranks take the same line: volume 2M, level 5, about 0.5 / 0.65 ms at r = 8 and 0.5 / 1.6 at r = 27 (from totals
+// over the levels).  Several right-hand sides multiply both sides, so a level that is over the line stays over it
+// (8 columns, all levels of a clustered 3M: 29.0 / 50.3 ms); one below it may be worth it for many columns, which
+// the plan does not know.
 static bool target_stationary_pays(const FarLevel &F) {
     const int64_t waves = (F.n_tgt + 128 * 152 - 1) / (128 * 152);
     return F.n_adm >= 4000 * (int64_t)F.n_trans * waves;
