@@ -28,8 +28,8 @@
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Calls return after
  *     enqueueing their work except where noted; ffm_plan synchronises its stream a
  *     few times (pair counts decide allocation sizes).
- *   - Sizes: at most 2^31 - 1 points in both sets together, and per level at most 2^32 - 1 near box pairs and
- *     2^32 - 1 admissible ones (more of the latter only where the target-stationary transfer takes the level, see
+ *   - Sizes: at most 2^31 - 1 points in both sets together, and per level at most 2^32 - 2^12 near box pairs and
+ *     2^32 - 2^12 admissible ones (more of the latter only where the target-stationary transfer takes the level, see
  *     lagrange_transfer); ffm_plan returns FFM_EUNSUPPORTED past these.
  *   - Functions return an ffm_status; no exception crosses the ABI.  On failure, output
  *     handles are set to NULL and ffm_last_error() describes the cause.

@@ -519,7 +519,7 @@ ffm_status ffm_plan_export(const ffm_plan_t *plan, int what, int level, void *ho
             const FarLevel &F = plan->far[level];
             *count = F.n_adm;
             if (!host_out || F.n_adm == 0) return;
-            if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs: the level has no list of them");
+            if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 2^12 admissible pairs: the level has no list of them");
             auto tgt = to_host(F.tgt, F.n_tgt, s);
             auto off = to_host(F.adm_off, F.n_tgt + 1, s);
             Alloc tmp;  // a level without pair lists gets them for this call

@@ -18,7 +18,9 @@ namespace ffm {
 
 constexpr int LMAX = 21;         // finest level of the Morton keys (3 x 21 bits)
 constexpr int R1MAX = 8;         // largest Chebyshev node count per axis
-constexpr int64_t MAX_LISTED = 0xffffffffll;  // pairs of a level that a list with 32-bit offsets holds
+// Pairs of a level that a list with 32-bit offsets holds.  4096 below 2^32: the kernels' 32-bit indices step past the end of a
+// list by up to a block's threads or a tile's pairs before they are compared with it, and must not wrap to its start.
+constexpr int64_t MAX_LISTED = 0xfffff000ll;
 constexpr int LAG_GEMM_BN = 32;  // pairs (GEMM columns) per tile of the Lagrange transfer
 constexpr int P2P_T = 128;        // threads per near-field block (the largest target chunk)
 constexpr int LAG_CHUNK = 512;    // points per block of the Lagrange point-wise kernels

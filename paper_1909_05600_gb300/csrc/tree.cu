@@ -1298,7 +1298,7 @@ __global__ void k_box_offsets(const uint32_t *__restrict__ tgt, const uint32_t *
 
 void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cudaStream_t s) {
     const FarLevel &F = p->far[l];
-    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs: the level has no list of them");
+    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 2^12 admissible pairs: the level has no list of them");
     Alloc tmp;
     tmp.stream = s;
     DescendArgs D{};
@@ -1333,7 +1333,7 @@ void fill_pair_lists(const ffm_plan_s *p, int l, uint32_t *src, uint32_t *t, cud
 void build_translation_groups(ffm_plan_s *p, int l, cudaStream_t s) {
     FarLevel &F = p->far[l];
     if (F.mode != 1 || F.n_adm == 0 || F.bt_off) return;
-    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs: the level has no list of them");
+    if (F.n_adm > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 2^12 admissible pairs: the level has no list of them");
     Alloc tmp;
     tmp.stream = s;
     if (!F.adm_src) {
@@ -1449,7 +1449,7 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
     FFM_CUDA(cudaStreamSynchronize(s));
     if (h.err) fail(FFM_ECUDA, "box translation outside the expected range");
     const int64_t na = (int64_t)h.na, nn = (int64_t)h.nn;
-    if (nn > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 near pairs at one level");
+    if (nn > MAX_LISTED) fail(FFM_EUNSUPPORTED, "more than 2^32 - 2^12 near pairs at one level");
     F.n_adm = na;
     p->info.n_adm[l] = na;
     const bool last = stop(nn);
@@ -1471,7 +1471,7 @@ static int64_t descend_level(ffm_plan_s *p, int l, DescendArgs D, Stop &&stop, N
         ts_first = ts_able && !root && F.tune_tc == 2;
     }
     if (na > MAX_LISTED && !ts_first)
-        fail(FFM_EUNSUPPORTED, "more than 2^32 - 1 admissible pairs at one level (only the target-stationary transfer "
+        fail(FFM_EUNSUPPORTED, "more than 2^32 - 2^12 admissible pairs at one level (only the target-stationary transfer "
                                "of the Laplace single layer does without a list of them)");
     if (na > 0 && !ts_first) {
         F.adm_src = p->mem.get<uint32_t>(na);
