@@ -283,14 +283,15 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(NearArgs N, const void *__restric
 // duplicated into both halves of a 64-bit register, and takes its sources four at a time
 // (one 16-byte shared load per array), so every arithmetic instruction is a packed f32x2
 // operation on two pairs: per coordinate the hi difference, the lo difference and their sum
-// ((x_hi - y_hi) + (x_lo - y_lo), exact in its hi part for nearby points), a multiply and two
-// fused multiply-adds for |x - y|^2, two hardware rsqrt, and one packed multiply-add into the
+// ((x_hi - y_hi) + (x_lo - y_lo), exact in its hi part for nearby points), three fused
+// multiply-adds for |x - y|^2 - tau^2, two hardware rsqrt, and one packed multiply-add into the
 // target's accumulator pair: 6.5 issue slots of FP32 arithmetic (13 FP32 operations) and one
 // special-function result per pair, against about 17 issue slots in the generic kernel.
 //
 // Coincident points: -tau^2 in the innermost multiply-add (where a multiply stood) leaves 0 or less, whose rsqrt
 // is +inf or NaN and makes the target's accumulator non-finite.  It changes no other pair: tau is at most 4e-9
-// of a leaf's edge at level 15.  (The third operand takes the kernel from 65.5 to 66.1 ms at 10M clustered points.)  Each thread checks its accumulators after every batch and recomputes that batch for the
+// of a leaf's edge at level 15.  (The third operand takes the kernel from 65.5 to 66.1 ms at 10M clustered
+// points.)  Each thread checks its accumulators after every batch and recomputes that batch for the
 // affected target with the pair test (pairs with |x - y|^2 - tau^2 below the smallest normal FP32
 // number contribute nothing, as in the generic kernel), starting again from the value it
 // had before the batch.
