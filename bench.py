@@ -350,8 +350,9 @@ def roofline(prof, info, steps, clk, pk, pk_kind, workload, nrhs=1):
     - NUFFT grid kernels: the FP32 pipe, 4 FLOP per complex x real multiply-add of a W^3
       kernel window (per direction and box, or per point).
     - Lagrange transfer: tensor cores, 2 r r_K FLOP per admissible pair (r_K = r, or 3 r for
-      the double layer's stacked component kernels; the single-precision GEMM; the TF32 hi/lo split triples the MMA work but not the algorithmic work), against
-      the measured BF16 peak times the nominal TF32/BF16 ratio (1.1 / 2.25).
+      the double layer's stacked component kernels, 8 r^2 for complex operators; the hi/lo split
+      triples the MMA work but not the algorithmic work), against the measured BF16 peak for the
+      transfers on f16 operands, times the nominal TF32/BF16 ratio (1.1 / 2.25) for those on TF32.
     - Plane-wave transforms of several right-hand sides on the tensor cores: 8 FLOP per
       (point, direction pair, right-hand side) (the real GEMMs P and Q over 2 columns per
       right-hand side), against the same TF32 peak.
